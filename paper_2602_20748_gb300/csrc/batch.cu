@@ -24,6 +24,7 @@
 #include "batch.h"
 #include "crpq.h"
 #include "device_common.cuh"
+#include "grid_barrier.cuh"
 #include "rpq_internal.h"
 
 namespace rpq {
@@ -123,37 +124,6 @@ __device__ __forceinline__ unsigned spill_reserve(unsigned long long *count, uns
   *at = first;
   if (first >= cap) return 0;
   return (unsigned)min((unsigned long long)chunks, cap - first);
-}
-
-__device__ bool bbarrier(BfsCtl *c, unsigned nblocks, u64 limit_ns) {
-  __shared__ unsigned stop;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    volatile unsigned *gen = &c->bar_gen;
-    unsigned g0 = *gen;
-    __threadfence();
-    unsigned arrived = atomicAdd(&c->bar_count, 1u);
-    if (arrived == nblocks - 1) {
-      atomicExch(&c->bar_count, 0u);
-      __threadfence();
-      atomicAdd(&c->bar_gen, 1u);
-    } else {
-      u64 t0 = globaltimer_ns();
-      unsigned spins = 0;
-      while (*gen == g0) {
-        __nanosleep(100);
-        if ((++spins & 63u) == 0 && globaltimer_ns() - t0 > limit_ns) {
-          atomicCAS(&c->err, 0u, (unsigned)(-RPQ_ERR_TIMEOUT));
-          break;
-        }
-        if (*(volatile unsigned *)&c->err) break;
-      }
-    }
-    __threadfence();
-    stop = *(volatile unsigned *)&c->err;
-  }
-  __syncthreads();
-  return stop == 0;
 }
 
 __device__ __forceinline__ u32 bdegsum(const BatchParams &p, const QueryDesc &qd, u32 q, u32 v) {
@@ -427,9 +397,10 @@ __device__ void bcommit(const BatchParams &p, int lp, u32 nxt, u64 *W, u64 *N, u
 
 __global__ void __launch_bounds__(BATCH_MAX_THREADS) batch_kernel(const __grid_constant__ BatchParams p) {
   BfsCtl *c = p.ctl;
+  unsigned epoch = 0;  // grid barriers passed
   u64 W = 0, N = 0, edges = 0, push_levels = 0;
   bseed(p, &W, &N);
-  if (!bbarrier(c, p.nblocks, p.time_limit_ns)) return;
+  if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
   u32 level = 0;
   for (;; level++) {
     const u32 cur = level % 3, nxt = (level + 1) % 3, old = (level + 2) % 3;
@@ -450,13 +421,13 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS) batch_kernel(const __grid_c
       push_levels++;
     }
     bpush(p, lp, cur, nxt, n_cur, &edges);
-    if (!bbarrier(c, p.nblocks, p.time_limit_ns)) return;
+    if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
     if (*(volatile unsigned long long *)&c->spill_count[cur] != 0) {
       bspill(p, lp, cur, nxt, &edges);
-      if (!bbarrier(c, p.nblocks, p.time_limit_ns)) return;
+      if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
     }
     bcommit(p, lp, nxt, &W, &N);
-    if (!bbarrier(c, p.nblocks, p.time_limit_ns)) return;
+    if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
   }
   W = warp_sum(W);
   N = warp_sum(N);
@@ -625,17 +596,18 @@ __device__ void serve_retire(const ServeParams &sp, u32 level) {
 __global__ void __launch_bounds__(BATCH_MAX_THREADS) serve_kernel(const __grid_constant__ ServeParams sp) {
   const BatchParams &p = sp.b;
   BfsCtl *c = p.ctl;
+  unsigned epoch = 0;  // grid barriers passed
   ServeState *st = sp.st;
   u64 W = 0, N = 0, edges = 0;
   if (blockIdx.x == 0 && threadIdx.x == 0) serve_decide(sp);
-  if (!bbarrier(c, p.nblocks, p.time_limit_ns)) return;
+  if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
   u32 level = 0;
   for (;; level++) {
     const u32 cur = level % 3, nxt = (level + 1) % 3, old = (level + 2) % 3;
     const int lp = level & 1;
     if (*(volatile unsigned *)&st->exit) break;
     serve_admit(sp, level, cur, lp, &W, &N);
-    if (!bbarrier(c, p.nblocks, p.time_limit_ns)) return;
+    if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
     u64 n_cur = *(volatile unsigned long long *)&c->n_list[cur];
     if (n_cur > p.list_cap) n_cur = p.list_cap;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
@@ -658,18 +630,18 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS) serve_kernel(const __grid_c
     }
     if (n_cur > 0) {
       bpush(p, lp, cur, nxt, n_cur, &edges);
-      if (!bbarrier(c, p.nblocks, p.time_limit_ns)) return;
+      if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
       if (*(volatile unsigned long long *)&c->spill_count[cur] != 0) {
         bspill(p, lp, cur, nxt, &edges);
-        if (!bbarrier(c, p.nblocks, p.time_limit_ns)) return;
+        if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
       }
       bcommit(p, lp, nxt, &W, &N, level + 1);
-      if (!bbarrier(c, p.nblocks, p.time_limit_ns)) return;
+      if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
     }
     serve_retire(sp, level);
-    if (!bbarrier(c, p.nblocks, p.time_limit_ns)) return;
+    if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
     if (blockIdx.x == 0 && threadIdx.x == 0) serve_decide(sp);
-    if (!bbarrier(c, p.nblocks, p.time_limit_ns)) return;
+    if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
   }
   W = warp_sum(W);
   N = warp_sum(N);

@@ -33,6 +33,7 @@
 // waits are bounded by a time limit (on expiry the kernel records
 // RPQ_ERR_TIMEOUT and returns).
 #include "device_common.cuh"
+#include "grid_barrier.cuh"
 #include "rpq_internal.h"
 
 namespace rpq {
@@ -109,41 +110,6 @@ __device__ __forceinline__ u32 popc_w(const Word<NW> &x) {
 template <int NW>
 __device__ __forceinline__ u64 widx(const BfsParams &p, u32 g, u32 q, u32 v) {
   return (((u64)q * p.n + v) * p.G + g) * NW;
-}
-
-// Grid-wide barrier for a cooperative launch.  Waits are bounded by the
-// deadline; on expiry the error word is set and every block returns at its
-// next check.  Returns false when the search must stop.
-__device__ bool grid_barrier(BfsCtl *c, unsigned nblocks, u64 limit_ns) {
-  __shared__ unsigned stop;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    volatile unsigned *gen = &c->bar_gen;
-    unsigned g0 = *gen;
-    __threadfence();
-    unsigned arrived = atomicAdd(&c->bar_count, 1u);
-    if (arrived == nblocks - 1) {
-      atomicExch(&c->bar_count, 0u);
-      __threadfence();
-      atomicAdd(&c->bar_gen, 1u);
-    } else {
-      u64 t0 = globaltimer_ns();
-      unsigned spins = 0;
-      while (*gen == g0) {
-        __nanosleep(100);
-        if ((++spins & 63u) == 0 && globaltimer_ns() - t0 > limit_ns) {
-          atomicCAS(&c->err, 0u, (unsigned)(-RPQ_ERR_TIMEOUT));
-          break;
-        }
-        if (*(volatile unsigned *)&c->err) break;
-      }
-    }
-    __threadfence();
-    stop = *(volatile unsigned *)&c->err;
-  }
-  __syncthreads();
-  // one reading per block, so all threads of a block take the same branch
-  return stop == 0;
 }
 
 // Automaton modes of a launch: one automaton for every lane, one per lane
@@ -1206,20 +1172,23 @@ __device__ void commit_phase(const BfsParams &p, int lp, u32 nxt, u64 n_cur, boo
 // Bytes a bottom-up level moves when the frontier holds the states `active`:
 // per target state with an active incoming transition, its visited words;
 // per such transition group, the row offsets and per in-edge a column id
-// and the gathered frontier words.
+// and the gathered frontier words.  An estimate in single precision: every
+// thread evaluates it at the start of every level, and in double precision it
+// took most of the 8 us between the end of one level's commit and the start of
+// the next (2 us now, the barrier).
 template <int NW>
-__device__ double pull_bytes(const BfsParams &p, u32 active) {
-  double b = 0;
-  const double wv = 8.0 * NW * p.G;
+__device__ float pull_bytes(const BfsParams &p, u32 active) {
+  float b = 0;
+  const float wv = 8.0f * NW * p.G, nf = (float)p.n;
   for (u32 q2 = 0; q2 < p.Q; q2++) {
     bool any = false;
     for (u32 j = p.q.in_begin[q2]; j < p.q.in_begin[q2 + 1]; j++) {
       const u32 f = p.q.in_from[j] & active, l = p.q.in_label[j];
       if (!f || l >= p.L) continue;
       any = true;
-      b += 8.0 * p.n + (double)p.label_edges[l] * (4.0 + wv * __popc(f));
+      b += 8.0f * nf + (float)p.label_edges[l] * (4.0f + wv * __popc(f));
     }
-    if (any) b += wv * p.n;
+    if (any) b += wv * nf;
   }
   return b;
 }
@@ -1231,10 +1200,11 @@ __global__ void __launch_bounds__(BFS_THREADS, 4) msbfs_kernel(const __grid_cons
 #pragma unroll
   for (int i = 0; i < ST_COUNT; i++) stat[i] = 0;
   BfsCtl *c = p.ctl;
+  unsigned epoch = 0;  // grid barriers passed
   const bool tracer = blockIdx.x == 0 && threadIdx.x == 0;
 
   seed_phase<NW, AM>(p, stat);
-  if (!grid_barrier(c, p.nblocks, p.time_limit_ns)) return;
+  if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
 
   u32 level = 0;
   for (;; level++) {
@@ -1244,8 +1214,8 @@ __global__ void __launch_bounds__(BFS_THREADS, 4) msbfs_kernel(const __grid_cons
     if (n_cur == 0) break;
     const u64 mf = *(volatile unsigned long long *)&c->mf[cur];
     const u32 active = *(volatile unsigned *)&c->smask[cur];
-    const double push_cost = (double)mf * (4.0 + 8.0 * NW) + (double)n_cur * (16.0 + 8.0 * NW);
-    const bool push = p.force == 1 || (p.force != 2 && (double)p.alpha * push_cost < pull_bytes<NW>(p, active));
+    const float push_cost = (float)mf * (4.0f + 8.0f * NW) + (float)n_cur * (16.0f + 8.0f * NW);
+    const bool push = p.force == 1 || (p.force != 2 && p.alpha * push_cost < pull_bytes<NW>(p, active));
     if (tracer) {
       // counters of the level after next start at zero
       c->n_list[old] = 0;
@@ -1269,10 +1239,10 @@ __global__ void __launch_bounds__(BFS_THREADS, 4) msbfs_kernel(const __grid_cons
     const u32 stamp = p.stamp_base + level + 2;  // the seeds used stamp_base + 1
     if (push) {
       push_level<NW, AM>(p, lp, cur, nxt, n_cur, stamp, stat);
-      if (!grid_barrier(c, p.nblocks, p.time_limit_ns)) return;
+      if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
       if (*(volatile unsigned long long *)&c->spill_count[cur] != 0) {
         spill_phase<NW>(p, lp, cur, nxt, stamp, stat);
-        if (!grid_barrier(c, p.nblocks, p.time_limit_ns)) return;
+        if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
       }
     } else {
       // a sparse frontier: test the frontier bitmap before each gather
@@ -1286,7 +1256,7 @@ __global__ void __launch_bounds__(BFS_THREADS, 4) msbfs_kernel(const __grid_cons
         pull_level<NW, true, AM>(p, lp, cur, nxt, active, stamp, bits, stat);
       else
         pull_level<NW, false, AM>(p, lp, cur, nxt, active, stamp, bits, stat);
-      if (!grid_barrier(c, p.nblocks, p.time_limit_ns)) return;
+      if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
     }
     {
       // bitmaps only where a bottom-up level may test them: a frontier with
@@ -1298,7 +1268,7 @@ __global__ void __launch_bounds__(BFS_THREADS, 4) msbfs_kernel(const __grid_cons
       if (tracer && level < (u32)TRACE_LEVELS) c->trace_c[level] = globaltimer_ns();
       commit_phase<NW, AM>(p, lp, nxt, n_cur, set_bits, clear_bits, stat);
     }
-    if (!grid_barrier(c, p.nblocks, p.time_limit_ns)) return;
+    if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
   }
   if (lane_id() == 0) {
 #pragma unroll

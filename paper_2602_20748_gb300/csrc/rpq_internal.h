@@ -102,8 +102,10 @@ constexpr unsigned int ERR_LIST_OVERFLOW = 1000u;   // BfsCtl::err: an append ra
 constexpr unsigned int APPEND_SEG = 128;             // list slots a warp reserves at a time
 
 struct BfsCtl {
-  unsigned int bar_count;
-  unsigned int bar_gen;
+  // grid barrier (grid_barrier.cuh): blocks that have arrived, over all
+  // barriers; the last barrier completed << 1 | error; a line each
+  alignas(128) unsigned int bar_count[32];
+  unsigned int bar_flag[32];
   unsigned int err;
   unsigned int err_where;
   unsigned long long n_list[3];
