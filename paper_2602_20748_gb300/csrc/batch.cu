@@ -25,6 +25,7 @@
 #include "crpq.h"
 #include "device_common.cuh"
 #include "grid_barrier.cuh"
+#include "push_split.cuh"
 #include "rpq_internal.h"
 
 namespace rpq {
@@ -112,20 +113,6 @@ __device__ __forceinline__ bool bad(const BatchParams &p, bool cond, unsigned wh
   return cond;
 }
 
-
-// Reserves up to `chunks` spill records with one atomic add and returns how
-// many of them fit below `cap` (their first index in *at).  Records below
-// the capacity are always written by their reserver, so the spill phase,
-// which reads min(count, cap) records, never reads one nobody wrote; the
-// chunks that do not fit are processed in place.
-__device__ __forceinline__ unsigned spill_reserve(unsigned long long *count, unsigned chunks, unsigned long long cap,
-                                                  unsigned long long *at) {
-  const unsigned long long first = atomicAdd(count, (unsigned long long)chunks);
-  *at = first;
-  if (first >= cap) return 0;
-  return (unsigned)min((unsigned long long)chunks, cap - first);
-}
-
 __device__ __forceinline__ u32 bdegsum(const BatchParams &p, const QueryDesc &qd, u32 q, u32 v) {
   u32 s = 0;
   for (u32 t = qd.out_begin[q]; t < qd.out_begin[q + 1]; t++) {
@@ -140,20 +127,21 @@ __device__ __forceinline__ u32 bdegsum(const BatchParams &p, const QueryDesc &qd
 // A warp's current run of reserved list slots [pos, end) (warp-uniform).
 struct BAppender {
   u64 pos = 0, end = 0;
+  u32 seg = 0;  // slots reserved at a time (0: exactly what is appended)
 };
 
 // Warp-aggregated append with a capacity check; a full list stops the search
 // with an error the host answers by splitting the batch.  The warp reserves
-// append_seg slots at a time with one atomic add (the list counter would
-// otherwise take one atomic per append from every warp); slots it does not
-// use hold NO_ENTRY (bappend_close).  Small lists use one atomic per append.
+// seg slots at a time with one atomic add (the list counter would otherwise
+// take one atomic per append from every warp); slots it does not use hold
+// NO_ENTRY (bappend_close).  Small lists use one atomic per append.
 __device__ __forceinline__ void bappend(const BatchParams &p, BAppender &a, bool take, u64 entry,
                                         unsigned long long *count, u64 *list) {
   const u32 b = __ballot_sync(FULL_MASK, take);
   if (!b) return;
   const u32 k = __popc(b), r = __popc(b & lanemask_lt());
   u64 at;
-  if (p.append_seg == 0) {
+  if (a.seg == 0) {
     u64 base = 0;
     if (lane_id() == __ffs(b) - 1) base = atomicAdd(count, (unsigned long long)k);
     at = __shfl_sync(FULL_MASK, base, __ffs(b) - 1) + r;
@@ -161,13 +149,13 @@ __device__ __forceinline__ void bappend(const BatchParams &p, BAppender &a, bool
     const u64 room = a.end - a.pos;
     u64 nb = 0;
     if (k > room) {
-      if (lane_id() == 0) nb = atomicAdd(count, (unsigned long long)p.append_seg);
+      if (lane_id() == 0) nb = atomicAdd(count, (unsigned long long)a.seg);
       nb = __shfl_sync(FULL_MASK, nb, 0);
     }
     at = r < room ? a.pos + r : nb + (r - room);
     if (k > room) {
       a.pos = nb + (k - room);
-      a.end = nb + p.append_seg;
+      a.end = nb + a.seg;
     } else {
       a.pos += k;
     }
@@ -218,6 +206,7 @@ __device__ __forceinline__ bool bvisit(const BatchParams &p, u32 i, u32 q2, u32 
 __device__ void bseed(const BatchParams &p, u64 *W, u64 *N) {
   const u64 stride = (u64)gridDim.x * blockDim.x;
   BAppender app;
+  u64 mf = 0;
   for (u64 base = (u64)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); base < p.nq; base += stride) {
     u64 i = base + lane_id();
     bool take = false;
@@ -228,6 +217,7 @@ __device__ void bseed(const BatchParams &p, u64 *W, u64 *N) {
       if (take) {
         const u32 d = bdegsum(p, p.qd[i], 0, s);
         *W += d;
+        mf += d;
         *N += 1;
         if (p.qn) {
           p.qn[i] = 1;
@@ -238,21 +228,26 @@ __device__ void bseed(const BatchParams &p, u64 *W, u64 *N) {
     bappend(p, app, take, bentry((u32)i, 0, s), &p.ctl->n_list[0], p.list0);
   }
   bappend_close(p, app, p.list0);
+  mf = warp_sum(mf);
+  if (lane_id() == 0 && mf) atomicAdd(&p.ctl->mf[0], mf);
 }
 
-__device__ void bpush(const BatchParams &p, int lp, u32 cur, u32 nxt, u64 n_cur, u64 *edges) {
+__device__ void bpush(const BatchParams &p, int lp, u32 cur, u32 nxt, u64 n_cur, u32 grab, u32 chunk, u32 seg,
+                      u64 *edges) {
   const u64 *list = lp ? p.list1 : p.list0;
   u64 *nlist = lp ? p.list0 : p.list1;
   const u32 lane = lane_id();
   BAppender app;
+  app.seg = seg;
   for (;;) {
     u64 base = 0;
-    if (lane == 0) base = atomicAdd(&p.ctl->cursor[cur], 32ull);
+    if (lane == 0) base = atomicAdd(&p.ctl->cursor[cur], (unsigned long long)grab);
     base = __shfl_sync(FULL_MASK, base, 0);
     if (base >= n_cur) break;
     const u64 idx = base + lane;
-    u64 e = idx < n_cur ? __ldcg(&list[idx]) : NO_ENTRY;
+    u64 e = lane < grab && idx < n_cur ? __ldcg(&list[idx]) : NO_ENTRY;
     const bool present = e != NO_ENTRY;
+    if (!__any_sync(FULL_MASK, present)) continue;
     if (!present) e = 0;
     const u32 i = (u32)(e >> 37), q = (u32)(e >> 32) & 31u, v = (u32)e;
     bool valid = present && !bad(p, i >= p.nq || v >= p.n, 10);
@@ -274,19 +269,27 @@ __device__ void bpush(const BatchParams &p, int lp, u32 cur, u32 nxt, u64 n_cur,
           if (bad(p, (u64)rbeg + rlen > p.m, 6)) rlen = 0;
         }
       }
-      if (rlen > SPILL_EDGES) {
-        const u32 chunks = (rlen + SPILL_EDGES - 1) / SPILL_EDGES;
+      // long rows, one at a time: the warp writes a row's chunk records together
+      for (u32 big = __ballot_sync(FULL_MASK, rlen > chunk); big; big &= big - 1) {
+        const u32 o = __ffs(big) - 1;
+        const u32 o_beg = __shfl_sync(FULL_MASK, rbeg, o), o_len = __shfl_sync(FULL_MASK, rlen, o);
+        const u32 o_i = __shfl_sync(FULL_MASK, i, o), o_q2 = __shfl_sync(FULL_MASK, q2, o);
         u64 at = 0;
-        const u32 fit = spill_reserve(&p.ctl->spill_count[cur], chunks, p.spill_cap, &at);
-        for (u32 c = 0; c < fit; c++) {
+        u32 fit = 0;
+        if (lane == 0) fit = spill_reserve(&p.ctl->spill_count[cur], (o_len + chunk - 1) / chunk, p.spill_cap, &at);
+        at = __shfl_sync(FULL_MASK, at, 0);
+        fit = __shfl_sync(FULL_MASK, fit, 0);
+        for (u32 c = lane; c < fit; c += 32) {
           u64 *rec = p.spill + (at + c) * 2;
-          rec[0] = bentry(i, q2, 0) | (rbeg + c * SPILL_EDGES);
-          rec[1] = min(SPILL_EDGES, rlen - c * SPILL_EDGES);
+          rec[0] = bentry(o_i, o_q2, 0) | (o_beg + c * chunk);
+          rec[1] = min(chunk, o_len - c * chunk);
         }
         // the chunks that did not fit stay with this warp
-        const u32 moved = min(rlen, fit * SPILL_EDGES);
-        rbeg += moved;
-        rlen -= moved;
+        if (lane == o) {
+          const u32 moved = min(rlen, fit * chunk);
+          rbeg += moved;
+          rlen -= moved;
+        }
       }
       u32 pre = rlen;
 #pragma unroll
@@ -322,11 +325,12 @@ __device__ void bpush(const BatchParams &p, int lp, u32 cur, u32 nxt, u64 n_cur,
   bappend_close(p, app, nlist);
 }
 
-__device__ void bspill(const BatchParams &p, int lp, u32 cur, u32 nxt, u64 *edges) {
+__device__ void bspill(const BatchParams &p, int lp, u32 cur, u32 nxt, u32 seg, u64 *edges) {
   u64 *nlist = lp ? p.list0 : p.list1;
   const u32 lane = lane_id();
   const u64 count = min(*(volatile unsigned long long *)&p.ctl->spill_count[cur], (unsigned long long)p.spill_cap);
   BAppender app;
+  app.seg = seg;
   for (;;) {
     u64 r = 0;
     if (lane == 0) r = atomicAdd(&p.ctl->spill_cursor[cur], 1ull);
@@ -356,6 +360,7 @@ __device__ void bcommit(const BatchParams &p, int lp, u32 nxt, u64 *W, u64 *N, u
   u64 n_next = *(volatile unsigned long long *)&p.ctl->n_list[nxt];
   if (n_next > p.list_cap) n_next = p.list_cap;
   const u64 stride = (u64)gridDim.x * blockDim.x;
+  u64 mf = 0;  // out-edges of the next frontier
   for (u64 j0 = (u64)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); j0 < n_next; j0 += stride) {
     const u64 j = j0 + lane_id();
     bool ok = j < n_next;
@@ -374,6 +379,7 @@ __device__ void bcommit(const BatchParams &p, int lp, u32 nxt, u64 *W, u64 *N, u
       if (ok && p.active) p.active[i] = stamp;
     }
     *W += d;
+    mf += d;
     *N += ok ? 1 : 0;
     if (p.qn) {
       // per-query counters; the entries of a warp usually share one query
@@ -393,6 +399,8 @@ __device__ void bcommit(const BatchParams &p, int lp, u32 nxt, u64 *W, u64 *N, u
       }
     }
   }
+  mf = warp_sum(mf);
+  if (lane_id() == 0 && mf) atomicAdd(&p.ctl->mf[nxt], mf);
 }
 
 __global__ void __launch_bounds__(BATCH_MAX_THREADS) batch_kernel(const __grid_constant__ BatchParams p) {
@@ -408,9 +416,13 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS) batch_kernel(const __grid_c
     u64 n_cur = *(volatile unsigned long long *)&c->n_list[cur];
     if (n_cur > p.list_cap) n_cur = p.list_cap;
     if (n_cur == 0) break;
+    const u64 mf = *(volatile unsigned long long *)&c->mf[cur];
+    const u64 n_warps = (u64)p.nblocks * (blockDim.x >> 5);
+    const u32 seg = mf < PUSH_EXACT ? 0u : p.append_seg;
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       c->n_list[old] = 0;
       c->cursor[old] = 0;
+      c->mf[old] = 0;
       c->spill_count[old] = 0;
       c->spill_cursor[old] = 0;
       if (level < (u32)TRACE_LEVELS) {
@@ -420,10 +432,10 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS) batch_kernel(const __grid_c
       }
       push_levels++;
     }
-    bpush(p, lp, cur, nxt, n_cur, &edges);
+    bpush(p, lp, cur, nxt, n_cur, push_grab(n_cur, n_warps), spill_chunk(mf, n_warps), seg, &edges);
     if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
     if (*(volatile unsigned long long *)&c->spill_count[cur] != 0) {
-      bspill(p, lp, cur, nxt, &edges);
+      bspill(p, lp, cur, nxt, seg, &edges);
       if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
     }
     bcommit(p, lp, nxt, &W, &N);
@@ -507,6 +519,7 @@ __device__ void serve_admit(const ServeParams &sp, u32 level, u32 cur, int lp, u
   const u64 nwarps = ((u64)gridDim.x * blockDim.x) >> 5;
   u64 *list = lp ? p.list1 : p.list0;
   BAppender app;
+  app.seg = p.append_seg;
   // warp-uniform loop: every lane of a warp takes the same requests
   for (u64 w = warp; w < k; w += nwarps) {
     const ServeReq *rq = sp.reqs + ((head + w) & (u64)(sp.ring - 1));
@@ -629,10 +642,12 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS) serve_kernel(const __grid_c
       }
     }
     if (n_cur > 0) {
-      bpush(p, lp, cur, nxt, n_cur, &edges);
+      // admissions between levels add out-edges that no commit counted: the longest chunks
+      bpush(p, lp, cur, nxt, n_cur, push_grab(n_cur, (u64)p.nblocks * (blockDim.x >> 5)), SPILL_EDGES, p.append_seg,
+            &edges);
       if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
       if (*(volatile unsigned long long *)&c->spill_count[cur] != 0) {
-        bspill(p, lp, cur, nxt, &edges);
+        bspill(p, lp, cur, nxt, p.append_seg, &edges);
         if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
       }
       bcommit(p, lp, nxt, &W, &N, level + 1);

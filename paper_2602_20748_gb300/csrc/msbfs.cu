@@ -34,6 +34,7 @@
 // RPQ_ERR_TIMEOUT and returns).
 #include "device_common.cuh"
 #include "grid_barrier.cuh"
+#include "push_split.cuh"
 #include "rpq_internal.h"
 
 namespace rpq {
@@ -177,35 +178,25 @@ __device__ __forceinline__ u32 la_degsum(const BfsParams &p, u32 q, u32 v, u32 g
   return s;
 }
 
-// Reserves up to `chunks` spill records with one atomic add and returns how
-// many of them fit below `cap` (their first index in *at).  Records below
-// the capacity are always written by their reserver, so the spill phase,
-// which reads min(count, cap) records, never reads one nobody wrote; the
-// chunks that do not fit are processed in place.
-__device__ __forceinline__ unsigned spill_reserve(unsigned long long *count, unsigned chunks, unsigned long long cap,
-                                                  unsigned long long *at) {
-  const unsigned long long first = atomicAdd(count, (unsigned long long)chunks);
-  *at = first;
-  if (first >= cap) return 0;
-  return (unsigned)min((unsigned long long)chunks, cap - first);
-}
-
-// A warp's current run of reserved list slots [pos, end) (warp-uniform).
+// A warp's current run of reserved list slots [pos, end) (warp-uniform) and
+// how many it reserves at a time in this phase (0: exactly what it appends).
 struct Appender {
   u64 pos = 0, end = 0;
+  u32 seg = 0;
 };
 
 // Warp-aggregated append of `entry` for the lanes with `take` set.  All 32
 // lanes must call it.  With segments, the warp fills its reserved slots and
-// reserves APPEND_SEG more with one atomic add when they run out, so the
-// list counter sees one atomic per segment instead of one per append.
+// reserves seg more with one atomic add when they run out, so the list
+// counter sees one atomic per segment instead of one per append; slots left
+// over are read (and skipped) by the next level and the commit.
 __device__ __forceinline__ void warp_append(const BfsParams &p, Appender &a, bool take, u64 entry,
                                             unsigned long long *count, u64 *list) {
   const u32 b = __ballot_sync(FULL_MASK, take);
   if (!b) return;
   const u32 k = __popc(b), r = __popc(b & lanemask_lt());
   u64 at;
-  if (p.append_seg == 0) {
+  if (a.seg == 0) {
     u64 base = 0;
     if (lane_id() == __ffs(b) - 1) base = atomicAdd(count, (unsigned long long)k);
     base = __shfl_sync(FULL_MASK, base, __ffs(b) - 1);
@@ -214,13 +205,13 @@ __device__ __forceinline__ void warp_append(const BfsParams &p, Appender &a, boo
     const u64 room = a.end - a.pos;
     u64 nb = 0;
     if (k > room) {
-      if (lane_id() == 0) nb = atomicAdd(count, (unsigned long long)p.append_seg);
+      if (lane_id() == 0) nb = atomicAdd(count, (unsigned long long)a.seg);
       nb = __shfl_sync(FULL_MASK, nb, 0);
     }
     at = r < room ? a.pos + r : nb + (r - room);
     if (k > room) {
       a.pos = nb + (k - room);
-      a.end = nb + p.append_seg;
+      a.end = nb + a.seg;
     } else {
       a.pos += k;
     }
@@ -301,6 +292,7 @@ __device__ void seed_phase(const BfsParams &p, u64 *stat) {
     if (mf) atomicAdd(&p.ctl->stats[ST_GROUP_W], mf);
     if (gx) atomicAdd(&p.ctl->stats[ST_GROUP_X], gx);
     if (mf) atomicAdd(&p.ctl->mf[0], mf);
+    if (gn) atomicAdd(&p.ctl->n_true[0], gn);
   }
   if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&p.ctl->smask[0], 1u);
 }
@@ -329,12 +321,13 @@ __device__ __forceinline__ bool relax(const BfsParams &p, u64 *FB, u32 tgq, u32 
   }
 }
 
-// Top-down expansion of the entries of the current list.  A warp takes 32
+// Top-down expansion of the entries of the current list.  A warp takes `grab`
 // entries at a time and spreads the edges of their rows evenly over its lanes
 // (prefix sum of row lengths, owner found by binary search); rows longer than
-// SPILL_EDGES are queued in chunks for the spill sub-phase.
+// `chunk` are queued in chunks for the spill sub-phase.
 template <int NW, int AM>
-__device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_cur, u32 stamp, u64 *stat) {
+__device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_cur, u32 grab, u32 chunk, u32 seg,
+                           u32 stamp, u64 *stat) {
   const u64 *list = lp ? p.list1 : p.list0;
   u64 *nlist = lp ? p.list0 : p.list1;
   const u64 *F = lp ? p.fr1 : p.fr0;
@@ -343,14 +336,16 @@ __device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_c
   const u32 lane = lane_id();
   u64 edges = 0, rows = 0, entries = 0;
   Appender app;
+  app.seg = seg;
   for (;;) {
     u64 base = 0;
-    if (lane == 0) base = atomicAdd(&p.ctl->cursor[cur], 32ull);
+    if (lane == 0) base = atomicAdd(&p.ctl->cursor[cur], (unsigned long long)grab);
     base = __shfl_sync(FULL_MASK, base, 0);
     if (base >= n_cur) break;
     u64 idx = base + lane;
-    u64 e = idx < n_cur ? __ldcg(&list[idx]) : NO_ENTRY;
+    u64 e = lane < grab && idx < n_cur ? __ldcg(&list[idx]) : NO_ENTRY;
     bool valid = e != NO_ENTRY;
+    if (!__any_sync(FULL_MASK, valid)) continue;
     if (!valid) e = 0;
     u32 gq = (u32)(e >> 32), v = (u32)e;
     u32 g = gq / Q, q = gq - g * Q;
@@ -394,21 +389,32 @@ __device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_c
           rows++;
         }
       }
-      if (p.spill && rlen > SPILL_EDGES) {
-        const u32 chunks = (rlen + SPILL_EDGES - 1) / SPILL_EDGES;
-        u64 at = 0;
-        const u32 fit = spill_reserve(&p.ctl->spill_count[cur], chunks, p.spill_cap, &at);
-        for (u32 c = 0; c < fit; c++) {
-          u64 *rec = p.spill + (at + c) * (2 + NW);
-          rec[0] = ((u64)tgq << 32) | (rbeg + c * SPILL_EDGES);
-          rec[1] = min(SPILL_EDGES, rlen - c * SPILL_EDGES);
+      // long rows, one at a time: the warp writes a row's chunk records together
+      for (u32 big = __ballot_sync(FULL_MASK, p.spill && rlen > chunk); big; big &= big - 1) {
+        const u32 o = __ffs(big) - 1;
+        const u32 o_beg = __shfl_sync(FULL_MASK, rbeg, o), o_len = __shfl_sync(FULL_MASK, rlen, o);
+        const u32 o_gq = __shfl_sync(FULL_MASK, tgq, o);
+        Word<NW> ofm;
 #pragma unroll
-          for (int t = 0; t < NW; t++) rec[2 + t] = fmt.w[t];
+        for (int i = 0; i < NW; i++) ofm.w[i] = __shfl_sync(FULL_MASK, fmt.w[i], o);
+        u64 at = 0;
+        u32 fit = 0;
+        if (lane == 0) fit = spill_reserve(&p.ctl->spill_count[cur], (o_len + chunk - 1) / chunk, p.spill_cap, &at);
+        at = __shfl_sync(FULL_MASK, at, 0);
+        fit = __shfl_sync(FULL_MASK, fit, 0);
+        for (u32 c = lane; c < fit; c += 32) {
+          u64 *rec = p.spill + (at + c) * (2 + NW);
+          rec[0] = ((u64)o_gq << 32) | (o_beg + c * chunk);
+          rec[1] = min(chunk, o_len - c * chunk);
+#pragma unroll
+          for (int t = 0; t < NW; t++) rec[2 + t] = ofm.w[t];
         }
         // the chunks that did not fit stay with this warp
-        const u32 moved = min(rlen, fit * SPILL_EDGES);
-        rbeg += moved;
-        rlen -= moved;
+        if (lane == o) {
+          const u32 moved = min(rlen, fit * chunk);
+          rbeg += moved;
+          rlen -= moved;
+        }
       }
       // exclusive prefix of row lengths across the warp
       u32 pre = rlen;
@@ -459,13 +465,14 @@ __device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_c
 
 // The queued chunks of long rows: a warp per chunk, taken dynamically.
 template <int NW>
-__device__ void spill_phase(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 stamp, u64 *stat) {
+__device__ void spill_phase(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 seg, u32 stamp, u64 *stat) {
   u64 *nlist = lp ? p.list0 : p.list1;
   u64 *FB = lp ? p.fr0 : p.fr1;
   const u32 lane = lane_id();
   const u64 count = min(*(volatile unsigned long long *)&p.ctl->spill_count[cur], (unsigned long long)p.spill_cap);
   u64 edges = 0;
   Appender app;
+  app.seg = seg;
   for (;;) {
     u64 r = 0;
     if (lane == 0) r = atomicAdd(&p.ctl->spill_cursor[cur], 1ull);
@@ -668,6 +675,8 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
   const u64 gword = 8ull * NW * p.G;  // bytes of the G words of one (state, vertex)
   u64 edges = 0, words = 0, bytes = 0;
   Appender app;
+  // small graphs: shorter segments, so that unused slots do not outnumber the entries
+  app.seg = (u64)n * Q * p.G >= n_warps * 2 * APPEND_SEG ? p.append_seg : min(p.append_seg, 32u);
   // lane mode by source state: this warp's per-target accumulators
   u64 *lane_acc = nullptr;
   if constexpr (AM == AM_LANE) {
@@ -1165,6 +1174,7 @@ __device__ void commit_phase(const BfsParams &p, int lp, u32 nxt, u64 n_cur, boo
     if (mf) atomicAdd(&p.ctl->stats[ST_GROUP_W], mf);
     if (gx) atomicAdd(&p.ctl->stats[ST_GROUP_X], gx);
     if (mf) atomicAdd(&p.ctl->mf[nxt], mf);
+    if (gv) atomicAdd(&p.ctl->n_true[nxt], gv);
     if (states) atomicOr(&p.ctl->smask[nxt], states);
   }
 }
@@ -1214,13 +1224,15 @@ __global__ void __launch_bounds__(BFS_THREADS, 4) msbfs_kernel(const __grid_cons
     if (n_cur == 0) break;
     const u64 mf = *(volatile unsigned long long *)&c->mf[cur];
     const u32 active = *(volatile unsigned *)&c->smask[cur];
-    const float push_cost = (float)mf * (4.0f + 8.0f * NW) + (float)n_cur * (16.0f + 8.0f * NW);
+    const u64 n_true = *(volatile unsigned long long *)&c->n_true[cur];
+    const float push_cost = (float)mf * (4.0f + 8.0f * NW) + (float)n_true * (16.0f + 8.0f * NW);
     const bool push = p.force == 1 || (p.force != 2 && p.alpha * push_cost < pull_bytes<NW>(p, active));
     if (tracer) {
       // counters of the level after next start at zero
       c->n_list[old] = 0;
       c->cursor[old] = 0;
       c->mf[old] = 0;
+      c->n_true[old] = 0;
       c->spill_count[old] = 0;
       c->spill_cursor[old] = 0;
       c->heavy_cursor[old] = 0;
@@ -1238,10 +1250,13 @@ __global__ void __launch_bounds__(BFS_THREADS, 4) msbfs_kernel(const __grid_cons
     }
     const u32 stamp = p.stamp_base + level + 2;  // the seeds used stamp_base + 1
     if (push) {
-      push_level<NW, AM>(p, lp, cur, nxt, n_cur, stamp, stat);
+      const u64 n_warps = (u64)p.nblocks * (BFS_THREADS / 32);
+      const u32 seg = mf < PUSH_EXACT ? 0u : p.append_seg;
+      push_level<NW, AM>(p, lp, cur, nxt, n_cur, push_grab(n_cur, n_warps), spill_chunk(mf, n_warps), seg, stamp,
+                         stat);
       if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
       if (*(volatile unsigned long long *)&c->spill_count[cur] != 0) {
-        spill_phase<NW>(p, lp, cur, nxt, stamp, stat);
+        spill_phase<NW>(p, lp, cur, nxt, seg, stamp, stat);
         if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
       }
     } else {

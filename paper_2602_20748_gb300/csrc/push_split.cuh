@@ -1,0 +1,46 @@
+// How a top-down level is split over the warps, for the bit-sliced and the
+// batched engine.
+#pragma once
+
+#include "device_common.cuh"
+#include "rpq_internal.h"
+
+namespace rpq {
+
+// Reserves up to `chunks` spill records with one atomic add and returns how
+// many of them fit below `cap` (their first index in *at).  Records below
+// the capacity are always written by their reserver, so the spill phase,
+// which reads min(count, cap) records, never reads one nobody wrote; the
+// chunks that do not fit are processed in place.
+__device__ __forceinline__ unsigned spill_reserve(unsigned long long *count, unsigned chunks, unsigned long long cap,
+                                                  unsigned long long *at) {
+  const unsigned long long first = atomicAdd(count, (unsigned long long)chunks);
+  *at = first;
+  if (first >= cap) return 0;
+  return (unsigned)min((unsigned long long)chunks, cap - first);
+}
+
+// Chunk length of a top-down level whose frontier has mf out-edges: long rows
+// are cut so that every warp gets about one chunk, within [SPILL_EDGES_MIN,
+// SPILL_EDGES].  A fixed 1,024 left a level of 36,830 edges from a hundred
+// entries to the four warps that held them (496 us on R-MAT 2^20, one source).
+__device__ __forceinline__ u32 spill_chunk(u64 mf, u64 n_warps) {
+  u32 s = SPILL_EDGES_MIN;
+  while (s < SPILL_EDGES && (u64)s * n_warps < mf) s <<= 1;
+  return s;
+}
+
+// Entries a warp takes at a time: 32 while every warp gets some, fewer for
+// short lists, down to one warp per entry.
+__device__ __forceinline__ u32 push_grab(u64 n_cur, u64 n_warps) {
+  u32 e = 32;
+  while (e > 1 && n_cur < n_warps * e) e >>= 1;
+  return e;
+}
+
+// List slots a warp reserves at a time in a top-down level of mf edges: below
+// PUSH_EXACT edges the appends are few enough for an atomic each, and the
+// lists stay free of unused slots, which the next level would read.
+constexpr u64 PUSH_EXACT = 1ull << 16;
+
+}  // namespace rpq

@@ -111,6 +111,7 @@ struct BfsCtl {
   unsigned long long n_list[3];
   unsigned long long cursor[3];
   unsigned long long mf[3];
+  unsigned long long n_true[3];        // frontier entries without the lists' unused slots
   unsigned long long spill_count[3];   // top-down row chunks queued this level
   unsigned long long spill_cursor[3];
   unsigned long long heavy_cursor[3];  // bottom-up row chunks taken
@@ -126,9 +127,11 @@ struct BfsCtl {
   unsigned long long trace_c[TRACE_LEVELS];   // start time (ns) of each level's commit phase
 };
 
-// A top-down row longer than SPILL_EDGES is cut into chunks of SPILL_EDGES
-// edges that all warps share in a sub-phase of the level.
+// A top-down row longer than the level's chunk length (at most SPILL_EDGES
+// edges, see spill_chunk) is cut into chunks that all warps share in a
+// sub-phase of the level.
 constexpr unsigned int SPILL_EDGES = 1024;
+constexpr unsigned int SPILL_EDGES_MIN = 64;
 constexpr unsigned long long SPILL_CAP = 1ull << 18;  // chunks per level
 
 struct BfsParams {
