@@ -1302,12 +1302,13 @@ bool serve_engine_graphed(ServeEngine *e) { return e->graph != nullptr; }
 int batch_run(rpq_ctx *ctx, const rpq_graph *g, uint32_t nq, const rpq_query *const *queries,
               const uint32_t *sources, bool materialize, const BatchTuning &tun, BatchOut *out) {
   const double t_start = host_seconds();
-  if (out->per_query && !materialize && tun.direct && tun.lanes > 0) {
+  const bool direct = out->per_query && !materialize && tun.direct && tun.lanes > 0;
+  if (direct) {
     // every query to the lane-mode launches
     out->qstats.assign(3ull * nq, 0);
     for (uint32_t i = 0; i < nq; i++) out->evicted_idx.push_back(i);
   }
-  for (uint32_t b0 = 0; b0 < nq && out->evicted_idx.empty();) {
+  for (uint32_t b0 = 0; b0 < nq && !direct;) {
     uint32_t k = std::min<uint32_t>(tun.queries_per_launch, nq - b0);
     for (;;) {
       int rc = batch_launch(ctx, g, b0, k, queries + b0, sources + b0, materialize, tun, out);

@@ -80,6 +80,22 @@ def test_batch_split_when_frontier_list_is_small(er):
     assert np.array_equal(got, oracle_batch_rows(og, regexes, sources))
 
 
+def test_split_batch_with_evictions_answers_every_query(er, monkeypatch):
+    # 1,200 seeds do not fit 1,024 list slots, so the batch is split; queries of its first part are evicted
+    monkeypatch.setenv("RPQ_BATCH_LIST_CAP", "1024")
+    c2 = rpq.Context(device=0)
+    rpq.rpq_set_option(c2, "batch_evict", 20)
+    g0, og, src = er
+    s0, d0, l0 = synth.er_graph(1000, 5000, 4, seed=synth.BASE_SEED + 3)
+    g = rpq.load_graph(c2, 1000, 4, s0, d0, l0)
+    regexes, sources = synth.batch_queries(1200, 4, 1.2, src, 1000, seed=48)
+    r = rpq.run_rpq_batch(c2, g, [rpq.compile_rpq(c2, x) for x in regexes], sources, flags=rpq.RPQ_PER_QUERY)
+    assert rpq.result_stats(r)["bfs_launches"] > 2 and rpq.result_stats(r)["evicted"] > 0
+    for i, (rx, s) in enumerate(zip(regexes, sources)):
+        want = oracle.pair_digest(oracle.rpq(og, rx, sources=[int(s)]).rows)
+        assert rpq.result_query_stats(r, i) == want, (i, rx, int(s))
+
+
 def test_batch_autotune_and_edge_cases(ctx, er):
     g, og, src = er
     regexes, sources = synth.batch_queries(100, 4, 1.2, src, 1000, seed=53)
