@@ -239,12 +239,9 @@ __device__ void bpush(const BatchParams &p, int lp, u32 cur, u32 nxt, u64 n_cur,
   const u32 lane = lane_id();
   BAppender app;
   app.seg = seg;
-  for (;;) {
-    u64 base = 0;
-    if (lane == 0) base = atomicAdd(&p.ctl->cursor[cur], (unsigned long long)grab);
-    base = __shfl_sync(FULL_MASK, base, 0);
-    if (base >= n_cur) break;
-    const u64 idx = base + lane;
+  Items it(grid_warp(), grid_warps(), grab);
+  for (; it.at < n_cur; it.next(&p.ctl->cursor[cur])) {
+    const u64 idx = it.at + lane;
     u64 e = lane < grab && idx < n_cur ? __ldcg(&list[idx]) : NO_ENTRY;
     const bool present = e != NO_ENTRY;
     if (!__any_sync(FULL_MASK, present)) continue;
@@ -331,11 +328,9 @@ __device__ void bspill(const BatchParams &p, int lp, u32 cur, u32 nxt, u32 seg, 
   const u64 count = min(*(volatile unsigned long long *)&p.ctl->spill_count[cur], (unsigned long long)p.spill_cap);
   BAppender app;
   app.seg = seg;
-  for (;;) {
-    u64 r = 0;
-    if (lane == 0) r = atomicAdd(&p.ctl->spill_cursor[cur], 1ull);
-    r = __shfl_sync(FULL_MASK, r, 0);
-    if (r >= count) break;
+  Items it(grid_warp(), grid_warps(), 1);
+  for (; it.at < count; it.next(&p.ctl->spill_cursor[cur])) {
+    const u64 r = it.at;
     const u64 h = __ldcg(p.spill + 2 * r);
     const u32 len = (u32)__ldcg(p.spill + 2 * r + 1);
     const u32 i = (u32)(h >> 37), q2 = (u32)(h >> 32) & 31u, b = (u32)h;

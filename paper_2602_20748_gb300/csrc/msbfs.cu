@@ -337,12 +337,9 @@ __device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_c
   u64 edges = 0, rows = 0, entries = 0;
   Appender app;
   app.seg = seg;
-  for (;;) {
-    u64 base = 0;
-    if (lane == 0) base = atomicAdd(&p.ctl->cursor[cur], (unsigned long long)grab);
-    base = __shfl_sync(FULL_MASK, base, 0);
-    if (base >= n_cur) break;
-    u64 idx = base + lane;
+  Items it(grid_warp(), grid_warps(), grab);
+  for (; it.at < n_cur; it.next(&p.ctl->cursor[cur])) {
+    u64 idx = it.at + lane;
     u64 e = lane < grab && idx < n_cur ? __ldcg(&list[idx]) : NO_ENTRY;
     bool valid = e != NO_ENTRY;
     if (!__any_sync(FULL_MASK, valid)) continue;
@@ -473,12 +470,9 @@ __device__ void spill_phase(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 se
   u64 edges = 0;
   Appender app;
   app.seg = seg;
-  for (;;) {
-    u64 r = 0;
-    if (lane == 0) r = atomicAdd(&p.ctl->spill_cursor[cur], 1ull);
-    r = __shfl_sync(FULL_MASK, r, 0);
-    if (r >= count) break;
-    const u64 *rec = p.spill + r * (2 + NW);
+  Items it(grid_warp(), grid_warps(), 1);
+  for (; it.at < count; it.next(&p.ctl->spill_cursor[cur])) {
+    const u64 *rec = p.spill + it.at * (2 + NW);
     const u64 h = __ldcg(rec);
     const u32 tgq = (u32)(h >> 32), b = (u32)h;
     const u32 len = (u32)__ldcg(rec + 1);
@@ -669,8 +663,11 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
   const u32 lane_off = li * PER;
   const u32 my_g = lane_on ? lane_off / NW : 0;
   const u64 wpv = (u64)p.G * NW;
-  const u64 warp = ((u64)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const u64 n_warps = ((u64)gridDim.x * blockDim.x) >> 5;
+  const u64 warp = grid_warp(), n_warps = grid_warps();
+  // vertices a warp takes at a time: 32, fewer (but no fewer than it works on
+  // at once) on graphs too small to give every warp two such chunks
+  u32 cv = 32;
+  while (cv > VPW && n < 2 * n_warps * cv) cv >>= 1;
   const bool chunked = p.hchunk != nullptr;
   const u64 gword = 8ull * NW * p.G;  // bytes of the G words of one (state, vertex)
   u64 edges = 0, words = 0, bytes = 0;
@@ -684,7 +681,7 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
     lane_acc = s_lane_acc[threadIdx.x >> 5];
   }
 
-  // A warp takes 32 consecutive vertices at a time: lane i first finds, with
+  // A warp takes cv consecutive vertices at a time: lane i first finds, with
   // coalesced reads of the in-row offsets, the target states into which
   // vertex c0 + i has a light in-row on an active transition; only those
   // (vertex, state) pairs are then visited, VPW vertices at a time (their
@@ -692,13 +689,9 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
   // a cursor (the level's list cursor, unused by bottom-up levels), so a
   // warp whose chunks had little work takes more of them; else chunk k goes
   // to warp k mod warps.
-  u64 c0 = warp * 32;
-  if (p.pull_dynamic) {
-    u64 t = 0;
-    if (lane == 0) t = atomicAdd(&p.ctl->cursor[cur], 32ull);
-    c0 = __shfl_sync(FULL_MASK, t, 0);
-  }
-  for (; c0 < n;) {
+  Items vit(warp, n_warps, cv);
+  for (; vit.at < n;) {
+    const u64 c0 = vit.at;
     // hmask: states with a long in-row (its chunks also produce); with a
     // sparse frontier (bits), lane i also tests up to PRESCAN in-edges of
     // its own vertex against the frontier bitmap, so that a state none of
@@ -707,7 +700,7 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
     // no hit yet -- the sub-warp tests the rest of them below
     constexpr u32 PRESCAN = 16;
     u32 qmask = 0, hmask = 0, tmask = 0;
-    if (c0 + lane < n) {
+    if (lane < cv && c0 + lane < n) {
       const u32 v = (u32)(c0 + lane);
       for (u32 q2 = 0; q2 < Q; q2++)
         for (u32 j = p.q.in_begin[q2]; j < p.q.in_begin[q2 + 1]; j++) {
@@ -923,13 +916,10 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
                            vis, acc);
     }
     }
-    if (p.pull_dynamic) {
-      u64 t = 0;
-      if (lane == 0) t = atomicAdd(&p.ctl->cursor[cur], 32ull);
-      c0 = __shfl_sync(FULL_MASK, t, 0);
-    } else {
-      c0 += n_warps * 32;
-    }
+    if (p.pull_dynamic)
+      vit.next(&p.ctl->cursor[cur]);
+    else
+      vit.at += n_warps * cv;
   }
 
   bool chunks_done = !chunked;
@@ -942,10 +932,8 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
       u64 lact = 0;  // labels with an active transition
       for (u32 j = 0; j < p.q.in_begin[Q]; j++)
         if ((p.q.in_from[j] & active) && p.q.in_label[j] < p.L) lact |= 1ull << p.q.in_label[j];
-      for (;;) {
-        u64 it = 0;
-        if (lane == 0) it = atomicAdd(&p.ctl->heavy_cursor[cur], 1ull);
-        it = __shfl_sync(FULL_MASK, it, 0);
+      for (Items hit(warp, n_warps, 1);; hit.next(&p.ctl->heavy_cursor[cur])) {
+        const u64 it = hit.at;
         u64 acc_base = 0, ci = 0;
         u32 ls = 0;
         bool found = false;
@@ -1033,10 +1021,8 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
     }
   }
   if (!chunks_done) {
-    for (;;) {
-      u64 it = 0;
-      if (lane == 0) it = atomicAdd(&p.ctl->heavy_cursor[cur], 1ull);
-      it = __shfl_sync(FULL_MASK, it, 0);
+    for (Items hit(warp, n_warps, 1);; hit.next(&p.ctl->heavy_cursor[cur])) {
+      const u64 it = hit.at;
       // map the item number to (target state, transition group, chunk)
       u64 acc_base = 0, ci = 0;
       u32 q2s = 0, from = 0, ls = 0, js = 0;

@@ -43,4 +43,25 @@ __device__ __forceinline__ u32 push_grab(u64 n_cur, u64 n_warps) {
 // lists stay free of unused slots, which the next level would read.
 constexpr u64 PUSH_EXACT = 1ull << 16;
 
+__device__ __forceinline__ u64 grid_warp() { return ((u64)blockIdx.x * blockDim.x + threadIdx.x) >> 5; }
+__device__ __forceinline__ u64 grid_warps() { return ((u64)gridDim.x * blockDim.x) >> 5; }
+
+// Work items of a phase, `step` consecutive ones at a time: a warp's first
+// item is its own (warp * step), the next ones come from the phase's cursor.
+// Phases with fewer items than warps touch no cursor: the 4,864 warps of a
+// full grid asking one counter for nothing took 8-10 us.
+struct Items {
+  u64 at;        // first item of the current grab
+  u64 n_first;   // items handed out by warp number
+  u32 step;
+  __device__ __forceinline__ Items(u64 warp, u64 n_warps, u32 step_)
+      : at(warp * step_), n_first(n_warps * step_), step(step_) {}
+  // warp-uniform; all lanes call it
+  __device__ __forceinline__ void next(unsigned long long *cursor) {
+    u64 t = 0;
+    if (lane_id() == 0) t = atomicAdd(cursor, (unsigned long long)step);
+    at = n_first + __shfl_sync(FULL_MASK, t, 0);
+  }
+};
+
 }  // namespace rpq
