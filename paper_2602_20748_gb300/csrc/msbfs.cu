@@ -324,9 +324,10 @@ __device__ __forceinline__ bool relax(const BfsParams &p, u64 *FB, u32 tgq, u32 
 // Top-down expansion of the entries of the current list.  A warp takes `grab`
 // entries at a time and spreads the edges of their rows evenly over its lanes
 // (prefix sum of row lengths, owner found by binary search); rows longer than
-// `chunk` are queued in chunks for the spill sub-phase.
+// `chunk` are queued in chunks for the spill sub-phase.  n_warps: the warps
+// that share the level, those of the grid or of block 0 alone.
 template <int NW, int AM>
-__device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_cur, u32 grab, u32 chunk, u32 seg,
+__device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_cur, u64 n_warps, u32 chunk, u32 seg,
                            u32 stamp, u64 *stat) {
   const u64 *list = lp ? p.list1 : p.list0;
   u64 *nlist = lp ? p.list0 : p.list1;
@@ -337,7 +338,8 @@ __device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_c
   u64 edges = 0, rows = 0, entries = 0;
   Appender app;
   app.seg = seg;
-  Items it(grid_warp(), grid_warps(), grab);
+  const u32 grab = push_grab(n_cur, n_warps);
+  Items it(grid_warp(), n_warps, grab);
   for (; it.at < n_cur; it.next(&p.ctl->cursor[cur])) {
     u64 idx = it.at + lane;
     u64 e = lane < grab && idx < n_cur ? __ldcg(&list[idx]) : NO_ENTRY;
@@ -1087,15 +1089,15 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
 // set_bits: the next frontier may be sparse enough for bottom-up levels to
 // test its bitmap, so its bits are set; clear_bits: this level's bits were set.
 template <int NW, int AM>
-__device__ void commit_phase(const BfsParams &p, int lp, u32 nxt, u64 n_cur, bool set_bits, bool clear_bits,
-                             u64 *stat) {
+__device__ void commit_phase(const BfsParams &p, int lp, u32 nxt, u64 n_cur, u64 n_warps, bool set_bits,
+                             bool clear_bits, u64 *stat) {
   const u64 *list = lp ? p.list1 : p.list0;
   const u64 *nlist = lp ? p.list0 : p.list1;
   u64 *F = lp ? p.fr1 : p.fr0;
   const u64 *FB = lp ? p.fr0 : p.fr1;
   const u32 Q = p.Q;
   const u64 n_next = *(volatile unsigned long long *)&p.ctl->n_list[nxt];
-  const u64 stride = (u64)gridDim.x * blockDim.x;
+  const u64 stride = n_warps * 32;
   const u64 tid = (u64)blockIdx.x * blockDim.x + threadIdx.x;
   u64 W = 0, N = 0, mf = 0, gv = 0, gx = 0;
   u32 states = 0;
@@ -1189,6 +1191,16 @@ __device__ float pull_bytes(const BfsParams &p, u32 active) {
   return b;
 }
 
+// Levels of at most SOLO_SLOTS list slots and SOLO_EDGES out-edges are run by
+// block 0 alone, with __syncthreads between the phases: a level is then the
+// latency of its loads and atomics (7-8 us for a handful of entries), where
+// the grid pays two more barriers and the wake-up of 4,864 warps (17-19 us).
+// Above 512 edges the block's eight warps take longer than that.  The other
+// blocks wait at a grid barrier, for at most SOLO_RUN levels at a time, so
+// that no wait comes near the time limit.
+constexpr u64 SOLO_SLOTS = 512, SOLO_EDGES = 512;
+constexpr u32 SOLO_RUN = 64;
+
 template <int NW, int AM>
 __global__ void __launch_bounds__(BFS_THREADS, 4) msbfs_kernel(const __grid_constant__ BfsParams p) {
   // per-warp statistics, summed into the control block at the end
@@ -1202,7 +1214,7 @@ __global__ void __launch_bounds__(BFS_THREADS, 4) msbfs_kernel(const __grid_cons
   seed_phase<NW, AM>(p, stat);
   if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
 
-  u32 level = 0;
+  u32 level = 0, run = 0;  // run: levels left of block 0's run, 0 outside one
   for (;; level++) {
     const u32 cur = level % 3, nxt = (level + 1) % 3, old = (level + 2) % 3;
     const int lp = level & 1;
@@ -1211,8 +1223,20 @@ __global__ void __launch_bounds__(BFS_THREADS, 4) msbfs_kernel(const __grid_cons
     const u64 mf = *(volatile unsigned long long *)&c->mf[cur];
     const u32 active = *(volatile unsigned *)&c->smask[cur];
     const u64 n_true = *(volatile unsigned long long *)&c->n_true[cur];
+    const bool solo = n_cur <= SOLO_SLOTS && mf <= SOLO_EDGES && p.force != 2;
+    if (solo && run == 0) {
+      // every block has read this level's counters before block 0 goes on
+      if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
+      if (blockIdx.x != 0) {
+        if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
+        level = *(volatile unsigned *)&c->next_level - 1;
+        continue;
+      }
+      run = SOLO_RUN;
+    }
     const float push_cost = (float)mf * (4.0f + 8.0f * NW) + (float)n_true * (16.0f + 8.0f * NW);
-    const bool push = p.force == 1 || (p.force != 2 && p.alpha * push_cost < pull_bytes<NW>(p, active));
+    const bool push =
+        solo || p.force == 1 || (p.force != 2 && p.alpha * push_cost < pull_bytes<NW>(p, active));
     if (tracer) {
       // counters of the level after next start at zero
       c->n_list[old] = 0;
@@ -1235,15 +1259,20 @@ __global__ void __launch_bounds__(BFS_THREADS, 4) msbfs_kernel(const __grid_cons
         stat[ST_PULL_LEVELS] += 1;
     }
     const u32 stamp = p.stamp_base + level + 2;  // the seeds used stamp_base + 1
-    if (push) {
-      const u64 n_warps = (u64)p.nblocks * (BFS_THREADS / 32);
+    const u64 n_warps = (run ? 1ull : (u64)p.nblocks) * (BFS_THREADS / 32);
+    if (mf == 0) {
+      // no out-edges: the next frontier is empty, only this one is cleared
+    } else if (push) {
       const u32 seg = mf < PUSH_EXACT ? 0u : p.append_seg;
-      push_level<NW, AM>(p, lp, cur, nxt, n_cur, push_grab(n_cur, n_warps), spill_chunk(mf, n_warps), seg, stamp,
-                         stat);
-      if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
-      if (*(volatile unsigned long long *)&c->spill_count[cur] != 0) {
-        spill_phase<NW>(p, lp, cur, nxt, seg, stamp, stat);
+      push_level<NW, AM>(p, lp, cur, nxt, n_cur, n_warps, run ? ~0u : spill_chunk(mf, n_warps), seg, stamp, stat);
+      if (run) {
+        __syncthreads();
+      } else {
         if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
+        if (*(volatile unsigned long long *)&c->spill_count[cur] != 0) {
+          spill_phase<NW>(p, lp, cur, nxt, seg, stamp, stat);
+          if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
+        }
       }
     } else {
       // a sparse frontier: test the frontier bitmap before each gather
@@ -1267,7 +1296,17 @@ __global__ void __launch_bounds__(BFS_THREADS, 4) msbfs_kernel(const __grid_cons
       const bool set_bits = p.fbits && n_next * 4 < sparse_cap;
       const bool clear_bits = p.fbits && (level == 0 || n_cur * 4 < sparse_cap);
       if (tracer && level < (u32)TRACE_LEVELS) c->trace_c[level] = globaltimer_ns();
-      commit_phase<NW, AM>(p, lp, nxt, n_cur, set_bits, clear_bits, stat);
+      commit_phase<NW, AM>(p, lp, nxt, n_cur, n_warps, set_bits, clear_bits, stat);
+      if (run) {
+        __syncthreads();
+        const u64 mf_next = *(volatile unsigned long long *)&c->mf[nxt];
+        if (--run == 0 || n_next == 0 || n_next > SOLO_SLOTS || mf_next > SOLO_EDGES) {
+          run = 0;
+          if (tracer) c->next_level = level + 1;
+          if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
+        }
+        continue;
+      }
     }
     if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
   }

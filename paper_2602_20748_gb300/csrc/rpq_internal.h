@@ -116,6 +116,7 @@ struct BfsCtl {
   unsigned long long spill_cursor[3];
   unsigned long long heavy_cursor[3];  // bottom-up row chunks taken
   unsigned int smask[3];               // DFA states present in each frontier
+  unsigned int next_level;             // first level after a run of one-block levels
   unsigned long long levels;
   unsigned long long stats[ST_COUNT];
   // per-level trace (first TRACE_LEVELS levels): start time (ns), frontier
