@@ -490,7 +490,8 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
     p.list1 = w.list1;
     p.ctl = ctx->ctl;
     p.stamp_base = ctx->stamp;
-    p.nblocks = (unsigned)blocks;
+    const int grid = bfs_grid(blocks, nw, Gb, n);
+    p.nblocks = (unsigned)grid;
     p.force = force;
     p.alpha = ctx->alpha;
     p.pull_dynamic = ctx->pull_dynamic;
@@ -501,7 +502,7 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
     CK(launch_vis_init(nw, p, w.empty, ctx->stream));
     CK(cudaMemsetAsync(ctx->ctl, 0, sizeof(BfsCtl), ctx->stream));
     CK(cudaEventRecord(ctx->ev[0], ctx->stream));
-    CK(launch_msbfs(nw, p, blocks, BFS_THREADS_HOST, ctx->stream));
+    CK(launch_msbfs(nw, p, grid, BFS_THREADS_HOST, ctx->stream));
     CK(cudaEventRecord(ctx->ev[1], ctx->stream));
     res->stats.launches += 3;
     res->stats.bfs_launches += 1;
@@ -1785,7 +1786,8 @@ int rpq_lane_stats_multi(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Mu
   p.list_cap = w.list_cap;
   p.ctl = ctx->ctl;
   p.stamp_base = ctx->stamp;
-  p.nblocks = (unsigned)blocks;
+  const int grid = bfs_grid(blocks, 1, G, n);
+  p.nblocks = (unsigned)grid;
   p.force = 0;
   p.alpha = ctx->alpha;
   p.pull_dynamic = ctx->pull_dynamic;
@@ -1806,7 +1808,7 @@ int rpq_lane_stats_multi(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Mu
   BfsCtl hctl;
   std::vector<uint64_t> hls(3ull * G * 64);
   if ((e = launch_vis_init(1, p, w.empty, st)) == cudaSuccess && (e = cudaMemsetAsync(ctx->ctl, 0, sizeof(BfsCtl), st)) == cudaSuccess &&
-      (e = cudaEventRecord(ctx->ev[0], st)) == cudaSuccess && (e = launch_msbfs_multi(p, blocks, BFS_THREADS_HOST, st)) == cudaSuccess &&
+      (e = cudaEventRecord(ctx->ev[0], st)) == cudaSuccess && (e = launch_msbfs_multi(p, grid, BFS_THREADS_HOST, st)) == cudaSuccess &&
       (e = cudaEventRecord(ctx->ev[1], st)) == cudaSuccess && (e = launch_emit_lane_stats(1, ep, ls, st)) == cudaSuccess &&
       (e = cudaEventRecord(ctx->ev[2], st)) == cudaSuccess)
     e = cudaMemcpyAsync(&hctl, ctx->ctl, sizeof(BfsCtl), cudaMemcpyDeviceToHost, st);
@@ -1982,6 +1984,13 @@ static int lane_launch(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Lane
     }
   }
   grp_begin[Q] = (uint16_t)grp.size();
+  std::vector<uint32_t> sl((size_t)Q * L, 0);
+  if (Q <= 8)
+    for (uint32_t q = 0; q < Q; q++)
+      for (uint32_t t = out_begin[q]; t < out_begin[q + 1]; t++) {
+        uint32_t &e = sl[(size_t)q * L + (trans[t] & 0xFFFFu)];
+        e = (e >> 16 ? e : t) | 1u << (16 + (trans[t] >> 16));
+      }
   if (grp.empty()) {  // no transition: keep the buffers non-empty
     grp.push_back(0xFFFFu);
     gmask.assign(GW, 0);
@@ -1992,7 +2001,7 @@ static int lane_launch(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Lane
   const size_t o_mask = 0, o_fin = o_mask + al(mask.size() * 8), o_emp = o_fin + al(fin.size() * 8),
                o_ob = o_emp + al(empty_q.size() * 8), o_tr = o_ob + al(b_ob), o_it = o_tr + al(b_tr),
                o_gm = o_it + al(b_it), o_gb = o_gm + al(gmask.size() * 8), o_gr = o_gb + al(grp_begin.size() * 2),
-               o_ls = o_gr + al(grp.size() * 4), tbytes = o_ls + al(24ull * G * K);
+               o_sl = o_gr + al(grp.size() * 4), o_ls = o_sl + al(sl.size() * 4), tbytes = o_ls + al(24ull * G * K);
   std::vector<unsigned char> host(o_ls);
   std::memcpy(host.data() + o_mask, mask.data(), mask.size() * 8);
   std::memcpy(host.data() + o_fin, fin.data(), fin.size() * 8);
@@ -2003,6 +2012,7 @@ static int lane_launch(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Lane
   std::memcpy(host.data() + o_gm, gmask.data(), gmask.size() * 8);
   std::memcpy(host.data() + o_gb, grp_begin.data(), grp_begin.size() * 2);
   std::memcpy(host.data() + o_gr, grp.data(), grp.size() * 4);
+  std::memcpy(host.data() + o_sl, sl.data(), sl.size() * 4);
   unsigned char *dt = nullptr;
   if ((rc = dalloc(ctx, &dt, tbytes))) return rc;
   cudaStream_t st = ctx->stream;
@@ -2042,7 +2052,8 @@ static int lane_launch(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Lane
   p.list_cap = w.list_cap;
   p.ctl = ctx->ctl;
   p.stamp_base = ctx->stamp;
-  p.nblocks = (unsigned)blocks;
+  const int grid = bfs_grid(blocks, nw, G, n);
+  p.nblocks = (unsigned)grid;
   p.force = 0;
   p.alpha = ctx->alpha;
   p.pull_dynamic = ctx->pull_dynamic;
@@ -2056,6 +2067,7 @@ static int lane_launch(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Lane
   p.la_in_t = reinterpret_cast<const unsigned short *>(dt + o_it);
   p.la_grp_begin = reinterpret_cast<const unsigned short *>(dt + o_gb);
   p.la_grp = reinterpret_cast<const unsigned int *>(dt + o_gr);
+  p.la_sl = reinterpret_cast<const unsigned int *>(dt + o_sl);
   p.la_gmask = reinterpret_cast<const unsigned long long *>(dt + o_gm);
   EmitParams ep{};
   ep.vis = w.vis;
@@ -2071,7 +2083,7 @@ static int lane_launch(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Lane
   if ((e = launch_vis_init_lane(nw, p, reinterpret_cast<const u64 *>(dt + o_emp), st)) == cudaSuccess &&
       (e = cudaMemsetAsync(ctx->ctl, 0, sizeof(BfsCtl), st)) == cudaSuccess &&
       (e = cudaEventRecord(ctx->ev[0], st)) == cudaSuccess &&
-      (e = launch_msbfs_lane(nw, p, blocks, BFS_THREADS_HOST, st)) == cudaSuccess &&
+      (e = launch_msbfs_lane(nw, p, grid, BFS_THREADS_HOST, st)) == cudaSuccess &&
       (e = cudaEventRecord(ctx->ev[1], st)) == cudaSuccess && (e = launch_emit_lane_stats(nw, ep, ls, st)) == cudaSuccess &&
       (e = cudaEventRecord(ctx->ev[2], st)) == cudaSuccess)
     e = rb_queue(ctx, 0, ctx->ctl, sizeof(BfsCtl));

@@ -239,9 +239,8 @@ __device__ void bpush(const BatchParams &p, int lp, u32 cur, u32 nxt, u64 n_cur,
   const u32 lane = lane_id();
   BAppender app;
   app.seg = seg;
-  Items it(grid_warp(), grid_warps(), grab);
-  for (; it.at < n_cur; it.next(&p.ctl->cursor[cur])) {
-    const u64 idx = it.at + lane;
+  for (u64 it = grid_warp() * grab; it < n_cur; it = next_item(&p.ctl->cursor[cur], grid_warps(), grab)) {
+    const u64 idx = it + lane;
     u64 e = lane < grab && idx < n_cur ? __ldcg(&list[idx]) : NO_ENTRY;
     const bool present = e != NO_ENTRY;
     if (!__any_sync(FULL_MASK, present)) continue;
@@ -328,9 +327,7 @@ __device__ void bspill(const BatchParams &p, int lp, u32 cur, u32 nxt, u32 seg, 
   const u64 count = min(*(volatile unsigned long long *)&p.ctl->spill_count[cur], (unsigned long long)p.spill_cap);
   BAppender app;
   app.seg = seg;
-  Items it(grid_warp(), grid_warps(), 1);
-  for (; it.at < count; it.next(&p.ctl->spill_cursor[cur])) {
-    const u64 r = it.at;
+  for (u64 r = grid_warp(); r < count; r = next_item(&p.ctl->spill_cursor[cur], grid_warps(), 1)) {
     const u64 h = __ldcg(p.spill + 2 * r);
     const u32 len = (u32)__ldcg(p.spill + 2 * r + 1);
     const u32 i = (u32)(h >> 37), q2 = (u32)(h >> 32) & 31u, b = (u32)h;

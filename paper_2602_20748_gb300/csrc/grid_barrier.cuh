@@ -21,8 +21,10 @@ namespace rpq {
 // is set and the block returns false.  An error recorded by any block before
 // the barrier makes it return false in every block: the releasing block hands
 // the error out with the epoch, so all threads of the grid take the same
-// branch.
-__device__ __forceinline__ bool grid_sync(BfsCtl *c, unsigned nblocks, unsigned &epoch, u64 limit_ns) {
+// branch.  before(): run by thread 0 when the block's other threads have
+// arrived, before the block does.
+template <typename F>
+__device__ __forceinline__ bool grid_sync(BfsCtl *c, unsigned nblocks, unsigned &epoch, u64 limit_ns, F before) {
   __shared__ unsigned s_go;
   epoch++;
   __syncthreads();
@@ -30,6 +32,7 @@ __device__ __forceinline__ bool grid_sync(BfsCtl *c, unsigned nblocks, unsigned 
     volatile unsigned *flag = &c->bar_flag[0];
     const unsigned want = epoch << 1;  // counter and epoch may wrap: compared for equality only
     unsigned go;
+    before();
     __threadfence();
     if (atomicAdd(&c->bar_count[0], 1u) + 1u == epoch * nblocks) {
       __threadfence();
@@ -57,6 +60,10 @@ __device__ __forceinline__ bool grid_sync(BfsCtl *c, unsigned nblocks, unsigned 
   }
   __syncthreads();
   return (s_go & 1u) == 0;
+}
+
+__device__ __forceinline__ bool grid_sync(BfsCtl *c, unsigned nblocks, unsigned &epoch, u64 limit_ns) {
+  return grid_sync(c, nblocks, epoch, limit_ns, [] {});
 }
 
 }  // namespace rpq

@@ -113,9 +113,10 @@ __device__ __forceinline__ u64 widx(const BfsParams &p, u32 g, u32 q, u32 v) {
   return (((u64)q * p.n + v) * p.G + g) * NW;
 }
 
-// Automaton modes of a launch: one automaton for every lane, one per lane
-// group (multi), or one per lane (lane mode).
-constexpr int AM_ONE = 0, AM_GROUP = 1, AM_LANE = 2;
+// Automaton modes of a launch: one automaton for every lane (of one lane
+// group, or of several), one per lane group (multi), or one per lane (lane
+// mode).
+constexpr int AM_ONE = 0, AM_GROUP = 1, AM_LANE = 2, AM_MANY = 3;
 // Lane-mode bottom-up by source state (see pull_level) for unions of at most
 // this many states; larger ones gather per target state.
 constexpr u32 LANE_SRC_Q = 8;
@@ -178,6 +179,10 @@ __device__ __forceinline__ u32 la_degsum(const BfsParams &p, u32 q, u32 v, u32 g
   return s;
 }
 
+// List entries are (group * Q + state) << 32 | vertex; this bit marks one that
+// the bottom-up phase that produced it has committed.
+constexpr u64 ENTRY_DONE = 1ull << 63;
+
 // A warp's current run of reserved list slots [pos, end) (warp-uniform) and
 // how many it reserves at a time in this phase (0: exactly what it appends).
 struct Appender {
@@ -229,6 +234,11 @@ __device__ __forceinline__ void append_close(const BfsParams &p, Appender &a, u6
   for (u64 i = a.pos + lane_id(); i < a.end; i += 32)
     if (i < p.list_cap) list[i] = NO_ENTRY;
   a.pos = a.end = 0;
+}
+
+// Adds v (the same in every lane) to one of the warp's statistics.
+__device__ __forceinline__ void stat_add(u64 *stat, int i, u64 v) {
+  if (lane_id() == 0) stat[i] += v;
 }
 
 template <int NW, int AM>
@@ -287,9 +297,6 @@ __device__ void seed_phase(const BfsParams &p, u64 *stat) {
   if (lane_id() == 0) {
     stat[ST_W] += W;
     stat[ST_N] += N;
-    stat[ST_GROUP_VERTICES] += gn;
-    // counted once per warp and phase: straight into the control block
-    if (mf) atomicAdd(&p.ctl->stats[ST_GROUP_W], mf);
     if (gx) atomicAdd(&p.ctl->stats[ST_GROUP_X], gx);
     if (mf) atomicAdd(&p.ctl->mf[0], mf);
     if (gn) atomicAdd(&p.ctl->n_true[0], gn);
@@ -297,17 +304,25 @@ __device__ void seed_phase(const BfsParams &p, u64 *stat) {
   if (blockIdx.x == 0 && threadIdx.x == 0) atomicOr(&p.ctl->smask[0], 1u);
 }
 
-// One top-down relaxation of edge (tgq, w) with source lanes fm: the lanes
-// not yet visited at (tgq, w) are OR-ed into the next frontier word; returns
-// whether this thread must list (tgq, w) in the next frontier.
+// Target of a top-down row: state and group, packed as in the rows' shared
+// records (relax runs once per edge and would pay a division to unpack a list
+// entry's group * Q + state).
+__device__ __forceinline__ u32 pack_target(u32 q2, u32 g) { return q2 << 16 | g; }
+__device__ __forceinline__ u64 target_entry(const BfsParams &p, u32 tg, u32 w) {
+  return (u64)((tg & 0xFFFFu) * p.Q + (tg >> 16)) << 32 | w;
+}
+
+// One top-down relaxation of an edge to (target tg, w) with source lanes fm:
+// the lanes not yet visited there are OR-ed into the next frontier word;
+// returns whether this thread must list the target in the next frontier.
 template <int NW>
-__device__ __forceinline__ bool relax(const BfsParams &p, u64 *FB, u32 tgq, u32 w, const Word<NW> &fm, u32 stamp) {
-  const u32 g = tgq / p.Q, q2 = tgq - g * p.Q;
+__device__ __forceinline__ bool relax(const BfsParams &p, u64 *FB, u32 tg, u32 w, const u64 *fm, u32 stamp) {
+  const u32 g = tg & 0xFFFFu, q2 = tg >> 16;
   const u64 wi = widx<NW>(p, g, q2, w);
   Word<NW> vis = load_cg<NW>(p.vis + wi);
   Word<NW> m;
 #pragma unroll
-  for (int i = 0; i < NW; i++) m.w[i] = fm.w[i] & ~vis.w[i];
+  for (int i = 0; i < NW; i++) m.w[i] = fm[i] & ~vis.w[i];
   if (!any_bits(m)) return false;
   if constexpr (NW == 1) {
     u64 old = atomicOr((unsigned long long *)(FB + wi), m.w[0]);
@@ -325,10 +340,18 @@ __device__ __forceinline__ bool relax(const BfsParams &p, u64 *FB, u32 tgq, u32 
 // entries at a time and spreads the edges of their rows evenly over its lanes
 // (prefix sum of row lengths, owner found by binary search); rows longer than
 // `chunk` are queued in chunks for the spill sub-phase.  n_warps: the warps
-// that share the level, those of the grid or of block 0 alone.
+// that share the level, those of the grid or of block 0 alone.  The entries'
+// frontier words and the rows' targets are kept in the warp's shared scratch:
+// an edge reads its owner's with three loads instead of ten shuffles, and the
+// words do not sit in registers through the edge loop.
 template <int NW, int AM>
 __device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_cur, u64 n_warps, u32 chunk, u32 seg,
-                           u32 stamp, u64 *stat) {
+                           u32 stamp, u64 *scratch, u64 *stat) {
+  // scratch: [32][NW] words of the entries, in lane mode [32][NW] of them
+  // masked by the row's transition, [32] (first edge - prefix, target)
+  u64 *s_fm = scratch + lane_id() * NW;
+  u64 *s_words = AM == AM_LANE ? scratch + 32 * NW : scratch;
+  uint2 *s_row = reinterpret_cast<uint2 *>(s_words + 32 * NW);
   const u64 *list = lp ? p.list1 : p.list0;
   u64 *nlist = lp ? p.list0 : p.list1;
   const u64 *F = lp ? p.fr1 : p.fr0;
@@ -339,19 +362,16 @@ __device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_c
   Appender app;
   app.seg = seg;
   const u32 grab = push_grab(n_cur, n_warps);
-  Items it(grid_warp(), n_warps, grab);
-  for (; it.at < n_cur; it.next(&p.ctl->cursor[cur])) {
-    u64 idx = it.at + lane;
+  for (u64 it = grid_warp() * grab; it < n_cur; it = next_item(&p.ctl->cursor[cur], n_warps, grab)) {
+    u64 idx = it + lane;
     u64 e = lane < grab && idx < n_cur ? __ldcg(&list[idx]) : NO_ENTRY;
     bool valid = e != NO_ENTRY;
     if (!__any_sync(FULL_MASK, valid)) continue;
     if (!valid) e = 0;
-    u32 gq = (u32)(e >> 32), v = (u32)e;
+    u32 gq = (u32)((e & ~ENTRY_DONE) >> 32), v = (u32)e;
     u32 g = gq / Q, q = gq - g * Q;
-    Word<NW> fm;
-#pragma unroll
-    for (int i = 0; i < NW; i++) fm.w[i] = 0;
-    if (valid) fm = load_cg<NW>(F + widx<NW>(p, g, q, v));
+    __syncwarp();  // the previous entries' edges are done
+    if (valid) store_w<NW>(s_fm, load_cg<NW>(F + widx<NW>(p, g, q, v)));
     entries += valid;
     const QueryDesc &qd = gdesc<AM>(p, valid ? g : 0);
     u32 t_beg, nt;
@@ -364,24 +384,29 @@ __device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_c
     }
     u32 max_nt = __reduce_max_sync(FULL_MASK, nt);
     for (u32 j = 0; j < max_nt; j++) {
-      u32 rbeg = 0, rlen = 0, tgq = 0;
-      Word<NW> fmt = fm;  // the entry's lanes that take this transition
+      u32 rbeg = 0, rlen = 0, tg = 0;
+      if (AM == AM_LANE && j) __syncwarp();  // the previous transition's edges are done
       if (j < nt) {
         u32 t = t_beg + j;
         u32 l, to;
+        bool any = true;
         if constexpr (AM == AM_LANE) {
+          // the entry's lanes that take this transition
           const u32 e = p.la_trans[t];
           l = e & 0xFFFFu;
           to = e >> 16;
           const u64 *mk = p.la_mask + (u64)t * ((u64)p.G * NW) + (u64)g * NW;
+          Word<NW> fmt;
 #pragma unroll
-          for (int k = 0; k < NW; k++) fmt.w[k] &= __ldg(mk + k);
+          for (int k = 0; k < NW; k++) fmt.w[k] = s_fm[k] & __ldg(mk + k);
+          any = any_bits(fmt);
+          store_w<NW>(s_words + lane * NW, fmt);
         } else {
           l = qd.out_label[t];
           to = qd.out_to[t];
         }
-        tgq = g * Q + to;
-        if (l < p.L && (AM != AM_LANE || any_bits(fmt))) {
+        tg = pack_target(to, g);
+        if (l < p.L && any) {
           const u32 *off = p.out_off + (u64)l * n1 + v;
           rbeg = __ldg(off);
           rlen = __ldg(off + 1) - rbeg;
@@ -389,13 +414,12 @@ __device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_c
         }
       }
       // long rows, one at a time: the warp writes a row's chunk records together
-      for (u32 big = __ballot_sync(FULL_MASK, p.spill && rlen > chunk); big; big &= big - 1) {
+      const u32 longs = __ballot_sync(FULL_MASK, p.spill && rlen > chunk);
+      if (longs) __syncwarp();
+      for (u32 big = longs; big; big &= big - 1) {
         const u32 o = __ffs(big) - 1;
         const u32 o_beg = __shfl_sync(FULL_MASK, rbeg, o), o_len = __shfl_sync(FULL_MASK, rlen, o);
-        const u32 o_gq = __shfl_sync(FULL_MASK, tgq, o);
-        Word<NW> ofm;
-#pragma unroll
-        for (int i = 0; i < NW; i++) ofm.w[i] = __shfl_sync(FULL_MASK, fmt.w[i], o);
+        const u32 o_tg = __shfl_sync(FULL_MASK, tg, o);
         u64 at = 0;
         u32 fit = 0;
         if (lane == 0) fit = spill_reserve(&p.ctl->spill_count[cur], (o_len + chunk - 1) / chunk, p.spill_cap, &at);
@@ -403,10 +427,10 @@ __device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_c
         fit = __shfl_sync(FULL_MASK, fit, 0);
         for (u32 c = lane; c < fit; c += 32) {
           u64 *rec = p.spill + (at + c) * (2 + NW);
-          rec[0] = ((u64)o_gq << 32) | (o_beg + c * chunk);
+          rec[0] = ((u64)o_tg << 32) | (o_beg + c * chunk);
           rec[1] = min(chunk, o_len - c * chunk);
 #pragma unroll
-          for (int t = 0; t < NW; t++) rec[2 + t] = ofm.w[t];
+          for (int t = 0; t < NW; t++) rec[2 + t] = s_words[o * NW + t];
         }
         // the chunks that did not fit stay with this warp
         if (lane == o) {
@@ -425,6 +449,10 @@ __device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_c
       u32 total = __shfl_sync(FULL_MASK, pre, 31);
       pre -= rlen;
       edges += (lane == 0) ? total : 0;
+      if (total == 0) continue;
+      if (AM != AM_LANE) __syncwarp();  // the previous transition's edges are done
+      s_row[lane] = make_uint2(rbeg - pre, tg);
+      __syncwarp();
       for (u32 k0 = 0; k0 < total; k0 += 32) {
         u32 k = k0 + lane;
         // owner: the largest lane o with pre[o] <= k
@@ -434,19 +462,14 @@ __device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_c
           u32 pv = __shfl_sync(FULL_MASK, pre, o + step);
           if (pv <= k) o += step;
         }
-        u32 o_beg = __shfl_sync(FULL_MASK, rbeg, o);
-        u32 o_pre = __shfl_sync(FULL_MASK, pre, o);
-        u32 o_gq = __shfl_sync(FULL_MASK, tgq, o);
-        Word<NW> ofm;
-#pragma unroll
-        for (int i = 0; i < NW; i++) ofm.w[i] = __shfl_sync(FULL_MASK, fmt.w[i], o);
+        const uint2 row = s_row[o];
         bool take = false;
         u32 w = 0;
         if (k < total) {
-          w = __ldg(p.out_col + o_beg + (k - o_pre));
-          take = relax<NW>(p, FB, o_gq, w, ofm, stamp);
+          w = __ldg(p.out_col + (u32)(row.x + k));
+          take = relax<NW>(p, FB, row.y, w, s_words + o * NW, stamp);
         }
-        warp_append(p, app, take, ((u64)o_gq << 32) | w, &p.ctl->n_list[nxt], nlist);
+        warp_append(p, app, take, target_entry(p, row.y, w), &p.ctl->n_list[nxt], nlist);
       }
     }
   }
@@ -454,12 +477,12 @@ __device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_c
   edges = warp_sum(edges);
   rows = warp_sum(rows);
   entries = warp_sum(entries);
-  stat[ST_GROUP_EDGES] += edges;
-  stat[ST_GROUP_ROWS] += rows;
+  stat_add(stat, ST_GROUP_EDGES, edges);
+  stat_add(stat, ST_GROUP_ROWS, rows);
   // per relaxation a column id and the target's visited word (the spilled
   // share is counted by the spill phase); per row its two offsets; per entry
   // the list entry and its frontier word
-  stat[ST_ALG_BYTES] += edges * (4 + 8 * NW) + rows * 8 + entries * (8 + 8 * NW);
+  stat_add(stat, ST_ALG_BYTES, edges * (4 + 8 * NW) + rows * 8 + entries * (8 + 8 * NW));
 }
 
 // The queued chunks of long rows: a warp per chunk, taken dynamically.
@@ -472,11 +495,10 @@ __device__ void spill_phase(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 se
   u64 edges = 0;
   Appender app;
   app.seg = seg;
-  Items it(grid_warp(), grid_warps(), 1);
-  for (; it.at < count; it.next(&p.ctl->spill_cursor[cur])) {
-    const u64 *rec = p.spill + it.at * (2 + NW);
+  for (u64 it = grid_warp(); it < count; it = next_item(&p.ctl->spill_cursor[cur], grid_warps(), 1)) {
+    const u64 *rec = p.spill + it * (2 + NW);
     const u64 h = __ldcg(rec);
-    const u32 tgq = (u32)(h >> 32), b = (u32)h;
+    const u32 tg = (u32)(h >> 32), b = (u32)h;
     const u32 len = (u32)__ldcg(rec + 1);
     Word<NW> fm;
 #pragma unroll
@@ -488,25 +510,24 @@ __device__ void spill_phase(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 se
       u32 w = 0;
       if (k < len) {
         w = __ldg(p.out_col + b + k);
-        take = relax<NW>(p, FB, tgq, w, fm, stamp);
+        take = relax<NW>(p, FB, tg, w, fm.w, stamp);
       }
-      warp_append(p, app, take, ((u64)tgq << 32) | w, &p.ctl->n_list[nxt], nlist);
+      warp_append(p, app, take, target_entry(p, tg, w), &p.ctl->n_list[nxt], nlist);
     }
   }
   append_close(p, app, nlist);
   edges = warp_sum(edges);
-  stat[ST_GROUP_EDGES] += edges;
-  stat[ST_ALG_BYTES] += edges * (4 + 8 * NW);
+  stat_add(stat, ST_GROUP_EDGES, edges);
+  stat_add(stat, ST_ALG_BYTES, edges * (4 + 8 * NW));
 }
 
 // Bottom-up work for target (q2, w) over in-edges [beg, end) of one
 // transition group with active source states `from`: every lane ORs the
-// gathered frontier words of its PER words into acc.  With EARLY (one lane
-// group: few enough lanes that a vertex can run out of unvisited ones) a lane
-// stops gathering once acc covers all its lanes not yet visited, and the
-// sub-warp (lanes sg_mask) leaves the row when all its lanes have (with many
-// groups a vertex practically never runs out, and the test costs more than it
-// saves).  Returns the in-edges examined.
+// gathered frontier words of its PER words into acc.  With EARLY (few enough
+// lanes that a vertex can run out of unvisited ones) a lane stops gathering
+// once acc covers all its lanes not yet visited, and the sub-warp (lanes
+// sg_mask) leaves the row when all its lanes have.  Returns the in-edges
+// examined.
 template <int NW, int PER, bool EARLY, bool LANE>
 __device__ __forceinline__ u32 gather_row(const BfsParams &p, const u64 *F, const u32 *bits, u32 from, u32 beg,
                                           u32 end, u32 lane_off, bool lane_on, u32 sg_mask,
@@ -639,6 +660,639 @@ __device__ __forceinline__ void pull_finish(const BfsParams &p, Appender &app, u
   warp_append(p, app, take, ((u64)(my_g * p.Q + q2) << 32) | w, &p.ctl->n_list[nxt], nlist);
 }
 
+// What a block's warps committed in a level, in shared memory: added to the
+// control block once per block and level.  One atomic per warp and counter
+// queued up to 4,864 x 5 of them on two lines: 4-5 us of every commit.
+struct CommitSums {
+  unsigned long long mf, gx, n_true;
+  unsigned int smask;
+};
+
+// By one thread, when the block's warps have committed.  gx is kept to the end.
+__device__ __forceinline__ void publish_sums(BfsCtl *c, CommitSums &s, u32 nxt) {
+  if (s.n_true == 0) return;
+  if (s.mf) atomicAdd(&c->mf[nxt], s.mf);
+  atomicAdd(&c->n_true[nxt], s.n_true);
+  atomicOr(&c->smask[nxt], s.smask);
+  s.mf = s.n_true = 0;
+  s.smask = 0;
+}
+
+// ---------------------------------------------------------------------------
+// Bottom-up expansion of several lane groups under one automaton (G > 1, 256
+// lanes each), the form of every large source list.
+//
+// What bounds it: gathers of G * 32 bytes from random rows of the frontier
+// array.  Walking one vertex's in-row after another, the row offsets, the
+// column ids and the gathers of every row were three dependent round trips,
+// with at most four gathers in flight and one in a row's tail.  Here the
+// gathers of 32 consecutive vertices are listed first, by all lanes together
+// (coalesced offsets and column ids, one round trip each for the whole list),
+// in shared memory; a vertex is then one round trip of up to eight gathers.
+// With a frontier bitmap only neighbours in the frontier are listed, and only
+// vertices with such a neighbour read their visited words.
+//
+// A vertex produced by one sub-warp alone (no chunks of long rows, no second
+// piece of the list) is also committed by it: it has the visited words in
+// registers, and the vertex's degrees, counted once per vertex by the lane
+// that lists it, serve all its groups; its entries carry ENTRY_DONE, and the
+// commit phase passes over them.
+// ---------------------------------------------------------------------------
+constexpr u32 STAGE = 256;           // gathers listed at a time per warp
+constexpr u64 STAGE_ROW = (1ull << 58) - 1;  // low bits: state * n + vertex; above: the owning vertex's lane
+
+
+// The k-th set bit of m (0-based).
+__device__ __forceinline__ u32 nth_bit(u32 m, u32 k) {
+  for (; k; k--) m &= m - 1;
+  return __ffs(m) - 1;
+}
+
+// ORs the listed rows lst[first], lst[first + step], ... below cnt into acc,
+// eight gathers in flight.  Lanes that are off must pass cnt = 0.
+__device__ __forceinline__ void gather_list(const u64 *F, u64 wpv, u32 lane_off, const u64 *lst, u32 first, u32 step,
+                                            u32 cnt, u64 (&acc)[2]) {
+  constexpr int DEEP = 8;
+  for (u32 k = first; k < cnt; k += DEEP * step) {
+    ulonglong2 a[DEEP];
+#pragma unroll
+    for (int t = 0; t < DEEP; t++) {
+      const u32 j = k + t * step;
+      a[t] = make_ulonglong2(0, 0);
+      if (j < cnt)
+        a[t] = __ldcg(reinterpret_cast<const ulonglong2 *>(F + (lst[j] & STAGE_ROW) * wpv + lane_off));
+    }
+#pragma unroll
+    for (int t = 0; t < DEEP; t++) {
+      acc[0] |= a[t].x;
+      acc[1] |= a[t].y;
+    }
+  }
+}
+
+template <int NW>
+__device__ void pull_staged(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 active, u32 stamp, const u32 *bits,
+                            u64 *scratch, CommitSums &sums, u64 *stat) {
+  static_assert(NW == 4, "two words per lane, two lanes per group");
+  const u64 *F = lp ? p.fr1 : p.fr0;
+  u64 *FB = lp ? p.fr0 : p.fr1;
+  u64 *nlist = lp ? p.list0 : p.list1;
+  const u32 n = p.n, Q = p.Q, n1 = p.n + 1;
+  const u32 lane = lane_id();
+  const u32 lanes_used = p.G * 2;
+  u32 SW = 1;
+  while (SW < lanes_used) SW <<= 1;
+  const u32 VPW = 32 / SW;  // vertices a warp works on at once
+  const u32 sg = lane / SW, li = lane % SW;
+  const bool lane_on = li < lanes_used;
+  const u32 lane_off = li * 2, my_g = li / 2;
+  const u64 wpv = (u64)p.G * NW;
+  u64 *lst = scratch;  // [STAGE]
+  // the listed vertices: lane | shared << 5 | rows << 6, first gather, gathers,
+  // out-degree
+  __shared__ uint4 s_vertex[BFS_THREADS / 32][32];
+  uint4 *vertex = s_vertex[threadIdx.x >> 5];
+  const bool chunked = p.hchunk != nullptr;
+  const u64 gword = 8ull * NW * p.G;  // bytes of the G words of one (state, vertex)
+  u64 W = 0, mf = 0;
+  u32 N = 0, gv = 0, gx = 0, states = 0;
+  Appender app;
+  app.seg = (u64)n * Q * p.G >= grid_warps() * 2 * APPEND_SEG ? p.append_seg : min(p.append_seg, 32u);
+
+  // Long in-rows first (the light rows' shorter items then fill the phase's
+  // end): their precomputed chunks, a warp per (target state, transition
+  // group, chunk), the sub-warps sharing the list.
+  if (chunked) {
+    for (u64 it = grid_warp();; it = next_item(&p.ctl->heavy_cursor[cur], grid_warps(), 1)) {
+      u64 acc_base = 0, ci = 0;
+      u32 q2 = 0, from = 0;
+      bool found = false;
+      for (u32 q = 0; q < Q && !found; q++)
+        for (u32 j = p.q.in_begin[q]; j < p.q.in_begin[q + 1]; j++) {
+          const u32 l = p.q.in_label[j];
+          if (!(p.q.in_from[j] & active) || l >= p.L) continue;
+          const u64 cnt = p.hchunk_off[l + 1] - p.hchunk_off[l];
+          if (it < acc_base + cnt) {
+            found = true;
+            q2 = q;
+            from = p.q.in_from[j] & active;
+            ci = p.hchunk_off[l] + (it - acc_base);
+            break;
+          }
+          acc_base += cnt;
+        }
+      if (!found) break;
+      const u32 *rec = p.hchunk + 3 * ci;
+      const u32 w = __ldg(rec), beg = __ldg(rec + 1), len = __ldg(rec + 2) - beg;
+      u64 vis[2], acc[2] = {0, 0};
+      load_vis<2>(p.vis + ((u64)q2 * n + w) * wpv + lane_off, lane_on, vis);
+      if (__all_sync(FULL_MASK, (vis[0] & vis[1]) == ~0ull)) continue;
+      for (u32 fb = from; fb; fb &= fb - 1) {
+        const u64 qb = (u64)(__ffs(fb) - 1) * n;
+        for (u32 e0 = 0; e0 < len; e0 += STAGE) {
+          u32 cnt = 0;
+          __syncwarp();  // the previous list is consumed
+          for (u32 k = e0; k < min(len, e0 + STAGE); k += 32) {
+            u64 row = 0;
+            bool in = k + lane < len;
+            if (in) {
+              row = qb + __ldg(p.in_col + beg + k + lane);
+              if (bits) in = (__ldcg(bits + (row >> 5)) >> (row & 31)) & 1u;
+            }
+            const u32 b = __ballot_sync(FULL_MASK, in);
+            if (in) lst[cnt + __popc(b & lanemask_lt())] = row;
+            cnt += __popc(b);
+          }
+          __syncwarp();
+          gather_list(F, wpv, lane_off, lst, sg, VPW, lane_on ? cnt : 0, acc);
+          stat_add(stat, ST_ALG_BYTES, cnt * gword);
+        }
+      }
+      for (u32 o = SW; o < 32; o <<= 1) {
+        acc[0] |= __shfl_xor_sync(FULL_MASK, acc[0], o);
+        acc[1] |= __shfl_xor_sync(FULL_MASK, acc[1], o);
+      }
+      stat_add(stat, ST_PULL_EDGES, len);
+      stat_add(stat, ST_PULL_VERTICES, 1);
+      stat_add(stat, ST_ALG_BYTES, gword + len * (bits ? 8 : 4));
+      pull_finish<NW, 2>(p, app, FB, nlist, nxt, q2, w, stamp, li, lane_on && sg == 0, my_g, true, vis, acc);
+    }
+  }
+
+  u32 cv = 32;  // vertices a warp takes at a time (see pull_level)
+  while (cv > VPW && n < 2 * grid_warps() * cv) cv >>= 1;
+  for (u64 c0 = grid_warp() * cv; c0 < n;) {
+    const u32 v = (u32)(c0 + lane);
+    const bool mine = lane < cv && c0 + lane < n;
+    for (u32 q2 = 0; q2 < Q; q2++) {
+      const u32 gb = p.q.in_begin[q2], ge = p.q.in_begin[q2 + 1];
+      // this lane's vertex: its light in-rows on active transitions (gathers
+      // to list), and whether chunks of a long one produce it too
+      u32 tot = 0, lens = 0;
+      bool shared = false;
+      if (mine)
+        for (u32 j = gb; j < ge; j++) {
+          const u32 from = p.q.in_from[j] & active, l = p.q.in_label[j];
+          if (!from || l >= p.L) continue;
+          const u32 *off = p.in_off + (u64)l * n1 + v;
+          const u32 len = __ldg(off + 1) - __ldg(off);
+          if (len >= HEAVY_ROW && chunked)
+            shared = true;
+          else
+            lens += len, tot += len * __popc(from);
+        }
+      u32 pre = tot;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const u32 t = __shfl_up_sync(FULL_MASK, pre, o);
+        if (lane >= (u32)o) pre += t;
+      }
+      const u32 T = __shfl_sync(FULL_MASK, pre, 31);
+      if (T == 0) continue;
+      pre -= tot;
+      lens = __reduce_add_sync(FULL_MASK, lens);
+      stat_add(stat, ST_PULL_EDGES, lens);
+      stat_add(stat, ST_ALG_BYTES, lens * (bits ? 8 : 4));
+      shared |= tot && pre / STAGE != (pre + tot - 1) / STAGE;  // listed in two pieces
+      // the vertex's out-degree over the labels leaving q2, for its commit
+      u32 rows = 0, deg = 0;
+      if (tot && !shared) deg = degsum(p, p.q, q2, v, &rows);
+      for (u32 p0 = 0; p0 < T; p0 += STAGE) {
+        const u32 pend = min(T, p0 + STAGE);
+        u32 listed = 0;
+        __syncwarp();  // the previous list is consumed
+        for (u32 k0 = p0; k0 < pend; k0 += 32) {
+          const u32 k = k0 + lane;
+          // owner: the largest lane o with pre[o] <= k
+          u32 o = 0;
+#pragma unroll
+          for (u32 step = 16; step > 0; step >>= 1) {
+            const u32 pv = __shfl_sync(FULL_MASK, pre, o + step);
+            if (pv <= k) o += step;
+          }
+          u32 r = k - __shfl_sync(FULL_MASK, pre, o);
+          bool in = k < pend;
+          u64 row = 0;
+          if (in) {
+            // the r-th gather of vertex c0 + o: its groups in order, every
+            // in-edge once per active source state
+            u32 col = 0, st = 0;
+            for (u32 j = gb; j < ge; j++) {
+              const u32 from = p.q.in_from[j] & active, l = p.q.in_label[j];
+              if (!from || l >= p.L) continue;
+              const u32 *off = p.in_off + (u64)l * n1 + (u32)(c0 + o);
+              const u32 beg = __ldg(off), len = __ldg(off + 1) - beg;
+              if (len >= HEAVY_ROW && chunked) continue;
+              const u32 np = __popc(from);
+              if (r < len * np) {
+                col = beg + (np == 1 ? r : r / np);
+                st = nth_bit(from, np == 1 ? 0 : r % np);
+                break;
+              }
+              r -= len * np;
+            }
+            row = (u64)st * n + __ldg(p.in_col + col);
+            if (bits) in = (__ldcg(bits + (row >> 5)) >> (row & 31)) & 1u;
+          }
+          const u32 b = __ballot_sync(FULL_MASK, in);
+          if (in) lst[listed + __popc(b & lanemask_lt())] = row | (u64)o << 58;
+          listed += __popc(b);
+        }
+        __syncwarp();
+        // this lane's vertex's part of the list: [first, first + cnt)
+        u32 first, cnt;
+        if (bits) {
+          u32 lo = 0, hi = listed;
+          while (lo < hi) {
+            const u32 mid = (lo + hi) >> 1;
+            if ((u32)(lst[mid] >> 58) < lane)
+              lo = mid + 1;
+            else
+              hi = mid;
+          }
+          first = lo;
+          const u32 up = __shfl_down_sync(FULL_MASK, lo, 1);
+          cnt = (lane == 31 ? listed : up) - lo;
+        } else {
+          const u32 s = max(pre, p0), e = min(pre + tot, pend);
+          first = s - p0;
+          cnt = e > s ? e - s : 0;
+        }
+        const u32 M = __ballot_sync(FULL_MASK, cnt != 0);
+        const u32 nz = __popc(M);
+        if (cnt) vertex[__popc(M & lanemask_lt())] = make_uint4(lane | (u32)shared << 5 | rows << 6, first, cnt, deg);
+        __syncwarp();
+        stat_add(stat, ST_PULL_VERTICES, nz);
+        stat_add(stat, ST_ALG_BYTES, (listed + nz) * gword);
+        for (u32 r0 = 0; r0 < nz; r0 += VPW) {
+          const bool work = r0 + sg < nz;
+          const uint4 x = vertex[work ? r0 + sg : 0];
+          const bool osh = (x.x >> 5) & 1u;
+          const bool on = work && lane_on;
+          const u32 w = (u32)c0 + (x.x & 31u);
+          const u64 base = ((u64)q2 * n + w) * wpv + lane_off;
+          u64 vis[2], acc[2] = {0, 0};
+          load_vis<2>(p.vis + base, on, vis);
+          gather_list(F, wpv, lane_off, lst + x.y, 0, 1, on ? x.z : 0, acc);
+          const u64 n0 = acc[0] & ~vis[0], n1w = acc[1] & ~vis[1];  // zero for lanes that are off
+          const bool nz_l = (n0 | n1w) != 0;
+          if (!__any_sync(FULL_MASK, nz_l)) continue;
+          if (nz_l) {
+            if (osh) {
+              if (n0) atomicOr((unsigned long long *)(FB + base), n0);
+              if (n1w) atomicOr((unsigned long long *)(FB + base + 1), n1w);
+            } else {
+              *reinterpret_cast<ulonglong2 *>(FB + base) = make_ulonglong2(n0, n1w);
+              *reinterpret_cast<ulonglong2 *>(p.vis + base) = make_ulonglong2(vis[0] | n0, vis[1] | n1w);
+              const u32 c = __popcll(n0) + __popcll(n1w);
+              N += c;
+              W += (u64)c * x.w;
+            }
+          }
+          // one lane per group lists the entry
+          bool take = __shfl_xor_sync(FULL_MASK, nz_l, 1) | nz_l;
+          take = take && on && (li & 1) == 0;
+          if (take && osh) take = atomicMax(p.claim + (((u64)q2 * n + w) * p.G + my_g), stamp) < stamp;
+          if (take && !osh) {
+            mf += x.w;
+            gx += x.x >> 6;
+            gv += 1;
+            states |= 1u << q2;
+          }
+          warp_append(p, app, take, ((u64)(my_g * Q + q2) << 32) | w | (osh ? 0ull : ENTRY_DONE),
+                      &p.ctl->n_list[nxt], nlist);
+        }
+      }
+    }
+    if (p.pull_dynamic)
+      c0 = next_item(&p.ctl->cursor[cur], grid_warps(), cv);
+    else
+      c0 += grid_warps() * cv;
+  }
+  append_close(p, app, nlist);
+  W = warp_sum(W);
+  mf = warp_sum(mf);
+  const u64 s_gv = warp_sum((u64)gv), s_gx = warp_sum((u64)gx);
+  states = __reduce_or_sync(FULL_MASK, states);
+  stat_add(stat, ST_W, W);
+  stat_add(stat, ST_N, warp_sum((u64)N));
+  // counted above: per in-edge a column id (and a bitmap word), per gather a
+  // frontier row, per vertex its visited words; here per entry committed its
+  // list entry, its new frontier word and its visited word written
+  stat_add(stat, ST_ALG_BYTES, s_gv * (8 + 16 * NW));
+  if (lane == 0 && s_gv) {
+    atomicAdd(&sums.mf, mf);
+    atomicAdd(&sums.gx, s_gx);
+    atomicAdd(&sums.n_true, s_gv);
+    atomicOr(&sums.smask, states);
+  }
+}
+
+// ---------------------------------------------------------------------------
+// Bottom-up expansion in lane mode, by source state, for launches whose lanes
+// fill a warp's row (G * 2 > 16 lanes of two words) and whose union automaton
+// has at most LANE_SRC_Q states.
+//
+// Target q2's new lanes at vertex w are the OR over the union's transitions
+// t = (s, l, q2) and the in-edges (v, w) of label l of F[s][v] & mask(t).  A
+// row F[s][v] serves every target of (s, l): it is gathered once and masked
+// into the targets' accumulators (shared memory, one 16-byte word per lane and
+// target).  What bounds it: the gathers, about one per in-edge and source
+// state.  A vertex's rows are short and spread over its labels, so walking
+// them one by one kept one or two gathers in flight, each behind its row's
+// offsets and column ids.  Here the gathers of 16 in-edges at a time are
+// listed by all lanes together, without the rows a frontier bitmap shows
+// empty, and read eight at once whatever rows and labels they belong to; a
+// row's gathers of one state are ORed before they are masked, and a vertex's
+// visited words are read together when its list ends.  A batch of 4,096
+// queries on R-MAT 2^22 (3,704 lanes, 8 states, 189 transitions): its three
+// dense levels 90 / 105 / 103 -> 51 / 58 / 56 ms.  Masking every gather by
+// itself (one apply per in-edge and state) took 82 / 101 / 99 ms: the masks
+// and accumulators pass the load/store unit once per target of each.  Three
+// blocks per SM (80 registers) beat four (314 against 327 ms of traversal).
+// ---------------------------------------------------------------------------
+constexpr u32 LANE_EDGES = 16;                          // in-edges listed at a time
+constexpr u32 LANE_LIST = LANE_EDGES * LANE_SRC_Q;      // their gathers
+constexpr u64 LANE_ROW = (1ull << 44) - 1;              // state * n + vertex; above: label * 8 + state, owner lane
+
+struct LaneTables {  // of a level, in shared memory
+  u32 grp[RPQ_MAX_LABELS * LANE_SRC_Q];  // [label][state]: first transition | targets << 16 (0: none, or state not active)
+  unsigned char act[RPQ_MAX_LABELS];     // [label]: active states with a transition on it
+};
+
+template <int NW>
+__device__ void pull_lanes(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 active, u32 stamp, const u32 *bits,
+                           u64 *scratch, LaneTables &tab, u64 *stat) {
+  static_assert(NW == 4, "two words per lane");
+  const u64 *F = lp ? p.fr1 : p.fr0;
+  u64 *FB = lp ? p.fr0 : p.fr1;
+  u64 *nlist = lp ? p.list0 : p.list1;
+  const u32 n = p.n, Q = p.Q, L = p.L, n1 = p.n + 1;
+  const u32 lane = lane_id();
+  const bool lane_on = lane < p.G * 2;
+  const u32 lane_off = lane * 2;
+  const u64 wpv = (u64)p.G * NW, gword = 8ull * NW * p.G;
+  ulonglong2 *sacc = reinterpret_cast<ulonglong2 *>(scratch) + lane;  // target q2's words at sacc[32 * q2]
+  u64 *lst = scratch + LANE_SRC_Q * 2 * 32;                           // [LANE_LIST]
+  const bool chunked = p.hchunk != nullptr;
+  Appender app;
+  app.seg = (u64)n * Q * p.G >= grid_warps() * 2 * APPEND_SEG ? p.append_seg : min(p.append_seg, 32u);
+
+  for (u32 i = threadIdx.x; i < L * LANE_SRC_Q; i += blockDim.x) {
+    const u32 l = i / LANE_SRC_Q, s = i % LANE_SRC_Q;
+    tab.grp[i] = s < Q && ((active >> s) & 1u) ? p.la_sl[s * L + l] : 0u;
+  }
+  __syncthreads();
+  u64 lset = 0;  // labels with an active transition
+  for (u32 l = 0; l < L; l++) {
+    u32 a = 0;
+    for (u32 s = 0; s < Q; s++) a |= (tab.grp[l * LANE_SRC_Q + s] >> 16 ? 1u : 0u) << s;
+    if (a) lset |= 1ull << l;
+    if (threadIdx.x == 0) tab.act[l] = (unsigned char)a;
+  }
+  __syncthreads();
+
+  u32 tmask = 0;  // targets with an accumulator
+  // row (words r) of a gather from (label, state) tag into its targets
+  auto apply = [&](u32 tag, const ulonglong2 r) {
+    const u32 e = tab.grp[tag];
+    u64 at = (u64)(e & 0xFFFFu) * wpv + lane_off;
+    for (u32 tm = e >> 16; tm; tm &= tm - 1, at += wpv) {
+      const u32 to = __ffs(tm) - 1;
+      ulonglong2 m = make_ulonglong2(0, 0);
+      if (lane_on) m = __ldg(reinterpret_cast<const ulonglong2 *>(p.la_mask + at));
+      m.x &= r.x;
+      m.y &= r.y;
+      if ((tmask >> to) & 1u) {
+        const ulonglong2 a = sacc[32 * to];
+        m.x |= a.x;
+        m.y |= a.y;
+      }
+      sacc[32 * to] = m;
+      tmask |= 1u << to;
+    }
+  };
+  // the accumulated vertex: lanes not yet visited go to the next frontier
+  auto flush = [&](u32 w, bool shared) {
+    ulonglong2 v[LANE_SRC_Q];
+#pragma unroll
+    for (u32 q2 = 0; q2 < LANE_SRC_Q; q2++) {
+      v[q2] = make_ulonglong2(~0ull, ~0ull);
+      if (lane_on && ((tmask >> q2) & 1u))
+        v[q2] = __ldcg(reinterpret_cast<const ulonglong2 *>(p.vis + ((u64)q2 * n + w) * wpv + lane_off));
+    }
+    u32 found = 0;
+#pragma unroll
+    for (u32 q2 = 0; q2 < LANE_SRC_Q; q2++)
+      if ((tmask >> q2) & 1u) {
+        ulonglong2 a = sacc[32 * q2];
+        a.x &= ~v[q2].x;
+        a.y &= ~v[q2].y;
+        sacc[32 * q2] = a;
+        if (a.x | a.y) found |= 1u << q2;
+      }
+    stat_add(stat, ST_PULL_VERTICES, __popc(tmask));
+    stat_add(stat, ST_ALG_BYTES, __popc(tmask) * gword);
+    u32 any = __reduce_or_sync(FULL_MASK, found);
+    for (; any; any &= any - 1) {
+      const u32 q2 = __ffs(any) - 1;
+      const bool nz = (found >> q2) & 1u;
+      const u64 base = ((u64)q2 * n + w) * wpv + lane_off;
+      if (nz) {
+        const ulonglong2 a = sacc[32 * q2];
+        if (shared) {
+          if (a.x) atomicOr((unsigned long long *)(FB + base), a.x);
+          if (a.y) atomicOr((unsigned long long *)(FB + base + 1), a.y);
+        } else {
+          *reinterpret_cast<ulonglong2 *>(FB + base) = a;
+        }
+      }
+      bool take = __shfl_xor_sync(FULL_MASK, nz, 1) | nz;
+      take = take && (lane & 1) == 0;
+      if (take && shared)
+        take = atomicMax(p.claim + (((u64)q2 * n + w) * p.G + lane / 2), stamp) < stamp;
+      warp_append(p, app, take, ((u64)(lane / 2 * Q + q2) << 32) | w, &p.ctl->n_list[nxt], nlist);
+    }
+    tmask = 0;
+  };
+
+  // Long in-rows first, an item per (label, chunk): the chunk's rows of each
+  // active source state are ORed together and masked once.
+  if (chunked) {
+    for (u64 it = grid_warp();; it = next_item(&p.ctl->heavy_cursor[cur], grid_warps(), 1)) {
+      u64 acc_base = 0, ci = 0;
+      u32 l = 0;
+      bool found = false;
+      for (u64 lb = lset; lb && !found; lb &= lb - 1) {
+        l = __ffsll((long long)lb) - 1;
+        const u64 cnt = p.hchunk_off[l + 1] - p.hchunk_off[l];
+        found = it < acc_base + cnt;
+        if (found) ci = p.hchunk_off[l] + (it - acc_base);
+        acc_base += cnt;
+      }
+      if (!found) break;
+      const u32 *rec = p.hchunk + 3 * ci;
+      const u32 w = __ldg(rec), beg = __ldg(rec + 1), len = __ldg(rec + 2) - beg;
+      for (u32 sm = tab.act[l]; sm; sm &= sm - 1) {
+        const u32 st = __ffs(sm) - 1;
+        u64 g[2] = {0, 0};
+        for (u32 e0 = 0; e0 < len; e0 += LANE_LIST) {
+          u32 cnt = 0;
+          __syncwarp();  // the previous list is consumed
+          for (u32 k = e0; k < min(len, e0 + LANE_LIST); k += 32) {
+            u64 row = 0;
+            bool in = k + lane < len;
+            if (in) {
+              row = (u64)st * n + __ldg(p.in_col + beg + k + lane);
+              if (bits) in = (__ldcg(bits + (row >> 5)) >> (row & 31)) & 1u;
+            }
+            const u32 b = __ballot_sync(FULL_MASK, in);
+            if (in) lst[cnt + __popc(b & lanemask_lt())] = row;
+            cnt += __popc(b);
+          }
+          __syncwarp();
+          gather_list(F, wpv, lane_off, lst, 0, 1, lane_on ? cnt : 0, g);
+          stat_add(stat, ST_ALG_BYTES, cnt * gword);
+        }
+        if (__any_sync(FULL_MASK, (g[0] | g[1]) != 0)) apply(l * LANE_SRC_Q + st, make_ulonglong2(g[0], g[1]));
+      }
+      stat_add(stat, ST_PULL_EDGES, len);
+      stat_add(stat, ST_ALG_BYTES, len * 4);
+      if (tmask) flush(w, true);
+    }
+  }
+
+  u32 cv = 32;  // vertices a warp takes at a time (see pull_level)
+  while (cv > 1 && n < 2 * grid_warps() * cv) cv >>= 1;
+  for (u64 c0 = grid_warp() * cv; c0 < n;) {
+    // this lane's vertex: its light in-edges on active labels, and whether
+    // chunks of a long row produce it too
+    u32 tot = 0;
+    bool sh = false;
+    if (lane < cv && c0 + lane < n)
+      for (u64 lb = lset; lb; lb &= lb - 1) {
+        const u32 *off = p.in_off + (u64)(__ffsll((long long)lb) - 1) * n1 + c0 + lane;
+        const u32 len = __ldg(off + 1) - __ldg(off);
+        if (len >= HEAVY_ROW && chunked)
+          sh = true;
+        else
+          tot += len;
+      }
+    const u32 shared = __ballot_sync(FULL_MASK, sh);
+    u32 pre = tot;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const u32 t = __shfl_up_sync(FULL_MASK, pre, o);
+      if (lane >= (u32)o) pre += t;
+    }
+    const u32 T = __shfl_sync(FULL_MASK, pre, 31);
+    pre -= tot;
+    stat_add(stat, ST_PULL_EDGES, T);
+    stat_add(stat, ST_ALG_BYTES, T * 4ull);
+    u32 own = 32;  // lane of the vertex being accumulated (32: none)
+    for (u32 p0 = 0; p0 < T; p0 += LANE_EDGES) {
+      // in-edges p0 + lane: owner, label, the states to gather it from
+      const u32 k = p0 + lane;
+      u32 o = 0;
+#pragma unroll
+      for (u32 step = 16; step > 0; step >>= 1) {
+        const u32 pv = __shfl_sync(FULL_MASK, pre, o + step);
+        if (pv <= k) o += step;
+      }
+      u32 r = k - __shfl_sync(FULL_MASK, pre, o);
+      u32 l = 0, u = 0, sm = 0;
+      if (lane < LANE_EDGES && k < T) {
+        for (u64 lb = lset; lb; lb &= lb - 1) {
+          l = __ffsll((long long)lb) - 1;
+          const u32 *off = p.in_off + (u64)l * n1 + c0 + o;
+          const u32 beg = __ldg(off), len = __ldg(off + 1) - beg;
+          if (len >= HEAVY_ROW && chunked) continue;
+          if (r < len) {
+            u = __ldg(p.in_col + beg + r);
+            sm = tab.act[l];
+            break;
+          }
+          r -= len;
+        }
+        if (bits)
+          for (u32 m = sm; m; m &= m - 1) {
+            const u32 st = __ffs(m) - 1;
+            const u64 row = (u64)st * n + u;
+            if (!((__ldcg(bits + (row >> 5)) >> (row & 31)) & 1u)) sm &= ~(1u << st);
+          }
+      }
+      u32 at = __popc(sm);
+#pragma unroll
+      for (int d = 1; d < 32; d <<= 1) {
+        const u32 t = __shfl_up_sync(FULL_MASK, at, d);
+        if (lane >= (u32)d) at += t;
+      }
+      const u32 listed = __shfl_sync(FULL_MASK, at, 31);
+      at -= __popc(sm);
+      // a row's gathers are listed state by state, so that a state's rows are
+      // ORed before they are masked (with a bitmap, where rows are missing,
+      // in-edge by in-edge)
+      u32 run = 1;
+      if (!bits) {
+        const u32 same = __match_any_sync(FULL_MASK, lane < LANE_EDGES && k < T ? o << 6 | l : 1u << 31 | lane);
+        run = __popc(same);
+        at = __shfl_sync(FULL_MASK, at, __ffs(same) - 1) + __popc(same & lanemask_lt());
+      }
+      __syncwarp();  // the previous list is consumed
+      for (u32 m = sm; m; m &= m - 1, at += run) {
+        const u32 st = __ffs(m) - 1;
+        lst[at] = ((u64)st * n + u) | (u64)(l * LANE_SRC_Q + st) << 44 | (u64)o << 58;
+      }
+      __syncwarp();
+      stat_add(stat, ST_ALG_BYTES, listed * gword);
+      for (u32 i = 0; i < listed;) {
+        const u32 o2 = (u32)(lst[i] >> 58);
+        if (o2 != own) {
+          if (tmask) flush((u32)c0 + own, (shared >> own) & 1u);
+          own = o2;
+        }
+        // the run of this vertex in the list: [i, j)
+        u32 j = i, hi = listed;
+        while (j < hi) {
+          const u32 mid = (j + hi) >> 1;
+          if ((u32)(lst[mid] >> 58) == o2)
+            j = mid + 1;
+          else
+            hi = mid;
+        }
+        constexpr u32 DEEP = 8;
+        ulonglong2 g = make_ulonglong2(0, 0);
+        for (; i < j; i += DEEP) {
+          ulonglong2 a[DEEP];
+#pragma unroll
+          for (u32 t = 0; t < DEEP; t++) {
+            a[t] = make_ulonglong2(0, 0);
+            if (lane_on && i + t < j)
+              a[t] = __ldcg(reinterpret_cast<const ulonglong2 *>(F + (lst[i + t] & LANE_ROW) * wpv + lane_off));
+          }
+#pragma unroll
+          for (u32 t = 0; t < DEEP; t++)
+            if (i + t < j) {
+              g.x |= a[t].x;
+              g.y |= a[t].y;
+              const u32 tag = (u32)(lst[i + t] >> 44);
+              if (i + t + 1 < j && (u32)(lst[i + t + 1] >> 44) == tag) continue;
+              if (__any_sync(FULL_MASK, (g.x | g.y) != 0)) apply(tag & (RPQ_MAX_LABELS * LANE_SRC_Q - 1), g);
+              g = make_ulonglong2(0, 0);
+            }
+        }
+        i = j;
+      }
+    }
+    if (tmask) flush((u32)c0 + own, (shared >> own) & 1u);
+    if (p.pull_dynamic)
+      c0 = next_item(&p.ctl->cursor[cur], grid_warps(), cv);
+    else
+      c0 += grid_warps() * cv;
+  }
+  append_close(p, app, nlist);
+}
+
 // Bottom-up expansion.  Light rows: one vertex per sub-warp of SW lanes (the
 // smallest power of two holding the vertex's G * NW words at PER words per
 // lane), all groups at once, so a warp covers 32 / SW vertices (32 for a
@@ -646,9 +1300,9 @@ __device__ __forceinline__ void pull_finish(const BfsParams &p, Appender &app, u
 // chunk taken dynamically over the (target state, transition group) pairs
 // whose source states are active; the sub-warps split the chunk's edges and
 // OR their gathers together.
-template <int NW, bool EARLY, int AM>
+template <int NW, int AM>
 __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 active, u32 stamp, const u32 *bits,
-                           u64 *stat) {
+                           u64 *scratch, u64 *stat) {
   constexpr int PER = (NW >= 2) ? 2 : 1;
   const u64 *F = lp ? p.fr1 : p.fr0;
   u64 *FB = lp ? p.fr0 : p.fr1;
@@ -677,11 +1331,7 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
   // small graphs: shorter segments, so that unused slots do not outnumber the entries
   app.seg = (u64)n * Q * p.G >= n_warps * 2 * APPEND_SEG ? p.append_seg : min(p.append_seg, 32u);
   // lane mode by source state: this warp's per-target accumulators
-  u64 *lane_acc = nullptr;
-  if constexpr (AM == AM_LANE) {
-    __shared__ u64 s_lane_acc[BFS_THREADS / 32][LANE_SRC_Q * 2 * 32];
-    lane_acc = s_lane_acc[threadIdx.x >> 5];
-  }
+  u64 *lane_acc = scratch;
 
   // A warp takes cv consecutive vertices at a time: lane i first finds, with
   // coalesced reads of the in-row offsets, the target states into which
@@ -691,9 +1341,7 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
   // a cursor (the level's list cursor, unused by bottom-up levels), so a
   // warp whose chunks had little work takes more of them; else chunk k goes
   // to warp k mod warps.
-  Items vit(warp, n_warps, cv);
-  for (; vit.at < n;) {
-    const u64 c0 = vit.at;
+  for (u64 c0 = warp * cv; c0 < n;) {
     // hmask: states with a long in-row (its chunks also produce); with a
     // sparse frontier (bits), lane i also tests up to PRESCAN in-edges of
     // its own vertex against the frontier bitmap, so that a state none of
@@ -879,7 +1527,7 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
           u32 lfrom = from;
           if constexpr (AM == AM_GROUP) lfrom = lane_on ? p.from_tab[((u64)my_g * Q + q2) * p.L + l] & active : 0u;
           u32 gat = 0;
-          const u32 ex = gather_row<NW, PER, EARLY, AM == AM_LANE>(p, F, bits, lfrom, beg, end, lane_off, lane_on,
+          const u32 ex = gather_row<NW, PER, true, AM == AM_LANE>(p, F, bits, lfrom, beg, end, lane_off, lane_on,
                                                                    sg_mask, vis, acc, gat,
                                                                    p.la_in_t + (u64)j * Q);
           edges += (li == 0) ? ex : 0;
@@ -897,31 +1545,19 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
         for (int k = 0; k < PER; k++) full &= vis[k] == ~0ull;
         return (__ballot_sync(FULL_MASK, full) & sg_mask) == sg_mask;
       };
-      bool work;
-      if constexpr (EARLY) {
-        // the gathers stop early on the visited words: read them first
-        const bool allv = all_visited();
-        work = any && !allv;
-        if (!__any_sync(FULL_MASK, work)) continue;
-        if (work) gather_all();
-      } else {
-        // the gathers do not read the visited words, so they are issued while
-        // those are in flight (a vertex whose lanes turn out all visited
-        // gathered for nothing: rare where many lanes never reach anything)
-        if (!__any_sync(FULL_MASK, any)) continue;
-        if (any) gather_all();
-        const bool allv = all_visited();
-        work = any && !allv;
-        if (!__any_sync(FULL_MASK, work)) continue;
-      }
+      // the gathers stop early on the visited words: read them first
+      const bool allv = all_visited();
+      const bool work = any && !allv;
+      if (!__any_sync(FULL_MASK, work)) continue;
+      if (work) gather_all();
       pull_finish<NW, PER>(p, app, FB, nlist, nxt, q2, w, stamp, li, lane_on && work, my_g, ((vh >> q2) & 1u) != 0,
                            vis, acc);
     }
     }
     if (p.pull_dynamic)
-      vit.next(&p.ctl->cursor[cur]);
+      c0 = next_item(&p.ctl->cursor[cur], n_warps, cv);
     else
-      vit.at += n_warps * cv;
+      c0 += n_warps * cv;
   }
 
   bool chunks_done = !chunked;
@@ -934,8 +1570,7 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
       u64 lact = 0;  // labels with an active transition
       for (u32 j = 0; j < p.q.in_begin[Q]; j++)
         if ((p.q.in_from[j] & active) && p.q.in_label[j] < p.L) lact |= 1ull << p.q.in_label[j];
-      for (Items hit(warp, n_warps, 1);; hit.next(&p.ctl->heavy_cursor[cur])) {
-        const u64 it = hit.at;
+      for (u64 it = warp;; it = next_item(&p.ctl->heavy_cursor[cur], n_warps, 1)) {
         u64 acc_base = 0, ci = 0;
         u32 ls = 0;
         bool found = false;
@@ -1023,8 +1658,7 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
     }
   }
   if (!chunks_done) {
-    for (Items hit(warp, n_warps, 1);; hit.next(&p.ctl->heavy_cursor[cur])) {
-      const u64 it = hit.at;
+    for (u64 it = warp;; it = next_item(&p.ctl->heavy_cursor[cur], n_warps, 1)) {
       // map the item number to (target state, transition group, chunk)
       u64 acc_base = 0, ci = 0;
       u32 q2s = 0, from = 0, ls = 0, js = 0;
@@ -1064,7 +1698,7 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
       u32 lfrom = from;
       if constexpr (AM == AM_GROUP) lfrom = lane_on ? p.from_tab[((u64)my_g * Q + q2s) * p.L + ls] & active : 0u;
       u32 gat = 0;
-      const u32 ex = gather_row<NW, PER, EARLY, AM == AM_LANE>(p, F, bits, lfrom, sb, se, lane_off, lane_on, sg_mask,
+      const u32 ex = gather_row<NW, PER, true, AM == AM_LANE>(p, F, bits, lfrom, sb, se, lane_off, lane_on, sg_mask,
                                                                vis, acc, gat, p.la_in_t + (u64)js * Q);
       for (u32 o = SW; o < 32; o <<= 1) {
 #pragma unroll
@@ -1079,9 +1713,9 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
     }
   }
   append_close(p, app, nlist);
-  stat[ST_PULL_EDGES] += warp_sum(edges);
-  stat[ST_PULL_VERTICES] += warp_sum(words);
-  stat[ST_ALG_BYTES] += warp_sum(bytes);
+  stat_add(stat, ST_PULL_EDGES, warp_sum(edges));
+  stat_add(stat, ST_PULL_VERTICES, warp_sum(words));
+  stat_add(stat, ST_ALG_BYTES, warp_sum(bytes));
 }
 
 // Commit of a level: fold the new frontier words into VIS, count work, note
@@ -1090,7 +1724,7 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
 // test its bitmap, so its bits are set; clear_bits: this level's bits were set.
 template <int NW, int AM>
 __device__ void commit_phase(const BfsParams &p, int lp, u32 nxt, u64 n_cur, u64 n_warps, bool set_bits,
-                             bool clear_bits, u64 *stat) {
+                             bool clear_bits, CommitSums &sums, u64 *stat) {
   const u64 *list = lp ? p.list1 : p.list0;
   const u64 *nlist = lp ? p.list0 : p.list1;
   u64 *F = lp ? p.fr1 : p.fr0;
@@ -1104,18 +1738,19 @@ __device__ void commit_phase(const BfsParams &p, int lp, u32 nxt, u64 n_cur, u64
   for (u64 j = tid; j < n_next; j += stride) {
     u64 e = __ldcg(&nlist[j]);
     if (e == NO_ENTRY) continue;
-    u32 gq = (u32)(e >> 32), w = (u32)e;
+    u32 gq = (u32)((e & ~ENTRY_DONE) >> 32), w = (u32)e;
     u32 g = gq / Q, q = gq - g * Q;
+    if (set_bits) {
+      const u64 bi = (u64)q * p.n + w;
+      atomicOr(p.fbits + (lp ? 0 : p.fbits_words) + (bi >> 5), 1u << (bi & 31));
+    }
+    if (e & ENTRY_DONE) continue;
     u64 wi = widx<NW>(p, g, q, w);
     Word<NW> m = load_cg<NW>(FB + wi);
     Word<NW> v = load_cg<NW>(p.vis + wi);
 #pragma unroll
     for (int t = 0; t < NW; t++) v.w[t] |= m.w[t];
     store_w<NW>(p.vis + wi, v);
-    if (set_bits) {
-      const u64 bi = (u64)q * p.n + w;
-      atomicOr(p.fbits + (lp ? 0 : p.fbits_words) + (bi >> 5), 1u << (bi & 31));
-    }
     u32 c = popc_w(m);
     u32 rows = 0, d;
     if constexpr (AM == AM_LANE) {
@@ -1136,7 +1771,7 @@ __device__ void commit_phase(const BfsParams &p, int lp, u32 nxt, u64 n_cur, u64
   for (u64 j = tid; j < n_cur; j += stride) {
     u64 e = __ldcg(&list[j]);
     if (e == NO_ENTRY) continue;
-    u32 gq = (u32)(e >> 32);
+    u32 gq = (u32)((e & ~ENTRY_DONE) >> 32);
     u32 g = gq / Q;
     store_w<NW>(F + widx<NW>(p, g, gq - g * Q, (u32)e), zero);
     if (clear_bits) {
@@ -1158,12 +1793,12 @@ __device__ void commit_phase(const BfsParams &p, int lp, u32 nxt, u64 n_cur, u64
   if (lane_id() == 0) {
     stat[ST_W] += W;
     stat[ST_N] += N;
-    stat[ST_GROUP_VERTICES] += gv;
-    if (mf) atomicAdd(&p.ctl->stats[ST_GROUP_W], mf);
-    if (gx) atomicAdd(&p.ctl->stats[ST_GROUP_X], gx);
-    if (mf) atomicAdd(&p.ctl->mf[nxt], mf);
-    if (gv) atomicAdd(&p.ctl->n_true[nxt], gv);
-    if (states) atomicOr(&p.ctl->smask[nxt], states);
+    if (gv) {
+      atomicAdd(&sums.mf, mf);
+      atomicAdd(&sums.gx, gx);
+      atomicAdd(&sums.n_true, gv);
+      atomicOr(&sums.smask, states);
+    }
   }
 }
 
@@ -1202,18 +1837,33 @@ constexpr u64 SOLO_SLOTS = 512, SOLO_EDGES = 512;
 constexpr u32 SOLO_RUN = 64;
 
 template <int NW, int AM>
-__global__ void __launch_bounds__(BFS_THREADS, 4) msbfs_kernel(const __grid_constant__ BfsParams p) {
-  // per-warp statistics, summed into the control block at the end
-  u64 stat[ST_COUNT];
-#pragma unroll
-  for (int i = 0; i < ST_COUNT; i++) stat[i] = 0;
+__global__ void __launch_bounds__(BFS_THREADS, AM == AM_LANE ? 3 : 4) msbfs_kernel(const __grid_constant__ BfsParams p) {
+  // per-warp statistics (lane 0 adds to them once per phase), summed into the
+  // control block at the end; in registers they were spilled by every phase
+  __shared__ u64 s_stat[BFS_THREADS / 32][ST_COUNT];
+  u64 *stat = s_stat[threadIdx.x >> 5];
+  if (lane_id() < ST_COUNT) stat[lane_id()] = 0;
+  __syncwarp();
   BfsCtl *c = p.ctl;
   unsigned epoch = 0;  // grid barriers passed
+  __shared__ CommitSums sums;
+  // per-warp scratch of the expansion phases: a push keeps its entries' words
+  // and rows there, lane mode its accumulators, pull_staged its lists
+  constexpr int SCRATCH = AM == AM_LANE ? LANE_SRC_Q * 2 * 32 + LANE_LIST : AM == AM_MANY ? STAGE : 32 * NW + 32;
+  __shared__ __align__(16) u64 s_scratch[BFS_THREADS / 32][SCRATCH];
+  u64 *scratch = s_scratch[threadIdx.x >> 5];
+  if (threadIdx.x == 0) sums = CommitSums{};  // seen by the block after the seeds' barrier
   const bool tracer = blockIdx.x == 0 && threadIdx.x == 0;
 
   seed_phase<NW, AM>(p, stat);
   if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
 
+  // lane mode: bottom-up levels by pull_lanes, whose lanes fill a warp's row.
+  // They cost less per byte than the estimate's: with its bytes taken at 0.4
+  // the batch above took 320 ms, at 1 342 ms (0.67: 343, 0.33 .. 0.17: 320).
+  constexpr float LANES_PULL = 0.4f;
+  const bool lanes_staged =
+      AM == AM_LANE && NW == 4 && p.lane_by_source && p.Q <= LANE_SRC_Q && p.G * NW / 2 > 16;
   u32 level = 0, run = 0;  // run: levels left of block 0's run, 0 outside one
   for (;; level++) {
     const u32 cur = level % 3, nxt = (level + 1) % 3, old = (level + 2) % 3;
@@ -1235,8 +1885,9 @@ __global__ void __launch_bounds__(BFS_THREADS, 4) msbfs_kernel(const __grid_cons
       run = SOLO_RUN;
     }
     const float push_cost = (float)mf * (4.0f + 8.0f * NW) + (float)n_true * (16.0f + 8.0f * NW);
-    const bool push =
-        solo || p.force == 1 || (p.force != 2 && p.alpha * push_cost < pull_bytes<NW>(p, active));
+    float pull_cost = pull_bytes<NW>(p, active);
+    if (lanes_staged) pull_cost *= LANES_PULL;
+    const bool push = solo || p.force == 1 || (p.force != 2 && p.alpha * push_cost < pull_cost);
     if (tracer) {
       // counters of the level after next start at zero
       c->n_list[old] = 0;
@@ -1253,6 +1904,8 @@ __global__ void __launch_bounds__(BFS_THREADS, 4) msbfs_kernel(const __grid_cons
         c->trace_mode[level] = push ? 1u : 2u;
         c->trace_mf[level] = mf;
       }
+      stat[ST_GROUP_W] += mf;
+      stat[ST_GROUP_VERTICES] += n_true;
       if (push)
         stat[ST_PUSH_LEVELS] += 1;
       else
@@ -1264,7 +1917,8 @@ __global__ void __launch_bounds__(BFS_THREADS, 4) msbfs_kernel(const __grid_cons
       // no out-edges: the next frontier is empty, only this one is cleared
     } else if (push) {
       const u32 seg = mf < PUSH_EXACT ? 0u : p.append_seg;
-      push_level<NW, AM>(p, lp, cur, nxt, n_cur, n_warps, run ? ~0u : spill_chunk(mf, n_warps), seg, stamp, stat);
+      push_level<NW, AM>(p, lp, cur, nxt, n_cur, n_warps, run ? ~0u : spill_chunk(mf, n_warps), seg, stamp, scratch,
+                         stat);
       if (run) {
         __syncthreads();
       } else {
@@ -1279,13 +1933,21 @@ __global__ void __launch_bounds__(BFS_THREADS, 4) msbfs_kernel(const __grid_cons
       // (implies n_cur * 4 < n * Q, so the commit that built this frontier set its bits)
       const bool sparse = p.fbits && n_cur * 4 < (u64)p.n * __popc(active);
       const u32 *bits = sparse ? p.fbits + (lp ? p.fbits_words : 0) : nullptr;
-      // early exit pays where few lanes are live: one lane group, the
-      // per-group automata of a multi launch (typically one start vertex
-      // each), or per-lane automata (lanes of short queries go quiet early)
-      if (p.G == 1 || AM != AM_ONE)
-        pull_level<NW, true, AM>(p, lp, cur, nxt, active, stamp, bits, stat);
-      else
-        pull_level<NW, false, AM>(p, lp, cur, nxt, active, stamp, bits, stat);
+      // pull_level's early exit pays where few lanes are live: one lane
+      // group, the per-group automata of a multi launch (typically one start
+      // vertex each), or per-lane automata (lanes of short queries go quiet
+      // early)
+      if constexpr (AM == AM_MANY) {
+        pull_staged<NW>(p, lp, cur, nxt, active, stamp, bits, scratch, sums, stat);
+      } else if constexpr (AM == AM_LANE && NW == 4) {
+        __shared__ LaneTables tab;
+        if (lanes_staged)
+          pull_lanes<NW>(p, lp, cur, nxt, active, stamp, bits, scratch, tab, stat);
+        else
+          pull_level<NW, AM>(p, lp, cur, nxt, active, stamp, bits, scratch, stat);
+      } else {
+        pull_level<NW, AM>(p, lp, cur, nxt, active, stamp, bits, scratch, stat);
+      }
       if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
     }
     {
@@ -1296,8 +1958,10 @@ __global__ void __launch_bounds__(BFS_THREADS, 4) msbfs_kernel(const __grid_cons
       const bool set_bits = p.fbits && n_next * 4 < sparse_cap;
       const bool clear_bits = p.fbits && (level == 0 || n_cur * 4 < sparse_cap);
       if (tracer && level < (u32)TRACE_LEVELS) c->trace_c[level] = globaltimer_ns();
-      commit_phase<NW, AM>(p, lp, nxt, n_cur, n_warps, set_bits, clear_bits, stat);
+      commit_phase<NW, AM>(p, lp, nxt, n_cur, n_warps, set_bits, clear_bits, sums, stat);
       if (run) {
+        __syncthreads();
+        if (threadIdx.x == 0) publish_sums(c, sums, nxt);
         __syncthreads();
         const u64 mf_next = *(volatile unsigned long long *)&c->mf[nxt];
         if (--run == 0 || n_next == 0 || n_next > SOLO_SLOTS || mf_next > SOLO_EDGES) {
@@ -1308,13 +1972,11 @@ __global__ void __launch_bounds__(BFS_THREADS, 4) msbfs_kernel(const __grid_cons
         continue;
       }
     }
-    if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
+    if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns, [&] { publish_sums(c, sums, nxt); })) return;
   }
-  if (lane_id() == 0) {
-#pragma unroll
-    for (int i = 0; i < ST_COUNT; i++)
-      if (stat[i]) atomicAdd(&c->stats[i], stat[i]);
-  }
+  if (threadIdx.x == 0 && sums.gx) atomicAdd(&c->stats[ST_GROUP_X], sums.gx);
+  __syncwarp();
+  if (lane_id() < ST_COUNT && stat[lane_id()]) atomicAdd(&c->stats[lane_id()], stat[lane_id()]);
   if (tracer) {
     c->levels = level;
     c->trace_t[level < (u32)TRACE_LEVELS ? level : TRACE_LEVELS] = globaltimer_ns();
@@ -1397,9 +2059,10 @@ cudaError_t launch_source_filter(const uint32_t *off, uint32_t n, uint32_t L, un
 
 cudaError_t launch_msbfs(int nw, const BfsParams &p, int blocks, int threads, cudaStream_t st) {
   void *args[] = {(void *)&p};
-  if (nw == 1)
-    return cudaLaunchCooperativeKernel((void *)msbfs_kernel<1, AM_ONE>, blocks, threads, args, 0, st);
-  return cudaLaunchCooperativeKernel((void *)msbfs_kernel<4, AM_ONE>, blocks, threads, args, 0, st);
+  void *kernel = nw == 1   ? (void *)msbfs_kernel<1, AM_ONE>
+                 : p.G == 1 ? (void *)msbfs_kernel<4, AM_ONE>
+                            : (void *)msbfs_kernel<4, AM_MANY>;
+  return cudaLaunchCooperativeKernel(kernel, blocks, threads, args, 0, st);
 }
 
 int msbfs_max_blocks(int nw, int threads, int *blocks_per_sm, int *sms) {

@@ -50,18 +50,12 @@ __device__ __forceinline__ u64 grid_warps() { return ((u64)gridDim.x * blockDim.
 // item is its own (warp * step), the next ones come from the phase's cursor.
 // Phases with fewer items than warps touch no cursor: the 4,864 warps of a
 // full grid asking one counter for nothing took 8-10 us.
-struct Items {
-  u64 at;        // first item of the current grab
-  u64 n_first;   // items handed out by warp number
-  u32 step;
-  __device__ __forceinline__ Items(u64 warp, u64 n_warps, u32 step_)
-      : at(warp * step_), n_first(n_warps * step_), step(step_) {}
-  // warp-uniform; all lanes call it
-  __device__ __forceinline__ void next(unsigned long long *cursor) {
-    u64 t = 0;
-    if (lane_id() == 0) t = atomicAdd(cursor, (unsigned long long)step);
-    at = n_first + __shfl_sync(FULL_MASK, t, 0);
-  }
-};
+// next_item: the first item of the warp's next grab (warp-uniform, all lanes
+// call it).
+__device__ __forceinline__ u64 next_item(unsigned long long *cursor, u64 n_warps, u32 step) {
+  u64 t = 0;
+  if (lane_id() == 0) t = atomicAdd(cursor, (unsigned long long)step);
+  return n_warps * step + __shfl_sync(FULL_MASK, t, 0);
+}
 
 }  // namespace rpq

@@ -108,14 +108,14 @@ struct BfsCtl {
   unsigned int bar_flag[32];
   unsigned int err;
   unsigned int err_where;
-  unsigned long long n_list[3];
-  unsigned long long cursor[3];
-  unsigned long long mf[3];
-  unsigned long long n_true[3];        // frontier entries without the lists' unused slots
+  alignas(128) unsigned long long n_list[3];
+  alignas(128) unsigned long long cursor[3];
+  alignas(128) unsigned long long mf[3];  // frontier out-edges
+  alignas(128) unsigned long long n_true[3];  // frontier entries without the lists' unused slots
   unsigned long long spill_count[3];   // top-down row chunks queued this level
   unsigned long long spill_cursor[3];
   unsigned long long heavy_cursor[3];  // bottom-up row chunks taken
-  unsigned int smask[3];               // DFA states present in each frontier
+  alignas(128) unsigned int smask[3];  // DFA states present in each frontier
   unsigned int next_level;             // first level after a run of one-block levels
   unsigned long long levels;
   unsigned long long stats[ST_COUNT];
@@ -197,6 +197,10 @@ struct BfsParams {
   const unsigned short *la_grp_begin;
   const unsigned int *la_grp;
   const unsigned long long *la_gmask;
+  // la_sl[s * L + l] (unions of at most 8 states): first transition of (state
+  // s, label l) | the set of its targets << 16; its transitions are
+  // consecutive, targets ascending
+  const unsigned int *la_sl;
   BfsCtl *ctl;
   unsigned int stamp_base;     // claim stamps continue across launches
   unsigned int nblocks;
@@ -223,6 +227,17 @@ cudaError_t launch_vis_init_lane(int nw, const BfsParams &p, const unsigned long
 cudaError_t launch_source_filter(const uint32_t *off, uint32_t n, uint32_t L, unsigned long long label_mask,
                                  const uint32_t *srcs, unsigned long long count, unsigned char *flag,
                                  cudaStream_t st);
+// Blocks of a traversal launch over n vertices: enough that a bottom-up level
+// gives every sub-warp a vertex (the lanes it uses per vertex, two words each,
+// rounded up to a power of two), at most max_blocks.  More blocks only make
+// the barriers of a small graph's levels dearer.
+inline int bfs_grid(int max_blocks, int nw, uint32_t G, uint32_t n) {
+  const uint32_t lanes = nw == 1 ? G : G * nw / 2;
+  uint64_t sw = 1;
+  while (sw < lanes) sw <<= 1;
+  const uint64_t want = (n * sw + 255) / 256;
+  return want < (uint64_t)max_blocks ? (int)want : max_blocks;
+}
 int msbfs_max_blocks(int nw, int threads, int *blocks_per_sm, int *sms);
 
 struct EmitParams {

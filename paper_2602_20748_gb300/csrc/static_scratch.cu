@@ -185,7 +185,8 @@ extern "C" int run_rpq_static(rpq_ctx *ctx, const rpq_graph *g, const rpq_query 
   p.stamp_base = 0;
   const int blocks = ctx_bfs_blocks(ctx, 1);
   if (blocks <= 0) return ctx_error(ctx, RPQ_ERR_CUDA, "traversal kernel cannot be made resident");
-  p.nblocks = (unsigned)blocks;
+  const int grid = bfs_grid(blocks, 1, 1, n);
+  p.nblocks = (unsigned)grid;
   p.force = 0;
   p.alpha = ctx_alpha(ctx);
   p.pull_dynamic = 1;
@@ -195,7 +196,7 @@ extern "C" int run_rpq_static(rpq_ctx *ctx, const rpq_graph *g, const rpq_query 
   p.time_limit_ns = ctx_time_limit_ns(ctx);
   p.q = qd;
   STATIC_CK(launch_vis_init(1, p, empty, st));
-  STATIC_CK(launch_msbfs(1, p, blocks, 256, st));
+  STATIC_CK(launch_msbfs(1, p, grid, 256, st));
 
   EmitParams ep{};
   ep.vis = vis;

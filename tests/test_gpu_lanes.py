@@ -150,3 +150,20 @@ def test_lanes_gather_order_match_oracle(by_source):
     regexes, sources = _mix(300, L, src, n, seed=93)
     r = _check(c, g, og, regexes, sources)
     assert rpq.result_stats(r)["evicted"] == len(regexes)
+
+
+@pytest.mark.parametrize("n_q,alpha", [(2400, 2), (2305, 1e9), (4000, 1e9)])
+def test_lanes_filling_a_warps_row_match_oracle(n_q, alpha):
+    """More than 2,304 lanes: bottom-up levels list their gathers (10 to 16
+    lane groups, the last one partly filled), with hub rows in chunks, dense
+    and sparse frontiers; the automatic direction and bottom-up only."""
+    n = 1500
+    src, dst, lab = _graph(n, 6000, 4, seed=91, hubs=True)
+    c = rpq.Context(device=0)
+    rpq.rpq_set_option(c, "batch_direct", 1)
+    rpq.rpq_set_option(c, "lane_alpha", alpha)
+    g = rpq.load_graph(c, n, 4, src, dst, lab)
+    og = oracle.Graph(n, 4, src, dst, lab)
+    regexes, sources = _mix(n_q, 4, src, n, seed=92 + n_q)
+    r = _check(c, g, og, regexes, sources)
+    assert rpq.result_stats(r)["pull_levels"] > 0
