@@ -298,12 +298,13 @@ void free_chunk(rpq_ctx *ctx, Chunk &c) {
 // min_len destinations, longest first, while the bitsets take at most half of
 // the budget left, and allocates them into c.  Returns the lanes' slots on
 // the host (NO_SOURCE: listed only).
-int pick_bit_lanes(rpq_ctx *ctx, const RowBitsReq &req, const u64 *off, uint32_t segs, uint32_t n, Chunk &c) {
+int pick_bit_lanes(rpq_ctx *ctx, const RowBitsReq &req, const u64 *off, uint32_t segs, uint32_t live, uint32_t n,
+                   Chunk &c) {
   std::vector<u64> lane_off(c.n_lanes + 1);
   u64 *d_lane_off = nullptr;
   int rc;
   if ((rc = dalloc(ctx, &d_lane_off, (uint64_t)c.n_lanes + 1))) return rc;
-  cudaError_t e = launch_gather_lane_off(off, segs, c.n_lanes, ctx->small + 2, d_lane_off, ctx->stream);
+  cudaError_t e = launch_gather_lane_off(off, segs, c.n_lanes, live, ctx->small + 2, d_lane_off, ctx->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(lane_off.data(), d_lane_off, lane_off.size() * 8, cudaMemcpyDeviceToHost, ctx->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
@@ -439,14 +440,14 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
     if (rc) return rc;
   }
   Workspace &w = ctx->ws;
-  const uint32_t segs = (n + EMIT_SEG - 1) / EMIT_SEG;
-
   std::vector<uint32_t> lanes;
   std::vector<uint64_t> empty;
   for (uint64_t g0 = 0; g0 < groups_total; g0 += G) {
     if (ctx->cancel.load(std::memory_order_relaxed)) return set_err(ctx, RPQ_ERR_CANCELLED, "cancelled");
     const uint32_t Gb = (uint32_t)std::min<uint64_t>(G, groups_total - g0);
     const uint32_t n_lanes = Gb * K;
+    const uint32_t live = (uint32_t)std::min<uint64_t>(n_lanes, srcs.size() - g0 * K);  // the others are empty
+    const uint32_t tiles = emit_tiles(nw, Gb, n), segs = emit_segs(tiles, n);
     lanes.assign(n_lanes, NO_SOURCE);
     empty.assign((size_t)Gb * nw, 0);
     for (uint32_t i = 0; i < n_lanes; i++) {
@@ -520,6 +521,7 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
       ep.Q = Q;
       ep.final_mask = qd.final_mask;
       ep.lanesrc = w.lanesrc;
+      ep.tiles = tiles;
       ep.segs = segs;
       CK(cudaMemsetAsync(ls, 0, 24ull * n_lanes, ctx->stream));
       CK(cudaEventRecord(ctx->ev[2], ctx->stream));
@@ -571,6 +573,7 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
     u32 *cnt = nullptr;
     u64 *off = nullptr, *tmp = nullptr;
     const uint64_t ncnt = (uint64_t)n_lanes * segs;
+    const uint64_t nscan = (uint64_t)live * segs;
     const uint64_t tmpw = scan_tmp_words(ncnt);
     int rc;
     if ((rc = dalloc(ctx, &cnt, ncnt)) || (rc = dalloc(ctx, &off, ncnt)) || (rc = dalloc(ctx, &tmp, tmpw))) {
@@ -586,6 +589,7 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
     ep.Q = Q;
     ep.final_mask = qd.final_mask;
     ep.lanesrc = w.lanesrc;
+    ep.tiles = tiles;
     ep.segs = segs;
     ep.cnt = cnt;
     ep.off = off;
@@ -594,7 +598,7 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
     CK(cudaMemsetAsync(ctx->small, 0, 3 * 8, ctx->stream));
     CK(cudaEventRecord(ctx->ev[2], ctx->stream));
     CK(launch_emit(nw, false, !materialize, ep, ctx->stream));
-    CK(exclusive_scan_u32_to_u64(cnt, off, ncnt, ctx->small + 2, tmp, ctx->stream));
+    CK(exclusive_scan_u32_to_u64(cnt, off, nscan, ctx->small + 2, tmp, ctx->stream));
     res->stats.launches += 2;
     BfsCtl hctl;
     u64 hsmall[3];
@@ -649,7 +653,7 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
       c.n_lanes = n_lanes;
       c.rows = total;
       if (bits_req) {
-        if ((rc = pick_bit_lanes(ctx, *bits_req, off, segs, n, c))) {
+        if ((rc = pick_bit_lanes(ctx, *bits_req, off, segs, live, n, c))) {
           free_chunk(ctx, c);
           dfree(ctx, cnt, ncnt);
           dfree(ctx, off, ncnt);
@@ -664,7 +668,7 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
           // bitset rows are not listed: offsets of the listed rows only
           u64 listed = 0;
           CK(launch_zero_lane_counts(cnt, segs, n_lanes, c.lane_slot, ctx->stream));
-          CK(exclusive_scan_u32_to_u64(cnt, off, ncnt, ctx->small + 2, tmp, ctx->stream));
+          CK(exclusive_scan_u32_to_u64(cnt, off, nscan, ctx->small + 2, tmp, ctx->stream));
           CK(cudaMemcpyAsync(&listed, ctx->small + 2, 8, cudaMemcpyDeviceToHost, ctx->stream));
           CK(cudaStreamSynchronize(ctx->stream));
           c.rows = listed;
@@ -681,10 +685,10 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
       }
       ep.dst = c.dst;
       CK(launch_emit(nw, true, false, ep, ctx->stream));
-      CK(launch_gather_lane_off(off, segs, n_lanes, ctx->small + 2, c.lane_off, ctx->stream));
+      CK(launch_gather_lane_off(off, segs, n_lanes, live, ctx->small + 2, c.lane_off, ctx->stream));
       CK(cudaMemcpyAsync(c.lanesrc, w.lanesrc, n_lanes * 4, cudaMemcpyDeviceToDevice, ctx->stream));
       // digest of the written rows (a block per source lane)
-      CK(launch_row_digest(w.lanesrc, c.lane_off, n_lanes, c.dst, ctx->small, ctx->stream));
+      CK(launch_row_digest(w.lanesrc, c.lane_off, live, c.dst, ctx->small, ctx->stream));
       res->chunks.push_back(c);
       CK(rb_queue(ctx, RB_SMALL, ctx->small, 16));
       res->stats.launches += 4;
@@ -1804,7 +1808,8 @@ int rpq_lane_stats_multi(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Mu
   ep.final_mask = un.final_mask;
   ep.final_g = d_fin;
   ep.lanesrc = w.lanesrc;
-  ep.segs = (n + EMIT_SEG - 1) / EMIT_SEG;
+  ep.tiles = emit_tiles(1, G, n);
+  ep.segs = emit_segs(ep.tiles, n);
   BfsCtl hctl;
   std::vector<uint64_t> hls(3ull * G * 64);
   if ((e = launch_vis_init(1, p, w.empty, st)) == cudaSuccess && (e = cudaMemsetAsync(ctx->ctl, 0, sizeof(BfsCtl), st)) == cudaSuccess &&
@@ -2077,7 +2082,8 @@ static int lane_launch(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Lane
   ep.final_mask = un.final_mask;
   ep.final_lane = reinterpret_cast<const unsigned long long *>(dt + o_fin);
   ep.lanesrc = w.lanesrc;
-  ep.segs = (n + EMIT_SEG - 1) / EMIT_SEG;
+  ep.tiles = emit_tiles(nw, G, n);
+  ep.segs = emit_segs(ep.tiles, n);
   BfsCtl hctl;
   std::vector<uint64_t> hls(3ull * G * K);
   if ((e = launch_vis_init_lane(nw, p, reinterpret_cast<const u64 *>(dt + o_emp), st)) == cudaSuccess &&

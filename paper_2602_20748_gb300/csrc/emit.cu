@@ -4,7 +4,7 @@
 // set of v with some accepting state q such that s's lane is set in the
 // visited word of (group g, state q, vertex v).  For lane group g, OR the
 // accepting states' words into a K-bit result word per vertex.  A block owns
-// a segment of EMIT_SEG vertices of one group and walks it in batches of
+// a segment of p.tiles * 32 vertices of one group and walks it in batches of
 // EMIT_BATCH 32-vertex tiles.  The block loads a batch cooperatively, whole
 // 32-byte sectors at a time (a vertex's K lane bits of the group are one
 // contiguous run), into shared memory laid out by lane column; warp c then
@@ -105,8 +105,8 @@ __device__ __forceinline__ void batch_store(const u64 (&pre)[4], u32 *s_vis) {
   }
 }
 
-__device__ __forceinline__ void digest_add(u64 src, u32 y, u64 &hsum, u64 &hxor) {
-  const u64 h = splitmix64(src | (u64)y);
+__device__ __forceinline__ void digest_add(const RowHash &rh, u32 y, u64 &hsum, u64 &hxor) {
+  const u64 h = rh(y);
   hsum += h;
   hxor ^= h;
 }
@@ -167,9 +167,9 @@ __global__ void __launch_bounds__(64 * NW, NW == 1 ? 16 : 4) emit_count_kernel(c
   const u64 glane = (u64)g * (64 * NW) + col * 32 + lane;
   const u32 src = p.lanesrc[glane];
   const u32 valid_cols = __ballot_sync(FULL_MASK, src != NO_SOURCE);
-  const u64 src_hi = (u64)src << 32;
-  const u32 w_begin = seg * EMIT_SEG;
-  const u32 n_tiles = min((u32)EMIT_TILES, (p.n - w_begin + 31) / 32);
+  const RowHash rh(src);
+  const u32 w_begin = seg * p.tiles * 32;
+  const u32 n_tiles = min(p.tiles, (p.n - w_begin + 31) / 32);
   constexpr int CNT_PLANES = 8;  // EMIT_TILES <= 2^CNT_PLANES - 1 vertices per thread
   static_assert(EMIT_TILES < (1 << CNT_PLANES), "count planes too narrow");
   u32 planes[CNT_PLANES];
@@ -190,7 +190,7 @@ __global__ void __launch_bounds__(64 * NW, NW == 1 ? 16 : 4) emit_count_kernel(c
         u32 m = warp_transpose32(x);
         cnt += __popc(m);
         const u32 w0 = w_begin + (tb + t) * 32;
-        for (; m; m &= m - 1) digest_add(src_hi, w0 + __ffs(m) - 1, hsum, hxor);
+        for (; m; m &= m - 1) digest_add(rh, w0 + __ffs(m) - 1, hsum, hxor);
       } else {
         u32 carry = x;
 #pragma unroll
@@ -241,8 +241,8 @@ __global__ void __launch_bounds__(64 * NW, NW == 1 ? 16 : 3) emit_write_kernel(c
     if (slot != NO_SOURCE) bs = reinterpret_cast<u32 *>(p.bits + (u64)slot * p.bwords);
   }
   const bool listed = !bs || p.keep_lists;
-  const u32 w_begin = seg * EMIT_SEG;
-  const u32 n_tiles = min((u32)EMIT_TILES, (p.n - w_begin + 31) / 32);
+  const u32 w_begin = seg * p.tiles * 32;
+  const u32 n_tiles = min(p.tiles, (p.n - w_begin + 31) / 32);
   u64 pre[4];
   batch_fetch<NW>(p, p.final_mask, g, w_begin, min(EMIT_BATCH, n_tiles) * 32, pre);
   for (u32 tb = 0; tb < n_tiles; tb += EMIT_BATCH) {
@@ -311,54 +311,54 @@ cudaError_t launch_emit(int nw, bool write, bool digest, const EmitParams &p, cu
   return cudaGetLastError();
 }
 
-// Digest of a materialized chunk's rows: block b takes lanes b, b +
-// gridDim.x, ...; the rows of lane i are contiguous (dst[lane_off[i] ..
-// lane_off[i + 1])) and all belong to source lanesrc[i].  The 16-byte aligned
-// middle of a lane's rows is read four rows per load, two loads in flight per
-// thread; the unaligned ends row by row.
-__global__ void row_digest_kernel(const u32 *__restrict__ lanesrc, const u64 *__restrict__ lane_off, u32 n_lanes,
+// Digest of a materialized chunk's rows: block (b, y) takes part y of the rows
+// of lanes b, b + gridDim.x, ...; the rows of lane i are contiguous
+// (dst[lane_off[i] .. lane_off[i + 1])) and all belong to source lanesrc[i].
+// The 16-byte aligned middle of a part is read four rows per load, two loads
+// in flight per thread; the unaligned ends row by row.  Bound by the integer
+// operations of the hash (see RowHash).
+__global__ void row_digest_kernel(const u32 *__restrict__ lanesrc, const u64 *__restrict__ lane_off, u32 live,
                                   const u32 *__restrict__ dst, u64 *__restrict__ digest) {
   u64 hsum = 0, hxor = 0;
-  for (u32 i = blockIdx.x; i < n_lanes; i += gridDim.x) {
-    const u64 src = (u64)lanesrc[i] << 32;
-    const u64 b = lane_off[i], e = lane_off[i + 1];
+  for (u32 i = blockIdx.x; i < live; i += gridDim.x) {
+    const RowHash rh(lanesrc[i]);
+    const u64 lb = lane_off[i], len = lane_off[i + 1] - lb;
+    const u64 b = lb + len * blockIdx.y / gridDim.y, e = lb + len * (blockIdx.y + 1) / gridDim.y;
     const u64 ab = min(e, (b + 3) & ~3ull), ae = max(ab, e & ~3ull);  // aligned middle [ab, ae)
-    for (u64 r = b + threadIdx.x; r < ab; r += blockDim.x) digest_add(src, __ldcs(dst + r), hsum, hxor);
-    for (u64 r = ae + threadIdx.x; r < e; r += blockDim.x) digest_add(src, __ldcs(dst + r), hsum, hxor);
+    for (u64 r = b + threadIdx.x; r < ab; r += blockDim.x) digest_add(rh, __ldcs(dst + r), hsum, hxor);
+    for (u64 r = ae + threadIdx.x; r < e; r += blockDim.x) digest_add(rh, __ldcs(dst + r), hsum, hxor);
     const uint4 *v = reinterpret_cast<const uint4 *>(dst + ab);
     const u64 nv = (ae - ab) / 4;
     u64 k = threadIdx.x;
     for (; k + blockDim.x < nv; k += 2ull * blockDim.x) {
       const uint4 x0 = __ldcs(v + k), x1 = __ldcs(v + k + blockDim.x);
-      digest_add(src, x0.x, hsum, hxor);
-      digest_add(src, x0.y, hsum, hxor);
-      digest_add(src, x0.z, hsum, hxor);
-      digest_add(src, x0.w, hsum, hxor);
-      digest_add(src, x1.x, hsum, hxor);
-      digest_add(src, x1.y, hsum, hxor);
-      digest_add(src, x1.z, hsum, hxor);
-      digest_add(src, x1.w, hsum, hxor);
+      digest_add(rh, x0.x, hsum, hxor);
+      digest_add(rh, x0.y, hsum, hxor);
+      digest_add(rh, x0.z, hsum, hxor);
+      digest_add(rh, x0.w, hsum, hxor);
+      digest_add(rh, x1.x, hsum, hxor);
+      digest_add(rh, x1.y, hsum, hxor);
+      digest_add(rh, x1.z, hsum, hxor);
+      digest_add(rh, x1.w, hsum, hxor);
     }
     if (k < nv) {
       const uint4 x0 = __ldcs(v + k);
-      digest_add(src, x0.x, hsum, hxor);
-      digest_add(src, x0.y, hsum, hxor);
-      digest_add(src, x0.z, hsum, hxor);
-      digest_add(src, x0.w, hsum, hxor);
+      digest_add(rh, x0.x, hsum, hxor);
+      digest_add(rh, x0.y, hsum, hxor);
+      digest_add(rh, x0.z, hsum, hxor);
+      digest_add(rh, x0.w, hsum, hxor);
     }
   }
-  hsum = warp_sum(hsum);
-  hxor = warp_xor(hxor);
-  if (lane_id() == 0 && (hsum | hxor)) {
-    atomicAdd(&digest[0], hsum);
-    atomicXor(&digest[1], hxor);
-  }
+  digest_flush(hsum, hxor, digest);
 }
 
-cudaError_t launch_row_digest(const uint32_t *lanesrc, const unsigned long long *lane_off, uint32_t n_lanes,
+cudaError_t launch_row_digest(const uint32_t *lanesrc, const unsigned long long *lane_off, uint32_t live,
                               const uint32_t *dst, unsigned long long *digest, cudaStream_t st) {
-  if (n_lanes == 0) return cudaSuccess;
-  row_digest_kernel<<<n_lanes, 256, 0, st>>>(lanesrc, lane_off, n_lanes, dst, digest);
+  if (live == 0) return cudaSuccess;
+  // a block per lane fills the chip from 608 lanes on; fewer lanes are split
+  // (the one lane of a lookup's 250,000 rows took one block 190 us)
+  const uint32_t parts = live >= 608 ? 1 : std::min<uint32_t>(256, (1216 + live - 1) / live);
+  row_digest_kernel<<<dim3(live, parts), 256, 0, st>>>(lanesrc, lane_off, live, dst, digest);
   return cudaGetLastError();
 }
 
@@ -377,9 +377,9 @@ __global__ void __launch_bounds__(64 * NW, NW == 1 ? 16 : 4) emit_lane_stats_ker
   const u64 glane = (u64)g * (64 * NW) + col * 32 + lane;
   const u32 src = p.lanesrc[glane];
   const u32 valid_cols = __ballot_sync(FULL_MASK, src != NO_SOURCE);
-  const u64 src_hi = (u64)src << 32;
-  const u32 w_begin = seg * EMIT_SEG;
-  const u32 n_tiles = min((u32)EMIT_TILES, (p.n - w_begin + 31) / 32);
+  const RowHash rh(src);
+  const u32 w_begin = seg * p.tiles * 32;
+  const u32 n_tiles = min(p.tiles, (p.n - w_begin + 31) / 32);
   u64 cnt = 0, hsum = 0, hxor = 0;
   for (u32 tb = 0; tb < n_tiles; tb += EMIT_BATCH) {
     const u32 nt = min(EMIT_BATCH, n_tiles - tb);
@@ -394,7 +394,7 @@ __global__ void __launch_bounds__(64 * NW, NW == 1 ? 16 : 4) emit_lane_stats_ker
       u32 m = warp_transpose32(x);
       cnt += __popc(m);
       const u32 w0 = w_begin + (tb + t) * 32;
-      for (; m; m &= m - 1) digest_add(src_hi, w0 + __ffs(m) - 1, hsum, hxor);
+      for (; m; m &= m - 1) digest_add(rh, w0 + __ffs(m) - 1, hsum, hxor);
     }
   }
   if (cnt) {
@@ -417,7 +417,8 @@ cudaError_t launch_emit_lane_stats(int nw, const EmitParams &p, unsigned long lo
 // caller's buffer (used by the entry point that allocates nothing, at most 64
 // start vertices): tile by tile, the warp transpose gives each lane its
 // members in vertex order; row k goes to out[2k], out[2k + 1].
-template <int NW>
+// ALIGNED: out is 8-byte aligned, so that a row is one store.
+template <int NW, bool ALIGNED>
 __global__ void emit_pairs_kernel(const EmitParams p, u32 *__restrict__ out) {
   const u32 seg = blockIdx.x, g = blockIdx.y;
   const u32 col = threadIdx.x >> 5, lane = lane_id();
@@ -427,8 +428,8 @@ __global__ void emit_pairs_kernel(const EmitParams p, u32 *__restrict__ out) {
   const u32 valid_cols = __ballot_sync(FULL_MASK, src != NO_SOURCE);
   const u32 *vis32 = reinterpret_cast<const u32 *>(p.vis);
   u64 pos = p.off[glane * p.segs + seg];
-  const u32 w_begin = seg * EMIT_SEG;
-  for (u32 t = 0; t < EMIT_TILES; t++) {
+  const u32 w_begin = seg * p.tiles * 32;
+  for (u32 t = 0; t < p.tiles; t++) {
     const u32 w0 = w_begin + t * 32;
     if (w0 >= p.n) break;
     const u32 w = w0 + lane;
@@ -442,8 +443,13 @@ __global__ void emit_pairs_kernel(const EmitParams p, u32 *__restrict__ out) {
     }
     const u32 mine = warp_transpose32(x & valid_cols);
     for (u32 b = mine; b; b &= b - 1) {
-      out[2 * pos] = src;
-      out[2 * pos + 1] = w0 + (__ffs(b) - 1);
+      const u32 y = w0 + (__ffs(b) - 1);
+      if (ALIGNED) {
+        reinterpret_cast<uint2 *>(out)[pos] = make_uint2(src, y);
+      } else {
+        out[2 * pos] = src;
+        out[2 * pos + 1] = y;
+      }
       pos++;
     }
   }
@@ -451,22 +457,26 @@ __global__ void emit_pairs_kernel(const EmitParams p, u32 *__restrict__ out) {
 
 cudaError_t launch_emit_pairs(const EmitParams &p, uint32_t *out, cudaStream_t st) {
   dim3 grid(p.segs, p.G);
-  emit_pairs_kernel<1><<<grid, 64, 0, st>>>(p, out);
+  if (reinterpret_cast<uintptr_t>(out) % 8 == 0)
+    emit_pairs_kernel<1, true><<<grid, 64, 0, st>>>(p, out);
+  else
+    emit_pairs_kernel<1, false><<<grid, 64, 0, st>>>(p, out);
   return cudaGetLastError();
 }
 
 cudaError_t preload_static_emit_kernels() {
   cudaFuncAttributes a;
   cudaError_t e = cudaFuncGetAttributes(&a, emit_count_kernel<1, false>);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, emit_pairs_kernel<1>);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, emit_pairs_kernel<1, true>);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, emit_pairs_kernel<1, false>);
   return e;
 }
 
-// lane_off[i] = off[i * segs] for every lane; lane_off[n_lanes] = total.
-__global__ void gather_lane_off(const u64 *__restrict__ off, u32 segs, u32 n_lanes, const u64 *__restrict__ total,
+__global__ void gather_lane_off(const u64 *__restrict__ off, u32 segs, u32 n_lanes, u32 live,
+                                const u64 *__restrict__ total,
                                 u64 *__restrict__ lane_off) {
   for (u32 i = blockIdx.x * blockDim.x + threadIdx.x; i <= n_lanes; i += gridDim.x * blockDim.x)
-    lane_off[i] = (i == n_lanes) ? *total : off[(u64)i * segs];
+    lane_off[i] = i >= live ? *total : off[(u64)i * segs];
 }
 
 __global__ void zero_lane_counts(u32 *__restrict__ cnt, u32 segs, u32 n_lanes, const u32 *__restrict__ lane_slot) {
@@ -482,9 +492,9 @@ cudaError_t launch_zero_lane_counts(u32 *cnt, u32 segs, u32 n_lanes, const u32 *
   return cudaGetLastError();
 }
 
-cudaError_t launch_gather_lane_off(const u64 *off, u32 segs, u32 n_lanes, const u64 *total, u64 *lane_off,
+cudaError_t launch_gather_lane_off(const u64 *off, u32 segs, u32 n_lanes, u32 live, const u64 *total, u64 *lane_off,
                                    cudaStream_t st) {
-  gather_lane_off<<<(n_lanes + 256) / 256, 256, 0, st>>>(off, segs, n_lanes, total, lane_off);
+  gather_lane_off<<<(n_lanes + 256) / 256, 256, 0, st>>>(off, segs, n_lanes, live, total, lane_off);
   return cudaGetLastError();
 }
 

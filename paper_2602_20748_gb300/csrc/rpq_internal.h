@@ -247,6 +247,7 @@ struct EmitParams {
   uint32_t Q;
   uint32_t final_mask;
   const uint32_t *lanesrc;
+  uint32_t tiles;                // 32-vertex tiles per segment (emit_tiles)
   uint32_t segs;                 // segments per group
   uint32_t *cnt;                 // [G * K][segs]
   const unsigned long long *off; // exclusive offsets of cnt (write pass)
@@ -267,12 +268,27 @@ struct EmitParams {
   uint64_t bwords;
   uint32_t keep_lists;
 };
-constexpr int EMIT_TILES = 128;  // 32-vertex tiles per segment
+constexpr int EMIT_TILES = 128;  // 32-vertex tiles per segment at most
+constexpr int EMIT_TILES_MIN = 8;
 constexpr int EMIT_SEG = 32 * EMIT_TILES;
+// Tiles per segment for a launch of G groups over n vertices, a block per
+// segment and group: as long as possible (a row's first and last 32 words in
+// a segment are stored word by word), but short enough for two blocks (12 of
+// the two-warp blocks of nw = 1) per residency slot of the write pass.  With
+// 4,096-vertex segments 300 sources on 65,537 vertices ran on 34 blocks, one
+// source on R-MAT 2^20 on 256 blocks of two warps.
+inline uint32_t emit_tiles(int nw, uint32_t G, uint32_t n) {
+  const uint64_t want = nw == 1 ? 152ull * 12 : 152ull * 6;
+  uint32_t t = EMIT_TILES;
+  while (t > EMIT_TILES_MIN && ((uint64_t)n + 32 * t - 1) / (32 * t) * G < want) t >>= 1;
+  return t;
+}
+inline uint32_t emit_segs(uint32_t tiles, uint32_t n) { return (uint32_t)(((uint64_t)n + 32 * tiles - 1) / (32 * tiles)); }
 cudaError_t launch_emit(int nw, bool write, bool digest, const EmitParams &p, cudaStream_t st);
 // Digest (sum, xor of splitmix64(src << 32 | dst)) of a materialized chunk's
 // rows, added into digest[0..1].
-cudaError_t launch_row_digest(const uint32_t *lanesrc, const unsigned long long *lane_off, uint32_t n_lanes,
+// live: the lanes that may have rows (the first ones).
+cudaError_t launch_row_digest(const uint32_t *lanesrc, const unsigned long long *lane_off, uint32_t live,
                               const uint32_t *dst, unsigned long long *digest, cudaStream_t st);
 // Per-lane row count and digest (lane_stats[3 * lane + {0, 1, 2}] = rows,
 // digest sum, digest xor over the lane's (source, y) rows); lane_stats zeroed
@@ -291,7 +307,9 @@ cudaError_t preload_scan_kernels();
 // cnt[lane][*] = 0 for every lane with lane_slot[lane] != NO_SOURCE.
 cudaError_t launch_zero_lane_counts(uint32_t *cnt, uint32_t segs, uint32_t n_lanes, const uint32_t *lane_slot,
                                     cudaStream_t st);
-cudaError_t launch_gather_lane_off(const unsigned long long *off, uint32_t segs, uint32_t n_lanes,
+// lane_off[i] = off[i * segs] for the first `live` lanes, *total from there to
+// lane_off[n_lanes] (lanes without a start vertex are the last ones).
+cudaError_t launch_gather_lane_off(const unsigned long long *off, uint32_t segs, uint32_t n_lanes, uint32_t live,
                                    const unsigned long long *total, unsigned long long *lane_off, cudaStream_t st);
 
 // Pair expansion for fetch: out[2k], out[2k+1] = (src, dst) of row first + k.

@@ -22,6 +22,7 @@
 // threads, other streams of the same device) race with each other; callers
 // serialize them.  The array keeps the previous call's contents; everything a
 // call needs zeroed is cleared by the call itself.
+#include <algorithm>
 #include <cstring>
 
 #include "crpq.h"
@@ -109,7 +110,11 @@ extern "C" int run_rpq_static(rpq_ctx *ctx, const rpq_graph *g, const rpq_query 
   const uint32_t Q = qd.n_states;
   if (Q == 0) return RPQ_OK;  // empty language: no rows
   const uint32_t n = dg.n;
-  const uint32_t segs = (n + EMIT_SEG - 1) / EMIT_SEG;
+  // the longest emission segments need the least; shorter ones where they fit
+  uint32_t tiles = emit_tiles(1, 1, n);
+  while (tiles < (uint32_t)EMIT_TILES && static_scratch_need(Q, n, emit_segs(tiles, n)) > STATIC_SCRATCH_BYTES)
+    tiles <<= 1;
+  const uint32_t segs = emit_segs(tiles, n);
   const size_t need = static_scratch_need(Q, n, segs);
   if (need > STATIC_SCRATCH_BYTES)
     return ctx_error(ctx, RPQ_ERR_OUT_OF_BUDGET,
@@ -181,6 +186,11 @@ extern "C" int run_rpq_static(rpq_ctx *ctx, const rpq_graph *g, const rpq_query 
   p.list1 = list1;
   p.list_cap = words;  // one append per (state, vertex) per level (no segments here)
   p.append_seg = 0;
+  // what the query leaves of the array holds the chunk records of long
+  // top-down rows; rows whose chunks do not fit are processed in place
+  p.spill = (u64 *)(base + at);
+  p.spill_cap = std::min<size_t>(SPILL_CAP, (STATIC_SCRATCH_BYTES - at) / (3 * sizeof(u64)));
+  if (p.spill_cap == 0) p.spill = nullptr;
   p.ctl = ctl;
   p.stamp_base = 0;
   const int blocks = ctx_bfs_blocks(ctx, 1);
@@ -191,7 +201,11 @@ extern "C" int run_rpq_static(rpq_ctx *ctx, const rpq_graph *g, const rpq_query 
   p.alpha = ctx_alpha(ctx);
   p.pull_dynamic = 1;
   p.lane_by_source = 1;
-  p.hchunk = nullptr;  // long rows are scanned in place
+  // chunks of long in-rows belong to the graph: scanned in place, one lane
+  // walked a row of up to 10^4 edges alone (64 start vertices on R-MAT 2^18:
+  // 3.2 ms a call)
+  p.hchunk = dg.hchunk_in;
+  for (uint32_t l = 0; l <= dg.L && l < dg.hchunk_in_off.size(); l++) p.hchunk_off[l] = dg.hchunk_in_off[l];
   for (uint32_t l = 0; l < dg.L; l++) p.label_edges[l] = dg.label_edges[l];
   p.time_limit_ns = ctx_time_limit_ns(ctx);
   p.q = qd;
@@ -205,13 +219,14 @@ extern "C" int run_rpq_static(rpq_ctx *ctx, const rpq_graph *g, const rpq_query 
   ep.Q = Q;
   ep.final_mask = qd.final_mask;
   ep.lanesrc = lanesrc;
+  ep.tiles = tiles;
   ep.segs = segs;
   ep.cnt = cnt;
   ep.off = off;
   ep.dst = nullptr;
   ep.digest = small;
   STATIC_CK(launch_emit(1, false, false, ep, st));
-  STATIC_CK(exclusive_scan_u32_to_u64(cnt, off, (size_t)64 * segs, small + 2, tmp, st));
+  STATIC_CK(exclusive_scan_u32_to_u64(cnt, off, (size_t)ns * segs, small + 2, tmp, st));
   unsigned int err = 0;
   u64 total = 0;
   STATIC_CK(cudaMemcpyAsync(&err, &ctl->err, sizeof(err), cudaMemcpyDeviceToHost, st));
