@@ -137,7 +137,8 @@ int rpq_set_stream(rpq_ctx *ctx, void *cuda_stream);
  *   "max_groups"   lane groups (256 start vertices each) per launch, 1 .. 16
  *   "time_limit_s" bound on each device-side wait (default 20 s)
  *   "batch_evict"  run_rpq_batch with RPQ_PER_QUERY: product vertices after
- *                  which a query leaves the shared launch (0: never)
+ *                  which, or 32 times as many product edges after which, a
+ *                  query leaves the shared launch (0: never)
  *   "batch_streams" helper contexts evaluating evicted queries side by
  *                  side, 1 .. 16 (default 4)
  *   "batch_lanes"  run_rpq_batch with RPQ_PER_QUERY: evicted queries run in

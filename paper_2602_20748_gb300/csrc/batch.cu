@@ -203,6 +203,17 @@ __device__ __forceinline__ bool bvisit(const BatchParams &p, u32 i, u32 q2, u32 
   return !(atomicOr((unsigned long long *)word, bit) & bit);
 }
 
+// Whether a query with N product vertices and W product edges so far leaves
+// the batch: past evict_at vertices, or past EVICT_EDGES times as many edges.
+// The edges of a frontier are known before it is expanded, so a query that is
+// about to outgrow the batch leaves it without the level that would do so: on
+// configuration 4's batch that level and the next were 26 of 28 ms.  The factor
+// lies at twice the edges that evict_at vertices of degree 16 have.
+constexpr u64 EVICT_EDGES = 32;
+__device__ __forceinline__ bool outgrown(const BatchParams &p, u64 N, u64 W) {
+  return p.evict_at && (N > p.evict_at || W > p.evict_at * EVICT_EDGES);
+}
+
 __device__ void bseed(const BatchParams &p, u64 *W, u64 *N) {
   const u64 stride = (u64)gridDim.x * blockDim.x;
   BAppender app;
@@ -222,6 +233,7 @@ __device__ void bseed(const BatchParams &p, u64 *W, u64 *N) {
         if (p.qn) {
           p.qn[i] = 1;
           p.qw[i] = d;
+          if (outgrown(p, 1, d)) p.evicted[i] = 1u;
         }
       }
     }
@@ -371,7 +383,8 @@ __device__ void bcommit(const BatchParams &p, int lp, u32 nxt, u64 *W, u64 *N, u
       if (ok && p.active) p.active[i] = stamp;
     }
     *W += d;
-    mf += d;
+    // evicted queries' entries are not expanded
+    if (ok && !(p.evict_at && __ldcg(&p.evicted[i]))) mf += d;
     *N += ok ? 1 : 0;
     if (p.qn) {
       // per-query counters; the entries of a warp usually share one query
@@ -380,14 +393,12 @@ __device__ void bcommit(const BatchParams &p, int lp, u32 nxt, u64 *W, u64 *N, u
       if (same) {
         const u64 dn = warp_sum((u64)(ok ? 1 : 0)), dw = warp_sum(d);
         if (lane_id() == 0 && dn) {
-          const u64 before = atomicAdd(&p.qn[i0], dn);
-          atomicAdd(&p.qw[i0], dw);
-          if (p.evict_at && before + dn > p.evict_at) p.evicted[i0] = 1u;
+          const u64 n_all = atomicAdd(&p.qn[i0], dn) + dn, w_all = atomicAdd(&p.qw[i0], dw) + dw;
+          if (outgrown(p, n_all, w_all)) p.evicted[i0] = 1u;
         }
       } else if (ok) {
-        const u64 before = atomicAdd(&p.qn[i], 1ull);
-        atomicAdd(&p.qw[i], d);
-        if (p.evict_at && before + 1 > p.evict_at) p.evicted[i] = 1u;
+        const u64 n_all = atomicAdd(&p.qn[i], 1ull) + 1, w_all = atomicAdd(&p.qw[i], d) + d;
+        if (outgrown(p, n_all, w_all)) p.evicted[i] = 1u;
       }
     }
   }
@@ -424,7 +435,8 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS) batch_kernel(const __grid_c
       }
       push_levels++;
     }
-    bpush(p, lp, cur, nxt, n_cur, push_grab(n_cur, n_warps), spill_chunk(mf, n_warps), seg, &edges);
+    bpush(p, lp, cur, nxt, n_cur, push_grab(n_cur, mf, n_warps), spill_chunk(mf, n_warps, p.spill_cap), seg,
+          &edges);
     if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
     if (*(volatile unsigned long long *)&c->spill_count[cur] != 0) {
       bspill(p, lp, cur, nxt, seg, &edges);
@@ -635,7 +647,7 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS) serve_kernel(const __grid_c
     }
     if (n_cur > 0) {
       // admissions between levels add out-edges that no commit counted: the longest chunks
-      bpush(p, lp, cur, nxt, n_cur, push_grab(n_cur, (u64)p.nblocks * (blockDim.x >> 5)), SPILL_EDGES, p.append_seg,
+      bpush(p, lp, cur, nxt, n_cur, push_grab(n_cur, 0, (u64)p.nblocks * (blockDim.x >> 5)), SPILL_EDGES, p.append_seg,
             &edges);
       if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
       if (*(volatile unsigned long long *)&c->spill_count[cur] != 0) {

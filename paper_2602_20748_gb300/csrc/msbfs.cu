@@ -345,8 +345,8 @@ __device__ __forceinline__ bool relax(const BfsParams &p, u64 *FB, u32 tg, u32 w
 // an edge reads its owner's with three loads instead of ten shuffles, and the
 // words do not sit in registers through the edge loop.
 template <int NW, int AM>
-__device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_cur, u64 n_warps, u32 chunk, u32 seg,
-                           u32 stamp, u64 *scratch, u64 *stat) {
+__device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_cur, u64 mf, u64 n_warps, u32 chunk,
+                           u32 seg, u32 stamp, u64 *scratch, u64 *stat) {
   // scratch: [32][NW] words of the entries, in lane mode [32][NW] of them
   // masked by the row's transition, [32] (first edge - prefix, target)
   u64 *s_fm = scratch + lane_id() * NW;
@@ -361,7 +361,7 @@ __device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_c
   u64 edges = 0, rows = 0, entries = 0;
   Appender app;
   app.seg = seg;
-  const u32 grab = push_grab(n_cur, n_warps);
+  const u32 grab = push_grab(n_cur, mf, n_warps);
   for (u64 it = grid_warp() * grab; it < n_cur; it = next_item(&p.ctl->cursor[cur], n_warps, grab)) {
     u64 idx = it + lane;
     u64 e = lane < grab && idx < n_cur ? __ldcg(&list[idx]) : NO_ENTRY;
@@ -1917,8 +1917,8 @@ __global__ void __launch_bounds__(BFS_THREADS, AM == AM_LANE ? 3 : 4) msbfs_kern
       // no out-edges: the next frontier is empty, only this one is cleared
     } else if (push) {
       const u32 seg = mf < PUSH_EXACT ? 0u : p.append_seg;
-      push_level<NW, AM>(p, lp, cur, nxt, n_cur, n_warps, run ? ~0u : spill_chunk(mf, n_warps), seg, stamp, scratch,
-                         stat);
+      push_level<NW, AM>(p, lp, cur, nxt, n_cur, mf, n_warps, run ? ~0u : spill_chunk(mf, n_warps, p.spill_cap), seg,
+                         stamp, scratch, stat);
       if (run) {
         __syncthreads();
       } else {

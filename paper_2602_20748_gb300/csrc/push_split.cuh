@@ -21,20 +21,26 @@ __device__ __forceinline__ unsigned spill_reserve(unsigned long long *count, uns
 }
 
 // Chunk length of a top-down level whose frontier has mf out-edges: long rows
-// are cut so that every warp gets about one chunk, within [SPILL_EDGES_MIN,
-// SPILL_EDGES].  A fixed 1,024 left a level of 36,830 edges from a hundred
-// entries to the four warps that held them (496 us on R-MAT 2^20, one source).
-__device__ __forceinline__ u32 spill_chunk(u64 mf, u64 n_warps) {
-  u32 s = SPILL_EDGES_MIN;
-  while (s < SPILL_EDGES && (u64)s * n_warps < mf) s <<= 1;
-  return s;
+// are cut so that every warp gets about eight chunks, from SPILL_EDGES_MIN to
+// SPILL_EDGES edges, up to 16 times longer where the records would not fit half
+// of the queue (rows that find it full stay whole with one warp).  One chunk per warp
+// left the last warp of a level at five times the first one's time; a fixed
+// 1,024 left a level of 36,830 edges from a hundred entries to the four warps
+// that held them.
+__device__ __forceinline__ u32 spill_chunk(u64 mf, u64 n_warps, u64 cap) {
+  u64 s = SPILL_EDGES_MIN;
+  while (s < SPILL_EDGES && s * n_warps * 8 < mf) s <<= 1;
+  while (s * cap < 2 * mf && s < SPILL_EDGES * 16) s <<= 1;
+  return (u32)s;
 }
 
-// Entries a warp takes at a time: 32 while every warp gets some, fewer for
-// short lists, down to one warp per entry.
-__device__ __forceinline__ u32 push_grab(u64 n_cur, u64 n_warps) {
+// Entries a warp takes at a time: 32 while every warp gets some, of at most
+// 4,096 edges on average, and in a level of more than 256 edges per warp while
+// it gets four grabs; fewer otherwise, down to one.
+__device__ __forceinline__ u32 push_grab(u64 n_cur, u64 mf, u64 n_warps) {
+  const u64 grabs = mf > n_warps * 256 ? 4 : 1;
   u32 e = 32;
-  while (e > 1 && n_cur < n_warps * e) e >>= 1;
+  while (e > 1 && (n_cur < n_warps * e * grabs || mf * e > 4096 * n_cur)) e >>= 1;
   return e;
 }
 
