@@ -318,6 +318,38 @@ struct LastParams {
 
 constexpr int CL_THREADS = 256;
 constexpr int CL_WARPS = CL_THREADS / 32;
+// A round of a DENSE item is 128 words (four per lane): DENSE_SPAN vertices,
+// aligned to their number.  Its new values, at most CL_LIST of them, are first
+// listed in shared memory (see count_last_kernel).
+constexpr u32 DENSE_SPAN = 128 * 64;
+constexpr u32 CL_LIST = 2048;
+
+// splitmix64(pre ^ z) for the values z = zb + y, y < DENSE_SPAN (zb a multiple
+// of DENSE_SPAN): the low 13 bits of pre ^ z are those of pre ^ y, the rest is
+// common, and adding the increment carries out of the low half for one pre in
+// 2^19 only (then ok is false).  What is left per value is RowHash's 20
+// operations and an xor.
+struct SpanHash {
+  u32 p13, r, k, c;
+  bool ok;
+  __device__ __forceinline__ SpanHash(u64 pre, u32 zb) {
+    const u64 x = pre ^ (u64)zb;
+    p13 = (u32)x & (DENSE_SPAN - 1);
+    const u64 rr = (x & ~(u64)(DENSE_SPAN - 1)) + 0x9E3779B97F4A7C15ull;
+    r = (u32)rr;
+    ok = r <= 0xFFFFFFFFu - (DENSE_SPAN - 1);
+    const u32 hi = (u32)(rr >> 32);
+    k = hi << 2;
+    c = (hi ^ (hi >> 30)) * 0x1CE4E5B9u;
+  }
+  __device__ __forceinline__ u64 operator()(u32 y) const {
+    const u32 lo = r + (p13 ^ y);
+    const u32 l1 = lo ^ (lo >> 30) ^ k;
+    u64 z = (u64)l1 * 0x1CE4E5B9u + ((u64)(l1 * 0xBF58476Du + c) << 32);
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    return z ^ (z >> 31);
+  }
+};
 
 // Per-warp state of an item: the rows of the tuple's constraints and the
 // tuple's bound values (declaration order).
@@ -350,6 +382,9 @@ __device__ __forceinline__ u64 last_hash(const LastParams &lp, const LastWarp &s
 
 __global__ void __launch_bounds__(CL_THREADS) count_last_kernel(const LastParams lp) {
   __shared__ LastWarp s_warp[CL_WARPS];
+  __shared__ unsigned short s_list[CL_WARPS][CL_LIST];
+  unsigned short *list = s_list[threadIdx.x >> 5];
+  const bool last_var = lp.newpos >= 2 && lp.newpos + 1 == lp.arity;  // splitmix64(pre ^ z) is the whole hash
   const StepParams &p = lp.p;
   LastWarp &sw = s_warp[threadIdx.x >> 5];
   const u32 lane = lane_id();
@@ -406,9 +441,12 @@ __global__ void __launch_bounds__(CL_THREADS) count_last_kernel(const LastParams
     const u32 c = (u32)(t - cur_beg);
     t++;
     if (gen == DENSE) {
-      // words w0 + lane + 32 j of the AND, four per round; a lane walks the
-      // set bits of its four words in one loop, so that lanes wait for the
-      // largest four-word count rather than the largest one-word count
+      // words w0 + lane + 32 j of the AND, four per round.  The lanes list
+      // their set bits in shared memory and hash them from there, 32 at a time
+      // with no lane idle: hashed where they are found, the lanes waited for
+      // the one with most bits, at 40 instructions a turn instead of the 8 that
+      // list one.  Rounds with more than CL_LIST bits, or whose hash does not
+      // fold, walk their bits in place.
       const u64 *b0 = sw.bits[0], *b1 = p.nc > 1 ? sw.bits[1] : nullptr;
       const u64 w0 = (u64)c * DENSE_WORDS, w1 = min(p.bwords, w0 + DENSE_WORDS);
       for (u64 wb = w0; wb < w1; wb += 128) {
@@ -424,6 +462,40 @@ __global__ void __launch_bounds__(CL_THREADS) count_last_kernel(const LastParams
             for (u32 k = 2; k < p.nc; k++) x &= sw.bits[k][w];
           }
           m[j] = x;
+        }
+        u32 n_bits = 0;
+#pragma unroll
+        for (int j = 0; j < 4; j++) n_bits += __popcll(m[j]);
+        u32 at = n_bits;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          const u32 t2 = __shfl_up_sync(FULL_MASK, at, d);
+          if (lane >= (u32)d) at += t2;
+        }
+        const u32 total = __shfl_sync(FULL_MASK, at, 31);
+        if (total == 0) continue;
+        const SpanHash sh(pre, (u32)(wb * 64));
+        if (last_var && total <= CL_LIST && sh.ok) {
+          unsigned short *out = list + (at - n_bits);
+          __syncwarp();  // the previous list is read
+#pragma unroll
+          for (int j = 0; j < 8; j++) {
+            u32 half = (u32)(m[j >> 1] >> ((j & 1) * 32));
+            const u32 y0 = lane * 64 + (j >> 1) * 2048 + (j & 1) * 32;
+            while (half) {
+              const u32 b = 31 - __clz(half);
+              *out++ = (unsigned short)(y0 + b);
+              half ^= 1u << b;
+            }
+          }
+          __syncwarp();
+          for (u32 k = lane; k < total; k += 32) {
+            const u64 h = sh(list[k]);
+            hs += h;
+            hx ^= h;
+          }
+          cnt += n_bits;
+          continue;
         }
         // the eight 32-bit halves in vertex order: half k covers vertices
         // base0 + (k / 2) * 2048 + (k % 2) * 32 ..

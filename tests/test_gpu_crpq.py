@@ -177,3 +177,24 @@ def test_rmat22_triangle_sampled(ctx, rmat22):
     want = oracle.crpq(og, 3, TRIANGLE, var_label=vlab, restrict0=sample)
     rows, info = crpq_gpu(ctx, g, 3, TRIANGLE, var_label=vlab, restrict0=sample)
     assert rows.tolist() == want.rows.tolist()
+
+
+@pytest.mark.parametrize("n,per_label", [(8191, 4), (8193, 4), (20000, 4), (20000, 1.25), (8193, 1.25)])
+def test_count_only_join_of_bitsets(ctx, n, per_label):
+    """Count-only last step over bitsets: rounds of 8,192 vertices (one word
+    less, one more, several), with more and with fewer new values than a round
+    lists in shared memory; the last variable last and first in declaration
+    order, and four variables."""
+    src, dst, lab = synth.random_graph(n, int(3 * per_label * n), 3, seed=n + int(10 * per_label))
+    g = rpq.load_graph(ctx, n, 3, src, dst, lab)
+    og = oracle.Graph(n, 3, src, dst, lab)
+    x = np.array([0, 1, 2, n // 2, n - 1], np.uint32)
+    rpq.rpq_set_option(ctx, "crpq_bitset_frac", 0)  # every non-empty row is a bitset
+    try:
+        for nv, atoms in ((3, [(0, "a", 1), (0, "b*", 2), (1, "c*", 2)]), (3, [(0, "a", 2), (0, "b*", 1), (2, "c*", 1)]),
+                          (4, [(0, "a", 1), (1, "b", 2), (0, "c*", 3), (2, "b*", 3)])):
+            want = oracle.crpq(og, nv, atoms, restrict0=x)
+            _, info = crpq_gpu(ctx, g, nv, atoms, restrict0=x, flags=rpq.RPQ_COUNT_ONLY)
+            assert (info[0], info[2], info[3]) == oracle.row_digest(want.rows), atoms
+    finally:
+        rpq.rpq_set_option(ctx, "crpq_bitset_frac", 1 / 64)
