@@ -11,10 +11,8 @@
 // reads lane column c (32 lanes) of each tile, thread i holding the 32 lane
 // bits of vertex w0 + i.
 //
-// Count pass: each thread adds its words into bit-sliced counters (plane k
-// holds bit k of each lane's count over the thread's vertices); at the end
-// each plane is transposed across the warp once and the (lane, segment)
-// counts come out as popcounts.  An exclusive scan over the counts laid out
+// Count pass: the visited words are added into bit-sliced counters, 64 lanes a
+// word (see emit_count_kernel).  An exclusive scan over the counts laid out
 // [lane][segment] gives every row its output position directly (lanes are in
 // source order, segments in vertex order).
 //
@@ -77,20 +75,35 @@ template <int NW>
 __device__ __forceinline__ void batch_fetch(const EmitParams &p, u32 final_mask, u32 g, u32 w_first, u32 nv,
                                             u64 (&pre)[4]) {
   static_assert(EMIT_BV * NW == 4 * 64 * NW, "four words per thread");
-#pragma unroll
-  for (u32 r = 0; r < 4; r++) {
+  auto load = [&](u32 q, u32 r) {
     const u32 k = threadIdx.x + r * (64 * NW);
     const u32 v = k / NW, h = k % NW;
     const u32 w = w_first + v;
-    u64 word = 0;
-    if (v < nv && w < p.n)
-      for (u32 fm = final_mask; fm; fm &= fm - 1) {
-        const u32 q = __ffs(fm) - 1;
-        u64 x = __ldg(p.vis + (((u64)q * p.n + w) * p.G + g) * NW + h);
-        if (p.final_lane) x &= __ldg(p.final_lane + ((u64)q * p.G + g) * NW + h);  // lane mode
-        word |= x;
-      }
-    pre[r] = word;
+    return v < nv && w < p.n ? __ldg(p.vis + (((u64)q * p.n + w) * p.G + g) * NW + h) : 0ull;
+  };
+  if ((final_mask & (final_mask - 1)) == 0 && final_mask && !p.final_lane) {
+    // one accepting state: nothing here waits for the loads (in a loop over
+    // the states each of the four was waited for, and none stayed in flight
+    // behind the current batch)
+    const u32 q = __ffs(final_mask) - 1;
+#pragma unroll
+    for (u32 r = 0; r < 4; r++) pre[r] = load(q, r);
+    return;
+  }
+#pragma unroll
+  for (u32 r = 0; r < 4; r++) pre[r] = 0;
+  for (u32 fm = final_mask; fm; fm &= fm - 1) {
+    const u32 q = __ffs(fm) - 1;
+    u64 x[4];
+#pragma unroll
+    for (u32 r = 0; r < 4; r++) x[r] = load(q, r);
+    if (p.final_lane) {  // lane mode
+      const u64 m = __ldg(p.final_lane + ((u64)q * p.G + g) * NW + threadIdx.x % NW);
+#pragma unroll
+      for (u32 r = 0; r < 4; r++) x[r] &= m;
+    }
+#pragma unroll
+    for (u32 r = 0; r < 4; r++) pre[r] |= x[r];
   }
 }
 
@@ -153,15 +166,117 @@ __device__ __forceinline__ void ring_flush(u32 R, u32 rd, u32 end, u32 *base, co
   __syncwarp();
 }
 
+// Stores the bitset words that the lanes set in B have collected: `chunks`
+// 16-byte pieces each, piece q of row j in its ring at slot q ^ (j & 7) (so
+// that neither the rows' writes nor the pieces' reads meet in a bank), to
+// dst_j.  Rows four at a time, eight lanes per row, 128 contiguous bytes.
+__device__ __forceinline__ void bits_flush(u32 B, u32 *dst, u32 chunks, const u32 *ring, u32 *slots) {
+  const u32 lane = lane_id();
+  if (B & (1u << lane)) slots[__popc(B & lanemask_lt())] = lane;
+  __syncwarp();
+  const u32 n_rows = __popc(B), q = lane & 7;
+  for (u32 r0 = 0; r0 < n_rows; r0 += 4) {
+    const u32 idx = r0 + (lane >> 3);
+    const u32 j = slots[idx < n_rows ? idx : 0];
+    uint4 *dj = reinterpret_cast<uint4 *>(__shfl_sync(FULL_MASK, reinterpret_cast<u64>(dst), j));
+    if (idx < n_rows && q < chunks)
+      dj[q] = *reinterpret_cast<const uint4 *>(ring + j * EMIT_RING + 4 * (q ^ (j & 7)));
+  }
+  __syncwarp();
+}
+
 }  // namespace
 
-// Count pass: cnt[lane][segment] = the lane's members in the segment; with
-// DIGEST, also the digest of those (source, y) rows (count-only results).
-template <int NW, bool DIGEST>
-__global__ void __launch_bounds__(64 * NW, NW == 1 ? 16 : 4) emit_count_kernel(const EmitParams p) {
-  __shared__ u32 s_vis[2 * NW * EMIT_BV];
+// Count pass: cnt[lane][segment] = the lane's members in the segment.
+//
+// A thread takes word h of every 64th vertex of the segment (four adjacent
+// threads read one vertex's 32 bytes) and adds the words, 64 lanes at a time,
+// into bit-sliced counters: four words by carry-save adders, then one carry
+// into the higher planes, 7 logic operations per word.  Nothing passes through
+// shared memory until the threads' counters are added up at the end, so the
+// pass is bound by its loads (on R-MAT 2^22, 16 groups, 2.1 GB: 1,300 -> 520 us;
+// spreading each batch by lane column in shared memory first cost two block
+// barriers per 256 vertices and 16 operations per 32 lanes).
+template <int NW>
+__global__ void __launch_bounds__(64 * NW, NW == 1 ? 16 : 6) emit_count_kernel(const EmitParams p) {
+  constexpr int PLANES = NW == 1 ? 11 : 9;  // highest of a warp's sums: 32 / NW threads x EMIT_TILES / 2 words each
+  static_assert(EMIT_TILES / 2 * (32 / NW) < (2 << PLANES), "planes too narrow");
+  constexpr int OWN = 7;  // of a thread's counters
+  static_assert(EMIT_TILES / 2 < (1 << OWN), "planes too narrow");
+  constexpr int WARPS = 2 * NW;
+  __shared__ u64 s_pl[WARPS][NW][PLANES + 1];
   // groups of one segment are adjacent blocks, so they read the same
   // visited lines close together in time
+  const u32 g = blockIdx.x % p.G, seg = blockIdx.x / p.G;
+  const u32 h = threadIdx.x % NW, v0 = threadIdx.x / NW;
+  const u32 w_begin = seg * p.tiles * 32;
+  const u32 nv = min(p.tiles * 32, p.n - w_begin);
+  const u64 step = 64ull * p.G * NW;  // words between this thread's vertices
+  u64 pl[PLANES + 1];
+#pragma unroll
+  for (int k = 0; k <= PLANES; k++) pl[k] = 0;
+  const u64 *base = p.vis + ((u64)(w_begin + v0) * p.G + g) * NW + h;
+  const u64 per_state = (u64)p.n * p.G * NW;
+  auto csa = [](u64 &sum, u64 a, u64 b) {  // sum + a + b = sum' + 2 * result
+    const u64 carry = (sum & a) | (sum & b) | (a & b);
+    sum ^= a ^ b;
+    return carry;
+  };
+#pragma unroll 2
+  for (u32 v = v0; v < nv; v += 256) {
+    // the OR over the accepting states of vertices w_begin + v + 64 r, a
+    // state's four words at a time (see batch_fetch)
+    const u64 *at = base + (u64)((v - v0) / 64) * step;
+    u64 a[4] = {0, 0, 0, 0};
+    for (u32 fm = p.final_mask; fm; fm &= fm - 1) {
+      const u64 *aq = at + (u64)(__ffs(fm) - 1) * per_state;
+      u64 x[4];
+#pragma unroll
+      for (u32 r = 0; r < 4; r++) x[r] = v + 64 * r < nv ? __ldg(aq + r * step) : 0ull;
+#pragma unroll
+      for (u32 r = 0; r < 4; r++) a[r] |= x[r];
+    }
+    const u64 t0 = csa(pl[0], a[0], a[1]), t1 = csa(pl[0], a[2], a[3]);
+    u64 carry = csa(pl[1], t0, t1);
+#pragma unroll
+    for (int k = 2; k < OWN; k++) {
+      const u64 x = pl[k] & carry;
+      pl[k] ^= carry;
+      carry = x;
+    }
+  }
+  // the warp's threads of one h: their counters added up bit by bit
+#pragma unroll
+  for (int o = NW; o < 32; o <<= 1) {
+    u64 carry = 0;
+#pragma unroll
+    for (int k = 0; k <= PLANES; k++) {
+      const u64 y = __shfl_xor_sync(FULL_MASK, pl[k], o);
+      const u64 x = pl[k];
+      pl[k] = x ^ y ^ carry;
+      carry = (x & y) | (x & carry) | (y & carry);
+    }
+  }
+  if (lane_id() < NW)
+#pragma unroll
+    for (int k = 0; k <= PLANES; k++) s_pl[threadIdx.x >> 5][lane_id()][k] = pl[k];
+  __syncthreads();
+  // thread t: lane t of the group
+  const u32 bit = threadIdx.x % 64;
+  const u64 glane = (u64)g * (64 * NW) + threadIdx.x;
+  u32 cnt = 0;
+  for (int wv = 0; wv < WARPS; wv++)
+#pragma unroll
+    for (int k = 0; k <= PLANES; k++) cnt += (u32)((s_pl[wv][threadIdx.x / 64][k] >> bit) & 1ull) << k;
+  p.cnt[glane * p.segs + seg] = p.lanesrc[glane] == NO_SOURCE ? 0u : cnt;
+}
+
+// Count pass of a count-only result: also the digest of the (source, y) rows.
+// Warp c reads lane column c of each tile from shared memory, transposes it
+// and hashes the members lane by lane.
+template <int NW>
+__global__ void __launch_bounds__(64 * NW, NW == 1 ? 16 : 4) emit_count_digest_kernel(const EmitParams p) {
+  __shared__ u32 s_vis[2 * NW * EMIT_BV];
   const u32 g = blockIdx.x % p.G, seg = blockIdx.x / p.G;
   const u32 col = threadIdx.x >> 5, lane = lane_id();
   const u64 glane = (u64)g * (64 * NW) + col * 32 + lane;
@@ -170,45 +285,28 @@ __global__ void __launch_bounds__(64 * NW, NW == 1 ? 16 : 4) emit_count_kernel(c
   const RowHash rh(src);
   const u32 w_begin = seg * p.tiles * 32;
   const u32 n_tiles = min(p.tiles, (p.n - w_begin + 31) / 32);
-  constexpr int CNT_PLANES = 8;  // EMIT_TILES <= 2^CNT_PLANES - 1 vertices per thread
-  static_assert(EMIT_TILES < (1 << CNT_PLANES), "count planes too narrow");
-  u32 planes[CNT_PLANES];
-#pragma unroll
-  for (int k = 0; k < CNT_PLANES; k++) planes[k] = 0;
   u32 cnt = 0;
   u64 hsum = 0, hxor = 0;
+  u64 pre[4];
+  batch_fetch<NW>(p, p.final_mask, g, w_begin, min(EMIT_BATCH, n_tiles) * 32, pre);
   for (u32 tb = 0; tb < n_tiles; tb += EMIT_BATCH) {
-    u64 pre[4];
-    batch_fetch<NW>(p, p.final_mask, g, w_begin + tb * 32, min(EMIT_BATCH, n_tiles - tb) * 32, pre);
     __syncthreads();  // the previous batch is consumed
     batch_store<NW>(pre, s_vis);
     __syncthreads();
+    if (tb + EMIT_BATCH < n_tiles)  // next batch in flight while this one is hashed
+      batch_fetch<NW>(p, p.final_mask, g, w_begin + (tb + EMIT_BATCH) * 32,
+                      min(EMIT_BATCH, n_tiles - tb - EMIT_BATCH) * 32, pre);
 #pragma unroll
     for (u32 t = 0; t < EMIT_BATCH; t++) {
-      const u32 x = s_vis[col * EMIT_BV + t * 32 + lane] & valid_cols;  // zero past the segment's end
-      if (DIGEST) {
-        u32 m = warp_transpose32(x);
-        cnt += __popc(m);
-        const u32 w0 = w_begin + (tb + t) * 32;
-        for (; m; m &= m - 1) digest_add(rh, w0 + __ffs(m) - 1, hsum, hxor);
-      } else {
-        u32 carry = x;
-#pragma unroll
-        for (int k = 0; k < CNT_PLANES; k++) {
-          const u32 c = planes[k] & carry;
-          planes[k] ^= carry;
-          carry = c;
-        }
-      }
+      // zero past the segment's end
+      u32 m = warp_transpose32(s_vis[col * EMIT_BV + t * 32 + lane] & valid_cols);
+      cnt += __popc(m);
+      const u32 w0 = w_begin + (tb + t) * 32;
+      for (; m; m &= m - 1) digest_add(rh, w0 + __ffs(m) - 1, hsum, hxor);
     }
   }
-  if (!DIGEST) {
-    // lane j's count = sum over planes k of 2^k * (thread bits j of plane k)
-#pragma unroll
-    for (int k = 0; k < CNT_PLANES; k++) cnt += (u32)__popc(warp_transpose32(planes[k])) << k;
-  }
   p.cnt[glane * p.segs + seg] = cnt;
-  if (DIGEST) digest_flush(hsum, hxor, p.digest);
+  digest_flush(hsum, hxor, p.digest);
 }
 
 // Write pass: dst[off[lane][segment] ...] = the lane's members in vertex
@@ -241,40 +339,65 @@ __global__ void __launch_bounds__(64 * NW, NW == 1 ? 16 : 3) emit_write_kernel(c
     if (slot != NO_SOURCE) bs = reinterpret_cast<u32 *>(p.bits + (u64)slot * p.bwords);
   }
   const bool listed = !bs || p.keep_lists;
+  const u32 unlisted = __ballot_sync(FULL_MASK, !listed);
   const u32 w_begin = seg * p.tiles * 32;
   const u32 n_tiles = min(p.tiles, (p.n - w_begin + 31) / 32);
   u64 pre[4];
   batch_fetch<NW>(p, p.final_mask, g, w_begin, min(EMIT_BATCH, n_tiles) * 32, pre);
   for (u32 tb = 0; tb < n_tiles; tb += EMIT_BATCH) {
-    const u32 nt = min(EMIT_BATCH, n_tiles - tb);
     __syncthreads();  // the previous batch is consumed
     batch_store<NW>(pre, s_vis);
     __syncthreads();
     if (tb + EMIT_BATCH < n_tiles)  // next batch in flight while this one is placed
       batch_fetch<NW>(p, p.final_mask, g, w_begin + (tb + EMIT_BATCH) * 32,
                       min(EMIT_BATCH, n_tiles - tb - EMIT_BATCH) * 32, pre);
+    // the batch's tiles turned around together: eight independent chains of
+    // shuffles (zero past the segment's end)
     u32 acc[EMIT_BATCH];
 #pragma unroll
-    for (u32 t = 0; t < EMIT_BATCH; t++) {
-      acc[t] = 0;
-      if (t >= nt) continue;  // uniform across the block
-      u32 m = warp_transpose32(s_vis[col * EMIT_BV + t * 32 + lane] & valid_cols);
-      acc[t] = m;
-      if (!listed) m = 0;
-      const u32 wb = w_begin + (tb + t) * 32 - 1;
-      // at most 31 words were pending, so the ring (64) holds this tile's 32
-      for (; m; m &= m - 1) myring[wr++ & (EMIT_RING - 1)] = wb + __ffs(m);
-      const bool full = wr > (rd | 31u);  // rd's 32-word chunk is complete
-      const u32 R = __ballot_sync(FULL_MASK, full);
-      if (R) {
-        ring_flush(R, rd, (rd | 31u) + 1u, base, ring, slots);
-        if (full) rd = (rd | 31u) + 1u;
+    for (u32 t = 0; t < EMIT_BATCH; t++)
+      acc[t] = warp_transpose32(s_vis[col * EMIT_BV + t * 32 + lane] & valid_cols);
+    if (unlisted != FULL_MASK)
+#pragma unroll
+      for (u32 t = 0; t < EMIT_BATCH; t++) {
+        u32 m = listed ? acc[t] : 0;
+        const u32 wb = w_begin + (tb + t) * 32;
+        // at most 31 words were pending, so the ring (64) holds this tile's
+        // 32; from the last member down, whose number one instruction finds
+        wr += __popc(m);
+        for (u32 at = wr; m;) {
+          const u32 b = 31 - __clz(m);
+          myring[--at & (EMIT_RING - 1)] = wb + b;
+          m ^= 1u << b;
+        }
+        const bool full = wr > (rd | 31u);  // rd's 32-word chunk is complete
+        const u32 R = __ballot_sync(FULL_MASK, full);
+        if (R) {
+          ring_flush(R, rd, (rd | 31u) + 1u, base, ring, slots);
+          if (full) rd = (rd | 31u) + 1u;
+        }
       }
-    }
-    if (bs) {  // the batch's 256 vertices start on a 32-byte boundary of the bitset
+    // bitset words: the batch's 256 vertices start on a 32-byte boundary.
+    // Lanes that are not listed collect four batches in their idle ring, so
+    // that a store covers four rows' whole lines instead of 32 of them (R-MAT
+    // 2^22, 4,096 bitset rows: 2,670 us a pass before, 1,830 with lines, loads
+    // in flight and tiles turned together).
+    if (bs && listed) {
       uint4 *d = reinterpret_cast<uint4 *>(bs + (w_begin + tb * 32) / 32);
       d[0] = make_uint4(acc[0], acc[1], acc[2], acc[3]);
       d[1] = make_uint4(acc[4], acc[5], acc[6], acc[7]);
+    }
+    if (unlisted) {
+      const u32 b4 = (tb / EMIT_BATCH) & 3;
+      if (!listed) {
+        uint4 *r = reinterpret_cast<uint4 *>(myring);
+        r[(2 * b4) ^ (lane & 7)] = make_uint4(acc[0], acc[1], acc[2], acc[3]);
+        r[(2 * b4 + 1) ^ (lane & 7)] = make_uint4(acc[4], acc[5], acc[6], acc[7]);
+      }
+      if (b4 == 3 || tb + EMIT_BATCH >= n_tiles) {
+        __syncwarp();
+        bits_flush(unlisted, bs + (w_begin + (tb - b4 * EMIT_BATCH) * 32) / 32, 2 * (b4 + 1), ring, slots);
+      }
     }
   }
   const u32 R = __ballot_sync(FULL_MASK, wr > rd);  // the partial last chunks
@@ -289,11 +412,9 @@ cudaError_t launch_emit(int nw, bool write, bool digest, const EmitParams &p, cu
   const int threads = nw == 1 ? 64 : 256;
   if (!write) {
     if (nw == 1)
-      digest ? emit_count_kernel<1, true><<<grid, threads, 0, st>>>(p)
-             : emit_count_kernel<1, false><<<grid, threads, 0, st>>>(p);
+      digest ? emit_count_digest_kernel<1><<<grid, threads, 0, st>>>(p) : emit_count_kernel<1><<<grid, threads, 0, st>>>(p);
     else
-      digest ? emit_count_kernel<4, true><<<grid, threads, 0, st>>>(p)
-             : emit_count_kernel<4, false><<<grid, threads, 0, st>>>(p);
+      digest ? emit_count_digest_kernel<4><<<grid, threads, 0, st>>>(p) : emit_count_kernel<4><<<grid, threads, 0, st>>>(p);
     return cudaGetLastError();
   }
   if (digest) return cudaErrorInvalidValue;  // the write pass does not fold the digest
@@ -466,7 +587,7 @@ cudaError_t launch_emit_pairs(const EmitParams &p, uint32_t *out, cudaStream_t s
 
 cudaError_t preload_static_emit_kernels() {
   cudaFuncAttributes a;
-  cudaError_t e = cudaFuncGetAttributes(&a, emit_count_kernel<1, false>);
+  cudaError_t e = cudaFuncGetAttributes(&a, emit_count_kernel<1>);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, emit_pairs_kernel<1, true>);
   if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, emit_pairs_kernel<1, false>);
   return e;
