@@ -1035,6 +1035,7 @@ __device__ void pull_lanes(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
   ulonglong2 *sacc = reinterpret_cast<ulonglong2 *>(scratch) + lane;  // target q2's words at sacc[32 * q2]
   u64 *lst = scratch + LANE_SRC_Q * 2 * 32;                           // [LANE_LIST]
   const bool chunked = p.hchunk != nullptr;
+  u32 *nbits = p.fbits ? p.fbits + (lp ? 0 : p.fbits_words) : nullptr;  // the next frontier's bitmap
   Appender app;
   app.seg = (u64)n * Q * p.G >= grid_warps() * 2 * APPEND_SEG ? p.append_seg : min(p.append_seg, 32u);
 
@@ -1044,10 +1045,12 @@ __device__ void pull_lanes(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
   }
   __syncthreads();
   u64 lset = 0;  // labels with an active transition
+  u32 sts_all = 0;  // states with one
   for (u32 l = 0; l < L; l++) {
     u32 a = 0;
     for (u32 s = 0; s < Q; s++) a |= (tab.grp[l * LANE_SRC_Q + s] >> 16 ? 1u : 0u) << s;
     if (a) lset |= 1ull << l;
+    sts_all |= a;
     if (threadIdx.x == 0) tab.act[l] = (unsigned char)a;
   }
   __syncthreads();
@@ -1097,6 +1100,10 @@ __device__ void pull_lanes(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
     for (; any; any &= any - 1) {
       const u32 q2 = __ffs(any) - 1;
       const bool nz = (found >> q2) & 1u;
+      if (lane == 0 && nbits) {
+        const u64 bi = (u64)q2 * n + w;
+        atomicOr(nbits + (bi >> 5), 1u << (bi & 31));
+      }
       const u64 base = ((u64)q2 * n + w) * wpv + lane_off;
       if (nz) {
         const ulonglong2 a = sacc[32 * q2];
@@ -1214,12 +1221,17 @@ __device__ void pull_lanes(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
           }
           r -= len;
         }
-        if (bits)
-          for (u32 m = sm; m; m &= m - 1) {
-            const u32 st = __ffs(m) - 1;
+        if (bits) {
+          u32 bw[LANE_SRC_Q];
+#pragma unroll
+          for (u32 st = 0; st < LANE_SRC_Q; st++) {
             const u64 row = (u64)st * n + u;
-            if (!((__ldcg(bits + (row >> 5)) >> (row & 31)) & 1u)) sm &= ~(1u << st);
+            bw[st] = (sm >> st) & 1u ? __ldcg(bits + (row >> 5)) >> (row & 31) : 0u;
           }
+          sm = 0;
+#pragma unroll
+          for (u32 st = 0; st < LANE_SRC_Q; st++) sm |= (bw[st] & 1u) << st;
+        }
       }
       u32 at = __popc(sm);
 #pragma unroll
@@ -1230,18 +1242,24 @@ __device__ void pull_lanes(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
       const u32 listed = __shfl_sync(FULL_MASK, at, 31);
       at -= __popc(sm);
       // a row's gathers are listed state by state, so that a state's rows are
-      // ORed before they are masked (with a bitmap, where rows are missing,
-      // in-edge by in-edge)
-      u32 run = 1;
-      if (!bits) {
-        const u32 same = __match_any_sync(FULL_MASK, lane < LANE_EDGES && k < T ? o << 6 | l : 1u << 31 | lane);
-        run = __popc(same);
-        at = __shfl_sync(FULL_MASK, at, __ffs(same) - 1) + __popc(same & lanemask_lt());
-      }
+      // ORed before they are masked: behind those of the row's smaller states
+      // and of its earlier in-edges
+      const u32 same = __match_any_sync(FULL_MASK, lane < LANE_EDGES && k < T ? o << 6 | l : 1u << 31 | lane);
+      at = __shfl_sync(FULL_MASK, at, __ffs(same) - 1);
       __syncwarp();  // the previous list is consumed
-      for (u32 m = sm; m; m &= m - 1, at += run) {
-        const u32 st = __ffs(m) - 1;
-        lst[at] = ((u64)st * n + u) | (u64)(l * LANE_SRC_Q + st) << 44 | (u64)o << 58;
+      auto entry = [&](u32 st) {
+        return ((u64)st * n + u) | (u64)(l * LANE_SRC_Q + st) << 44 | (u64)o << 58;
+      };
+      if (bits) {
+        for (u32 sts = sts_all; sts; sts &= sts - 1) {
+          const u32 st = __ffs(sts) - 1;
+          const u32 has = __ballot_sync(FULL_MASK, (sm >> st) & 1u) & same;
+          if ((sm >> st) & 1u) lst[at + __popc(has & lanemask_lt())] = entry(st);
+          at += __popc(has);
+        }
+      } else {  // every in-edge of the row has the same states
+        at += __popc(same & lanemask_lt());
+        for (u32 m = sm; m; m &= m - 1, at += __popc(same)) lst[at] = entry(__ffs(m) - 1);
       }
       __syncwarp();
       stat_add(stat, ST_ALG_BYTES, listed * gword);
@@ -1721,10 +1739,12 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
 // Commit of a level: fold the new frontier words into VIS, count work, note
 // the DFA states present in the new frontier, clear the old frontier words.
 // set_bits: the next frontier may be sparse enough for bottom-up levels to
-// test its bitmap, so its bits are set; clear_bits: this level's bits were set.
+// test its bitmap, so its bits are set (pull_lanes has set its own);
+// clear_bits: this level's bits were set and are cleared, entry by entry (1)
+// or all words (2).
 template <int NW, int AM>
 __device__ void commit_phase(const BfsParams &p, int lp, u32 nxt, u64 n_cur, u64 n_warps, bool set_bits,
-                             bool clear_bits, CommitSums &sums, u64 *stat) {
+                             int clear_bits, CommitSums &sums, u64 *stat) {
   const u64 *list = lp ? p.list1 : p.list0;
   const u64 *nlist = lp ? p.list0 : p.list1;
   u64 *F = lp ? p.fr1 : p.fr0;
@@ -1774,12 +1794,14 @@ __device__ void commit_phase(const BfsParams &p, int lp, u32 nxt, u64 n_cur, u64
     u32 gq = (u32)((e & ~ENTRY_DONE) >> 32);
     u32 g = gq / Q;
     store_w<NW>(F + widx<NW>(p, g, gq - g * Q, (u32)e), zero);
-    if (clear_bits) {
+    if (clear_bits == 1) {
       // the retired frontier's bitmap: every set bit belongs to one of these entries
       const u64 bi = (u64)(gq - g * Q) * p.n + (u32)e;
       p.fbits[(lp ? p.fbits_words : 0) + (bi >> 5)] = 0u;
     }
   }
+  if (clear_bits == 2)  // a dense frontier's: all of it
+    for (u64 j = tid; j < ((u64)p.n * Q + 31) / 32; j += stride) p.fbits[(lp ? p.fbits_words : 0) + j] = 0u;
   if (tid == 0) stat[ST_ALG_BYTES] += n_cur * (8 + 8 * NW);
   W = warp_sum(W);
   N = warp_sum(N);
@@ -1859,11 +1881,12 @@ __global__ void __launch_bounds__(BFS_THREADS, AM == AM_LANE ? 3 : 4) msbfs_kern
   if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
 
   // lane mode: bottom-up levels by pull_lanes, whose lanes fill a warp's row.
-  // They cost less per byte than the estimate's: with its bytes taken at 0.4
-  // the batch above took 320 ms, at 1 342 ms (0.67: 343, 0.33 .. 0.17: 320).
+  // With a bitmap they cost less than the estimate's bytes: the batch above
+  // goes top-down in its second level at a factor above 0.4 (60 ms, not 22).
   constexpr float LANES_PULL = 0.4f;
   const bool lanes_staged =
       AM == AM_LANE && NW == 4 && p.lane_by_source && p.Q <= LANE_SRC_Q && p.G * NW / 2 > 16;
+  bool have_bits = p.fbits != nullptr;  // this level's frontier has a bitmap (the seeds set theirs)
   u32 level = 0, run = 0;  // run: levels left of block 0's run, 0 outside one
   for (;; level++) {
     const u32 cur = level % 3, nxt = (level + 1) % 3, old = (level + 2) % 3;
@@ -1880,13 +1903,19 @@ __global__ void __launch_bounds__(BFS_THREADS, AM == AM_LANE ? 3 : 4) msbfs_kern
       if (blockIdx.x != 0) {
         if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
         level = *(volatile unsigned *)&c->next_level - 1;
+        // a top-down level of block 0 built this frontier
+        have_bits = p.fbits && *(volatile unsigned long long *)&c->n_list[(level + 1) % 3] * 4 < (u64)p.n * p.Q;
         continue;
       }
       run = SOLO_RUN;
     }
     const float push_cost = (float)mf * (4.0f + 8.0f * NW) + (float)n_true * (16.0f + 8.0f * NW);
     float pull_cost = pull_bytes<NW>(p, active);
-    if (lanes_staged) pull_cost *= LANES_PULL;
+    // pull_lanes tests the frontier's bitmap up to a seventh of the words: the
+    // rows it shows empty outweigh the test then (second and third level of the
+    // batch above 31 -> 22 and 50 -> 48 ms, its dense levels 57 -> 61)
+    const bool lanes_bits = lanes_staged && have_bits && n_cur * 7 < (u64)p.n * __popc(active) * p.G;
+    if (lanes_bits) pull_cost *= LANES_PULL;
     const bool push = solo || p.force == 1 || (p.force != 2 && p.alpha * push_cost < pull_cost);
     if (tracer) {
       // counters of the level after next start at zero
@@ -1930,8 +1959,9 @@ __global__ void __launch_bounds__(BFS_THREADS, AM == AM_LANE ? 3 : 4) msbfs_kern
       }
     } else {
       // a sparse frontier: test the frontier bitmap before each gather
-      // (implies n_cur * 4 < n * Q, so the commit that built this frontier set its bits)
-      const bool sparse = p.fbits && n_cur * 4 < (u64)p.n * __popc(active);
+      // (implies n_cur * 4 < n * Q, so the commit that built this frontier set
+      // its bits)
+      const bool sparse = lanes_staged ? lanes_bits : p.fbits && n_cur * 4 < (u64)p.n * __popc(active);
       const u32 *bits = sparse ? p.fbits + (lp ? p.fbits_words : 0) : nullptr;
       // pull_level's early exit pays where few lanes are live: one lane
       // group, the per-group automata of a multi launch (typically one start
@@ -1955,8 +1985,10 @@ __global__ void __launch_bounds__(BFS_THREADS, AM == AM_LANE ? 3 : 4) msbfs_kern
       // fewer than n * Q / 4 entries (the seeds always set theirs)
       const u64 n_next = *(volatile unsigned long long *)&c->n_list[nxt];
       const u64 sparse_cap = (u64)p.n * p.Q;
-      const bool set_bits = p.fbits && n_next * 4 < sparse_cap;
-      const bool clear_bits = p.fbits && (level == 0 || n_cur * 4 < sparse_cap);
+      const bool pulled_lanes = lanes_staged && mf != 0 && !push;
+      const bool set_bits = p.fbits && n_next * 4 < sparse_cap && !pulled_lanes;
+      const int clear_bits = !have_bits ? 0 : level == 0 || n_cur * 4 < sparse_cap ? 1 : 2;
+      have_bits = p.fbits && (n_next * 4 < sparse_cap || pulled_lanes);
       if (tracer && level < (u32)TRACE_LEVELS) c->trace_c[level] = globaltimer_ns();
       commit_phase<NW, AM>(p, lp, nxt, n_cur, n_warps, set_bits, clear_bits, sums, stat);
       if (run) {
