@@ -466,12 +466,8 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
     p.in_off = reverse ? g.out_off : g.in_off;
     p.in_col = reverse ? g.out_col : g.in_col;
     // bottom-up levels read the in-direction of the traversal
-    p.hchunk = reverse ? g.hchunk_out : g.hchunk_in;
-    {
-      const std::vector<uint32_t> &ho = reverse ? g.hchunk_out_off : g.hchunk_in_off;
-      for (uint32_t l = 0; l <= g.L && l < ho.size(); l++) p.hchunk_off[l] = ho[l];
-      for (uint32_t l = 0; l < g.L; l++) p.label_edges[l] = g.label_edges[l];
-    }
+    set_chunks(p, reverse ? g.hchunk_out : g.hchunk_in, reverse ? g.hchunk_out_off : g.hchunk_in_off, g.L, live);
+    for (uint32_t l = 0; l < g.L; l++) p.label_edges[l] = g.label_edges[l];
     p.n = n;
     p.L = g.L;
     p.G = Gb;
@@ -1768,8 +1764,7 @@ int rpq_lane_stats_multi(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Mu
   p.out_col = g.out_col;
   p.in_off = g.in_off;
   p.in_col = g.in_col;
-  p.hchunk = g.hchunk_in;
-  for (uint32_t l = 0; l <= g.L && l < g.hchunk_in_off.size(); l++) p.hchunk_off[l] = g.hchunk_in_off[l];
+  set_chunks(p, g.hchunk_in, g.hchunk_in_off, g.L, total_lanes);
   for (uint32_t l = 0; l < g.L; l++) p.label_edges[l] = g.label_edges[l];
   p.n = n;
   p.L = L;
@@ -2035,8 +2030,7 @@ static int lane_launch(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Lane
   p.out_col = g.out_col;
   p.in_off = g.in_off;
   p.in_col = g.in_col;
-  p.hchunk = g.hchunk_in;
-  for (uint32_t l = 0; l <= g.L && l < g.hchunk_in_off.size(); l++) p.hchunk_off[l] = g.hchunk_in_off[l];
+  set_chunks(p, g.hchunk_in, g.hchunk_in_off, g.L, k);
   for (uint32_t l = 0; l < g.L; l++) p.label_edges[l] = g.label_edges[l];
   p.n = n;
   p.L = L;

@@ -129,27 +129,39 @@ __global__ void label_bounds(const uint32_t *__restrict__ off, uint32_t n, uint3
   }
 }
 
-// Chunks of long rows: cnt[v] = number of HCHUNK-edge chunks of row v of one
-// label's CSR when the row has at least HEAVY_ROW edges, else 0.
-__global__ void count_chunks(const uint32_t *__restrict__ off, uint32_t n, u32 *__restrict__ cnt) {
-  for (u64 v = (u64)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (u64)gridDim.x * blockDim.x) {
-    uint32_t len = off[v + 1] - off[v];
-    cnt[v] = len >= HEAVY_ROW ? (len + HCHUNK - 1) / HCHUNK : 0u;
-  }
-}
-
-// Chunk records (vertex, first edge, end edge) at out[3 * (base + pos[v] + c)].
-__global__ void write_chunks(const uint32_t *__restrict__ off, uint32_t n, const u64 *__restrict__ pos, u64 base,
-                             uint32_t *__restrict__ out) {
-  for (u64 v = (u64)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += (u64)gridDim.x * blockDim.x) {
-    uint32_t b = off[v], len = off[v + 1] - b;
-    if (len < HEAVY_ROW) continue;
-    uint32_t k = (len + HCHUNK - 1) / HCHUNK;
-    for (uint32_t c = 0; c < k; c++) {
-      u64 r = 3 * (base + pos[v] + c);
-      out[r] = (uint32_t)v;
-      out[r + 1] = b + c * HCHUNK;
-      out[r + 2] = min(b + (c + 1) * HCHUNK, b + len);
+// Chunk lists of long rows, all labels at once (blockIdx.y = label): a list per
+// label and class, rows of at least LONG_ROW edges (class 0) and rows of
+// HEAVY_ROW .. LONG_ROW - 1 (class 1).  Without out, next[2 * label + class]
+// counts the chunks; with out, it is the place of the list's next record
+// (vertex, first edge, end edge), taken a warp at a time.
+__global__ void row_chunks(const uint32_t *__restrict__ off, uint32_t n, u32 *__restrict__ next,
+                           uint32_t *__restrict__ out) {
+  const uint32_t *row = off + (u64)blockIdx.y * (n + 1);
+  next += 2 * blockIdx.y;
+  const u64 step = (u64)gridDim.x * blockDim.x;
+  for (u64 v0 = (u64)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); v0 < n; v0 += step) {
+    const u64 v = v0 + lane_id();
+    const uint32_t b = v < n ? row[v] : 0u, len = v < n ? row[v + 1] - b : 0u;
+    for (int cls = 0; cls < 2; cls++) {
+      const bool mine = cls == 0 ? len >= LONG_ROW : len >= HEAVY_ROW && len < LONG_ROW;
+      if (!__any_sync(FULL_MASK, mine)) continue;
+      const u32 k = mine ? (len + HCHUNK - 1) / HCHUNK : 0u;
+      u32 at = k;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const u32 t = __shfl_up_sync(FULL_MASK, at, o);
+        if (lane_id() >= (u32)o) at += t;
+      }
+      u32 base = 0;
+      if (lane_id() == 31) base = atomicAdd(&next[cls], at);
+      base = __shfl_sync(FULL_MASK, base, 31) + at - k;
+      if (out)
+        for (u32 c = 0; c < k; c++) {
+          const u64 r = 3ull * (base + c);
+          out[r] = (uint32_t)v;
+          out[r + 1] = b + c * HCHUNK;
+          out[r + 2] = min(b + (c + 1) * HCHUNK, b + len);
+        }
     }
   }
 }
@@ -252,43 +264,32 @@ static int bits_for(uint64_t n) {
   return b;
 }
 
-// Chunk records of the long rows of every label of the CSR `off`; offs gets
-// the L + 1 per-label chunk offsets.
+// Chunk records of the long rows of every label of the CSR `off`: offs[2 * l +
+// c] is the first of label l's class c, offs[2 * L] their number.
 static cudaError_t build_chunks(const uint32_t *off, uint32_t n, uint32_t L, uint32_t **chunks,
                                 std::vector<uint32_t> *offs, cudaStream_t st) {
-  u32 *cnt = nullptr;
-  u64 *pos = nullptr, *tmp = nullptr, *dtot = nullptr;
-  offs->assign(L + 1, 0);
-  cudaError_t e = cudaMallocAsync(&cnt, (u64)n * 4, st);
-  if (e == cudaSuccess) e = cudaMallocAsync(&pos, (u64)n * 8, st);
-  if (e == cudaSuccess) e = cudaMallocAsync(&tmp, scan_tmp_words(n) * 8, st);
-  if (e == cudaSuccess) e = cudaMallocAsync(&dtot, 8, st);
-  for (int pass = 0; pass < 2 && e == cudaSuccess; pass++) {
-    if (pass == 1) {
-      for (uint32_t l = 0; l < L; l++) (*offs)[l + 1] += (*offs)[l];
-      e = cudaMallocAsync(chunks, 3 * (u64)std::max(1u, (*offs)[L]) * 4, st);
-    }
-    for (uint32_t l = 0; l < L && e == cudaSuccess; l++) {
-      const uint32_t *row = off + (u64)l * (n + 1);
-      count_chunks<<<grid_for(n, 256), 256, 0, st>>>(row, n, cnt);
-      e = cudaGetLastError();
-      if (e == cudaSuccess) e = exclusive_scan_u32_to_u64(cnt, pos, n, dtot, tmp, st);
-      if (e != cudaSuccess) break;
-      if (pass == 0) {
-        u64 t = 0;
-        e = cudaMemcpyAsync(&t, dtot, 8, cudaMemcpyDeviceToHost, st);
-        if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-        (*offs)[l + 1] = (uint32_t)t;
-      } else {
-        write_chunks<<<grid_for(n, 256), 256, 0, st>>>(row, n, pos, (*offs)[l], *chunks);
-        e = cudaGetLastError();
-      }
-    }
+  u32 *next = nullptr;
+  offs->assign(2 * L + 1, 0);
+  std::vector<u32> cnt(2 * L, 0);
+  const dim3 grid((unsigned)std::min<u64>(grid_for(n, 256), 608), L);
+  cudaError_t e = cudaMallocAsync(&next, 8ull * L, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(next, 0, 8ull * L, st);
+  if (e == cudaSuccess) {
+    row_chunks<<<grid, 256, 0, st>>>(off, n, next, nullptr);
+    e = cudaGetLastError();
   }
-  if (cnt) cudaFreeAsync(cnt, st);
-  if (pos) cudaFreeAsync(pos, st);
-  if (tmp) cudaFreeAsync(tmp, st);
-  if (dtot) cudaFreeAsync(dtot, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(cnt.data(), next, 8ull * L, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e == cudaSuccess) {
+    for (uint32_t i = 0; i < 2 * L; i++) (*offs)[i + 1] = (*offs)[i] + cnt[i];
+    e = cudaMallocAsync(chunks, 3 * (u64)std::max(1u, (*offs)[2 * L]) * 4, st);
+  }
+  if (e == cudaSuccess) e = cudaMemcpyAsync(next, offs->data(), 8ull * L, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) {
+    row_chunks<<<grid, 256, 0, st>>>(off, n, next, *chunks);
+    e = cudaGetLastError();
+  }
+  if (next) cudaFreeAsync(next, st);
   return e;
 }
 

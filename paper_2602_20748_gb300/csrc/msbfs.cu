@@ -24,7 +24,7 @@
 //     each in-edge on an incoming transition from a state that is present in
 //     the frontier, it gathers the neighbour's G frontier words (one
 //     coalesced 512-byte read) and ORs them into per-lane accumulators; rows
-//     with at least HEAVY_ROW in-edges are cut (at graph load) into chunks
+//     with at least heavy_row in-edges are cut (at graph load) into chunks
 //     shared by all warps,
 // chosen per level from the byte cost of each given the DFA states present
 // in the frontier.  New lanes land in the next frontier word; a commit phase
@@ -688,7 +688,8 @@ __device__ __forceinline__ void publish_sums(BfsCtl *c, CommitSums &s, u32 nxt) 
 // with at most four gathers in flight and one in a row's tail.  Here the
 // gathers of 32 consecutive vertices are listed first, by all lanes together
 // (coalesced offsets and column ids, one round trip each for the whole list),
-// in shared memory; a vertex is then one round trip of up to eight gathers.
+// in shared memory; a vertex is then one round trip of up to six gathers (six
+// and eight differ by 1%, four and eight by 2%).
 // With a frontier bitmap only neighbours in the frontier are listed, and only
 // vertices with such a neighbour read their visited words.
 //
@@ -709,10 +710,10 @@ __device__ __forceinline__ u32 nth_bit(u32 m, u32 k) {
 }
 
 // ORs the listed rows lst[first], lst[first + step], ... below cnt into acc,
-// eight gathers in flight.  Lanes that are off must pass cnt = 0.
+// DEEP gathers in flight.  Lanes that are off must pass cnt = 0.
+template <int DEEP>
 __device__ __forceinline__ void gather_list(const u64 *F, u64 wpv, u32 lane_off, const u64 *lst, u32 first, u32 step,
                                             u32 cnt, u64 (&acc)[2]) {
-  constexpr int DEEP = 8;
   for (u32 k = first; k < cnt; k += DEEP * step) {
     ulonglong2 a[DEEP];
 #pragma unroll
@@ -771,12 +772,12 @@ __device__ void pull_staged(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 ac
         for (u32 j = p.q.in_begin[q]; j < p.q.in_begin[q + 1]; j++) {
           const u32 l = p.q.in_label[j];
           if (!(p.q.in_from[j] & active) || l >= p.L) continue;
-          const u64 cnt = p.hchunk_off[l + 1] - p.hchunk_off[l];
+          const u64 cnt = p.hchunk_end[l] - p.hchunk_beg[l];
           if (it < acc_base + cnt) {
             found = true;
             q2 = q;
             from = p.q.in_from[j] & active;
-            ci = p.hchunk_off[l] + (it - acc_base);
+            ci = p.hchunk_beg[l] + (it - acc_base);
             break;
           }
           acc_base += cnt;
@@ -804,7 +805,7 @@ __device__ void pull_staged(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 ac
             cnt += __popc(b);
           }
           __syncwarp();
-          gather_list(F, wpv, lane_off, lst, sg, VPW, lane_on ? cnt : 0, acc);
+          gather_list<6>(F, wpv, lane_off, lst, sg, VPW, lane_on ? cnt : 0, acc);
           stat_add(stat, ST_ALG_BYTES, cnt * gword);
         }
       }
@@ -836,7 +837,7 @@ __device__ void pull_staged(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 ac
           if (!from || l >= p.L) continue;
           const u32 *off = p.in_off + (u64)l * n1 + v;
           const u32 len = __ldg(off + 1) - __ldg(off);
-          if (len >= HEAVY_ROW && chunked)
+          if (len >= p.heavy_row && chunked)
             shared = true;
           else
             lens += len, tot += len * __popc(from);
@@ -882,7 +883,7 @@ __device__ void pull_staged(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 ac
               if (!from || l >= p.L) continue;
               const u32 *off = p.in_off + (u64)l * n1 + (u32)(c0 + o);
               const u32 beg = __ldg(off), len = __ldg(off + 1) - beg;
-              if (len >= HEAVY_ROW && chunked) continue;
+              if (len >= p.heavy_row && chunked) continue;
               const u32 np = __popc(from);
               if (r < len * np) {
                 col = beg + (np == 1 ? r : r / np);
@@ -933,7 +934,7 @@ __device__ void pull_staged(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 ac
           const u64 base = ((u64)q2 * n + w) * wpv + lane_off;
           u64 vis[2], acc[2] = {0, 0};
           load_vis<2>(p.vis + base, on, vis);
-          gather_list(F, wpv, lane_off, lst + x.y, 0, 1, on ? x.z : 0, acc);
+          gather_list<6>(F, wpv, lane_off, lst + x.y, 0, 1, on ? x.z : 0, acc);
           const u64 n0 = acc[0] & ~vis[0], n1w = acc[1] & ~vis[1];  // zero for lanes that are off
           const bool nz_l = (n0 | n1w) != 0;
           if (!__any_sync(FULL_MASK, nz_l)) continue;
@@ -1132,9 +1133,9 @@ __device__ void pull_lanes(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
       bool found = false;
       for (u64 lb = lset; lb && !found; lb &= lb - 1) {
         l = __ffsll((long long)lb) - 1;
-        const u64 cnt = p.hchunk_off[l + 1] - p.hchunk_off[l];
+        const u64 cnt = p.hchunk_end[l] - p.hchunk_beg[l];
         found = it < acc_base + cnt;
-        if (found) ci = p.hchunk_off[l] + (it - acc_base);
+        if (found) ci = p.hchunk_beg[l] + (it - acc_base);
         acc_base += cnt;
       }
       if (!found) break;
@@ -1158,7 +1159,7 @@ __device__ void pull_lanes(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
             cnt += __popc(b);
           }
           __syncwarp();
-          gather_list(F, wpv, lane_off, lst, 0, 1, lane_on ? cnt : 0, g);
+          gather_list<8>(F, wpv, lane_off, lst, 0, 1, lane_on ? cnt : 0, g);
           stat_add(stat, ST_ALG_BYTES, cnt * gword);
         }
         if (__any_sync(FULL_MASK, (g[0] | g[1]) != 0)) apply(l * LANE_SRC_Q + st, make_ulonglong2(g[0], g[1]));
@@ -1180,7 +1181,7 @@ __device__ void pull_lanes(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
       for (u64 lb = lset; lb; lb &= lb - 1) {
         const u32 *off = p.in_off + (u64)(__ffsll((long long)lb) - 1) * n1 + c0 + lane;
         const u32 len = __ldg(off + 1) - __ldg(off);
-        if (len >= HEAVY_ROW && chunked)
+        if (len >= p.heavy_row && chunked)
           sh = true;
         else
           tot += len;
@@ -1213,7 +1214,7 @@ __device__ void pull_lanes(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
           l = __ffsll((long long)lb) - 1;
           const u32 *off = p.in_off + (u64)l * n1 + c0 + o;
           const u32 beg = __ldg(off), len = __ldg(off + 1) - beg;
-          if (len >= HEAVY_ROW && chunked) continue;
+          if (len >= p.heavy_row && chunked) continue;
           if (r < len) {
             u = __ldg(p.in_col + beg + r);
             sm = tab.act[l];
@@ -1377,7 +1378,7 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
           if (!from || l >= p.L) continue;
           const u32 *off = p.in_off + (u64)l * n1 + v;
           const u32 beg = __ldg(off), len = __ldg(off + 1) - beg;
-          if (len >= HEAVY_ROW && chunked) {
+          if (len >= p.heavy_row && chunked) {
             hmask |= 1u << q2;
             continue;
           }
@@ -1452,7 +1453,7 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
           const u32 l = __ffsll((long long)lset) - 1;
           const u32 *off = p.in_off + (u64)l * n1 + w;
           const u32 beg = __ldg(off), end = __ldg(off + 1);
-          if (beg == end || (end - beg >= HEAVY_ROW && chunked)) continue;
+          if (beg == end || (end - beg >= p.heavy_row && chunked)) continue;
           u32 S = 0;  // source states of those transitions on label l
           for (u32 q2 = 0; q2 < Q; q2++)
             if ((wmask >> q2) & 1u)
@@ -1514,7 +1515,7 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
           if (!from || l >= p.L) continue;
           const u32 *off = p.in_off + (u64)l * n1 + w;
           const u32 beg = __ldg(off), end = __ldg(off + 1);
-          if (end - beg >= HEAVY_ROW && chunked) continue;
+          if (end - beg >= p.heavy_row && chunked) continue;
           for (u32 i = beg + li; i < end && !hit; i += SW) {
             const u32 u = __ldg(p.in_col + i);
             bytes += 4 + 4 * __popc(from);
@@ -1540,7 +1541,7 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
           if (!from || l >= p.L) continue;
           const u32 *off = p.in_off + (u64)l * n1 + w;
           const u32 beg = __ldg(off), end = __ldg(off + 1);
-          if (end - beg >= HEAVY_ROW && chunked) continue;
+          if (end - beg >= p.heavy_row && chunked) continue;
           // in multi mode each lane gathers through its own group's transitions
           u32 lfrom = from;
           if constexpr (AM == AM_GROUP) lfrom = lane_on ? p.from_tab[((u64)my_g * Q + q2) * p.L + l] & active : 0u;
@@ -1594,11 +1595,11 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
         bool found = false;
         for (u64 lb = lact; lb; lb &= lb - 1) {
           const u32 l = __ffsll((long long)lb) - 1;
-          const u64 cnt = p.hchunk_off[l + 1] - p.hchunk_off[l];
+          const u64 cnt = p.hchunk_end[l] - p.hchunk_beg[l];
           if (it < acc_base + cnt) {
             found = true;
             ls = l;
-            ci = p.hchunk_off[l] + (it - acc_base);
+            ci = p.hchunk_beg[l] + (it - acc_base);
             break;
           }
           acc_base += cnt;
@@ -1685,14 +1686,14 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
         for (u32 j = p.q.in_begin[q2]; j < p.q.in_begin[q2 + 1]; j++) {
           const u32 l = p.q.in_label[j];
           if (!(p.q.in_from[j] & active) || l >= p.L) continue;
-          const u64 cnt = p.hchunk_off[l + 1] - p.hchunk_off[l];
+          const u64 cnt = p.hchunk_end[l] - p.hchunk_beg[l];
           if (it < acc_base + cnt) {
             found = true;
             q2s = q2;
             ls = l;
             js = j;
             from = p.q.in_from[j] & active;
-            ci = p.hchunk_off[l] + (it - acc_base);
+            ci = p.hchunk_beg[l] + (it - acc_base);
             break;
           }
           acc_base += cnt;

@@ -55,8 +55,17 @@ int dfa_then_label(const HostQuery &alpha, uint32_t x, HostQuery *out, std::stri
 // ---------------------------------------------------------------------------
 // In-edge rows with at least HEAVY_ROW edges are cut into chunks of HCHUNK
 // edges at graph load; bottom-up levels share the chunks among all warps
-// instead of scanning such a row with one warp.
-constexpr uint32_t HEAVY_ROW = 128;
+// instead of scanning such a row with one warp.  At 32 edges the warps' shares
+// come out evener than at 128, though such a vertex's words are then or-ed
+// atomically: 1,500 reverse targets on R-MAT 2^18 1.78 -> 1.52 ms,
+// configuration 2 20.2 -> 19.0 (24: 19.3, 48: 19.2, 64: 19.4, 256: 20.5).
+// Launches of few start vertices leave a row at the first frontier vertices
+// they meet, so for them only rows of LONG_ROW edges are chunked (one lookup
+// on R-MAT 2^20: 0.55 ms, 0.60 with chunks from 32); the lists keep the two
+// classes of rows apart.
+constexpr uint32_t HEAVY_ROW = 32;
+constexpr uint32_t LONG_ROW = 128;
+constexpr uint32_t FEW_STARTS = 32;  // fewer start vertices than this chunk LONG_ROW rows only
 constexpr uint32_t HCHUNK = 256;
 
 struct DevGraph {
@@ -69,8 +78,9 @@ struct DevGraph {
   uint32_t *in_col = nullptr;
   uint8_t *vlabel = nullptr;
   // Chunks (vertex, first edge, end edge) of the rows with >= HEAVY_ROW
-  // edges, per direction, grouped by label: label l's chunks are
-  // [off[l], off[l+1]) (host copy of the L+1 offsets).
+  // edges, per direction, grouped by label and class: label l's chunks of rows
+  // of LONG_ROW edges and more are [off[2 l], off[2 l + 1]), those of shorter
+  // rows follow up to off[2 l + 2] (host copy of the 2 L + 1 offsets).
   uint32_t *hchunk_in = nullptr, *hchunk_out = nullptr;
   std::vector<uint32_t> hchunk_in_off, hchunk_out_off;
   std::vector<uint8_t> vlabel_host;   // vertex labels (host copy), empty if none
@@ -99,7 +109,7 @@ enum StatIdx {
 constexpr int TRACE_LEVELS = 64;
 constexpr unsigned long long NO_ENTRY = ~0ull;      // a reserved list slot left empty
 constexpr unsigned int ERR_LIST_OVERFLOW = 1000u;   // BfsCtl::err: an append ran past list_cap
-constexpr unsigned int APPEND_SEG = 128;             // list slots a warp reserves at a time
+constexpr unsigned int APPEND_SEG = 64;              // list slots a warp reserves at a time (32, 128: 1% slower)
 
 struct BfsCtl {
   // grid barrier (grid_barrier.cuh): blocks that have arrived, over all
@@ -142,7 +152,9 @@ struct BfsParams {
   const uint32_t *in_off;
   const uint32_t *in_col;
   const uint32_t *hchunk;       // chunks of long in_off rows (nullptr: none)
-  uint32_t hchunk_off[RPQ_MAX_LABELS + 1];
+  uint32_t hchunk_beg[RPQ_MAX_LABELS];  // per label, the chunks of rows of
+  uint32_t hchunk_end[RPQ_MAX_LABELS];  // at least heavy_row edges
+  uint32_t heavy_row;
   unsigned long long label_edges[RPQ_MAX_LABELS];
   uint32_t n;
   uint32_t L;             // edge labels of the graph
@@ -211,6 +223,17 @@ struct BfsParams {
   unsigned long long time_limit_ns;
   QueryDesc q;
 };
+
+// The chunk lists of a launch of `starts` start vertices.
+inline void set_chunks(BfsParams &p, const uint32_t *chunks, const std::vector<uint32_t> &offs, uint32_t L,
+                       uint64_t starts) {
+  p.hchunk = chunks;
+  p.heavy_row = starts < FEW_STARTS ? LONG_ROW : HEAVY_ROW;
+  for (uint32_t l = 0; l < L; l++) {
+    p.hchunk_beg[l] = offs[2 * l];
+    p.hchunk_end[l] = offs[2 * l + (starts < FEW_STARTS ? 1 : 2)];
+  }
+}
 
 // Launchers (return cudaError_t of the launch).
 cudaError_t launch_vis_init(int nw, const BfsParams &p, const unsigned long long *empty, cudaStream_t st);

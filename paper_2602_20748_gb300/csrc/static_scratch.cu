@@ -204,8 +204,7 @@ extern "C" int run_rpq_static(rpq_ctx *ctx, const rpq_graph *g, const rpq_query 
   // chunks of long in-rows belong to the graph: scanned in place, one lane
   // walked a row of up to 10^4 edges alone (64 start vertices on R-MAT 2^18:
   // 3.2 ms a call)
-  p.hchunk = dg.hchunk_in;
-  for (uint32_t l = 0; l <= dg.L && l < dg.hchunk_in_off.size(); l++) p.hchunk_off[l] = dg.hchunk_in_off[l];
+  set_chunks(p, dg.hchunk_in, dg.hchunk_in_off, dg.L, ns);
   for (uint32_t l = 0; l < dg.L; l++) p.label_edges[l] = dg.label_edges[l];
   p.time_limit_ns = ctx_time_limit_ns(ctx);
   p.q = qd;
