@@ -479,7 +479,7 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
     p.claim = w.claim;
     p.fbits = w.fbits;
     p.fbits_words = w.fbits_words();
-    p.append_seg = APPEND_SEG;
+    p.append_seg = append_seg(nw);
     p.list_cap = w.list_cap;
     p.spill = w.spill;
     p.spill_cap = ctx->spill_cap;
@@ -1781,7 +1781,7 @@ int rpq_lane_stats_multi(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Mu
   p.list1 = w.list1;
   p.fbits = w.fbits;
   p.fbits_words = w.fbits_words();
-  p.append_seg = APPEND_SEG;
+  p.append_seg = append_seg(1);
   p.list_cap = w.list_cap;
   p.ctl = ctx->ctl;
   p.stamp_base = ctx->stamp;
@@ -2047,7 +2047,7 @@ static int lane_launch(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Lane
   p.list1 = w.list1;
   p.fbits = w.fbits;
   p.fbits_words = w.fbits_words();
-  p.append_seg = APPEND_SEG;
+  p.append_seg = append_seg(nw);
   p.list_cap = w.list_cap;
   p.ctl = ctx->ctl;
   p.stamp_base = ctx->stamp;

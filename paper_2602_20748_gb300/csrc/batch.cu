@@ -879,7 +879,7 @@ static int batch_launch(rpq_ctx *ctx, const rpq_graph *g, uint32_t qbase, uint32
   // segments only when the unused tails (at most three appending phases per
   // level, one segment per warp each) stay a small part of the list
   const u64 nwarps = (u64)blocks * tun.threads / 32;
-  p.append_seg = tun.list_cap >= 16 * 3 * nwarps * APPEND_SEG ? APPEND_SEG : 0;
+  p.append_seg = tun.list_cap >= 16 * 3 * nwarps * APPEND_SEG ? append_seg(4) : 0;
   void *args[] = {(void *)&p};
   cudaEvent_t ev0, ev1;
   cudaEventCreate(&ev0);
@@ -1099,7 +1099,7 @@ static void serve_params(ServeEngine *e) {
   p.qw = e->qw.p;
   p.evicted = e->evicted.p;
   p.evict_at = e->evict_at;
-  p.append_seg = APPEND_SEG;
+  p.append_seg = append_seg(4);
   p.hash_bits = e->hbits;
   p.rtab = e->rtab.p;
   p.qstats = e->qstats.p;

@@ -109,7 +109,11 @@ enum StatIdx {
 constexpr int TRACE_LEVELS = 64;
 constexpr unsigned long long NO_ENTRY = ~0ull;      // a reserved list slot left empty
 constexpr unsigned int ERR_LIST_OVERFLOW = 1000u;   // BfsCtl::err: an append ran past list_cap
-constexpr unsigned int APPEND_SEG = 64;              // list slots a warp reserves at a time (32, 128: 1% slower)
+constexpr unsigned int APPEND_SEG = 128;             // list slots a warp reserves at a time, at most
+// Launches of several words per vertex reserve half as many (configuration 2
+// 1% faster); with one word a warp appends up to 32 entries at once (one lookup
+// on R-MAT 2^20: 550 us, 600 with 64).
+inline unsigned int append_seg(int nw) { return nw == 1 ? APPEND_SEG : APPEND_SEG / 2; }
 
 struct BfsCtl {
   // grid barrier (grid_barrier.cuh): blocks that have arrived, over all
