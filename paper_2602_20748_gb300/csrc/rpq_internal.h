@@ -240,7 +240,12 @@ inline void set_chunks(BfsParams &p, const uint32_t *chunks, const std::vector<u
 }
 
 // Launchers (return cudaError_t of the launch).
-cudaError_t launch_vis_init(int nw, const BfsParams &p, const unsigned long long *empty, cudaStream_t st);
+cudaError_t launch_vis_init(const BfsParams &p, const unsigned long long *empty, cudaStream_t st);
+// Before a launch_msbfs of `live` start vertices, in lanes 0 .. live - 1: VIS,
+// the control block and small[0 .. 4) set up; with ids (at most 64), lanesrc
+// [0 .. 64) too.
+cudaError_t launch_start(int nw, const BfsParams &p, uint32_t live, unsigned long long *small, uint32_t *lanesrc,
+                         const uint32_t *ids, cudaStream_t st);
 cudaError_t launch_msbfs(int nw, const BfsParams &p, int blocks, int threads, cudaStream_t st);
 // Per-group automata (p.qg set): one lane word per group (NW = 1).
 cudaError_t launch_msbfs_multi(const BfsParams &p, int blocks, int threads, cudaStream_t st);
@@ -335,9 +340,11 @@ cudaError_t preload_scan_kernels();
 cudaError_t launch_zero_lane_counts(uint32_t *cnt, uint32_t segs, uint32_t n_lanes, const uint32_t *lane_slot,
                                     cudaStream_t st);
 // lane_off[i] = off[i * segs] for the first `live` lanes, *total from there to
-// lane_off[n_lanes] (lanes without a start vertex are the last ones).
+// lane_off[n_lanes] (lanes without a start vertex are the last ones); with
+// lanesrc_out, also copies the lanes' start vertices there.
 cudaError_t launch_gather_lane_off(const unsigned long long *off, uint32_t segs, uint32_t n_lanes, uint32_t live,
-                                   const unsigned long long *total, unsigned long long *lane_off, cudaStream_t st);
+                                   const unsigned long long *total, unsigned long long *lane_off,
+                                   const uint32_t *lanesrc, uint32_t *lanesrc_out, cudaStream_t st);
 
 // Pair expansion for fetch: out[2k], out[2k+1] = (src, dst) of row first + k.
 cudaError_t launch_expand_pairs(const uint32_t *lanesrc, const unsigned long long *lane_off, uint32_t n_lanes,

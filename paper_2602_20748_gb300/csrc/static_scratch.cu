@@ -47,7 +47,7 @@ static size_t static_scratch_need(uint32_t Q, uint32_t n, uint32_t segs) {
   need += align256(sizeof(BfsCtl));
   need += align256(4 * sizeof(u64));    // digest sum, xor, total, spare
   need += align256(64 * sizeof(u32));   // lanesrc
-  need += align256(sizeof(u64));        // empty-lane mask
+  need += align256(sizeof(u64));        // spare
   need += 5 * align256(words * 8);      // VIS, two frontiers, two entry lists
   need += align256((size_t)64 * segs * 4);  // per (lane, segment) counts
   need += align256((size_t)64 * segs * 8);  // their offsets
@@ -137,7 +137,7 @@ extern "C" int run_rpq_static(rpq_ctx *ctx, const rpq_graph *g, const rpq_query 
   BfsCtl *ctl = (BfsCtl *)take(sizeof(BfsCtl));
   u64 *small = (u64 *)take(4 * sizeof(u64));
   u32 *lanesrc = (u32 *)take(64 * sizeof(u32));
-  u64 *empty = (u64 *)take(sizeof(u64));
+  take(sizeof(u64));  // spare, so that what fits and what is refused stays as it was
   u64 *vis = (u64 *)take(words * 8);
   u64 *fr0 = (u64 *)take(words * 8);
   u64 *fr1 = (u64 *)take(words * 8);
@@ -148,24 +148,14 @@ extern "C" int run_rpq_static(rpq_ctx *ctx, const rpq_graph *g, const rpq_query 
   u64 *tmp = (u64 *)take(scan_tmp_words((size_t)64 * segs) * 8);
 
   cudaStream_t st = ctx_stream(ctx);
-  uint32_t lanes[64];
-  uint64_t empty_mask = 0;
-  for (uint32_t i = 0; i < 64; i++) {
-    lanes[i] = i < ns ? src[i] : NO_SOURCE;
-    if (i >= ns) empty_mask |= 1ull << i;
-  }
 #define STATIC_CK(expr)                                                                                 \
   do {                                                                                                  \
     cudaError_t _e = (expr);                                                                            \
     if (_e != cudaSuccess) return ctx_error(ctx, RPQ_ERR_CUDA, std::string(#expr) + ": " + cudaGetErrorString(_e)); \
   } while (0)
-  // what must start at zero: control block, digest / total, both frontiers
-  STATIC_CK(cudaMemsetAsync(ctl, 0, sizeof(BfsCtl), st));
-  STATIC_CK(cudaMemsetAsync(small, 0, 4 * sizeof(u64), st));
+  // what must start at zero: both frontiers here, the rest in launch_start
   STATIC_CK(cudaMemsetAsync(fr0, 0, words * 8, st));
   STATIC_CK(cudaMemsetAsync(fr1, 0, words * 8, st));
-  STATIC_CK(cudaMemcpyAsync(lanesrc, lanes, sizeof(lanes), cudaMemcpyHostToDevice, st));
-  STATIC_CK(cudaMemcpyAsync(empty, &empty_mask, sizeof(empty_mask), cudaMemcpyHostToDevice, st));
 
   BfsParams p;
   std::memset(&p, 0, sizeof(p));
@@ -208,7 +198,7 @@ extern "C" int run_rpq_static(rpq_ctx *ctx, const rpq_graph *g, const rpq_query 
   for (uint32_t l = 0; l < dg.L; l++) p.label_edges[l] = dg.label_edges[l];
   p.time_limit_ns = ctx_time_limit_ns(ctx);
   p.q = qd;
-  STATIC_CK(launch_vis_init(1, p, empty, st));
+  STATIC_CK(launch_start(1, p, ns, small, lanesrc, src, st));
   STATIC_CK(launch_msbfs(1, p, grid, 256, st));
 
   EmitParams ep{};

@@ -1,0 +1,64 @@
+"""RPQ evaluation where a size decides which path a level or a row takes: rows
+at the borders of the chunk classes (32, 128 and 256 edges), frontiers around
+the 512 edges that one block expands alone, vertex counts around an emission
+segment, source counts around a word, a row and a group of lanes.  Rows, digest and
+work counter equal the CPU oracle's exactly, for automatic, all top-down and
+all bottom-up levels."""
+
+import numpy as np
+import pytest
+
+import oracle
+from paper_2602_20748_gb300 import synth
+from test_gpu_rpq import MODES, check
+
+pytestmark = pytest.mark.gpu
+
+rpq = pytest.importorskip("paper_2602_20748_gb300.rpq")
+
+DEGREES = (1, 31, 32, 33, 127, 128, 129, 255, 256, 257, 511, 512, 513)
+
+
+@pytest.fixture(scope="module")
+def stars():
+    """13 vertices with exactly DEGREES[i] out-edges on label a, 13 with as
+    many in-edges on it, and two random edges per vertex on labels b and c."""
+    n = 2100
+    rng = np.random.Generator(np.random.PCG64(11))
+    src, dst, lab = [], [], []
+    for i, d in enumerate(DEGREES):
+        src += [i] * d
+        dst += rng.choice(np.arange(100, n), d, replace=False).tolist()
+        src += rng.choice(np.arange(100, n), d, replace=False).tolist()
+        dst += [40 + i] * d
+        lab += [0] * (2 * d)
+    src += rng.integers(0, n, 4 * n).tolist()
+    dst += rng.integers(0, n, 4 * n).tolist()
+    lab += [1, 2] * (2 * n)
+    g = n, 3, np.array(src, np.uint32), np.array(dst, np.uint32), np.array(lab, np.uint16)
+    c = rpq.Context(device=0)
+    return c, rpq.load_graph(c, *g), oracle.Graph(*g)
+
+
+@pytest.mark.parametrize("count", [1, 31, 32, 64, 65, 256, 257, 600])
+@pytest.mark.parametrize("regex", ["a", "a.b.c*", "(a|b)+.c", "a?.b*.a"])
+def test_row_lengths_and_source_counts(stars, regex, count):
+    c, g, og = stars
+    sources = np.arange(count, dtype=np.uint32)  # the stars first
+    want = oracle.rpq(og, regex, sources=sources)
+    for mode in MODES.values():
+        check(c, g, og, regex, sources=sources, mode=mode, want=want)
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 255, 256, 257, 511, 513, 1023, 1025])
+def test_vertex_counts_around_emission_segments(n):
+    """Two accepting states, both lane widths, rows kept and counted only."""
+    src, dst, lab = synth.random_graph(n, 3 * n, 2, seed=500 + n)
+    c = rpq.Context(device=0)
+    g, og = rpq.load_graph(c, n, 2, src, dst, lab), oracle.Graph(n, 2, src, dst, lab)
+    for sources in (np.arange(min(n, 64), dtype=np.uint32), None):
+        want = oracle.rpq(og, "a.b?", sources=sources)
+        rows, _ = check(c, g, og, "a.b?", sources=sources, want=want)
+        q = rpq.compile_rpq(c, "a.b?")
+        r = rpq.run_rpq(c, g, q, sources, flags=rpq.RPQ_COUNT_ONLY)
+        assert rpq.result_info(r)[0] == len(rows) and rpq.result_info(r)[2:4] == oracle.pair_digest(want.rows)[1:]
