@@ -175,9 +175,10 @@ __device__ __forceinline__ void bappend_close(const BatchParams &p, BAppender &a
 }
 
 // Test-and-set of (query i, state q2, vertex w); true when this thread set it.
+template <bool HASH>
 __device__ __forceinline__ bool bvisit(const BatchParams &p, u32 i, u32 q2, u32 w) {
   if (bad(p, i >= p.nq, 1) || bad(p, w >= p.n, 2)) return false;
-  if (p.hash_bits) {
+  if constexpr (HASH) {
     if (bad(p, q2 >= p.qd[i].n_states, 3)) return false;
     const int r = hinsert(p.vis + ((u64)i << p.hash_bits), p.hash_bits, (((u64)q2 << 32) | w) + 1);
     if (r < 0) p.evicted[i] = 1u;  // table full: the query leaves the batch
@@ -203,6 +204,47 @@ __device__ __forceinline__ bool bvisit(const BatchParams &p, u32 i, u32 q2, u32 
   return !(atomicOr((unsigned long long *)word, bit) & bit);
 }
 
+// Edges a lane takes at once in a push.  With bitmaps the words of four edges
+// are read together and the ones that need it set together: an edge's read, its
+// atomic and its append are a chain of three trips to L2, and a warp has no
+// other work in flight (48 queries on 2^16 vertices: 1,108 us one at a time,
+// 951 two, 915 four, 1,034 eight; at 64 registers for two blocks of 512 threads
+// an SM; with the 105 that the compiler takes unasked 1,020).  Hash probes are loops of their own and stay one at a
+// time (4,096 queries on 2^22 vertices: 279 ms either way).
+template <bool HASH>
+constexpr int PUSH_WIDE = HASH ? 1 : 4;
+
+template <bool HASH, int N>
+__device__ __forceinline__ void bvisit_wide(const BatchParams &p, const u32 (&i)[N], const u32 (&q2)[N],
+                                            const u32 (&w)[N], bool (&take)[N]) {
+  if constexpr (HASH) {
+#pragma unroll
+    for (int k = 0; k < N; k++) take[k] = take[k] && bvisit<true>(p, i[k], q2[k], w[k]);
+    return;
+  }
+  u64 *word[N];
+#pragma unroll
+  for (int k = 0; k < N; k++) {
+    word[k] = p.vis;
+    if (!take[k]) continue;
+    take[k] = !bad(p, i[k] >= p.nq, 1) && !bad(p, w[k] >= p.n, 2);
+    if (!take[k]) continue;
+    const u64 at = p.vis_off[i[k]] + (u64)q2[k] * p.wps + (w[k] >> 6);
+    take[k] = !bad(p, at >= p.vis_words || q2[k] >= p.qd[i[k]].n_states, 3);
+    if (take[k]) word[k] += at;
+  }
+  u64 seen[N];
+#pragma unroll
+  for (int k = 0; k < N; k++) seen[k] = take[k] ? __ldcg(word[k]) : ~0ull;
+#pragma unroll
+  for (int k = 0; k < N; k++) {
+    const u64 bit = 1ull << (w[k] & 63);
+    if (!(seen[k] & bit)) seen[k] = atomicOr((unsigned long long *)word[k], bit);
+  }
+#pragma unroll
+  for (int k = 0; k < N; k++) take[k] = !((seen[k] >> (w[k] & 63)) & 1ull);
+}
+
 // Whether a query with N product vertices and W product edges so far leaves
 // the batch: past evict_at vertices, or past EVICT_EDGES times as many edges.
 // The edges of a frontier are known before it is expanded, so a query that is
@@ -214,6 +256,7 @@ __device__ __forceinline__ bool outgrown(const BatchParams &p, u64 N, u64 W) {
   return p.evict_at && (N > p.evict_at || W > p.evict_at * EVICT_EDGES);
 }
 
+template <bool HASH>
 __device__ void bseed(const BatchParams &p, u64 *W, u64 *N) {
   const u64 stride = (u64)gridDim.x * blockDim.x;
   BAppender app;
@@ -224,7 +267,7 @@ __device__ void bseed(const BatchParams &p, u64 *W, u64 *N) {
     u32 s = 0;
     if (i < p.nq && p.qd[i].n_states > 0) {
       s = p.srcs[i];
-      take = bvisit(p, (u32)i, 0, s);
+      take = bvisit<HASH>(p, (u32)i, 0, s);
       if (take) {
         const u32 d = bdegsum(p, p.qd[i], 0, s);
         *W += d;
@@ -244,10 +287,12 @@ __device__ void bseed(const BatchParams &p, u64 *W, u64 *N) {
   if (lane_id() == 0 && mf) atomicAdd(&p.ctl->mf[0], mf);
 }
 
+template <bool HASH>
 __device__ void bpush(const BatchParams &p, int lp, u32 cur, u32 nxt, u64 n_cur, u32 grab, u32 chunk, u32 seg,
                       u64 *edges) {
   const u64 *list = lp ? p.list1 : p.list0;
   u64 *nlist = lp ? p.list0 : p.list1;
+  constexpr int WIDE = PUSH_WIDE<HASH>;
   const u32 lane = lane_id();
   BAppender app;
   app.seg = seg;
@@ -308,33 +353,42 @@ __device__ void bpush(const BatchParams &p, int lp, u32 cur, u32 nxt, u64 n_cur,
       const u32 total = __shfl_sync(FULL_MASK, pre, 31);
       pre -= rlen;
       *edges += (lane == 0) ? total : 0;
-      for (u32 k0 = 0; k0 < total; k0 += 32) {
-        const u32 k = k0 + lane;
-        u32 o = 0;
+      for (u32 k0 = 0; k0 < total; k0 += 32 * WIDE) {
+        bool take[WIDE];
+        u32 w[WIDE], to_q[WIDE], to_i[WIDE];
 #pragma unroll
-        for (u32 step = 16; step > 0; step >>= 1) {
-          u32 pv = __shfl_sync(FULL_MASK, pre, o + step);
-          if (pv <= k) o += step;
+        for (int x = 0; x < WIDE; x++) {
+          take[x] = false;
+          w[x] = to_q[x] = to_i[x] = 0;
+          if (x > 0 && k0 + 32 * x >= total) continue;  // uniform
+          const u32 k = k0 + 32 * x + lane;
+          u32 o = 0;
+#pragma unroll
+          for (u32 step = 16; step > 0; step >>= 1) {
+            u32 pv = __shfl_sync(FULL_MASK, pre, o + step);
+            if (pv <= k) o += step;
+          }
+          const u32 o_beg = __shfl_sync(FULL_MASK, rbeg, o);
+          const u32 o_pre = __shfl_sync(FULL_MASK, pre, o);
+          to_q[x] = __shfl_sync(FULL_MASK, q2, o);
+          to_i[x] = __shfl_sync(FULL_MASK, i, o);
+          take[x] = k < total && !bad(p, (u64)o_beg + (k - o_pre) >= p.m, 7);
+          w[x] = take[x] ? __ldg(p.out_col + o_beg + (k - o_pre)) : 0;
         }
-        const u32 o_beg = __shfl_sync(FULL_MASK, rbeg, o);
-        const u32 o_pre = __shfl_sync(FULL_MASK, pre, o);
-        const u32 o_q2 = __shfl_sync(FULL_MASK, q2, o);
-        const u32 o_i = __shfl_sync(FULL_MASK, i, o);
-        bool take = false;
-        u32 w = 0;
-        if (k < total && !bad(p, (u64)o_beg + (k - o_pre) >= p.m, 7)) {
-          w = __ldg(p.out_col + o_beg + (k - o_pre));
-          take = bvisit(p, o_i, o_q2, w);
-        }
-        bappend(p, app, take, bentry(o_i, o_q2, w), &p.ctl->n_list[nxt], nlist);
+        bvisit_wide<HASH>(p, to_i, to_q, w, take);
+#pragma unroll
+        for (int x = 0; x < WIDE; x++)
+          bappend(p, app, take[x], bentry(to_i[x], to_q[x], w[x]), &p.ctl->n_list[nxt], nlist);
       }
     }
   }
   bappend_close(p, app, nlist);
 }
 
+template <bool HASH>
 __device__ void bspill(const BatchParams &p, int lp, u32 cur, u32 nxt, u32 seg, u64 *edges) {
   u64 *nlist = lp ? p.list0 : p.list1;
+  constexpr int WIDE = PUSH_WIDE<HASH>;
   const u32 lane = lane_id();
   const u64 count = min(*(volatile unsigned long long *)&p.ctl->spill_count[cur], (unsigned long long)p.spill_cap);
   BAppender app;
@@ -345,15 +399,22 @@ __device__ void bspill(const BatchParams &p, int lp, u32 cur, u32 nxt, u32 seg, 
     const u32 i = (u32)(h >> 37), q2 = (u32)(h >> 32) & 31u, b = (u32)h;
     if (p.evict_at && i < p.nq && __ldcg(&p.evicted[i])) continue;  // warp-uniform
     *edges += (lane == 0) ? len : 0;
-    for (u32 k0 = 0; k0 < len; k0 += 32) {
-      const u32 k = k0 + lane;
-      bool take = false;
-      u32 w = 0;
-      if (k < len && !bad(p, (u64)b + k >= p.m, 8)) {
-        w = __ldg(p.out_col + b + k);
-        take = bvisit(p, i, q2, w);
+    for (u32 k0 = 0; k0 < len; k0 += 32 * WIDE) {
+      bool take[WIDE];
+      u32 w[WIDE];
+      u32 to_i[WIDE], to_q[WIDE];
+#pragma unroll
+      for (int x = 0; x < WIDE; x++) {
+        const u32 k = k0 + 32 * x + lane;
+        to_i[x] = i;
+        to_q[x] = q2;
+        take[x] = k < len && !bad(p, (u64)b + k >= p.m, 8);
+        w[x] = take[x] ? __ldg(p.out_col + b + k) : 0;
       }
-      bappend(p, app, take, bentry(i, q2, w), &p.ctl->n_list[nxt], nlist);
+      bvisit_wide<HASH>(p, to_i, to_q, w, take);
+#pragma unroll
+      for (int x = 0; x < WIDE; x++)
+        bappend(p, app, take[x], bentry(i, q2, w[x]), &p.ctl->n_list[nxt], nlist);
     }
   }
   bappend_close(p, app, nlist);
@@ -406,11 +467,12 @@ __device__ void bcommit(const BatchParams &p, int lp, u32 nxt, u64 *W, u64 *N, u
   if (lane_id() == 0 && mf) atomicAdd(&p.ctl->mf[nxt], mf);
 }
 
-__global__ void __launch_bounds__(BATCH_MAX_THREADS) batch_kernel(const __grid_constant__ BatchParams p) {
+template <bool HASH>
+__global__ void __launch_bounds__(BATCH_MAX_THREADS, 2) batch_kernel(const __grid_constant__ BatchParams p) {
   BfsCtl *c = p.ctl;
   unsigned epoch = 0;  // grid barriers passed
   u64 W = 0, N = 0, edges = 0, push_levels = 0;
-  bseed(p, &W, &N);
+  bseed<HASH>(p, &W, &N);
   if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
   u32 level = 0;
   for (;; level++) {
@@ -435,11 +497,11 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS) batch_kernel(const __grid_c
       }
       push_levels++;
     }
-    bpush(p, lp, cur, nxt, n_cur, push_grab(n_cur, mf, n_warps), spill_chunk(mf, n_warps, p.spill_cap), seg,
+    bpush<HASH>(p, lp, cur, nxt, n_cur, push_grab(n_cur, mf, n_warps), spill_chunk(mf, n_warps, p.spill_cap), seg,
           &edges);
     if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
     if (*(volatile unsigned long long *)&c->spill_count[cur] != 0) {
-      bspill(p, lp, cur, nxt, seg, &edges);
+      bspill<HASH>(p, lp, cur, nxt, seg, &edges);
       if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
     }
     bcommit(p, lp, nxt, &W, &N);
@@ -549,7 +611,7 @@ __device__ void serve_admit(const ServeParams &sp, u32 level, u32 cur, int lp, u
       }
       __syncwarp();
       if (lane == 0 && src < p.n && sp.slot_qd[slot].n_states > 0) {
-        take = bvisit(p, slot, 0, src);
+        take = bvisit<true>(p, slot, 0, src);
         if (take) {
           const u32 d = bdegsum(p, sp.slot_qd[slot], 0, src);
           p.qn[slot] = 1;
@@ -647,11 +709,11 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS) serve_kernel(const __grid_c
     }
     if (n_cur > 0) {
       // admissions between levels add out-edges that no commit counted: the longest chunks
-      bpush(p, lp, cur, nxt, n_cur, push_grab(n_cur, 0, (u64)p.nblocks * (blockDim.x >> 5)), SPILL_EDGES, p.append_seg,
+      bpush<true>(p, lp, cur, nxt, n_cur, push_grab(n_cur, 0, (u64)p.nblocks * (blockDim.x >> 5)), SPILL_EDGES, p.append_seg,
             &edges);
       if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
       if (*(volatile unsigned long long *)&c->spill_count[cur] != 0) {
-        bspill(p, lp, cur, nxt, p.append_seg, &edges);
+        bspill<true>(p, lp, cur, nxt, p.append_seg, &edges);
         if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
       }
       bcommit(p, lp, nxt, &W, &N, level + 1);
@@ -869,10 +931,11 @@ static int batch_launch(rpq_ctx *ctx, const rpq_graph *g, uint32_t qbase, uint32
   p.spill_cap = tun.spill_cap;
   p.ctl = d_ctl.p;
   p.time_limit_ns = ctx_time_limit_ns(ctx);
+  void (*const kernel)(BatchParams) = use_hash ? batch_kernel<true> : batch_kernel<false>;
   int bpsm = 0, sms = 0, dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bpsm, batch_kernel, tun.threads, 0)) != cudaSuccess)
+  if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bpsm, kernel, tun.threads, 0)) != cudaSuccess)
     return berr(ctx, e, "occupancy");
   const int blocks = std::max(1, std::min(sms, ctx_sm_share(ctx))) * bpsm;
   p.nblocks = (unsigned)blocks;
@@ -885,7 +948,7 @@ static int batch_launch(rpq_ctx *ctx, const rpq_graph *g, uint32_t qbase, uint32
   cudaEventCreate(&ev0);
   cudaEventCreate(&ev1);
   cudaEventRecord(ev0, st);
-  e = cudaLaunchCooperativeKernel((void *)batch_kernel, blocks, tun.threads, args, 0, st);
+  e = cudaLaunchCooperativeKernel((void *)kernel, blocks, tun.threads, args, 0, st);
   cudaEventRecord(ev1, st);
   if (e != cudaSuccess) {
     cudaEventDestroy(ev0);

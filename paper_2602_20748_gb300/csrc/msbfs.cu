@@ -2043,8 +2043,7 @@ cudaError_t launch_vis_init(const BfsParams &p, const unsigned long long *empty,
 // own parameters.  One launch for what took five calls, and with one
 // allocation and one read-back where there were three and two, a lookup on a
 // 1,000-vertex graph takes 98 us for 112, and one on 2^20 vertices 536 for 553.
-// More than 64 start vertices are copied from the host as before: parameters
-// hold 1,000 of them at most, and a launch of that size takes 0.5 ms or more.
+// More than 64 start vertices are copied from the host as before.
 struct StartLanes {
   u32 id[64];
 };

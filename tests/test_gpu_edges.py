@@ -62,3 +62,23 @@ def test_vertex_counts_around_emission_segments(n):
         q = rpq.compile_rpq(c, "a.b?")
         r = rpq.run_rpq(c, g, q, sources, flags=rpq.RPQ_COUNT_ONLY)
         assert rpq.result_info(r)[0] == len(rows) and rpq.result_info(r)[2:4] == oracle.pair_digest(want.rows)[1:]
+
+
+@pytest.mark.parametrize("flags", [rpq.RPQ_MATERIALIZE, rpq.RPQ_PER_QUERY])
+@pytest.mark.parametrize("regex", ["a", "a.a", "(a|b)+.c?"])
+def test_batch_row_lengths(stars, regex, flags):
+    """A query per star: the lists of a push hold 1 to 513 edges, and several
+    rows meet in one warp."""
+    c, g, og = stars
+    sources = np.arange(len(DEGREES) + 40, dtype=np.uint32)
+    r = rpq.run_rpq_batch(c, g, [rpq.compile_rpq(c, regex)] * len(sources), sources, flags=flags)
+    rows, W = [], 0
+    for i, s in enumerate(sources):
+        want = oracle.rpq(og, regex, sources=[int(s)])
+        W += want.W
+        rows += [(i, int(y)) for y in want.rows[:, 1]]
+        if flags == rpq.RPQ_PER_QUERY:
+            assert rpq.result_query_stats(r, i) == oracle.pair_digest(want.rows)
+    assert rpq.result_stats(r)["product_edges"] == W
+    if flags == rpq.RPQ_MATERIALIZE:
+        assert np.array_equal(rpq.fetch_pairs(r), np.array(rows, np.uint32).reshape(-1, 2))
