@@ -454,7 +454,7 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
     const uint32_t Gb = (uint32_t)std::min<uint64_t>(G, groups_total - g0);
     const uint32_t n_lanes = Gb * K;
     const uint32_t live = (uint32_t)std::min<uint64_t>(n_lanes, srcs.size() - g0 * K);  // the others are empty
-    const uint32_t tiles = emit_tiles(nw, Gb, n), segs = emit_segs(tiles, n);
+    uint32_t tiles = emit_tiles(nw, Gb, n), segs = emit_segs(tiles, n);
     if (n_lanes > 64) {
       lanes.assign(n_lanes, NO_SOURCE);
       std::copy(srcs.begin() + g0 * K, srcs.begin() + g0 * K + live, lanes.begin());
@@ -568,13 +568,22 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
     }
 
     // emission pass 1: counts and digest
-    const uint64_t ncnt = (uint64_t)n_lanes * segs;
-    const uint64_t nscan = (uint64_t)live * segs;
-    // one allocation: the offsets, the scan's scratch, the counts
-    const uint64_t tmpw = scan_tmp_words(ncnt), nscratch = ncnt + tmpw + (ncnt + 1) / 2;
+    // one allocation: the offsets, the scan's scratch, the counts; where the
+    // budget has no room for short segments, longer ones (down to what the
+    // longest need)
+    uint64_t ncnt, tmpw, nscratch;
     u64 *off = nullptr;
     int rc;
-    if ((rc = dalloc(ctx, &off, nscratch))) return rc;
+    for (;;) {
+      ncnt = (uint64_t)n_lanes * segs;
+      tmpw = scan_tmp_words(ncnt);
+      nscratch = ncnt + tmpw + (ncnt + 1) / 2;
+      if ((rc = dalloc(ctx, &off, nscratch)) == RPQ_OK) break;
+      if (tiles >= (uint32_t)EMIT_TILES) return rc;
+      tiles <<= 1;
+      segs = emit_segs(tiles, n);
+    }
+    const uint64_t nscan = (uint64_t)live * segs;
     u64 *const tmp = off + ncnt;
     u32 *const cnt = reinterpret_cast<u32 *>(tmp + tmpw);
     EmitParams ep{};

@@ -9,8 +9,8 @@
 // shared frontier list of (query, state, vertex) entries.  A level is
 // expanded top-down: a warp takes 32 entries, spreads the out-edges of their
 // transition rows evenly over its lanes, and test-and-sets the target bits
-// (a plain read first, the atomic only when the bit is clear); rows longer
-// than SPILL_EDGES are cut into chunks shared by all warps.  Results are the
+// (a plain read first, the atomic only when the bit is clear); long rows are
+// cut into chunks shared by all warps (spill_chunk).  Results are the
 // accepting states' bitmaps, emitted as (query index, vertex) rows.
 #include <algorithm>
 #include <atomic>
@@ -209,8 +209,9 @@ __device__ __forceinline__ bool bvisit(const BatchParams &p, u32 i, u32 q2, u32 
 // atomic and its append are a chain of three trips to L2, and a warp has no
 // other work in flight (48 queries on 2^16 vertices: 1,108 us one at a time,
 // 951 two, 915 four, 1,034 eight; at 64 registers for two blocks of 512 threads
-// an SM; with the 105 that the compiler takes unasked 1,020).  Hash probes are loops of their own and stay one at a
-// time (4,096 queries on 2^22 vertices: 279 ms either way).
+// an SM; with the 105 that the compiler takes unasked 1,020).  Hash probes are
+// loops of their own and stay one at a time (4,096 queries on 2^22 vertices:
+// 276 ms either way).
 template <bool HASH>
 constexpr int PUSH_WIDE = HASH ? 1 : 4;
 

@@ -383,6 +383,10 @@ int build_graph(DevGraph *g, uint32_t n, uint32_t L, uint64_t m, const uint32_t 
     g->label_edges.assign(L, 0);
     for (uint32_t l = 0; l < L; l++) g->label_edges[l] = (uint64_t)ends[2 * l + 1] - ends[2 * l];
   }
+  // the sort's buffers go first, so that the chunk lists do not raise the peak
+  if (ka) cudaFreeAsync(ka, st);
+  if (kb) cudaFreeAsync(kb, st);
+  ka = kb = nullptr;
   RPQ_TRY(build_chunks(g->in_off, n, L, &g->hchunk_in, &g->hchunk_in_off, st));
   RPQ_TRY(build_chunks(g->out_off, n, L, &g->hchunk_out, &g->hchunk_out_off, st));
 done:

@@ -18,14 +18,18 @@
 //   * top-down ("push"): the sparse list of (group, state, vertex) frontier
 //     entries is scanned, the out-edges on the labels of the state's
 //     transitions are spread evenly over the lanes of a warp, and the new
-//     lanes are OR-ed into the next frontier word with atomics; rows longer
-//     than SPILL_EDGES are cut into chunks shared by all warps; or
-//   * bottom-up ("pull"): a warp takes one vertex and all groups at once: for
+//     lanes are OR-ed into the next frontier word with atomics; long rows are
+//     cut into chunks shared by all warps (spill_chunk gives their length);
+//   * bottom-up ("pull"): a warp takes 32 vertices and all groups at once: for
 //     each in-edge on an incoming transition from a state that is present in
 //     the frontier, it gathers the neighbour's G frontier words (one
-//     coalesced 512-byte read) and ORs them into per-lane accumulators; rows
-//     with at least heavy_row in-edges are cut (at graph load) into chunks
-//     shared by all warps,
+//     coalesced 512-byte read) and ORs them into the vertex's; the gathers of
+//     a warp's vertices are listed first and read several at a time
+//     (pull_staged; pull_lanes with an automaton per lane); rows with at least
+//     heavy_row in-edges are cut (at graph load) into chunks shared by all
+//     warps; or
+//   * top-down by block 0 alone when the frontier has few entries and edges
+//     (SOLO_SLOTS, SOLO_EDGES): no grid barrier between such levels,
 // chosen per level from the byte cost of each given the DFA states present
 // in the frontier.  New lanes land in the next frontier word; a commit phase
 // folds them into VIS and clears the old frontier.  The whole search is one

@@ -82,3 +82,32 @@ def test_batch_row_lengths(stars, regex, flags):
     assert rpq.result_stats(r)["product_edges"] == W
     if flags == rpq.RPQ_MATERIALIZE:
         assert np.array_equal(rpq.fetch_pairs(r), np.array(rows, np.uint32).reshape(-1, 2))
+
+
+def test_smallest_budget_that_is_accepted():
+    """At the smallest memory budget a count is accepted with, the emission's
+    scratch is what its longest segments need, and the result is the same."""
+    n = 65536
+    src, dst, lab = synth.random_graph(n, 2 * n, 2, seed=77)
+    sources = np.arange(64, dtype=np.uint32)
+    want = oracle.rpq(oracle.Graph(n, 2, src, dst, lab), "a.b*", sources=sources)
+
+    def count(budget):
+        c = rpq.Context(device=0, mem_budget_bytes=budget)
+        try:
+            r = rpq.run_rpq(c, rpq.load_graph(c, n, 2, src, dst, lab), rpq.compile_rpq(c, "a.b*"), sources,
+                            flags=rpq.RPQ_COUNT_ONLY)
+        except rpq.RPQError:
+            return None
+        return rpq.result_info(r)[0], rpq.result_info(r)[2], rpq.result_info(r)[3]
+
+    refused, accepted = 1 << 16, 1 << 30
+    assert count(refused) is None and count(accepted) == oracle.pair_digest(want.rows)
+    while accepted - refused > 1 << 14:
+        b = (refused + accepted) // 2
+        got = count(b)
+        if got is None:
+            refused = b
+        else:
+            assert got == oracle.pair_digest(want.rows)
+            accepted = b
