@@ -254,7 +254,7 @@ __device__ __forceinline__ void bvisit_wide(const BatchParams &p, const u32 (&i)
 // lies at twice the edges that evict_at vertices of degree 16 have.
 constexpr u64 EVICT_EDGES = 32;
 __device__ __forceinline__ bool outgrown(const BatchParams &p, u64 N, u64 W) {
-  return p.evict_at && (N > p.evict_at || W > p.evict_at * EVICT_EDGES);
+  return p.evict_at && (N > p.evict_at || W / EVICT_EDGES > p.evict_at);
 }
 
 template <bool HASH>

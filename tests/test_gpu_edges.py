@@ -19,8 +19,7 @@ rpq = pytest.importorskip("paper_2602_20748_gb300.rpq")
 DEGREES = (1, 31, 32, 33, 127, 128, 129, 255, 256, 257, 511, 512, 513)
 
 
-@pytest.fixture(scope="module")
-def stars():
+def star_edges():
     """13 vertices with exactly DEGREES[i] out-edges on label a, 13 with as
     many in-edges on it, and two random edges per vertex on labels b and c."""
     n = 2100
@@ -35,7 +34,12 @@ def stars():
     src += rng.integers(0, n, 4 * n).tolist()
     dst += rng.integers(0, n, 4 * n).tolist()
     lab += [1, 2] * (2 * n)
-    g = n, 3, np.array(src, np.uint32), np.array(dst, np.uint32), np.array(lab, np.uint16)
+    return n, 3, np.array(src, np.uint32), np.array(dst, np.uint32), np.array(lab, np.uint16)
+
+
+@pytest.fixture(scope="module")
+def stars():
+    g = star_edges()
     c = rpq.Context(device=0)
     return c, rpq.load_graph(c, *g), oracle.Graph(*g)
 
@@ -111,3 +115,16 @@ def test_smallest_budget_that_is_accepted():
         else:
             assert got == oracle.pair_digest(want.rows)
             accepted = b
+
+
+@pytest.mark.parametrize("evict_at", [2.0**59, 2.0**60, 2.0**62])
+def test_a_bound_no_query_reaches_evicts_none(stars, evict_at):
+    og = stars[2]
+    c = rpq.Context(device=0)
+    rpq.rpq_set_option(c, "batch_evict", evict_at)
+    g = rpq.load_graph(c, *star_edges())
+    sources = np.arange(40, dtype=np.uint32)
+    r = rpq.run_rpq_batch(c, g, [rpq.compile_rpq(c, "(a|b)+.c")] * 40, sources, flags=rpq.RPQ_PER_QUERY)
+    assert rpq.result_stats(r)["evicted"] == 0
+    for i in range(40):
+        assert rpq.result_query_stats(r, i) == oracle.pair_digest(oracle.rpq(og, "(a|b)+.c", sources=[i]).rows)
