@@ -494,7 +494,7 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS, 2) batch_kernel(const __gri
       if (level < (u32)TRACE_LEVELS) {
         c->trace_t[level] = globaltimer_ns();
         c->trace_n[level] = n_cur;
-        c->trace_mode[level] = 1u;
+        c->trace_mode[level] = 1;
       }
       push_levels++;
     }
@@ -705,7 +705,7 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS) serve_kernel(const __grid_c
       if (level < (u32)TRACE_LEVELS) {
         c->trace_t[level] = globaltimer_ns();
         c->trace_n[level] = n_cur;
-        c->trace_mode[level] = 1u;
+        c->trace_mode[level] = 1;
       }
     }
     if (n_cur > 0) {

@@ -29,12 +29,12 @@ __device__ __forceinline__ bool grid_sync(BfsCtl *c, unsigned nblocks, unsigned 
   epoch++;
   __syncthreads();
   if (threadIdx.x == 0) {
-    volatile unsigned *flag = &c->bar_flag[0];
+    volatile unsigned *flag = &c->bar_flag;
     const unsigned want = epoch << 1;  // counter and epoch may wrap: compared for equality only
     unsigned go;
     before();
     __threadfence();
-    if (atomicAdd(&c->bar_count[0], 1u) + 1u == epoch * nblocks) {
+    if (atomicAdd(&c->bar_count, 1u) + 1u == epoch * nblocks) {
       __threadfence();
       go = want | (*(volatile unsigned *)&c->err ? 1u : 0u);
       *flag = go;

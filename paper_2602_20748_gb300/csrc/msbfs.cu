@@ -1937,7 +1937,7 @@ __global__ void __launch_bounds__(BFS_THREADS, AM == AM_LANE ? 3 : 4) msbfs_kern
       if (level < (u32)TRACE_LEVELS) {
         c->trace_t[level] = globaltimer_ns();
         c->trace_n[level] = n_cur;
-        c->trace_mode[level] = push ? 1u : 2u;
+        c->trace_mode[level] = push ? 1 : 2;
         c->trace_mf[level] = mf;
       }
       stat[ST_GROUP_W] += mf;

@@ -115,32 +115,41 @@ constexpr unsigned int APPEND_SEG = 128;             // list slots a warp reserv
 // on R-MAT 2^20: 550 us, 600 with 64).
 inline unsigned int append_seg(int nw) { return nw == 1 ? APPEND_SEG : APPEND_SEG / 2; }
 
+// The words that all blocks poll or add to lie 128 bytes and more apart, with
+// the trace, which one thread writes, between them: a line each, at the size of
+// the words alone.  The size counts: what run_rpq_static takes and the serving
+// slots that fit a budget depend on it.
 struct BfsCtl {
   // grid barrier (grid_barrier.cuh): blocks that have arrived, over all
-  // barriers; the last barrier completed << 1 | error; a line each
-  alignas(128) unsigned int bar_count[32];
-  unsigned int bar_flag[32];
+  // barriers; the last barrier completed << 1 | error
+  unsigned int bar_count;
+  unsigned int pad0[31];
+  unsigned int bar_flag;
   unsigned int err;
   unsigned int err_where;
-  alignas(128) unsigned long long n_list[3];
-  alignas(128) unsigned long long cursor[3];
-  alignas(128) unsigned long long mf[3];  // frontier out-edges
-  alignas(128) unsigned long long n_true[3];  // frontier entries without the lists' unused slots
+  unsigned int pad1;
+  // per-level trace (first TRACE_LEVELS levels): start time (ns), frontier
+  // entries and out-edges, start time (ns) of the commit phase, direction (1
+  // top-down, 2 bottom-up)
+  unsigned long long trace_c[TRACE_LEVELS];
+  unsigned long long n_list[3];
+  unsigned long long trace_n[TRACE_LEVELS];
+  unsigned long long cursor[3];
+  unsigned long long trace_mf[TRACE_LEVELS];
+  unsigned long long mf[3];  // frontier out-edges
+  unsigned long long trace_t[TRACE_LEVELS + 1];
+  unsigned long long n_true[3];        // frontier entries without the lists' unused slots
   unsigned long long spill_count[3];   // top-down row chunks queued this level
   unsigned long long spill_cursor[3];
   unsigned long long heavy_cursor[3];  // bottom-up row chunks taken
-  alignas(128) unsigned int smask[3];  // DFA states present in each frontier
-  unsigned int next_level;             // first level after a run of one-block levels
+  unsigned char trace_mode[TRACE_LEVELS];
   unsigned long long levels;
   unsigned long long stats[ST_COUNT];
-  // per-level trace (first TRACE_LEVELS levels): start time (ns), frontier
-  // entries, direction (1 top-down, 2 bottom-up)
-  unsigned long long trace_t[TRACE_LEVELS + 1];
-  unsigned long long trace_n[TRACE_LEVELS];
-  unsigned int trace_mode[TRACE_LEVELS];
-  unsigned long long trace_mf[TRACE_LEVELS];  // frontier out-edges (top-down cost)
-  unsigned long long trace_c[TRACE_LEVELS];   // start time (ns) of each level's commit phase
+  unsigned int smask[3];    // DFA states present in each frontier
+  unsigned int next_level;  // first level after a run of one-block levels
+  unsigned int pad2[10];
 };
+static_assert(sizeof(BfsCtl) == 2592, "see above");
 
 // A top-down row longer than the level's chunk length (at most SPILL_EDGES
 // edges, see spill_chunk) is cut into chunks that all warps share in a
