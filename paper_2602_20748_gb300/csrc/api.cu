@@ -303,10 +303,11 @@ void free_chunk(rpq_ctx *ctx, Chunk &c) {
 // Picks the lanes of a chunk whose rows become bitsets (bits_req): reads the
 // lanes' row counts from the scanned offsets, keeps the rows of at least
 // min_len destinations, longest first, while the bitsets take at most half of
-// the budget left, and allocates them into c.  Returns the lanes' slots on
-// the host (NO_SOURCE: listed only).
+// the budget left (`spare` bytes of what is taken can be given back), and
+// allocates them into c.  Returns the lanes' slots on the host (NO_SOURCE:
+// listed only).
 int pick_bit_lanes(rpq_ctx *ctx, const RowBitsReq &req, const u64 *off, uint32_t segs, uint32_t live, uint32_t n,
-                   Chunk &c) {
+                   uint64_t spare, Chunk &c) {
   std::vector<u64> lane_off(c.n_lanes + 1);
   u64 *d_lane_off = nullptr;
   int rc;
@@ -326,7 +327,7 @@ int pick_bit_lanes(rpq_ctx *ctx, const RowBitsReq &req, const u64 *off, uint32_t
     return lane_off[a + 1] - lane_off[a] > lane_off[b + 1] - lane_off[b];
   });
   const uint64_t bwords = ((uint64_t)n + 255) / 256 * 4;
-  const uint64_t left = ctx->used < ctx->budget ? ctx->budget - ctx->used : 0;
+  const uint64_t left = ctx->used < ctx->budget + spare ? ctx->budget + spare - ctx->used : 0;
   const uint64_t cap = left / 2 / (bwords * 8);
   if (sel.size() > cap) sel.resize(cap);
   if (sel.empty()) return RPQ_OK;
@@ -567,25 +568,18 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
       continue;
     }
 
-    // emission pass 1: counts and digest
-    // one allocation: the offsets, the scan's scratch, the counts; where the
-    // budget has no room for short segments, longer ones (down to what the
-    // longest need)
+    // emission pass 1: counts and digest, in one allocation: the offsets, the
+    // scan's scratch, the counts.  Where the budget has no room for short
+    // segments, longer ones (down to what the longest need)
     uint64_t ncnt, tmpw, nscratch;
-    u64 *off = nullptr;
-    int rc;
-    for (;;) {
-      ncnt = (uint64_t)n_lanes * segs;
+    u64 *off = nullptr, *tmp = nullptr;
+    u32 *cnt = nullptr;
+    auto scratch_words = [&](uint32_t sg) {
+      ncnt = (uint64_t)n_lanes * sg;
       tmpw = scan_tmp_words(ncnt);
-      nscratch = ncnt + tmpw + (ncnt + 1) / 2;
-      if ((rc = dalloc(ctx, &off, nscratch)) == RPQ_OK) break;
-      if (tiles >= (uint32_t)EMIT_TILES) return rc;
-      tiles <<= 1;
-      segs = emit_segs(tiles, n);
-    }
-    const uint64_t nscan = (uint64_t)live * segs;
-    u64 *const tmp = off + ncnt;
-    u32 *const cnt = reinterpret_cast<u32 *>(tmp + tmpw);
+      return ncnt + tmpw + (ncnt + 1) / 2;
+    };
+    const uint64_t min_scratch = scratch_words(emit_segs(EMIT_TILES, n));
     EmitParams ep{};
     ep.vis = w.vis;
     ep.n = n;
@@ -593,16 +587,31 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
     ep.Q = Q;
     ep.final_mask = qd.final_mask;
     ep.lanesrc = w.lanesrc;
-    ep.tiles = tiles;
-    ep.segs = segs;
-    ep.cnt = cnt;
-    ep.off = off;
     ep.dst = nullptr;
     ep.digest = ctx->small;
+    auto count_rows = [&]() -> int {
+      for (;;) {
+        nscratch = scratch_words(segs);
+        const int r = dalloc(ctx, &off, nscratch);
+        if (r == RPQ_OK) break;
+        if (tiles >= (uint32_t)EMIT_TILES) return r;
+        tiles <<= 1;
+        segs = emit_segs(tiles, n);
+      }
+      tmp = off + ncnt;
+      cnt = reinterpret_cast<u32 *>(tmp + tmpw);
+      ep.tiles = tiles;
+      ep.segs = segs;
+      ep.cnt = cnt;
+      ep.off = off;
+      CK(launch_emit(nw, false, !materialize, ep, ctx->stream));
+      CK(exclusive_scan_u32_to_u64(cnt, off, (uint64_t)live * segs, ctx->small + 2, tmp, ctx->stream));
+      res->stats.launches += 2;
+      return RPQ_OK;
+    };
     CK(cudaEventRecord(ctx->ev[2], ctx->stream));
-    CK(launch_emit(nw, false, !materialize, ep, ctx->stream));
-    CK(exclusive_scan_u32_to_u64(cnt, off, nscan, ctx->small + 2, tmp, ctx->stream));
-    res->stats.launches += 2;
+    int rc = count_rows();
+    if (rc) return rc;
     BfsCtl hctl;
     u64 hsmall[3];
     CK(rb_queue(ctx, 0, ctx->ctl, sizeof(BfsCtl), RB_SMALL, ctx->small, 3 * 8));
@@ -650,31 +659,42 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
 
     if (materialize) {
       Chunk c;
-      c.n_lanes = n_lanes;
-      c.rows = total;
-      if (bits_req) {
-        if ((rc = pick_bit_lanes(ctx, *bits_req, off, segs, live, n, c))) {
-          free_chunk(ctx, c);
-          dfree(ctx, off, nscratch);
-          return rc;
+      // the rows' buffers; the scratch of short segments gives way to them
+      auto room_for_rows = [&]() -> int {
+        c = Chunk();
+        c.n_lanes = n_lanes;
+        c.rows = total;
+        int r;
+        if (bits_req) {
+          if ((r = pick_bit_lanes(ctx, *bits_req, off, segs, live, n, (nscratch - min_scratch) * 8, c))) return r;
+          ep.lane_slot = c.lane_slot;
+          ep.bits = c.bits;
+          ep.bwords = c.bwords;
+          ep.keep_lists = c.lists_kept ? 1u : 0u;
+          if (c.bits && !c.lists_kept) {
+            // bitset rows are not listed: offsets of the listed rows only
+            u64 listed = 0;
+            CK(launch_zero_lane_counts(cnt, segs, n_lanes, c.lane_slot, ctx->stream));
+            CK(exclusive_scan_u32_to_u64(cnt, off, (uint64_t)live * segs, ctx->small + 2, tmp, ctx->stream));
+            CK(cudaMemcpyAsync(&listed, ctx->small + 2, 8, cudaMemcpyDeviceToHost, ctx->stream));
+            CK(cudaStreamSynchronize(ctx->stream));
+            c.rows = listed;
+            res->stats.launches += 2;
+          }
         }
-        ep.lane_slot = c.lane_slot;
-        ep.bits = c.bits;
-        ep.bwords = c.bwords;
-        ep.keep_lists = c.lists_kept ? 1u : 0u;
-        if (c.bits && !c.lists_kept) {
-          // bitset rows are not listed: offsets of the listed rows only
-          u64 listed = 0;
-          CK(launch_zero_lane_counts(cnt, segs, n_lanes, c.lane_slot, ctx->stream));
-          CK(exclusive_scan_u32_to_u64(cnt, off, nscan, ctx->small + 2, tmp, ctx->stream));
-          CK(cudaMemcpyAsync(&listed, ctx->small + 2, 8, cudaMemcpyDeviceToHost, ctx->stream));
-          CK(cudaStreamSynchronize(ctx->stream));
-          c.rows = listed;
-          res->stats.launches += 2;
-        }
+        if ((r = dalloc(ctx, &c.lanesrc, n_lanes)) || (r = dalloc(ctx, &c.lane_off, (uint64_t)n_lanes + 1))) return r;
+        return dalloc(ctx, &c.dst, c.rows);
+      };
+      rc = room_for_rows();
+      if (rc == RPQ_ERR_OUT_OF_BUDGET && nscratch > min_scratch) {
+        free_chunk(ctx, c);
+        dfree(ctx, off, nscratch);
+        tiles = EMIT_TILES;
+        segs = emit_segs(tiles, n);
+        if ((rc = count_rows())) return rc;
+        rc = room_for_rows();
       }
-      if ((rc = dalloc(ctx, &c.lanesrc, n_lanes)) || (rc = dalloc(ctx, &c.lane_off, (uint64_t)n_lanes + 1)) ||
-          (rc = dalloc(ctx, &c.dst, c.rows))) {
+      if (rc) {
         free_chunk(ctx, c);
         dfree(ctx, off, nscratch);
         return rc;
