@@ -3,9 +3,11 @@
 // traversal and emission kernels, results and fetch.
 #include <algorithm>
 #include <atomic>
+#include <condition_variable>
 #include <cstdio>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -47,6 +49,10 @@ struct rpq_ctx {
   cudaMemPool_t pool = nullptr;  // the context's own pool: freed blocks stay reserved for reuse
   uint64_t budget = 0;
   uint64_t used = 0;
+  // chunk lists of shorter rows of this context's graphs: held while the budget
+  // has room beside everything else, so that what fits it does not depend on them
+  uint64_t shorter_bytes = 0;
+  std::vector<rpq_graph *> graphs;  // whose lists these are
   std::string err;
   Workspace ws;
   BfsCtl *ctl = nullptr;
@@ -84,6 +90,12 @@ struct rpq_graph {
   rpq_ctx *ctx = nullptr;
   DevGraph g;
   uint64_t bytes = 0;
+  uint64_t shorter_bytes = 0;
+  // evaluations on other contexts that read the lists of shorter rows
+  mutable std::mutex mu;
+  mutable std::condition_variable cv;
+  mutable int users = 0;
+  bool giving_back = false;
 };
 
 struct rpq_query {
@@ -139,8 +151,34 @@ int cuda_err(rpq_ctx *c, cudaError_t e, const char *what) {
     if (_e != cudaSuccess) return cuda_err(ctx, _e, #expr); \
   } while (0)
 
+// Frees the lists of shorter rows of one of ctx's graphs (see ShorterChunks):
+// waits for the other contexts' evaluations that read them; new ones go without.
+void give_back_shorter(rpq_graph *g) {
+  rpq_ctx *ctx = g->ctx;
+  {
+    std::unique_lock<std::mutex> lk(g->mu);
+    g->giving_back = true;
+    g->cv.wait(lk, [&] { return g->users == 0; });
+    for (ChunkLists *c : {&g->g.chunks_in, &g->g.chunks_out}) {
+      if (c->shorter.rec) cudaFreeAsync(c->shorter.rec, ctx->stream);
+      c->shorter.rec = nullptr;
+    }
+  }
+  ctx->shorter_bytes -= g->shorter_bytes;
+  g->shorter_bytes = 0;
+  ctx->graphs.erase(std::find(ctx->graphs.begin(), ctx->graphs.end(), g));
+}
+
+// Makes `bytes` more fit the budget beside the lists of shorter rows, or gives
+// these back.
+void room_for(rpq_ctx *ctx, uint64_t bytes) {
+  if (ctx->used + ctx->shorter_bytes + bytes <= ctx->budget) return;
+  while (!ctx->graphs.empty()) give_back_shorter(ctx->graphs.back());
+}
+
 int dev_alloc(rpq_ctx *ctx, void **p, uint64_t bytes) {
   if (bytes == 0) bytes = 16;
+  room_for(ctx, bytes);
   if (ctx->used + bytes > ctx->budget)
     return set_err(ctx, RPQ_ERR_OUT_OF_BUDGET,
                    "device memory budget exceeded (" + std::to_string(ctx->used + bytes) + " > " +
@@ -419,6 +457,7 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
     if (q0_final) res->count += skipped;
   }
   const std::vector<uint32_t> &srcs = filter ? kept : srcs_in;
+  const ShorterChunks shorter(ctx, gr);
   res->stats.lane_words = srcs.size() <= 64 ? 1 : 4;
   if (srcs.empty()) return RPQ_OK;
   const int nw = srcs.size() <= 64 ? 1 : 4;
@@ -470,7 +509,7 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
     p.in_off = reverse ? g.out_off : g.in_off;
     p.in_col = reverse ? g.out_col : g.in_col;
     // bottom-up levels read the in-direction of the traversal
-    set_chunks(p, reverse ? g.hchunk_out : g.hchunk_in, reverse ? g.hchunk_out_off : g.hchunk_in_off, g.L, live);
+    set_chunks(p, reverse ? g.chunks_out : g.chunks_in, g.L, live, shorter.there());
     for (uint32_t l = 0; l < g.L; l++) p.label_edges[l] = g.label_edges[l];
     p.n = n;
     p.L = g.L;
@@ -980,6 +1019,7 @@ int load_graph(rpq_ctx *ctx, uint32_t n_vertices, uint32_t n_labels, uint64_t n_
   const uint64_t gbytes = rows * 8 + m * 8 + (vertex_label ? n_vertices : 0);
   // sort scratch (keys x3, flags, histograms) comes from the same budget
   const uint64_t scratch = m * 30 + (64ull << 20);
+  room_for(ctx, gbytes + scratch + m * 10);
   if (ctx->used + gbytes + scratch + m * 10 > ctx->budget) {
     delete gr;
     release_handle(ctx);
@@ -1015,14 +1055,19 @@ int load_graph(rpq_ctx *ctx, uint32_t n_vertices, uint32_t n_labels, uint64_t n_
   {
     // the graph arrays were allocated inside build_graph outside the budget
     // accounting; account for them now
-    uint64_t b = rows * 8 + gr->g.m * 8 +
-                 12ull * ((uint64_t)gr->g.hchunk_in_off.back() + gr->g.hchunk_out_off.back());
+    const DevGraph &dg = gr->g;
+    uint64_t b = rows * 8 + dg.m * 8 +
+                 12ull * ((uint64_t)dg.chunks_in.longer.off.back() + dg.chunks_out.longer.off.back());
     ctx->used += b;
     gr->bytes = b;
+    gr->shorter_bytes = 12ull * ((uint64_t)dg.chunks_in.shorter.off.back() + dg.chunks_out.shorter.off.back());
+    ctx->shorter_bytes += gr->shorter_bytes;
+    ctx->graphs.push_back(gr);
   }
   dfree(ctx, d_src, m);
   dfree(ctx, d_dst, m);
   dfree(ctx, d_lab, m);
+  room_for(ctx, 0);
   {
     cudaError_t e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) {
@@ -1037,12 +1082,7 @@ fail:
   dfree(ctx, d_src, m);
   dfree(ctx, d_dst, m);
   dfree(ctx, d_lab, m);
-  if (gr->g.out_off) cudaFreeAsync(gr->g.out_off, st);
-  if (gr->g.in_off) cudaFreeAsync(gr->g.in_off, st);
-  if (gr->g.out_col) cudaFreeAsync(gr->g.out_col, st);
-  if (gr->g.in_col) cudaFreeAsync(gr->g.in_col, st);
-  if (gr->g.hchunk_in) cudaFreeAsync(gr->g.hchunk_in, st);
-  if (gr->g.hchunk_out) cudaFreeAsync(gr->g.hchunk_out, st);
+  free_graph_arrays(&gr->g, st);
   if (gr->g.vlabel) dfree(ctx, gr->g.vlabel, n_vertices);
   delete gr;
   release_handle(ctx);
@@ -1062,12 +1102,8 @@ void free_graph(rpq_graph *g) {
   rpq_ctx *ctx = g->ctx;
   cudaSetDevice(ctx->device);
   cudaStream_t st = ctx->stream;
-  cudaFreeAsync(g->g.out_off, st);
-  cudaFreeAsync(g->g.in_off, st);
-  cudaFreeAsync(g->g.out_col, st);
-  cudaFreeAsync(g->g.in_col, st);
-  cudaFreeAsync(g->g.hchunk_in, st);
-  cudaFreeAsync(g->g.hchunk_out, st);
+  if (std::find(ctx->graphs.begin(), ctx->graphs.end(), g) != ctx->graphs.end()) give_back_shorter(g);
+  free_graph_arrays(&g->g, st);
   ctx->used -= std::min(ctx->used, g->bytes);
   if (g->g.vlabel) dfree(ctx, g->g.vlabel, g->g.n);
   delete g;
@@ -1262,12 +1298,7 @@ int run_rpq_middle(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *alpha, co
   dfree(ctx, d_lab, m2);
   // 4. alpha . X over the temporary graph, from the requested start vertices
   if (rc == RPQ_OK) rc = eval_rpq(ctx, &g2, &qx, srcs, flags, res);
-  if (g2.g.out_off) cudaFreeAsync(g2.g.out_off, st);
-  if (g2.g.in_off) cudaFreeAsync(g2.g.in_off, st);
-  if (g2.g.out_col) cudaFreeAsync(g2.g.out_col, st);
-  if (g2.g.in_col) cudaFreeAsync(g2.g.in_col, st);
-  if (g2.g.hchunk_in) cudaFreeAsync(g2.g.hchunk_in, st);
-  if (g2.g.hchunk_out) cudaFreeAsync(g2.g.hchunk_out, st);
+  free_graph_arrays(&g2.g, st);
   if (rc) {
     free_result(res);
     return rc;
@@ -1566,6 +1597,21 @@ void ctx_release_workspace(rpq_ctx *ctx) {
   if (ctx->pool) cudaMemPoolTrimTo(ctx->pool, 0);
 }
 const DevGraph &graph_dev(const rpq_graph *g) { return g->g; }
+
+ShorterChunks::ShorterChunks(rpq_ctx *ctx, const rpq_graph *g) : ctx_(ctx), g_(g) {
+  if (ctx == g->ctx) return;  // one call at a time: only its own allocations free them
+  std::lock_guard<std::mutex> lk(g->mu);
+  held_ = !g->giving_back && g->g.chunks_in.shorter.rec;
+  if (held_) g->users++;
+}
+ShorterChunks::~ShorterChunks() {
+  if (!held_) return;
+  cudaStreamSynchronize(ctx_->stream);  // an evaluation that failed may have left a launch running
+  std::lock_guard<std::mutex> lk(g_->mu);
+  if (--g_->users == 0) g_->cv.notify_all();
+}
+bool ShorterChunks::there() const { return ctx_ == g_->ctx ? g_->g.chunks_in.shorter.rec != nullptr : held_; }
+
 const HostQuery &query_host(const rpq_query *q) { return q->hq; }
 
 // Runs an RPQ from the given sorted distinct sources, materialized, and hands
@@ -1780,7 +1826,8 @@ int rpq_lane_stats_multi(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Mu
   p.out_col = g.out_col;
   p.in_off = g.in_off;
   p.in_col = g.in_col;
-  set_chunks(p, g.hchunk_in, g.hchunk_in_off, g.L, total_lanes);
+  const ShorterChunks shorter(ctx, gr);
+  set_chunks(p, g.chunks_in, g.L, total_lanes, shorter.there());
   for (uint32_t l = 0; l < g.L; l++) p.label_edges[l] = g.label_edges[l];
   p.n = n;
   p.L = L;
@@ -2046,7 +2093,8 @@ static int lane_launch(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Lane
   p.out_col = g.out_col;
   p.in_off = g.in_off;
   p.in_col = g.in_col;
-  set_chunks(p, g.hchunk_in, g.hchunk_in_off, g.L, k);
+  const ShorterChunks shorter(ctx, gr);
+  set_chunks(p, g.chunks_in, g.L, k, shorter.there());
   for (uint32_t l = 0; l < g.L; l++) p.label_edges[l] = g.label_edges[l];
   p.n = n;
   p.L = L;

@@ -68,6 +68,24 @@ void *ctx_static_scratch(rpq_ctx *ctx);
 void ctx_release_workspace(rpq_ctx *ctx);
 int static_scratch_prepare(void **addr, std::string *msg);
 const DevGraph &graph_dev(const rpq_graph *g);
+// The use of a graph's chunk lists of shorter rows by an evaluation on ctx: the
+// graph's own context gives them back when its budget needs the room, in its
+// stream's order; evaluations on other contexts keep them until they are done.
+class ShorterChunks {
+ public:
+  ShorterChunks(rpq_ctx *ctx, const rpq_graph *g);
+  ~ShorterChunks();
+  ShorterChunks(const ShorterChunks &) = delete;
+  ShorterChunks &operator=(const ShorterChunks &) = delete;
+  // Whether a launch that is issued next may read them (asked when no more
+  // memory is allocated before it).
+  bool there() const;
+
+ private:
+  rpq_ctx *ctx_;
+  const rpq_graph *g_;
+  bool held_ = false;  // counted in the graph's users
+};
 const HostQuery &query_host(const rpq_query *q);
 int rpq_rows_for_sources(rpq_ctx *ctx, const rpq_graph *g, const rpq_query *q, std::vector<uint32_t> &srcs,
                          bool reverse, std::vector<RowChunk> *chunks, rpq_stats *stats, uint64_t *dsum = nullptr,

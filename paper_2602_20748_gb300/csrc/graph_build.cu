@@ -131,11 +131,11 @@ __global__ void label_bounds(const uint32_t *__restrict__ off, uint32_t n, uint3
 
 // Chunk lists of long rows, all labels at once (blockIdx.y = label): a list per
 // label and class, rows of at least LONG_ROW edges (class 0) and rows of
-// HEAVY_ROW .. LONG_ROW - 1 (class 1).  Without out, next[2 * label + class]
-// counts the chunks; with out, it is the place of the list's next record
-// (vertex, first edge, end edge), taken a warp at a time.
+// HEAVY_ROW .. LONG_ROW - 1 (class 1).  Without out0 and out1,
+// next[2 * label + class] counts the chunks; with them, it is the place of the
+// list's next record (vertex, first edge, end edge), taken a warp at a time.
 __global__ void row_chunks(const uint32_t *__restrict__ off, uint32_t n, u32 *__restrict__ next,
-                           uint32_t *__restrict__ out) {
+                           uint32_t *__restrict__ out0, uint32_t *__restrict__ out1) {
   const uint32_t *row = off + (u64)blockIdx.y * (n + 1);
   next += 2 * blockIdx.y;
   const u64 step = (u64)gridDim.x * blockDim.x;
@@ -155,6 +155,7 @@ __global__ void row_chunks(const uint32_t *__restrict__ off, uint32_t n, u32 *__
       u32 base = 0;
       if (lane_id() == 31) base = atomicAdd(&next[cls], at);
       base = __shfl_sync(FULL_MASK, base, 31) + at - k;
+      uint32_t *out = cls == 0 ? out0 : out1;
       if (out)
         for (u32 c = 0; c < k; c++) {
           const u64 r = 3ull * (base + c);
@@ -264,33 +265,43 @@ static int bits_for(uint64_t n) {
   return b;
 }
 
-// Chunk records of the long rows of every label of the CSR `off`: offs[2 * l +
-// c] is the first of label l's class c, offs[2 * L] their number.
-static cudaError_t build_chunks(const uint32_t *off, uint32_t n, uint32_t L, uint32_t **chunks,
-                                std::vector<uint32_t> *offs, cudaStream_t st) {
+// Chunk records of the long rows of every label of the CSR `off`.
+static cudaError_t build_chunks(const uint32_t *off, uint32_t n, uint32_t L, ChunkLists *lists, cudaStream_t st) {
   u32 *next = nullptr;
-  offs->assign(2 * L + 1, 0);
+  ChunkList *cls[2] = {&lists->longer, &lists->shorter};
+  for (ChunkList *c : cls) c->off.assign(L + 1, 0);
   std::vector<u32> cnt(2 * L, 0);
   const dim3 grid((unsigned)std::min<u64>(grid_for(n, 256), 608), L);
   cudaError_t e = cudaMallocAsync(&next, 8ull * L, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(next, 0, 8ull * L, st);
   if (e == cudaSuccess) {
-    row_chunks<<<grid, 256, 0, st>>>(off, n, next, nullptr);
+    row_chunks<<<grid, 256, 0, st>>>(off, n, next, nullptr, nullptr);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(cnt.data(), next, 8ull * L, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e == cudaSuccess) {
-    for (uint32_t i = 0; i < 2 * L; i++) (*offs)[i + 1] = (*offs)[i] + cnt[i];
-    e = cudaMallocAsync(chunks, 3 * (u64)std::max(1u, (*offs)[2 * L]) * 4, st);
+  for (int c = 0; c < 2 && e == cudaSuccess; c++) {
+    for (uint32_t l = 0; l < L; l++) {
+      cls[c]->off[l + 1] = cls[c]->off[l] + cnt[2 * l + c];
+      cnt[2 * l + c] = cls[c]->off[l];
+    }
+    e = cudaMallocAsync(&cls[c]->rec, 3 * (u64)std::max(1u, cls[c]->off[L]) * 4, st);
   }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(next, offs->data(), 8ull * L, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(next, cnt.data(), 8ull * L, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) {
-    row_chunks<<<grid, 256, 0, st>>>(off, n, next, *chunks);
+    row_chunks<<<grid, 256, 0, st>>>(off, n, next, cls[0]->rec, cls[1]->rec);
     e = cudaGetLastError();
   }
   if (next) cudaFreeAsync(next, st);
   return e;
+}
+
+void free_graph_arrays(DevGraph *g, cudaStream_t st) {
+  for (uint32_t **p : {&g->out_off, &g->in_off, &g->out_col, &g->in_col, &g->chunks_in.longer.rec,
+                       &g->chunks_in.shorter.rec, &g->chunks_out.longer.rec, &g->chunks_out.shorter.rec}) {
+    if (*p) cudaFreeAsync(*p, st);
+    *p = nullptr;
+  }
 }
 
 int graph_key_bits(uint32_t n, uint32_t L) { return ((L > 1) ? bits_for(L) : 0) + 2 * bits_for(n); }
@@ -387,8 +398,8 @@ int build_graph(DevGraph *g, uint32_t n, uint32_t L, uint64_t m, const uint32_t 
   if (ka) cudaFreeAsync(ka, st);
   if (kb) cudaFreeAsync(kb, st);
   ka = kb = nullptr;
-  RPQ_TRY(build_chunks(g->in_off, n, L, &g->hchunk_in, &g->hchunk_in_off, st));
-  RPQ_TRY(build_chunks(g->out_off, n, L, &g->hchunk_out, &g->hchunk_out_off, st));
+  RPQ_TRY(build_chunks(g->in_off, n, L, &g->chunks_in, st));
+  RPQ_TRY(build_chunks(g->out_off, n, L, &g->chunks_out, st));
 done:
   if (ka) cudaFreeAsync(ka, st);
   if (kb) cudaFreeAsync(kb, st);

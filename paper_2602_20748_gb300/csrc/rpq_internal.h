@@ -68,6 +68,17 @@ constexpr uint32_t LONG_ROW = 128;
 constexpr uint32_t FEW_STARTS = 32;  // fewer start vertices than this chunk LONG_ROW rows only
 constexpr uint32_t HCHUNK = 256;
 
+// The chunks of one class of rows, grouped by label: label l's are [off[l],
+// off[l + 1]) (host copy of the L + 1 offsets).
+struct ChunkList {
+  uint32_t *rec = nullptr;
+  std::vector<uint32_t> off;
+};
+struct ChunkLists {
+  ChunkList longer;   // rows of LONG_ROW edges and more
+  ChunkList shorter;  // HEAVY_ROW .. LONG_ROW - 1 edges; given back when the budget needs the room
+};
+
 struct DevGraph {
   uint32_t n = 0;
   uint32_t L = 0;
@@ -78,11 +89,9 @@ struct DevGraph {
   uint32_t *in_col = nullptr;
   uint8_t *vlabel = nullptr;
   // Chunks (vertex, first edge, end edge) of the rows with >= HEAVY_ROW
-  // edges, per direction, grouped by label and class: label l's chunks of rows
-  // of LONG_ROW edges and more are [off[2 l], off[2 l + 1]), those of shorter
-  // rows follow up to off[2 l + 2] (host copy of the 2 L + 1 offsets).
-  uint32_t *hchunk_in = nullptr, *hchunk_out = nullptr;
-  std::vector<uint32_t> hchunk_in_off, hchunk_out_off;
+  // edges, per direction: of the rows of LONG_ROW edges and more, and of the
+  // shorter ones.
+  ChunkLists chunks_in, chunks_out;
   std::vector<uint8_t> vlabel_host;   // vertex labels (host copy), empty if none
   std::vector<uint64_t> label_edges;  // edges per label (host copy)
 };
@@ -164,9 +173,11 @@ struct BfsParams {
   const uint32_t *out_col;
   const uint32_t *in_off;
   const uint32_t *in_col;
-  const uint32_t *hchunk;       // chunks of long in_off rows (nullptr: none)
-  uint32_t hchunk_beg[RPQ_MAX_LABELS];  // per label, the chunks of rows of
-  uint32_t hchunk_end[RPQ_MAX_LABELS];  // at least heavy_row edges
+  // chunks of the in_off rows of at least heavy_row edges: per label and
+  // class (longer rows, shorter rows) their records and number
+  const uint32_t *chunk_rec[2];
+  uint32_t chunk_beg[2][RPQ_MAX_LABELS];
+  uint32_t chunk_n[2][RPQ_MAX_LABELS];
   uint32_t heavy_row;
   unsigned long long label_edges[RPQ_MAX_LABELS];
   uint32_t n;
@@ -237,14 +248,18 @@ struct BfsParams {
   QueryDesc q;
 };
 
-// The chunk lists of a launch of `starts` start vertices.
-inline void set_chunks(BfsParams &p, const uint32_t *chunks, const std::vector<uint32_t> &offs, uint32_t L,
-                       uint64_t starts) {
-  p.hchunk = chunks;
-  p.heavy_row = starts < FEW_STARTS ? LONG_ROW : HEAVY_ROW;
+// The chunk lists of a launch of `starts` start vertices (shorter: the graph
+// still has its lists of shorter rows).
+inline void set_chunks(BfsParams &p, const ChunkLists &c, uint32_t L, uint64_t starts, bool shorter) {
+  shorter = shorter && starts >= FEW_STARTS;
+  p.heavy_row = shorter ? HEAVY_ROW : LONG_ROW;
+  p.chunk_rec[0] = c.longer.rec;
+  p.chunk_rec[1] = shorter ? c.shorter.rec : nullptr;
   for (uint32_t l = 0; l < L; l++) {
-    p.hchunk_beg[l] = offs[2 * l];
-    p.hchunk_end[l] = offs[2 * l + (starts < FEW_STARTS ? 1 : 2)];
+    p.chunk_beg[0][l] = c.longer.off[l];
+    p.chunk_n[0][l] = c.longer.off[l + 1] - c.longer.off[l];
+    p.chunk_beg[1][l] = shorter ? c.shorter.off[l] : 0;
+    p.chunk_n[1][l] = shorter ? c.shorter.off[l + 1] - c.shorter.off[l] : 0;
   }
 }
 
@@ -379,6 +394,7 @@ cudaError_t launch_chunk_triples(const uint32_t *lanesrc, const unsigned long lo
 // Graph construction.  Returns RPQ_OK or an error code with *msg set.
 int build_graph(DevGraph *g, uint32_t n, uint32_t L, uint64_t m, const uint32_t *d_src, const uint32_t *d_dst,
                 const uint16_t *d_lab, cudaStream_t st, std::string *msg);
+void free_graph_arrays(DevGraph *g, cudaStream_t st);  // all but vlabel
 int graph_key_bits(uint32_t n, uint32_t L);
 
 // Stable LSD radix sort of 64-bit keys over bits [lo_bit, hi_bit); the result

@@ -194,7 +194,8 @@ extern "C" int run_rpq_static(rpq_ctx *ctx, const rpq_graph *g, const rpq_query 
   // chunks of long in-rows belong to the graph: scanned in place, one lane
   // walked a row of up to 10^4 edges alone (64 start vertices on R-MAT 2^18:
   // 3.2 ms a call)
-  set_chunks(p, dg.hchunk_in, dg.hchunk_in_off, dg.L, ns);
+  const ShorterChunks shorter(ctx, g);
+  set_chunks(p, dg.chunks_in, dg.L, ns, shorter.there());
   for (uint32_t l = 0; l < dg.L; l++) p.label_edges[l] = dg.label_edges[l];
   p.time_limit_ns = ctx_time_limit_ns(ctx);
   p.q = qd;

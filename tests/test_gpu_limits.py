@@ -84,3 +84,60 @@ def test_rows_need_no_more_than_the_counts_and_themselves(reach):
     for more in (0, 1, 1 << 19, 1 << 20, (1 << 21) + rows // 2, 1 << 22):
         assert run_with(low + rows + more, graph, "a.b", sources, rpq.RPQ_MATERIALIZE) == want
     assert run_with(low + rows - 1, graph, "a.b", sources, rpq.RPQ_MATERIALIZE) is None
+
+
+def test_lists_of_shorter_rows_take_nothing_from_the_budget():
+    """As many edges in rows of 16 and in rows of 64: what a budget accepts is
+    the same, and so are the rows of 64 at its limit, by bottom-up levels."""
+    n, m = 1 << 20, 1 << 18
+    sources = np.arange(100, dtype=np.uint32)
+    lows = []
+    for row in (16, 64):
+        src = np.repeat(np.arange(m // row, dtype=np.uint32), row)
+        dst = (np.arange(m, dtype=np.uint64) * 2654435761 % n).astype(np.uint32)
+        for graph in ((n, 1, src, dst, np.zeros(m, np.uint16)), (n, 1, dst, src, np.zeros(m, np.uint16))):
+            flags = rpq.RPQ_COUNT_ONLY | rpq.RPQ_FORCE_PULL
+            want = run_with(1 << 33, graph, "a.a", sources, rpq.RPQ_COUNT_ONLY)
+            lows.append(smallest(lambda b: run_with(b, graph, "a.a", sources, flags) == want, 1 << 28, 1 << 30))
+    assert len(set(lows)) == 1
+
+
+def test_lists_given_back_while_other_contexts_read_them():
+    """A call that the budget refuses gives the lists of shorter rows back, in
+    the middle of a server's requests on the same graph; replies and later calls
+    are what they were."""
+    n = 12000
+    rng = np.random.default_rng(7)
+    graph = (n, 3, *(rng.integers(0, k, 120 * n).astype(t) for k, t in ((n, np.uint32), (n, np.uint32), (3, np.uint16))))
+    c = rpq.Context(device=0, mem_budget_bytes=500 << 20)
+    g = rpq.load_graph(c, *graph)
+    queries = [rpq.compile_rpq(c, x) for x in ("a.b*", "(a|b)+.c", "c.a?.b")]
+
+    def summary(q, sources, flags=rpq.RPQ_COUNT_ONLY):
+        return [rpq.result_info(rpq.run_rpq(c, g, q, sources, flags=flags))[k] for k in (0, 2, 3)]
+
+    def batch():
+        r = rpq.run_rpq_batch(c, g, queries * 40, rng2, flags=rpq.RPQ_PER_QUERY)
+        return [rpq.result_query_stats(r, i) for i in range(120)]
+
+    rng2 = np.arange(120, dtype=np.uint32) * 97
+    rpq.rpq_set_option(c, "batch_direct", 1)
+    modes = (0, rpq.RPQ_REVERSE, rpq.RPQ_FORCE_PULL, rpq.RPQ_FORCE_PUSH)
+    lists = (np.arange(40, dtype=np.uint32), np.arange(600, dtype=np.uint32))
+    before = [summary(q, s, rpq.RPQ_COUNT_ONLY | f) for q in queries for s in lists for f in modes] + batch()
+    singles = [(q, int(s), summary(q, [int(s)])) for q in queries for s in rng.integers(0, n, 60)]
+    everything = [summary(q, None) for q in queries]
+    server = rpq.Server(c, g, mem_budget_bytes=8 << 30)
+    try:
+        tickets = [(server.submit_allpairs(q), w) for q, w in zip(queries, everything)]
+        tickets += [(server.submit_single(q, s), w) for q, s, w in singles]
+        with pytest.raises(rpq.RPQError) as e:
+            rpq.run_rpq(c, g, queries[0], None, flags=rpq.RPQ_MATERIALIZE)  # 140 million rows
+        assert e.value.code == rpq.RPQ_ERR_OUT_OF_BUDGET
+        tickets += [(server.submit_single(q, s), w) for q, s, w in singles]
+        for t, want in tickets:
+            rep = server.wait(t, timeout_s=60)
+            assert [rep["status"], rep["count"], rep["digest_sum"], rep["digest_xor"]] == [0, *want]
+    finally:
+        server.close()
+    assert [summary(q, s, rpq.RPQ_COUNT_ONLY | f) for q in queries for s in lists for f in modes] + batch() == before
