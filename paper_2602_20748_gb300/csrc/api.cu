@@ -530,14 +530,14 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
     p.list1 = w.list1;
     p.ctl = ctx->ctl;
     p.stamp_base = ctx->stamp;
-    const int grid = bfs_grid(blocks, nw, Gb, n);
-    p.nblocks = (unsigned)grid;
     p.force = force;
     p.alpha = ctx->alpha;
     p.pull_dynamic = ctx->pull_dynamic;
     p.lane_by_source = ctx->lane_by_source;
     p.time_limit_ns = ctx->time_limit_ns;
     p.q = qd;
+    const int grid = bfs_grid(blocks, nw, Gb, n, label_edges(p));
+    p.nblocks = (unsigned)grid;
 
     CK(launch_start(nw, p, live, ctx->small, w.lanesrc, n_lanes > 64 ? nullptr : srcs.data() + g0 * K, ctx->stream));
     CK(cudaEventRecord(ctx->ev[0], ctx->stream));
@@ -1848,14 +1848,14 @@ int rpq_lane_stats_multi(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Mu
   p.list_cap = w.list_cap;
   p.ctl = ctx->ctl;
   p.stamp_base = ctx->stamp;
-  const int grid = bfs_grid(blocks, 1, G, n);
-  p.nblocks = (unsigned)grid;
   p.force = 0;
   p.alpha = ctx->alpha;
   p.pull_dynamic = ctx->pull_dynamic;
   p.lane_by_source = ctx->lane_by_source;
   p.time_limit_ns = ctx->time_limit_ns;
   p.q = un;
+  const int grid = bfs_grid(blocks, 1, G, n, label_edges(p));
+  p.nblocks = (unsigned)grid;
   p.qg = d_desc;
   p.from_tab = d_ft;
   EmitParams ep{};
@@ -2115,14 +2115,14 @@ static int lane_launch(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Lane
   p.list_cap = w.list_cap;
   p.ctl = ctx->ctl;
   p.stamp_base = ctx->stamp;
-  const int grid = bfs_grid(blocks, nw, G, n);
-  p.nblocks = (unsigned)grid;
   p.force = 0;
   p.alpha = ctx->alpha;
   p.pull_dynamic = ctx->pull_dynamic;
   p.lane_by_source = ctx->lane_by_source;
   p.time_limit_ns = ctx->time_limit_ns;
   p.q = un;
+  const int grid = bfs_grid(blocks, nw, G, n, label_edges(p));
+  p.nblocks = (unsigned)grid;
   p.alpha = ctx->lane_alpha;
   p.la_out_begin = reinterpret_cast<const unsigned short *>(dt + o_ob);
   p.la_trans = reinterpret_cast<const unsigned int *>(dt + o_tr);

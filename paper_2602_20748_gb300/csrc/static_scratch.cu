@@ -185,8 +185,6 @@ extern "C" int run_rpq_static(rpq_ctx *ctx, const rpq_graph *g, const rpq_query 
   p.stamp_base = 0;
   const int blocks = ctx_bfs_blocks(ctx, 1);
   if (blocks <= 0) return ctx_error(ctx, RPQ_ERR_CUDA, "traversal kernel cannot be made resident");
-  const int grid = bfs_grid(blocks, 1, 1, n);
-  p.nblocks = (unsigned)grid;
   p.force = 0;
   p.alpha = ctx_alpha(ctx);
   p.pull_dynamic = 1;
@@ -199,6 +197,8 @@ extern "C" int run_rpq_static(rpq_ctx *ctx, const rpq_graph *g, const rpq_query 
   for (uint32_t l = 0; l < dg.L; l++) p.label_edges[l] = dg.label_edges[l];
   p.time_limit_ns = ctx_time_limit_ns(ctx);
   p.q = qd;
+  const int grid = bfs_grid(blocks, 1, 1, n, label_edges(p));
+  p.nblocks = (unsigned)grid;
   STATIC_CK(launch_start(1, p, ns, small, lanesrc, src, st));
   STATIC_CK(launch_msbfs(1, p, grid, 256, st));
 
