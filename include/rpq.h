@@ -462,7 +462,8 @@ typedef struct {
   double bfs_ms;             /* device time of the traversal kernels          */
   double emit_ms;            /* device time of the emission kernels           */
   uint64_t bfs_launches;     /* traversal kernel launches                     */
-  uint64_t launches;         /* all kernel launches of the evaluation         */
+  uint64_t launches;         /* all kernel launches of the evaluation (a scan
+                                counts as one)                               */
   uint64_t alg_bytes;        /* bytes the traversal kernels must move for the
                                 work they did (column ids, offsets, visited and
                                 frontier words, list entries)                 */

@@ -543,7 +543,7 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
     CK(cudaEventRecord(ctx->ev[0], ctx->stream));
     CK(launch_msbfs(nw, p, grid, BFS_THREADS_HOST, ctx->stream));
     CK(cudaEventRecord(ctx->ev[1], ctx->stream));
-    res->stats.launches += 3;
+    res->stats.launches += 2;
     res->stats.bfs_launches += 1;
 
     if (lane_stats && !materialize) {

@@ -128,3 +128,12 @@ def test_a_bound_no_query_reaches_evicts_none(stars, evict_at):
     assert rpq.result_stats(r)["evicted"] == 0
     for i in range(40):
         assert rpq.result_query_stats(r, i) == oracle.pair_digest(oracle.rpq(og, "(a|b)+.c", sources=[i]).rows)
+
+
+@pytest.mark.parametrize("flags,launches", [(rpq.RPQ_COUNT_ONLY, 5), (rpq.RPQ_MATERIALIZE, 9)])
+def test_launches_of_a_call(stars, flags, launches):
+    """Start, traversal, counts, scan, read-back; with rows also their writing,
+    their offsets, the digest and its read-back."""
+    c, g, _ = stars
+    r = rpq.run_rpq(c, g, rpq.compile_rpq(c, "a.b"), np.arange(20, dtype=np.uint32), flags=flags)
+    assert rpq.result_stats(r)["launches"] == launches
