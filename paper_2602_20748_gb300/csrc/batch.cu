@@ -66,6 +66,7 @@ struct BatchParams {
   unsigned long long *qw;  // product edges per query (W)
   u32 *evicted;            // 1 = query left the batch (too large)
   u64 evict_at;            // evict a query once qn exceeds this (0: never)
+  u64 evict_edges;         // or once qw exceeds this (0: qn alone counts)
   u32 append_seg;          // list slots a warp reserves at a time (0: one atomic per append)
   // Visited representation.  hash_bits == 0: dense bitmaps (vis, vis_off).
   // Otherwise query i owns an open-addressing table of 2^hash_bits slots at
@@ -247,14 +248,12 @@ __device__ __forceinline__ void bvisit_wide(const BatchParams &p, const u32 (&i)
 }
 
 // Whether a query with N product vertices and W product edges so far leaves
-// the batch: past evict_at vertices, or past EVICT_EDGES times as many edges.
-// The edges of a frontier are known before it is expanded, so a query that is
-// about to outgrow the batch leaves it without the level that would do so: on
-// configuration 4's batch that level and the next were 26 of 28 ms.  The factor
-// lies at twice the edges that evict_at vertices of degree 16 have.
-constexpr u64 EVICT_EDGES = 32;
+// the batch.  The edges of a frontier are known before it is expanded, so a
+// query that is about to outgrow the batch leaves it without the level that
+// would do so: on configuration 4's batch that level and the next were 26 of
+// 28 ms.
 __device__ __forceinline__ bool outgrown(const BatchParams &p, u64 N, u64 W) {
-  return p.evict_at && (N > p.evict_at || W / EVICT_EDGES > p.evict_at);
+  return p.evict_at && (N > p.evict_at || (p.evict_edges && W > p.evict_edges));
 }
 
 template <bool HASH>
@@ -854,6 +853,15 @@ BatchTuning batch_default_tuning() {
   return BatchTuning{BATCH_THREADS, 4096, 1ull << 28, SPILL_CAP, 1ull << 16, false, 4, 4096, false, false};
 }
 
+// The product edges that stand for evict_at product vertices: twice as many as
+// these have at the graph's mean degree, and at least 32 each.  A fixed 32 sent
+// queries away that could not outgrow anything (48 queries on 1,000 vertices
+// with 10^6 edges, bound 65,536: none leaves now, 22 did).
+static u64 evict_edges(u64 evict_at, const DevGraph &g) {
+  const u64 per = std::max<u64>(32, 2 * ((g.m + g.n - 1) / g.n));
+  return evict_at > ~0ull / per ? ~0ull : evict_at * per;
+}
+
 // One launch over queries [0, nq) of the arrays; appends rows to `out`.
 static int batch_launch(rpq_ctx *ctx, const rpq_graph *g, uint32_t qbase, uint32_t nq,
                         const rpq_query *const *queries, const uint32_t *sources, bool materialize,
@@ -914,6 +922,7 @@ static int batch_launch(rpq_ctx *ctx, const rpq_graph *g, uint32_t qbase, uint32
   p.qw = evict ? d_qw.p : nullptr;
   p.evicted = evict ? d_ev.p : nullptr;
   p.evict_at = evict ? (tun.evict_at ? tun.evict_at : (1ull << hbits) / 2) : 0;
+  p.evict_edges = evict_edges(p.evict_at, dg);
   p.hash_bits = hbits;
   p.rtab = use_hash ? d_rtab.p : nullptr;
   p.qstats = use_hash ? d_hq.p : nullptr;

@@ -201,3 +201,20 @@ def test_batch_spill_capacity_overflow():
     qs = [rpq.compile_rpq(c3, r) for r in regexes]
     got = rpq.fetch_pairs(rpq.run_rpq_batch(c3, g, qs, sources))
     assert np.array_equal(got, oracle_batch_rows(og, regexes, sources))
+
+
+def test_queries_on_a_dense_graph_stay_below_the_vertex_bound(ctx):
+    """1,000 vertices of degree 600: no query reaches 16,384 product vertices,
+    whatever its product edges."""
+    n = 1000
+    rng = np.random.default_rng(3)
+    src, dst, lab = (rng.integers(0, k, 600 * n).astype(t) for k, t in ((n, np.uint32), (n, np.uint32), (4, np.uint16)))
+    g, og = rpq.load_graph(ctx, n, 4, src, dst, lab), oracle.Graph(n, 4, src, dst, lab)
+    regexes = ["(a|b)+.c", "a.b*.c", "a*", "(a|b|c|d)+"] * 8
+    sources = np.arange(32, dtype=np.uint32)
+    rpq.rpq_set_option(ctx, "batch_evict", 16384)
+    r = rpq.run_rpq_batch(ctx, g, [rpq.compile_rpq(ctx, x) for x in regexes], sources, flags=rpq.RPQ_PER_QUERY)
+    assert rpq.result_stats(r)["evicted"] == 0
+    for i in range(4):
+        want = oracle.rpq(og, regexes[i], sources=sources[i:i + 1])
+        assert rpq.result_query_stats(r, i) == oracle.pair_digest(want.rows)
