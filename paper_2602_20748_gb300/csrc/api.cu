@@ -61,7 +61,7 @@ struct rpq_ctx {
   int sms = 0;
   int bpsm[2] = {0, 0};  // resident traversal blocks per SM for NW = 1, 4
   int bpsm_multi = 0;    // the same for the per-group-automata kernel (set on first use)
-  int bpsm_lane[2] = {0, 0};  // and for the per-lane-automata kernel, NW = 1, 4 (set on first use)
+  int bpsm_lane[3] = {0, 0, 0};  // and for the per-lane-automata kernels, NW = 1, 4, 4 staged (set on first use)
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
   float alpha = 16.0f;
   float lane_alpha = 2.0f;  // the same trade-off for lane-mode launches
@@ -2004,8 +2004,9 @@ static int lane_launch(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Lane
   }
   un.final_mask &= Q >= 32 ? ~0u : ((1u << Q) - 1u);
   // resident blocks of the lane-mode kernel
-  int &bpsm = ctx->bpsm_lane[nw == 1 ? 0 : 1];
-  if (bpsm == 0 && msbfs_lane_max_blocks(nw, BFS_THREADS_HOST, &bpsm))
+  const bool staged = lanes_staged(nw, G, Q, ctx->lane_by_source != 0);
+  int &bpsm = ctx->bpsm_lane[nw == 1 ? 0 : staged ? 2 : 1];
+  if (bpsm == 0 && msbfs_lane_max_blocks(nw, staged, BFS_THREADS_HOST, &bpsm))
     return set_err(ctx, RPQ_ERR_CUDA, "occupancy query failed");
   const int blocks = ctx_sm_share(ctx) * bpsm;
   if (blocks <= 0) return set_err(ctx, RPQ_ERR_CUDA, "traversal kernel cannot be made resident");
@@ -2048,7 +2049,7 @@ static int lane_launch(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Lane
   }
   grp_begin[Q] = (uint16_t)grp.size();
   std::vector<uint32_t> sl((size_t)Q * L, 0);
-  if (Q <= 8)
+  if (staged)
     for (uint32_t q = 0; q < Q; q++)
       for (uint32_t t = out_begin[q]; t < out_begin[q + 1]; t++) {
         uint32_t &e = sl[(size_t)q * L + (trans[t] & 0xFFFFu)];

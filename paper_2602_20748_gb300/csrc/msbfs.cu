@@ -121,11 +121,9 @@ __device__ __forceinline__ u64 widx(const BfsParams &p, u32 g, u32 q, u32 v) {
 
 // Automaton modes of a launch: one automaton for every lane (of one lane
 // group, or of several), one per lane group (multi), or one per lane (lane
-// mode).
-constexpr int AM_ONE = 0, AM_GROUP = 1, AM_LANE = 2, AM_MANY = 3;
-// Lane-mode bottom-up by source state (see pull_level) for unions of at most
-// this many states; larger ones gather per target state.
-constexpr u32 LANE_SRC_Q = 8;
+// mode; AM_LANES where its bottom-up levels are pull_lanes).
+constexpr int AM_ONE = 0, AM_GROUP = 1, AM_LANE = 2, AM_MANY = 3, AM_LANES = 4;
+constexpr bool per_lane(int am) { return am == AM_LANE || am == AM_LANES; }
 
 // Automaton of group g: its own in multi mode, else the launch's (the union
 // in lane mode).
@@ -283,7 +281,7 @@ __device__ void seed_phase(const BfsParams &p, u64 *stat) {
         entry = ((u64)g * p.Q << 32) | s;
         if (take && p.fbits) atomicOr(p.fbits + (s >> 5), 1u << (s & 31));  // state 0, bitmap 0
         u32 rows = 0, d;
-        if constexpr (AM == AM_LANE) {
+        if constexpr (per_lane(AM)) {
           Word<NW> me;
 #pragma unroll
           for (int k = 0; k < NW; k++) me.w[k] = (lane / 64 == (u32)k) ? bit : 0ull;
@@ -364,7 +362,7 @@ __device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_c
   // scratch: [32][NW] words of the entries, in lane mode [32][NW] of them
   // masked by the row's transition, [32] (first edge - prefix, target)
   u64 *s_fm = scratch + lane_id() * NW;
-  u64 *s_words = AM == AM_LANE ? scratch + 32 * NW : scratch;
+  u64 *s_words = per_lane(AM) ? scratch + 32 * NW : scratch;
   uint2 *s_row = reinterpret_cast<uint2 *>(s_words + 32 * NW);
   const u64 *list = lp ? p.list1 : p.list0;
   u64 *nlist = lp ? p.list0 : p.list1;
@@ -389,7 +387,7 @@ __device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_c
     entries += valid;
     const QueryDesc &qd = gdesc<AM>(p, valid ? g : 0);
     u32 t_beg, nt;
-    if constexpr (AM == AM_LANE) {
+    if constexpr (per_lane(AM)) {
       t_beg = valid ? p.la_out_begin[q] : 0;
       nt = valid ? p.la_out_begin[q + 1] - t_beg : 0;
     } else {
@@ -399,12 +397,12 @@ __device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_c
     u32 max_nt = __reduce_max_sync(FULL_MASK, nt);
     for (u32 j = 0; j < max_nt; j++) {
       u32 rbeg = 0, rlen = 0, tg = 0;
-      if (AM == AM_LANE && j) __syncwarp();  // the previous transition's edges are done
+      if (per_lane(AM) && j) __syncwarp();  // the previous transition's edges are done
       if (j < nt) {
         u32 t = t_beg + j;
         u32 l, to;
         bool any = true;
-        if constexpr (AM == AM_LANE) {
+        if constexpr (per_lane(AM)) {
           // the entry's lanes that take this transition
           const u32 e = p.la_trans[t];
           l = e & 0xFFFFu;
@@ -464,7 +462,7 @@ __device__ void push_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u64 n_c
       pre -= rlen;
       edges += (lane == 0) ? total : 0;
       if (total == 0) continue;
-      if (AM != AM_LANE) __syncwarp();  // the previous transition's edges are done
+      if (!per_lane(AM)) __syncwarp();  // the previous transition's edges are done
       s_row[lane] = make_uint2(rbeg - pre, tg);
       __syncwarp();
       for (u32 k0 = 0; k0 < total; k0 += 32) {
@@ -1781,7 +1779,7 @@ __device__ void commit_phase(const BfsParams &p, int lp, u32 nxt, u64 n_cur, u64
     store_w<NW>(p.vis + wi, v);
     u32 c = popc_w(m);
     u32 rows = 0, d;
-    if constexpr (AM == AM_LANE) {
+    if constexpr (per_lane(AM)) {
       d = la_degsum<NW>(p, q, w, g, m, W, &rows);
     } else {
       d = degsum(p, gdesc<AM>(p, g), q, w, &rows);
@@ -1867,7 +1865,7 @@ constexpr u64 SOLO_SLOTS = 512, SOLO_EDGES = 512;
 constexpr u32 SOLO_RUN = 64;
 
 template <int NW, int AM>
-__global__ void __launch_bounds__(BFS_THREADS, AM == AM_LANE ? 3 : 4) msbfs_kernel(const __grid_constant__ BfsParams p) {
+__global__ void __launch_bounds__(BFS_THREADS, AM == AM_LANES ? 3 : 4) msbfs_kernel(const __grid_constant__ BfsParams p) {
   // per-warp statistics (lane 0 adds to them once per phase), summed into the
   // control block at the end; in registers they were spilled by every phase
   __shared__ u64 s_stat[BFS_THREADS / 32][ST_COUNT];
@@ -1879,7 +1877,10 @@ __global__ void __launch_bounds__(BFS_THREADS, AM == AM_LANE ? 3 : 4) msbfs_kern
   __shared__ CommitSums sums;
   // per-warp scratch of the expansion phases: a push keeps its entries' words
   // and rows there, lane mode its accumulators, pull_staged its lists
-  constexpr int SCRATCH = AM == AM_LANE ? LANE_SRC_Q * 2 * 32 + LANE_LIST : AM == AM_MANY ? STAGE : 32 * NW + 32;
+  constexpr int SCRATCH = AM == AM_LANES  ? LANE_SRC_Q * 2 * 32 + LANE_LIST
+                          : AM == AM_LANE ? LANE_SRC_Q * 2 * 32
+                          : AM == AM_MANY ? STAGE
+                                          : 32 * NW + 32;
   __shared__ __align__(16) u64 s_scratch[BFS_THREADS / 32][SCRATCH];
   u64 *scratch = s_scratch[threadIdx.x >> 5];
   if (threadIdx.x == 0) sums = CommitSums{};  // seen by the block after the seeds' barrier
@@ -1888,12 +1889,11 @@ __global__ void __launch_bounds__(BFS_THREADS, AM == AM_LANE ? 3 : 4) msbfs_kern
   seed_phase<NW, AM>(p, stat);
   if (!grid_sync(c, p.nblocks, epoch, p.time_limit_ns)) return;
 
-  // lane mode: bottom-up levels by pull_lanes, whose lanes fill a warp's row.
-  // With a bitmap they cost less than the estimate's bytes: the batch above
-  // goes top-down in its second level at a factor above 0.4 (60 ms, not 22).
+  // Bottom-up levels by pull_lanes cost less than the estimate's bytes with a
+  // bitmap: the batch above goes top-down in its second level at a factor above
+  // 0.4 (60 ms, not 22).
   constexpr float LANES_PULL = 0.4f;
-  const bool lanes_staged =
-      AM == AM_LANE && NW == 4 && p.lane_by_source && p.Q <= LANE_SRC_Q && p.G * NW / 2 > 16;
+  constexpr bool lanes_staged = AM == AM_LANES;
   bool have_bits = p.fbits != nullptr;  // this level's frontier has a bitmap (the seeds set theirs)
   u32 level = 0, run = 0;  // run: levels left of block 0's run, 0 outside one
   for (;; level++) {
@@ -1977,12 +1977,9 @@ __global__ void __launch_bounds__(BFS_THREADS, AM == AM_LANE ? 3 : 4) msbfs_kern
       // early)
       if constexpr (AM == AM_MANY) {
         pull_staged<NW>(p, lp, cur, nxt, active, stamp, bits, scratch, sums, stat);
-      } else if constexpr (AM == AM_LANE && NW == 4) {
+      } else if constexpr (AM == AM_LANES) {
         __shared__ LaneTables tab;
-        if (lanes_staged)
-          pull_lanes<NW>(p, lp, cur, nxt, active, stamp, bits, scratch, tab, stat);
-        else
-          pull_level<NW, AM>(p, lp, cur, nxt, active, stamp, bits, scratch, stat);
+        pull_lanes<NW>(p, lp, cur, nxt, active, stamp, bits, scratch, tab, stat);
       } else {
         pull_level<NW, AM>(p, lp, cur, nxt, active, stamp, bits, scratch, stat);
       }
@@ -2164,20 +2161,23 @@ cudaError_t launch_msbfs_multi(const BfsParams &p, int blocks, int threads, cuda
   return cudaLaunchCooperativeKernel((void *)msbfs_kernel<1, AM_GROUP>, blocks, threads, args, 0, st);
 }
 
-cudaError_t launch_msbfs_lane(int nw, const BfsParams &p, int blocks, int threads, cudaStream_t st) {
-  void *args[] = {(void *)&p};
-  if (nw == 1)
-    return cudaLaunchCooperativeKernel((void *)msbfs_kernel<1, AM_LANE>, blocks, threads, args, 0, st);
-  return cudaLaunchCooperativeKernel((void *)msbfs_kernel<4, AM_LANE>, blocks, threads, args, 0, st);
+static void *lane_kernel(int nw, bool staged) {
+  return nw == 1  ? (void *)msbfs_kernel<1, AM_LANE>
+         : staged ? (void *)msbfs_kernel<4, AM_LANES>
+                  : (void *)msbfs_kernel<4, AM_LANE>;
 }
 
-int msbfs_lane_max_blocks(int nw, int threads, int *blocks_per_sm) {
-  cudaError_t e;
-  if (nw == 1)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, msbfs_kernel<1, AM_LANE>, threads, 0);
-  else
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, msbfs_kernel<4, AM_LANE>, threads, 0);
-  return e == cudaSuccess ? 0 : -1;
+cudaError_t launch_msbfs_lane(int nw, const BfsParams &p, int blocks, int threads, cudaStream_t st) {
+  void *args[] = {(void *)&p};
+  const bool staged = lanes_staged(nw, p.G, p.Q, p.lane_by_source != 0);
+  return cudaLaunchCooperativeKernel(lane_kernel(nw, staged), blocks, threads, args, 0, st);
+}
+
+int msbfs_lane_max_blocks(int nw, bool staged, int threads, int *blocks_per_sm) {
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, lane_kernel(nw, staged), threads, 0) ==
+                 cudaSuccess
+             ? 0
+             : -1;
 }
 
 int msbfs_multi_max_blocks(int threads, int *blocks_per_sm) {

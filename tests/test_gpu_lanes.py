@@ -167,3 +167,17 @@ def test_lanes_filling_a_warps_row_match_oracle(n_q, alpha):
     regexes, sources = _mix(n_q, 4, src, n, seed=92 + n_q)
     r = _check(c, g, og, regexes, sources)
     assert rpq.result_stats(r)["pull_levels"] > 0
+
+
+@pytest.mark.parametrize("n_q", [2040, 2100])
+def test_lanes_of_eight_and_nine_groups_match_oracle(n_q):
+    """Either side of the 2,048 lanes above which bottom-up levels are staged."""
+    n = 1500
+    src, dst, lab = _graph(n, 6000, 4, seed=91, hubs=True)
+    c = rpq.Context(device=0)
+    rpq.rpq_set_option(c, "batch_direct", 1)
+    rpq.rpq_set_option(c, "lane_alpha", 1e9)
+    g = rpq.load_graph(c, n, 4, src, dst, lab)
+    regexes, sources = _mix(n_q, 4, src, n, seed=94)
+    r = _check(c, g, oracle.Graph(n, 4, src, dst, lab), regexes, sources)
+    assert rpq.result_stats(r)["pull_levels"] > 0

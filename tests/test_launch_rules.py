@@ -19,6 +19,9 @@ def rules(tmp_path_factory):
 extern "C" int grid(int nw, unsigned groups, unsigned n, unsigned long long edges) {
   return rpq::bfs_grid(608, nw, groups, n, edges);
 }
+extern "C" int staged(int nw, unsigned groups, unsigned states, int by_source) {
+  return rpq::lanes_staged(nw, groups, states, by_source != 0);
+}
 """)
     cuda = os.path.join(os.path.dirname(os.path.realpath(build._nvcc())), "..", "include")
     subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", f"-I{build.CSRC}", f"-I{build.INCLUDE}", f"-I{cuda}",
@@ -38,3 +41,8 @@ def test_grid_grows_with_vertices_and_edges(rules, nw, groups, n):
     assert grids == sorted(grids) and grids[-1] <= MAX_BLOCKS
     # 4 million edges are spread over every block, whatever the number of vertices
     assert rules.grid(nw, groups, n, 4_000_000) == MAX_BLOCKS
+
+
+def test_staged_lane_levels_need_a_full_row_of_lanes(rules):
+    assert [rules.staged(4, g, 8, 1) for g in (1, 4, 8, 9, 16)] == [0, 0, 0, 1, 1]
+    assert not any((rules.staged(1, 16, 8, 1), rules.staged(4, 16, 9, 1), rules.staged(4, 16, 8, 0)))
