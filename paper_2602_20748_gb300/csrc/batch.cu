@@ -426,7 +426,12 @@ __device__ void bcommit(const BatchParams &p, int lp, u32 nxt, u64 *W, u64 *N, u
   u64 n_next = *(volatile unsigned long long *)&p.ctl->n_list[nxt];
   if (n_next > p.list_cap) n_next = p.list_cap;
   const u64 stride = (u64)gridDim.x * blockDim.x;
-  u64 mf = 0;  // out-edges of the next frontier, which batches split its level by
+  // out-edges of the next frontier, which batches split its level by.  Entries
+  // that find their query outgrown are not expanded and do not count; a read of
+  // evicted[i] to see it waited for the stores of the other warps that find the
+  // same (48 queries, 30 of them evicted, on a star of 200,000 vertices: 8.3 ms,
+  // 1.4 without)
+  u64 mf = 0;
   for (u64 j0 = (u64)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); j0 < n_next; j0 += stride) {
     const u64 j = j0 + lane_id();
     bool ok = j < n_next;
@@ -445,10 +450,6 @@ __device__ void bcommit(const BatchParams &p, int lp, u32 nxt, u64 *W, u64 *N, u
       if (ok && p.active) p.active[i] = stamp;
     }
     *W += d;
-    // entries of queries that leave count too: a read of evicted[i] here waited
-    // for the stores of the other warps that find the query outgrown (48 queries,
-    // 30 of them evicted, on a star of 200,000 vertices: 1.4 ms, 9.6 with it)
-    if (!SERVE) mf += d;
     *N += ok ? 1 : 0;
     if (p.qn) {
       // per-query counters; the entries of a warp usually share one query
@@ -458,12 +459,20 @@ __device__ void bcommit(const BatchParams &p, int lp, u32 nxt, u64 *W, u64 *N, u
         const u64 dn = warp_sum((u64)(ok ? 1 : 0)), dw = warp_sum(d);
         if (lane_id() == 0 && dn) {
           const u64 n_all = atomicAdd(&p.qn[i0], dn) + dn, w_all = atomicAdd(&p.qw[i0], dw) + dw;
-          if (outgrown(p, n_all, w_all)) p.evicted[i0] = 1u;
+          if (outgrown(p, n_all, w_all))
+            p.evicted[i0] = 1u;
+          else
+            mf += dw;
         }
       } else if (ok) {
         const u64 n_all = atomicAdd(&p.qn[i], 1ull) + 1, w_all = atomicAdd(&p.qw[i], d) + d;
-        if (outgrown(p, n_all, w_all)) p.evicted[i] = 1u;
+        if (outgrown(p, n_all, w_all))
+          p.evicted[i] = 1u;
+        else
+          mf += d;
       }
+    } else {
+      mf += d;
     }
   }
   if (SERVE) return;
