@@ -137,9 +137,9 @@ int rpq_set_stream(rpq_ctx *ctx, void *cuda_stream);
  *   "max_groups"   lane groups (256 start vertices each) per launch, 1 .. 16
  *   "time_limit_s" bound on each device-side wait (default 20 s)
  *   "batch_evict"  run_rpq_batch with RPQ_PER_QUERY: product vertices after
- *                  which a query leaves the shared launch, or once it has
- *                  product edges for twice as many at the graph's mean degree
- *                  (32 per vertex at least) (0: never)
+ *                  which a query leaves the shared launch, or 32 times as
+ *                  many product edges after which it does where it could
+ *                  still have that many product vertices (0: never)
  *   "batch_streams" helper contexts evaluating evicted queries side by
  *                  side, 1 .. 16 (default 4)
  *   "batch_lanes"  run_rpq_batch with RPQ_PER_QUERY: evicted queries run in
@@ -260,8 +260,8 @@ int run_rpq_middle(rpq_ctx *ctx, const rpq_graph *g, const rpq_query *alpha, con
  * are counted and digested as run_rpq(queries[i], {sources[i]}) would report
  * them (result_query_stats), and result_info totals those summaries.  In
  * that mode a query whose product graph grows past a threshold (option
- * "batch_evict", product vertices, or product edges in proportion; default
- * 65,536) leaves the shared launch,
+ * "batch_evict", product vertices, or 32 times as many product edges;
+ * default 65,536) leaves the shared launch,
  * and such queries are then evaluated together by the multi-source engine in
  * lane-mode launches: one bit lane per query, each lane with its own
  * automaton (option "batch_lanes"; "batch_direct" sends every query there).

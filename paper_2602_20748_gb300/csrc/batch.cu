@@ -66,7 +66,7 @@ struct BatchParams {
   unsigned long long *qw;  // product edges per query (W)
   u32 *evicted;            // 1 = query left the batch (too large)
   u64 evict_at;            // evict a query once qn exceeds this (0: never)
-  u64 evict_edges;         // or once qw exceeds this (0: qn alone counts)
+  u64 evict_edges;         // or once qw exceeds this and qn still can (0: qn alone counts)
   u32 append_seg;          // list slots a warp reserves at a time (0: one atomic per append)
   // Visited representation.  hash_bits == 0: dense bitmaps (vis, vis_off).
   // Otherwise query i owns an open-addressing table of 2^hash_bits slots at
@@ -247,13 +247,20 @@ __device__ __forceinline__ void bvisit_wide(const BatchParams &p, const u32 (&i)
   for (int k = 0; k < N; k++) take[k] = !((seen[k] >> (w[k] & 63)) & 1ull);
 }
 
-// Whether a query with N product vertices and W product edges so far leaves
-// the batch.  The edges of a frontier are known before it is expanded, so a
-// query that is about to outgrow the batch leaves it without the level that
-// would do so: on configuration 4's batch that level and the next were 26 of
-// 28 ms.
-__device__ __forceinline__ bool outgrown(const BatchParams &p, u64 N, u64 W) {
-  return p.evict_at && (N > p.evict_at || (p.evict_edges && W > p.evict_edges));
+// Whether query i with N product vertices and W product edges so far leaves the
+// batch: past evict_at vertices, or past evict_edges edges where its product
+// graph has more vertices than evict_at.  The edges of a frontier are known
+// before it is expanded, so a query that is about to outgrow the batch leaves it
+// without the level that would do so: on configuration 4's batch that level and
+// the next were 26 of 28 ms.  32 edges stand for a vertex, twice the degree of
+// that graph; at twice the mean degree of a denser one (R-MAT 2^16, degree 57)
+// 1,500 queries took 12% longer.  On small dense graphs edges say nothing: 48
+// queries on 1,000 vertices with 2.5 * 10^6 edges, bound 65,536, and 22 left.
+constexpr u64 EVICT_EDGES = 32;
+__device__ __forceinline__ bool outgrown(const BatchParams &p, u32 i, u64 N, u64 W) {
+  if (!p.evict_at) return false;
+  if (N > p.evict_at) return true;
+  return p.evict_edges && W > p.evict_edges && (u64)p.qd[i].n_states * p.n > p.evict_at;
 }
 
 template <bool HASH>
@@ -276,7 +283,7 @@ __device__ void bseed(const BatchParams &p, u64 *W, u64 *N) {
         if (p.qn) {
           p.qn[i] = 1;
           p.qw[i] = d;
-          if (outgrown(p, 1, d)) p.evicted[i] = 1u;
+          if (outgrown(p, (u32)i, 1, d)) p.evicted[i] = 1u;
         }
       }
     }
@@ -459,14 +466,14 @@ __device__ void bcommit(const BatchParams &p, int lp, u32 nxt, u64 *W, u64 *N, u
         const u64 dn = warp_sum((u64)(ok ? 1 : 0)), dw = warp_sum(d);
         if (lane_id() == 0 && dn) {
           const u64 n_all = atomicAdd(&p.qn[i0], dn) + dn, w_all = atomicAdd(&p.qw[i0], dw) + dw;
-          if (outgrown(p, n_all, w_all))
+          if (outgrown(p, i0, n_all, w_all))
             p.evicted[i0] = 1u;
           else
             mf += dw;
         }
       } else if (ok) {
         const u64 n_all = atomicAdd(&p.qn[i], 1ull) + 1, w_all = atomicAdd(&p.qw[i], d) + d;
-        if (outgrown(p, n_all, w_all))
+        if (outgrown(p, i, n_all, w_all))
           p.evicted[i] = 1u;
         else
           mf += d;
@@ -862,15 +869,6 @@ BatchTuning batch_default_tuning() {
   return BatchTuning{BATCH_THREADS, 4096, 1ull << 28, SPILL_CAP, 1ull << 16, false, 4, 4096, false, false};
 }
 
-// The product edges that stand for evict_at product vertices: twice as many as
-// these have at the graph's mean degree, and at least 32 each.  A fixed 32 sent
-// queries away that could not outgrow anything (48 queries on 1,000 vertices
-// with 10^6 edges, bound 65,536: none leaves now, 22 did).
-static u64 evict_edges(u64 evict_at, const DevGraph &g) {
-  const u64 per = std::max<u64>(32, 2 * ((g.m + g.n - 1) / g.n));
-  return evict_at > ~0ull / per ? ~0ull : evict_at * per;
-}
-
 // One launch over queries [0, nq) of the arrays; appends rows to `out`.
 static int batch_launch(rpq_ctx *ctx, const rpq_graph *g, uint32_t qbase, uint32_t nq,
                         const rpq_query *const *queries, const uint32_t *sources, bool materialize,
@@ -931,7 +929,7 @@ static int batch_launch(rpq_ctx *ctx, const rpq_graph *g, uint32_t qbase, uint32
   p.qw = evict ? d_qw.p : nullptr;
   p.evicted = evict ? d_ev.p : nullptr;
   p.evict_at = evict ? (tun.evict_at ? tun.evict_at : (1ull << hbits) / 2) : 0;
-  p.evict_edges = evict_edges(p.evict_at, dg);
+  p.evict_edges = p.evict_at > ~0ull / EVICT_EDGES ? ~0ull : p.evict_at * EVICT_EDGES;
   p.hash_bits = hbits;
   p.rtab = use_hash ? d_rtab.p : nullptr;
   p.qstats = use_hash ? d_hq.p : nullptr;

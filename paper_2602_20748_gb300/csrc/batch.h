@@ -17,9 +17,9 @@ struct BatchTuning {
   uint32_t queries_per_launch;  // queries sharing one launch
   uint64_t list_cap;            // frontier list capacity (entries)
   uint64_t spill_cap;           // long-row chunks per level (<= SPILL_CAP)
-  uint64_t evict_at;            // per-query mode: a query with more product vertices (or the product
-                                // edges that stand for them) leaves the batch and is evaluated with
-                                // the multi-source engine (0: never)
+  uint64_t evict_at;            // per-query mode: a query with more product vertices (or 32 times as
+                                // many product edges) leaves the batch and is evaluated with the
+                                // multi-source engine (0: never)
   bool multi;                   // evicted small automaton groups share multi-automaton launches
   uint32_t streams;             // helper contexts evaluating evicted queries side by side
   uint32_t lanes;               // per-query mode: evicted queries run in lane-mode launches of up to this
