@@ -294,25 +294,28 @@ cudaError_t launch_vis_init_lane(int nw, const BfsParams &p, const unsigned long
 cudaError_t launch_source_filter(const uint32_t *off, uint32_t n, uint32_t L, unsigned long long label_mask,
                                  const uint32_t *srcs, unsigned long long count, unsigned char *flag,
                                  cudaStream_t st);
-// Edges on the labels that a launch's automaton takes.
+// Edges per label that a launch's automaton takes, on average.
 inline uint64_t label_edges(const BfsParams &p) {
-  uint64_t seen = 0, m = 0;
+  uint64_t seen = 0, m = 0, n_labels = 0;
   for (uint32_t j = 0; j < p.q.in_begin[p.q.n_states]; j++) {
     const uint32_t l = p.q.in_label[j];
     if (l >= p.L || (seen >> l) & 1u) continue;
     seen |= 1ull << l;
     m += p.label_edges[l];
+    n_labels++;
   }
-  return m;
+  return n_labels ? m / n_labels : 0;
 }
-// Blocks of a traversal launch over n vertices and `edges` edges: enough that a
-// bottom-up level gives every sub-warp (the lanes it uses per vertex, two words
-// each, rounded up to a power of two) a vertex, or GRID_EDGES edges where
-// vertices have more, at most max_blocks.  Beyond that, blocks only make the
-// barriers of a small graph's levels dearer; sized by vertices alone, 64 start
-// vertices on 1,000 vertices with 2.5 * 10^6 edges ran on four blocks, 3,382 us
-// for (a|b)+.c where the full grid takes 294 and this rule 177.  4 edges differ
-// by up to 5% either way, 64 lose 40% with 6 * 10^5 edges.
+// Blocks of a traversal launch over n vertices with `edges` edges per label:
+// enough that a bottom-up level gives every sub-warp (the lanes it uses per
+// vertex, two words each, rounded up to a power of two) a vertex, or GRID_EDGES
+// edges where vertices have more, at most max_blocks.  Beyond that, blocks only
+// make the barriers of a small graph's levels dearer (by the labels' sum instead
+// of their average 600 lanes on 8,000 vertices of degree 100 took 3.35 ms for
+// 2.95); sized by vertices alone, 64 start vertices on 1,000 vertices with 2.5 *
+// 10^6 edges ran on four blocks, 3,390 us for (a|b)+.c where the full grid takes
+// 299 and this rule 199.  Of a* there 4 edges are up to 13% faster and up to 5%
+// slower, 64 lose 40% with 2 * 10^5 edges.
 constexpr uint32_t GRID_EDGES = 16;
 inline int bfs_grid(int max_blocks, int nw, uint32_t G, uint32_t n, uint64_t edges) {
   const uint32_t lanes = nw == 1 ? G : G * nw / 2;
