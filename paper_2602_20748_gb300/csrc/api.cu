@@ -61,7 +61,7 @@ struct rpq_ctx {
   int sms = 0;
   int bpsm[2] = {0, 0};  // resident traversal blocks per SM for NW = 1, 4
   int bpsm_multi = 0;    // the same for the per-group-automata kernel (set on first use)
-  int bpsm_lane[3] = {0, 0, 0};  // and for the per-lane-automata kernels, NW = 1, 4, 4 staged (set on first use)
+  int bpsm_lane[2][3] = {};  // and for the per-lane-automata kernels, by NW = 1, 4 and LaneKernel (set on first use)
   cudaEvent_t ev[4] = {nullptr, nullptr, nullptr, nullptr};
   float alpha = 16.0f;
   float lane_alpha = 2.0f;  // the same trade-off for lane-mode launches
@@ -2005,10 +2005,12 @@ static int lane_launch(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Lane
   un.final_mask &= Q >= 32 ? ~0u : ((1u << Q) - 1u);
   // resident blocks of the lane-mode kernel
   const bool staged = lanes_staged(nw, G, Q, ctx->lane_by_source != 0);
-  int &bpsm = ctx->bpsm_lane[nw == 1 ? 0 : staged ? 2 : 1];
-  if (bpsm == 0 && msbfs_lane_max_blocks(nw, staged, BFS_THREADS_HOST, &bpsm))
-    return set_err(ctx, RPQ_ERR_CUDA, "occupancy query failed");
-  const int blocks = ctx_sm_share(ctx) * bpsm;
+  LaneKernel kernel = staged ? LaneKernel::staged : LaneKernel::plain;
+  int *const bpsm = ctx->bpsm_lane[nw == 1 ? 0 : 1];
+  for (LaneKernel k : {kernel, LaneKernel::few})
+    if (bpsm[(int)k] == 0 && msbfs_lane_max_blocks(nw, k, BFS_THREADS_HOST, &bpsm[(int)k]))
+      return set_err(ctx, RPQ_ERR_CUDA, "occupancy query failed");
+  const int blocks = ctx_sm_share(ctx) * bpsm[(int)kernel];
   if (blocks <= 0) return set_err(ctx, RPQ_ERR_CUDA, "traversal kernel cannot be made resident");
   const uint64_t slack = 2ull * blocks * (BFS_THREADS_HOST / 32) * APPEND_SEG;
   const uint64_t words = (uint64_t)G * Q * n * nw;
@@ -2124,6 +2126,7 @@ static int lane_launch(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Lane
   p.q = un;
   const int grid = bfs_grid(blocks, nw, G, n, label_edges(p));
   p.nblocks = (unsigned)grid;
+  if (kernel == LaneKernel::plain && grid <= ctx_sm_share(ctx) * bpsm[(int)LaneKernel::few]) kernel = LaneKernel::few;
   p.alpha = ctx->lane_alpha;
   p.la_out_begin = reinterpret_cast<const unsigned short *>(dt + o_ob);
   p.la_trans = reinterpret_cast<const unsigned int *>(dt + o_tr);
@@ -2148,7 +2151,7 @@ static int lane_launch(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Lane
   if ((e = launch_vis_init_lane(nw, p, reinterpret_cast<const u64 *>(dt + o_emp), st)) == cudaSuccess &&
       (e = cudaMemsetAsync(ctx->ctl, 0, sizeof(BfsCtl), st)) == cudaSuccess &&
       (e = cudaEventRecord(ctx->ev[0], st)) == cudaSuccess &&
-      (e = launch_msbfs_lane(nw, p, grid, BFS_THREADS_HOST, st)) == cudaSuccess &&
+      (e = launch_msbfs_lane(nw, kernel, p, grid, BFS_THREADS_HOST, st)) == cudaSuccess &&
       (e = cudaEventRecord(ctx->ev[1], st)) == cudaSuccess && (e = launch_emit_lane_stats(nw, ep, ls, st)) == cudaSuccess &&
       (e = cudaEventRecord(ctx->ev[2], st)) == cudaSuccess)
     e = rb_queue(ctx, 0, ctx->ctl, sizeof(BfsCtl));

@@ -1864,8 +1864,8 @@ __device__ float pull_bytes(const BfsParams &p, u32 active) {
 constexpr u64 SOLO_SLOTS = 512, SOLO_EDGES = 512;
 constexpr u32 SOLO_RUN = 64;
 
-template <int NW, int AM>
-__global__ void __launch_bounds__(BFS_THREADS, AM == AM_LANES ? 3 : 4) msbfs_kernel(const __grid_constant__ BfsParams p) {
+template <int NW, int AM, int BLOCKS = AM == AM_LANES ? 3 : 4>
+__global__ void __launch_bounds__(BFS_THREADS, BLOCKS) msbfs_kernel(const __grid_constant__ BfsParams p) {
   // per-warp statistics (lane 0 adds to them once per phase), summed into the
   // control block at the end; in registers they were spilled by every phase
   __shared__ u64 s_stat[BFS_THREADS / 32][ST_COUNT];
@@ -2161,21 +2161,19 @@ cudaError_t launch_msbfs_multi(const BfsParams &p, int blocks, int threads, cuda
   return cudaLaunchCooperativeKernel((void *)msbfs_kernel<1, AM_GROUP>, blocks, threads, args, 0, st);
 }
 
-static void *lane_kernel(int nw, bool staged) {
-  return nw == 1  ? (void *)msbfs_kernel<1, AM_LANE>
-         : staged ? (void *)msbfs_kernel<4, AM_LANES>
-                  : (void *)msbfs_kernel<4, AM_LANE>;
+static void *lane_kernel(int nw, LaneKernel k) {
+  if (k == LaneKernel::staged) return (void *)msbfs_kernel<4, AM_LANES>;
+  if (k == LaneKernel::few) return nw == 1 ? (void *)msbfs_kernel<1, AM_LANE, 3> : (void *)msbfs_kernel<4, AM_LANE, 3>;
+  return nw == 1 ? (void *)msbfs_kernel<1, AM_LANE> : (void *)msbfs_kernel<4, AM_LANE>;
 }
 
-cudaError_t launch_msbfs_lane(int nw, const BfsParams &p, int blocks, int threads, cudaStream_t st) {
+cudaError_t launch_msbfs_lane(int nw, LaneKernel k, const BfsParams &p, int blocks, int threads, cudaStream_t st) {
   void *args[] = {(void *)&p};
-  const bool staged = lanes_staged(nw, p.G, p.Q, p.lane_by_source != 0);
-  return cudaLaunchCooperativeKernel(lane_kernel(nw, staged), blocks, threads, args, 0, st);
+  return cudaLaunchCooperativeKernel(lane_kernel(nw, k), blocks, threads, args, 0, st);
 }
 
-int msbfs_lane_max_blocks(int nw, bool staged, int threads, int *blocks_per_sm) {
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, lane_kernel(nw, staged), threads, 0) ==
-                 cudaSuccess
+int msbfs_lane_max_blocks(int nw, LaneKernel k, int threads, int *blocks_per_sm) {
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, lane_kernel(nw, k), threads, 0) == cudaSuccess
              ? 0
              : -1;
 }

@@ -268,7 +268,10 @@ inline void set_chunks(BfsParams &p, const ChunkLists &c, uint32_t L, uint64_t s
 // pull_lanes, in launches whose lanes fill a warp's row.  It needs 80 registers,
 // so its kernel runs three blocks per SM; the plain form is a kernel of its own,
 // at four: 1,797 lanes on R-MAT 2^24 (0.55 of the SMs), its three dense levels
-// 636 / 777 / 767 ms, 853 / 1,049 / 1,038 at three.
+// 636 / 777 / 767 ms, 853 / 1,049 / 1,038 at three.  Launches whose grid fits
+// three blocks per SM anyway take a third build, the plain levels at 80 registers
+// (200 lanes on 30,000 vertices of degree 40: 2.05 ms, 2.30 at 64).
+enum class LaneKernel { plain, few, staged };
 constexpr uint32_t LANE_SRC_Q = 8;
 inline bool lanes_staged(int nw, uint32_t G, uint32_t Q, bool by_source) {
   return nw == 4 && by_source && Q <= LANE_SRC_Q && G * nw / 2 > 16;
@@ -287,8 +290,8 @@ cudaError_t launch_msbfs_multi(const BfsParams &p, int blocks, int threads, cuda
 int msbfs_multi_max_blocks(int threads, int *blocks_per_sm);
 // Per-lane automata (p.la_* set), NW = 1 or 4.  VIS starts as empty_q[(q * G +
 // g) * NW + k]: the lanes that are empty or whose automaton has no state q.
-cudaError_t launch_msbfs_lane(int nw, const BfsParams &p, int blocks, int threads, cudaStream_t st);
-int msbfs_lane_max_blocks(int nw, bool staged, int threads, int *blocks_per_sm);
+cudaError_t launch_msbfs_lane(int nw, LaneKernel k, const BfsParams &p, int blocks, int threads, cudaStream_t st);
+int msbfs_lane_max_blocks(int nw, LaneKernel k, int threads, int *blocks_per_sm);
 cudaError_t launch_vis_init_lane(int nw, const BfsParams &p, const unsigned long long *empty_q, cudaStream_t st);
 // flag[i] = whether srcs[i] has an edge (offsets `off`, per label) on a label of label_mask.
 cudaError_t launch_source_filter(const uint32_t *off, uint32_t n, uint32_t L, unsigned long long label_mask,
