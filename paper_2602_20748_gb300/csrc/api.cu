@@ -508,8 +508,6 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
     p.out_col = reverse ? g.in_col : g.out_col;
     p.in_off = reverse ? g.out_off : g.in_off;
     p.in_col = reverse ? g.out_col : g.in_col;
-    // bottom-up levels read the in-direction of the traversal
-    set_chunks(p, reverse ? g.chunks_out : g.chunks_in, g.L, live, shorter.there());
     for (uint32_t l = 0; l < g.L; l++) p.label_edges[l] = g.label_edges[l];
     p.n = n;
     p.L = g.L;
@@ -536,6 +534,8 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
     p.lane_by_source = ctx->lane_by_source;
     p.time_limit_ns = ctx->time_limit_ns;
     p.q = qd;
+    // bottom-up levels read the in-direction of the traversal
+    set_chunks(p, reverse ? g.chunks_out : g.chunks_in, live, shorter.there());
     const int grid = bfs_grid(blocks, nw, Gb, n, label_edges(p));
     p.nblocks = (unsigned)grid;
 
@@ -1826,8 +1826,6 @@ int rpq_lane_stats_multi(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Mu
   p.out_col = g.out_col;
   p.in_off = g.in_off;
   p.in_col = g.in_col;
-  const ShorterChunks shorter(ctx, gr);
-  set_chunks(p, g.chunks_in, g.L, total_lanes, shorter.there());
   for (uint32_t l = 0; l < g.L; l++) p.label_edges[l] = g.label_edges[l];
   p.n = n;
   p.L = L;
@@ -1854,6 +1852,8 @@ int rpq_lane_stats_multi(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Mu
   p.lane_by_source = ctx->lane_by_source;
   p.time_limit_ns = ctx->time_limit_ns;
   p.q = un;
+  const ShorterChunks shorter(ctx, gr);
+  set_chunks(p, g.chunks_in, total_lanes, shorter.there());
   const int grid = bfs_grid(blocks, 1, G, n, label_edges(p));
   p.nblocks = (unsigned)grid;
   p.qg = d_desc;
@@ -2096,8 +2096,6 @@ static int lane_launch(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Lane
   p.out_col = g.out_col;
   p.in_off = g.in_off;
   p.in_col = g.in_col;
-  const ShorterChunks shorter(ctx, gr);
-  set_chunks(p, g.chunks_in, g.L, k, shorter.there());
   for (uint32_t l = 0; l < g.L; l++) p.label_edges[l] = g.label_edges[l];
   p.n = n;
   p.L = L;
@@ -2124,6 +2122,8 @@ static int lane_launch(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Lane
   p.lane_by_source = ctx->lane_by_source;
   p.time_limit_ns = ctx->time_limit_ns;
   p.q = un;
+  const ShorterChunks shorter(ctx, gr);
+  set_chunks(p, g.chunks_in, k, shorter.there(), staged);
   const int grid = bfs_grid(blocks, nw, G, n, label_edges(p));
   p.nblocks = (unsigned)grid;
   if (kernel == LaneKernel::plain && grid <= ctx_sm_share(ctx) * bpsm[(int)LaneKernel::few]) kernel = LaneKernel::few;

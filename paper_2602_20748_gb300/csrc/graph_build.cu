@@ -132,16 +132,19 @@ __global__ void label_bounds(const uint32_t *__restrict__ off, uint32_t n, uint3
 // Chunk lists of long rows, all labels at once (blockIdx.y = label): a list per
 // label and class, rows of at least LONG_ROW edges (class 0) and rows of
 // HEAVY_ROW .. LONG_ROW - 1 (class 1).  Without out0 and out1,
-// next[2 * label + class] counts the chunks; with them, it is the place of the
-// list's next record (vertex, first edge, end edge), taken a warp at a time.
-__global__ void row_chunks(const uint32_t *__restrict__ off, uint32_t n, u32 *__restrict__ next,
+// next[2 * label + class] counts the chunks and light[label] the edges in rows
+// below HEAVY_ROW; with them, next is the place of the list's next record
+// (vertex, first edge, end edge), taken a warp at a time.
+__global__ void row_chunks(const uint32_t *__restrict__ off, uint32_t n, u32 *__restrict__ next, u32 *__restrict__ light,
                            uint32_t *__restrict__ out0, uint32_t *__restrict__ out1) {
   const uint32_t *row = off + (u64)blockIdx.y * (n + 1);
   next += 2 * blockIdx.y;
   const u64 step = (u64)gridDim.x * blockDim.x;
+  u32 few = 0;
   for (u64 v0 = (u64)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); v0 < n; v0 += step) {
     const u64 v = v0 + lane_id();
     const uint32_t b = v < n ? row[v] : 0u, len = v < n ? row[v + 1] - b : 0u;
+    if (len < HEAVY_ROW) few += len;
     for (int cls = 0; cls < 2; cls++) {
       const bool mine = cls == 0 ? len >= LONG_ROW : len >= HEAVY_ROW && len < LONG_ROW;
       if (!__any_sync(FULL_MASK, mine)) continue;
@@ -165,6 +168,9 @@ __global__ void row_chunks(const uint32_t *__restrict__ off, uint32_t n, u32 *__
         }
     }
   }
+  if (out0) return;
+  few = warp_sum(few);
+  if (lane_id() == 0 && few) atomicAdd(&light[blockIdx.y], few);
 }
 
 // (label | src | dst) -> (label | dst | src)
@@ -270,16 +276,17 @@ static cudaError_t build_chunks(const uint32_t *off, uint32_t n, uint32_t L, Chu
   u32 *next = nullptr;
   ChunkList *cls[2] = {&lists->longer, &lists->shorter};
   for (ChunkList *c : cls) c->off.assign(L + 1, 0);
-  std::vector<u32> cnt(2 * L, 0);
+  std::vector<u32> cnt(3 * L, 0);
   const dim3 grid((unsigned)std::min<u64>(grid_for(n, 256), 608), L);
-  cudaError_t e = cudaMallocAsync(&next, 8ull * L, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(next, 0, 8ull * L, st);
+  cudaError_t e = cudaMallocAsync(&next, 12ull * L, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(next, 0, 12ull * L, st);
   if (e == cudaSuccess) {
-    row_chunks<<<grid, 256, 0, st>>>(off, n, next, nullptr, nullptr);
+    row_chunks<<<grid, 256, 0, st>>>(off, n, next, next + 2 * L, nullptr, nullptr);
     e = cudaGetLastError();
   }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(cnt.data(), next, 8ull * L, cudaMemcpyDeviceToHost, st);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(cnt.data(), next, 12ull * L, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  lists->light.assign(cnt.begin() + 2 * L, cnt.end());
   for (int c = 0; c < 2 && e == cudaSuccess; c++) {
     for (uint32_t l = 0; l < L; l++) {
       cls[c]->off[l + 1] = cls[c]->off[l] + cnt[2 * l + c];
@@ -289,7 +296,7 @@ static cudaError_t build_chunks(const uint32_t *off, uint32_t n, uint32_t L, Chu
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(next, cnt.data(), 8ull * L, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) {
-    row_chunks<<<grid, 256, 0, st>>>(off, n, next, cls[0]->rec, cls[1]->rec);
+    row_chunks<<<grid, 256, 0, st>>>(off, n, next, nullptr, cls[0]->rec, cls[1]->rec);
     e = cudaGetLastError();
   }
   if (next) cudaFreeAsync(next, st);

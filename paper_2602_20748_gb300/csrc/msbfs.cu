@@ -692,7 +692,9 @@ __device__ __forceinline__ void publish_sums(BfsCtl *c, CommitSums &s, u32 nxt) 
 
 // ---------------------------------------------------------------------------
 // Bottom-up expansion of several lane groups under one automaton (G > 1, 256
-// lanes each), the form of every large source list.
+// lanes each), the form of large source lists on graphs with rows of very
+// different lengths (where all rows are long pull_level is faster, see
+// set_chunks).
 //
 // What bounds it: gathers of G * 32 bytes from random rows of the frontier
 // array.  Walking one vertex's in-row after another, the row offsets, the
@@ -2132,8 +2134,8 @@ cudaError_t launch_source_filter(const uint32_t *off, uint32_t n, uint32_t L, un
 cudaError_t launch_msbfs(int nw, const BfsParams &p, int blocks, int threads, cudaStream_t st) {
   void *args[] = {(void *)&p};
   void *kernel = nw == 1   ? (void *)msbfs_kernel<1, AM_ONE>
-                 : p.G == 1 ? (void *)msbfs_kernel<4, AM_ONE>
-                            : (void *)msbfs_kernel<4, AM_MANY>;
+                 : p.G == 1 || p.walk_rows ? (void *)msbfs_kernel<4, AM_ONE>
+                                           : (void *)msbfs_kernel<4, AM_MANY>;
   return cudaLaunchCooperativeKernel(kernel, blocks, threads, args, 0, st);
 }
 

@@ -59,6 +59,7 @@ int dfa_then_label(const HostQuery &alpha, uint32_t x, HostQuery *out, std::stri
 // come out evener than at 128, though such a vertex's words are then or-ed
 // atomically: 1,500 reverse targets on R-MAT 2^18 1.78 -> 1.52 ms,
 // configuration 2 20.2 -> 19.0 (24: 19.3, 48: 19.2, 64: 19.4, 256: 20.5).
+// Where most rows are that long they may stay whole (see set_chunks).
 // Launches of few start vertices leave a row at the first frontier vertices
 // they meet, so for them only rows of LONG_ROW edges are chunked (one lookup
 // on R-MAT 2^20: 0.55 ms, 0.60 with chunks from 32); the lists keep the two
@@ -77,6 +78,7 @@ struct ChunkList {
 struct ChunkLists {
   ChunkList longer;   // rows of LONG_ROW edges and more
   ChunkList shorter;  // HEAVY_ROW .. LONG_ROW - 1 edges; given back when the budget needs the room
+  std::vector<uint32_t> light;  // per label, the edges in rows below HEAVY_ROW
 };
 
 struct DevGraph {
@@ -179,6 +181,7 @@ struct BfsParams {
   uint32_t chunk_beg[2][RPQ_MAX_LABELS];
   uint32_t chunk_n[2][RPQ_MAX_LABELS];
   uint32_t heavy_row;
+  bool walk_rows;  // several lane groups: bottom-up levels walk each row (see set_chunks)
   unsigned long long label_edges[RPQ_MAX_LABELS];
   uint32_t n;
   uint32_t L;             // edge labels of the graph
@@ -248,14 +251,56 @@ struct BfsParams {
   QueryDesc q;
 };
 
+// The labels that a launch's automaton takes and the graph has.
+inline uint64_t label_set(const BfsParams &p) {
+  uint64_t set = 0;
+  for (uint32_t j = 0; j < p.q.in_begin[p.q.n_states]; j++)
+    if (p.q.in_label[j] < p.L) set |= 1ull << p.q.in_label[j];
+  return set;
+}
 // The chunk lists of a launch of `starts` start vertices (shorter: the graph
-// still has its lists of shorter rows).
-inline void set_chunks(BfsParams &p, const ChunkLists &c, uint32_t L, uint64_t starts, bool shorter) {
-  shorter = shorter && starts >= FEW_STARTS;
+// still has its lists of shorter rows), and how launches of several lane groups
+// read the other rows bottom-up.
+//
+// Where rows of 32 to 127 edges are the ordinary ones, more than one vertex in
+// eight over the launch's labels, they stay whole: an item per row costs more
+// than the row, and there is nothing to even out.  500,000 vertices of degree 40,
+// a* from 64 start vertices: 1,825 us with their chunks, 512 without.  In R-MAT
+// graphs of degree 16 to 100 at most one vertex in eleven has such a row, and the
+// chunks make the calls 1.05 to 1.4 times as fast.
+//
+// There, and where the rows below 32 edges are long on average, levels walk a
+// vertex's rows (pull_level) instead of listing the gathers of 32 vertices
+// (pull_staged): the list costs more than it hides, the more so the fewer words a
+// gather reads.  300 start vertices (two groups) on 500,000 of degree 40 / 20:
+// 2,068 / 1,636 us listed, 1,313 / 1,274 walked; 4,096 on degree 20: 7.40 and
+// 7.23 ms, degree 10: 6.8 and 7.4.  R-MAT 2^20 of degree 64, 300: 3.14 ms listed,
+// 3.94 walked; its rows below 32 edges have 4 on average.
+//
+// Both need vertices enough for every warp to work on several at a time: of
+// degree 100, 300 start vertices take 244 us on 16,000 vertices by chunks and
+// lists, 290 by whole rows (32,000: 300 and 309; 64,000: 461 and 441), of degree
+// 25 per label 296 listed and 352 walked on 32,000 (128,000: 534 and 437).
+// Launches of one group have rows enough on any graph; the staged lane levels
+// list rows anyhow (3,000 lanes on 128,000 vertices of degree 50 per label: 54 ms
+// by chunks, 68 without).
+constexpr uint32_t WHOLE_MIN = 1u << 15, WALK_MIN = 1u << 17;
+inline void set_chunks(BfsParams &p, const ChunkLists &c, uint64_t starts, bool shorter, bool lanes_staged = false) {
+  const uint64_t labels = label_set(p);
+  uint64_t rows = 0, light = 0, vertices = 0;  // over the labels
+  for (uint32_t l = 0; l < p.L; l++)
+    if ((labels >> l) & 1u) {
+      rows += c.shorter.off[l + 1] - c.shorter.off[l];
+      light += c.light[l];
+      vertices += p.n;
+    }
+  const bool whole = rows * 8 > vertices && (p.G == 1 || p.n >= WHOLE_MIN) && !lanes_staged;
+  p.walk_rows = whole || (p.n >= WALK_MIN && light > vertices * (p.G <= 4 ? 8 : 16));
+  shorter = shorter && starts >= FEW_STARTS && !whole;
   p.heavy_row = shorter ? HEAVY_ROW : LONG_ROW;
   p.chunk_rec[0] = c.longer.rec;
   p.chunk_rec[1] = shorter ? c.shorter.rec : nullptr;
-  for (uint32_t l = 0; l < L; l++) {
+  for (uint32_t l = 0; l < p.L; l++) {
     p.chunk_beg[0][l] = c.longer.off[l];
     p.chunk_n[0][l] = c.longer.off[l + 1] - c.longer.off[l];
     p.chunk_beg[1][l] = shorter ? c.shorter.off[l] : 0;
@@ -299,14 +344,12 @@ cudaError_t launch_source_filter(const uint32_t *off, uint32_t n, uint32_t L, un
                                  cudaStream_t st);
 // Edges per label that a launch's automaton takes, on average.
 inline uint64_t label_edges(const BfsParams &p) {
-  uint64_t seen = 0, m = 0, n_labels = 0;
-  for (uint32_t j = 0; j < p.q.in_begin[p.q.n_states]; j++) {
-    const uint32_t l = p.q.in_label[j];
-    if (l >= p.L || (seen >> l) & 1u) continue;
-    seen |= 1ull << l;
-    m += p.label_edges[l];
-    n_labels++;
-  }
+  uint64_t m = 0, n_labels = 0;
+  for (uint64_t set = label_set(p), l = 0; l < p.L; l++)
+    if ((set >> l) & 1u) {
+      m += p.label_edges[l];
+      n_labels++;
+    }
   return n_labels ? m / n_labels : 0;
 }
 // Blocks of a traversal launch over n vertices with `edges` edges per label:

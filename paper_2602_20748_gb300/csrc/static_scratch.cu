@@ -189,14 +189,14 @@ extern "C" int run_rpq_static(rpq_ctx *ctx, const rpq_graph *g, const rpq_query 
   p.alpha = ctx_alpha(ctx);
   p.pull_dynamic = 1;
   p.lane_by_source = 1;
+  for (uint32_t l = 0; l < dg.L; l++) p.label_edges[l] = dg.label_edges[l];
+  p.time_limit_ns = ctx_time_limit_ns(ctx);
+  p.q = qd;
   // chunks of long in-rows belong to the graph: scanned in place, one lane
   // walked a row of up to 10^4 edges alone (64 start vertices on R-MAT 2^18:
   // 3.2 ms a call)
   const ShorterChunks shorter(ctx, g);
-  set_chunks(p, dg.chunks_in, dg.L, ns, shorter.there());
-  for (uint32_t l = 0; l < dg.L; l++) p.label_edges[l] = dg.label_edges[l];
-  p.time_limit_ns = ctx_time_limit_ns(ctx);
-  p.q = qd;
+  set_chunks(p, dg.chunks_in, ns, shorter.there());
   const int grid = bfs_grid(blocks, 1, 1, n, label_edges(p));
   p.nblocks = (unsigned)grid;
   STATIC_CK(launch_start(1, p, ns, small, lanesrc, src, st));

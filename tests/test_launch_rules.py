@@ -22,12 +22,39 @@ extern "C" int grid(int nw, unsigned groups, unsigned n, unsigned long long edge
 extern "C" int staged(int nw, unsigned groups, unsigned states, int by_source) {
   return rpq::lanes_staged(nw, groups, states, by_source != 0);
 }
+// Labels 0 and 1 with `longer` and `shorter` chunked rows each and `light` edges
+// in the others, a launch that takes label 0: 1 its longer rows are chunked, 2 its
+// shorter ones too, 4 its rows are walked.
+extern "C" int chunked(unsigned n, unsigned longer, unsigned shorter, unsigned light, unsigned groups,
+                       unsigned long long starts, int there, int lanes_staged) {
+  static unsigned rec[2];
+  rpq::ChunkLists c;
+  c.longer.rec = rec;
+  c.shorter.rec = rec + 1;
+  c.longer.off = {0, longer, 2 * longer};
+  c.shorter.off = {0, shorter, 2 * shorter};
+  c.light = {light, 100 * n};
+  rpq::BfsParams p{};
+  p.n = n;
+  p.L = 2;
+  p.G = groups;
+  p.q.n_states = 1;
+  p.q.in_begin[1] = 1;
+  p.q.in_label[0] = 0;
+  rpq::set_chunks(p, c, starts, there != 0, lanes_staged != 0);
+  const bool shorts = p.heavy_row == rpq::HEAVY_ROW;
+  if (shorts != (p.chunk_rec[1] != nullptr) || p.chunk_n[1][0] != (shorts ? shorter : 0) ||
+      p.chunk_n[0][0] != longer || (!shorts && p.heavy_row != rpq::LONG_ROW))
+    return -1;
+  return (p.chunk_rec[0] ? 1 : 0) | (shorts ? 2 : 0) | (p.walk_rows ? 4 : 0);
+}
 """)
     cuda = os.path.join(os.path.dirname(os.path.realpath(build._nvcc())), "..", "include")
     subprocess.run(["g++", "-std=c++17", "-shared", "-fPIC", f"-I{build.CSRC}", f"-I{build.INCLUDE}", f"-I{cuda}",
                     str(d / "rules.cpp"), "-o", str(d / "rules.so")], check=True)
     lib = ctypes.CDLL(str(d / "rules.so"))
     lib.grid.argtypes = [ctypes.c_int, ctypes.c_uint, ctypes.c_uint, ctypes.c_ulonglong]
+    lib.chunked.argtypes = [ctypes.c_uint] * 5 + [ctypes.c_ulonglong, ctypes.c_int, ctypes.c_int]
     return lib
 
 
@@ -46,3 +73,21 @@ def test_grid_grows_with_vertices_and_edges(rules, nw, groups, n):
 def test_staged_lane_levels_need_a_full_row_of_lanes(rules):
     assert [rules.staged(4, g, 8, 1) for g in (1, 4, 8, 9, 16)] == [0, 0, 0, 1, 1]
     assert not any((rules.staged(1, 16, 8, 1), rules.staged(4, 16, 9, 1), rules.staged(4, 16, 8, 0)))
+
+
+K, BIG = 1 << 15, 1 << 17
+
+
+@pytest.mark.parametrize("n,longer,shorter,light,groups,starts,there,want", [
+    (K, 3, 0, 0, 2, 100, 1, 3), (K, 3, K // 8, 0, 2, 100, 1, 3), (K, 3, K // 8 + 1, 0, 2, 100, 1, 5),
+    (K, 0, K - 9, 0, 16, 4096, 1, 5), (K - 8, 3, K // 2, 0, 2, 100, 1, 3), (K - 8, 3, K // 2, 0, 1, 100, 1, 5),
+    (K, 3, 50, 0, 1, 31, 1, 1), (K, 3, 50, 0, 1, 32, 1, 3), (K, 3, 50, 0, 2, 100, 0, 1), (K, 3, K, 0, 1, 1, 0, 5),
+    (BIG, 3, 50, 8 * BIG, 2, 300, 1, 3), (BIG, 3, 50, 8 * BIG + 1, 2, 300, 1, 7),
+    (BIG, 3, 50, 8 * BIG + 1, 4, 1000, 1, 7), (BIG, 3, 50, 16 * BIG, 5, 1200, 1, 3),
+    (BIG, 3, 50, 16 * BIG + 1, 16, 4096, 1, 7), (BIG - 8, 3, 50, 20 * BIG, 2, 300, 1, 3)])
+def test_rows_that_are_chunked_and_rows_that_are_walked(rules, n, longer, shorter, light, groups, starts, there, want):
+    assert rules.chunked(n, longer, shorter, light, groups, starts, there, 0) == want
+
+
+def test_staged_lane_levels_keep_the_chunks(rules):
+    assert rules.chunked(K, 3, K, 0, 12, 3000, 1, 1) == 3
