@@ -2143,12 +2143,18 @@ int msbfs_max_blocks(int nw, int threads, int *blocks_per_sm, int *sms) {
   int dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaError_t e;
   if (nw == 1)
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, msbfs_kernel<1, AM_ONE>, threads, 0);
-  else
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, msbfs_kernel<4, AM_ONE>, threads, 0);
-  return e == cudaSuccess ? 0 : -1;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, msbfs_kernel<1, AM_ONE>, threads, 0) ==
+                   cudaSuccess
+               ? 0
+               : -1;
+  // launch_msbfs takes either kernel: the grid has to fit both
+  int many = 0;
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, msbfs_kernel<4, AM_ONE>, threads, 0) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&many, msbfs_kernel<4, AM_MANY>, threads, 0) != cudaSuccess)
+    return -1;
+  *blocks_per_sm = std::min(*blocks_per_sm, many);
+  return 0;
 }
 
 cudaError_t preload_static_msbfs_kernels() {
