@@ -843,6 +843,18 @@ int berr(rpq_ctx *ctx, cudaError_t e, const char *what) {
   return ctx_error(ctx, RPQ_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
 }
 
+// Device memory for a launch of this engine.  The workspace that an earlier
+// multi-source evaluation left on the context may hold the room; nothing here
+// uses it, so it goes back first.
+int balloc(rpq_ctx *ctx, void **p, uint64_t bytes) {
+  int rc = ctx_alloc(ctx, p, bytes);
+  if (rc == RPQ_ERR_OUT_OF_BUDGET) {
+    ctx_release_workspace(ctx);
+    rc = ctx_alloc(ctx, p, bytes);
+  }
+  return rc;
+}
+
 template <typename T>
 struct DBuf {
   rpq_ctx *ctx = nullptr;
@@ -851,7 +863,7 @@ struct DBuf {
   int alloc(rpq_ctx *c, uint64_t count) {
     ctx = c;
     n = std::max<uint64_t>(count, 1);
-    return ctx_alloc(c, (void **)&p, n * sizeof(T));
+    return balloc(c, (void **)&p, n * sizeof(T));
   }
   T *release_ownership() {
     T *q = p;
@@ -1085,7 +1097,7 @@ static int batch_launch(rpq_ctx *ctx, const rpq_graph *g, uint32_t qbase, uint32
   out->dxor ^= hsmall[1];
   if (materialize && total) {
     u32 *rows = nullptr;
-    if ((rc = ctx_alloc(ctx, (void **)&rows, total * 8))) return rc;
+    if ((rc = balloc(ctx, (void **)&rows, total * 8))) return rc;
     ep.rows = rows;
     batch_emit<true><<<grid, BEMIT_WORDS, 0, st>>>(ep);
     if ((e = cudaGetLastError()) != cudaSuccess) {

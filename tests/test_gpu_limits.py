@@ -3,6 +3,8 @@
 import numpy as np
 import pytest
 
+from paper_2602_20748_gb300 import synth
+
 pytestmark = pytest.mark.gpu
 
 rpq = pytest.importorskip("paper_2602_20748_gb300.rpq")
@@ -141,3 +143,32 @@ def test_lists_given_back_while_other_contexts_read_them():
     finally:
         server.close()
     assert [summary(q, s, rpq.RPQ_COUNT_ONLY | f) for q in queries for s in lists for f in modes] + batch() == before
+
+
+def test_a_batch_is_accepted_again_after_its_lane_launches(monkeypatch):
+    """The workspace that the lane-mode launches of a batch leave does not stand
+    in the way of the next batch's shared launch."""
+    monkeypatch.setenv("RPQ_BATCH_LIST_CAP", str(1 << 24))  # 256 MiB of lists
+    n = 1 << 18
+    src, dst, lab = synth.rmat_graph(18, 4 << 18, 4, 1.2, seed=11)
+    regexes, sources = synth.batch_queries(512, 4, 1.2, src, n, seed=12)
+
+    def batches(budget, times):
+        c = rpq.Context(device=0, mem_budget_bytes=budget)
+        rpq.rpq_set_option(c, "batch_evict", 64)
+        try:
+            g = rpq.load_graph(c, n, 4, src, dst, lab)
+            qs = [rpq.compile_rpq(c, x) for x in regexes]
+            out = []
+            for _ in range(times):
+                r = rpq.run_rpq_batch(c, g, qs, sources, flags=rpq.RPQ_PER_QUERY)
+                out.append([rpq.result_query_stats(r, i) for i in range(len(qs))])
+                assert rpq.result_stats(r)["evicted"] > 64
+            return out
+        except rpq.RPQError as e:
+            assert e.code == rpq.RPQ_ERR_OUT_OF_BUDGET
+            return None
+
+    want = batches(8 << 30, 1)
+    low = smallest(lambda b: batches(b & ~0xFFFFF, 1) == want, 64 << 20, 2 << 30) & ~0xFFFFF
+    assert batches(low, 2) == want * 2
