@@ -692,7 +692,7 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
         std::fprintf(stderr, "[rpq trace]   level %2u %s n=%10llu mf=%12llu %9.3f ms (commit %7.3f ms)\n", l,
                      hctl.trace_mode[l] == 1 ? "push" : "pull", (unsigned long long)hctl.trace_n[l],
                      (unsigned long long)hctl.trace_mf[l], (hctl.trace_t[l + 1] - hctl.trace_t[l]) * 1e-6,
-                     hctl.trace_c[l] ? (hctl.trace_t[l + 1] - hctl.trace_c[l]) * 1e-6 : 0.0);
+                     hctl.trace_c[l] ? (uint32_t)((uint32_t)hctl.trace_t[l + 1] - hctl.trace_c[l]) * 1e-6 : 0.0);
     }
     ctx->stamp += (uint32_t)hctl.levels + 3;
 
@@ -2175,7 +2175,7 @@ static int lane_launch(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Lane
       std::fprintf(stderr, "[rpq trace]   level %2u %s n=%10llu mf=%12llu %9.3f ms (commit %7.3f ms)\n", l,
                    hctl.trace_mode[l] == 1 ? "push" : "pull", (unsigned long long)hctl.trace_n[l],
                    (unsigned long long)hctl.trace_mf[l], (hctl.trace_t[l + 1] - hctl.trace_t[l]) * 1e-6,
-                   hctl.trace_c[l] ? (hctl.trace_t[l + 1] - hctl.trace_c[l]) * 1e-6 : 0.0);
+                   hctl.trace_c[l] ? (uint32_t)((uint32_t)hctl.trace_t[l + 1] - hctl.trace_c[l]) * 1e-6 : 0.0);
   }
   if (stats) {
     float ms_bfs = 0, ms_emit = 0;

@@ -512,7 +512,7 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS, 2) batch_kernel(const __gri
       c->spill_cursor[old] = 0;
       if (level < (u32)TRACE_LEVELS) {
         c->trace_t[level] = globaltimer_ns();
-        c->trace_n[level] = n_cur;
+        c->trace_n[level] = (u32)min(n_cur, (u64)~0u);
         c->trace_mode[level] = 1;
       }
       push_levels++;
@@ -723,7 +723,7 @@ __global__ void __launch_bounds__(BATCH_MAX_THREADS) serve_kernel(const __grid_c
       c->spill_cursor[old] = 0;
       if (level < (u32)TRACE_LEVELS) {
         c->trace_t[level] = globaltimer_ns();
-        c->trace_n[level] = n_cur;
+        c->trace_n[level] = (u32)min(n_cur, (u64)~0u);
         c->trace_mode[level] = 1;
       }
     }

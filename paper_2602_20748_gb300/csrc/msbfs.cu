@@ -1939,7 +1939,7 @@ __global__ void __launch_bounds__(BFS_THREADS, BLOCKS) msbfs_kernel(const __grid
       c->smask[old] = 0;
       if (level < (u32)TRACE_LEVELS) {
         c->trace_t[level] = globaltimer_ns();
-        c->trace_n[level] = n_cur;
+        c->trace_n[level] = (u32)min(n_cur, (u64)~0u);
         c->trace_mode[level] = push ? 1 : 2;
         c->trace_mf[level] = mf;
       }
@@ -1996,7 +1996,7 @@ __global__ void __launch_bounds__(BFS_THREADS, BLOCKS) msbfs_kernel(const __grid
       const bool set_bits = p.fbits && n_next * 4 < sparse_cap && !pulled_lanes;
       const int clear_bits = !have_bits ? 0 : level == 0 || n_cur * 4 < sparse_cap ? 1 : 2;
       have_bits = p.fbits && (n_next * 4 < sparse_cap || pulled_lanes);
-      if (tracer && level < (u32)TRACE_LEVELS) c->trace_c[level] = globaltimer_ns();
+      if (tracer && level < (u32)TRACE_LEVELS) c->trace_c[level] = (u32)globaltimer_ns();
       commit_phase<NW, AM>(p, lp, nxt, n_cur, n_warps, set_bits, clear_bits, sums, stat);
       if (run) {
         __syncthreads();

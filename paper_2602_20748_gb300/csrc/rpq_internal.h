@@ -126,10 +126,10 @@ constexpr unsigned int APPEND_SEG = 128;             // list slots a warp reserv
 // on R-MAT 2^20: 550 us, 600 with 64).
 inline unsigned int append_seg(int nw) { return nw == 1 ? APPEND_SEG : APPEND_SEG / 2; }
 
-// The words that all blocks poll or add to lie 128 bytes and more apart, with
-// the trace, which one thread writes, between them: a line each, at the size of
-// the words alone.  The size counts: what run_rpq_static takes and the serving
-// slots that fit a budget depend on it.
+// The words that all blocks poll or add to, and that every level reads, have a
+// 128-byte line each (a trace entry written into the line of the barrier's flag
+// or of a counter cost the small calls 2-3%).  The size counts: what
+// run_rpq_static takes and the serving slots that fit a budget depend on it.
 struct BfsCtl {
   // grid barrier (grid_barrier.cuh): blocks that have arrived, over all
   // barriers; the last barrier completed << 1 | error
@@ -138,27 +138,31 @@ struct BfsCtl {
   unsigned int bar_flag;
   unsigned int err;
   unsigned int err_where;
-  unsigned int pad1;
-  // per-level trace (first TRACE_LEVELS levels): start time (ns), frontier
-  // entries and out-edges, start time (ns) of the commit phase, direction (1
-  // top-down, 2 bottom-up)
-  unsigned long long trace_c[TRACE_LEVELS];
+  unsigned int pad1[29];
   unsigned long long n_list[3];
-  unsigned long long trace_n[TRACE_LEVELS];
+  unsigned long long pad2[13];
   unsigned long long cursor[3];
-  unsigned long long trace_mf[TRACE_LEVELS];
+  unsigned long long pad3[13];
   unsigned long long mf[3];  // frontier out-edges
-  unsigned long long trace_t[TRACE_LEVELS + 1];
+  unsigned long long pad4[13];
   unsigned long long n_true[3];        // frontier entries without the lists' unused slots
   unsigned long long spill_count[3];   // top-down row chunks queued this level
   unsigned long long spill_cursor[3];
   unsigned long long heavy_cursor[3];  // bottom-up row chunks taken
-  unsigned char trace_mode[TRACE_LEVELS];
-  unsigned long long levels;
-  unsigned long long stats[ST_COUNT];
+  unsigned long long pad5[4];
   unsigned int smask[3];    // DFA states present in each frontier
   unsigned int next_level;  // first level after a run of one-block levels
-  unsigned int pad2[10];
+  unsigned long long levels;
+  unsigned long long stats[ST_COUNT];
+  unsigned long long pad6[12];
+  // per-level trace (first TRACE_LEVELS levels): start time (ns), frontier
+  // out-edges and entries (at most 2^32 - 1), start time of the commit phase (its
+  // low half), direction (1 top-down, 2 bottom-up)
+  unsigned long long trace_t[TRACE_LEVELS + 1];
+  unsigned long long trace_mf[TRACE_LEVELS];
+  unsigned int trace_n[TRACE_LEVELS];
+  unsigned int trace_c[TRACE_LEVELS];
+  unsigned char trace_mode[TRACE_LEVELS];
 };
 static_assert(sizeof(BfsCtl) == 2592, "see above");
 
