@@ -49,10 +49,11 @@ struct rpq_ctx {
   cudaMemPool_t pool = nullptr;  // the context's own pool: freed blocks stay reserved for reuse
   uint64_t budget = 0;
   uint64_t used = 0;
-  // chunk lists of shorter rows of this context's graphs: held while the budget
-  // has room beside everything else, so that what fits it does not depend on them
+  // chunks of shorter rows in the lists of this context's graphs: held while the
+  // budget has room beside everything else, so that what fits it does not depend
+  // on them
   uint64_t shorter_bytes = 0;
-  std::vector<rpq_graph *> graphs;  // whose lists these are
+  std::vector<rpq_graph *> graphs;  // whose chunks these are
   std::string err;
   Workspace ws;
   BfsCtl *ctl = nullptr;
@@ -91,7 +92,7 @@ struct rpq_graph {
   DevGraph g;
   uint64_t bytes = 0;
   uint64_t shorter_bytes = 0;
-  // evaluations on other contexts that read the lists of shorter rows
+  // evaluations on other contexts that read the chunk lists (see ChunkUse)
   mutable std::mutex mu;
   mutable std::condition_variable cv;
   mutable int users = 0;
@@ -151,25 +152,26 @@ int cuda_err(rpq_ctx *c, cudaError_t e, const char *what) {
     if (_e != cudaSuccess) return cuda_err(ctx, _e, #expr); \
   } while (0)
 
-// Frees the lists of shorter rows of one of ctx's graphs (see ShorterChunks):
-// waits for the other contexts' evaluations that read them; new ones go without.
+// The chunk lists of one of a context's graphs without the shorter rows: waits for
+// the other contexts' evaluations that read them; new ones wait for the new lists.
 void give_back_shorter(rpq_graph *g) {
   rpq_ctx *ctx = g->ctx;
+  ctx->shorter_bytes -= g->shorter_bytes;
+  g->shorter_bytes = 0;
+  ctx->graphs.erase(std::find(ctx->graphs.begin(), ctx->graphs.end(), g));
   {
     std::unique_lock<std::mutex> lk(g->mu);
     g->giving_back = true;
     g->cv.wait(lk, [&] { return g->users == 0; });
-    for (ChunkLists *c : {&g->g.chunks_in, &g->g.chunks_out}) {
-      if (c->shorter.rec) cudaFreeAsync(c->shorter.rec, ctx->stream);
-      c->shorter.rec = nullptr;
-    }
   }
-  ctx->shorter_bytes -= g->shorter_bytes;
-  g->shorter_bytes = 0;
-  ctx->graphs.erase(std::find(ctx->graphs.begin(), ctx->graphs.end(), g));
+  if (g->g.chunks_in.shorter) drop_shorter_chunks(g->g.in_off, g->g.n, g->g.L, &g->g.chunks_in, ctx->stream);
+  if (g->g.chunks_out.shorter) drop_shorter_chunks(g->g.out_off, g->g.n, g->g.L, &g->g.chunks_out, ctx->stream);
+  std::lock_guard<std::mutex> lk(g->mu);
+  g->giving_back = false;
+  g->cv.notify_all();
 }
 
-// Makes `bytes` more fit the budget beside the lists of shorter rows, or gives
+// Makes `bytes` more fit the budget beside the chunks of shorter rows, or gives
 // these back.
 void room_for(rpq_ctx *ctx, uint64_t bytes) {
   if (ctx->used + ctx->shorter_bytes + bytes <= ctx->budget) return;
@@ -457,7 +459,7 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
     if (q0_final) res->count += skipped;
   }
   const std::vector<uint32_t> &srcs = filter ? kept : srcs_in;
-  const ShorterChunks shorter(ctx, gr);
+  const ChunkUse use(ctx, gr);
   res->stats.lane_words = srcs.size() <= 64 ? 1 : 4;
   if (srcs.empty()) return RPQ_OK;
   const int nw = srcs.size() <= 64 ? 1 : 4;
@@ -535,7 +537,7 @@ int eval_rpq(rpq_ctx *ctx, const rpq_graph *gr, const rpq_query *qr, const std::
     p.time_limit_ns = ctx->time_limit_ns;
     p.q = qd;
     // bottom-up levels read the in-direction of the traversal
-    set_chunks(p, reverse ? g.chunks_out : g.chunks_in, live, shorter.there());
+    set_chunks(p, reverse ? g.chunks_out : g.chunks_in, live);
     const int grid = bfs_grid(blocks, nw, Gb, n, label_edges(p));
     p.nblocks = (unsigned)grid;
 
@@ -1056,11 +1058,12 @@ int load_graph(rpq_ctx *ctx, uint32_t n_vertices, uint32_t n_labels, uint64_t n_
     // the graph arrays were allocated inside build_graph outside the budget
     // accounting; account for them now
     const DevGraph &dg = gr->g;
-    uint64_t b = rows * 8 + dg.m * 8 +
-                 12ull * ((uint64_t)dg.chunks_in.longer.off.back() + dg.chunks_out.longer.off.back());
+    const uint64_t shorter = (uint64_t)dg.chunks_in.shorter + dg.chunks_out.shorter;
+    const uint64_t chunks = (uint64_t)dg.chunks_in.off.back() + dg.chunks_out.off.back();
+    uint64_t b = rows * 8 + dg.m * 8 + 12 * (chunks - shorter);
     ctx->used += b;
     gr->bytes = b;
-    gr->shorter_bytes = 12ull * ((uint64_t)dg.chunks_in.shorter.off.back() + dg.chunks_out.shorter.off.back());
+    gr->shorter_bytes = 12 * shorter;
     ctx->shorter_bytes += gr->shorter_bytes;
     ctx->graphs.push_back(gr);
   }
@@ -1102,7 +1105,11 @@ void free_graph(rpq_graph *g) {
   rpq_ctx *ctx = g->ctx;
   cudaSetDevice(ctx->device);
   cudaStream_t st = ctx->stream;
-  if (std::find(ctx->graphs.begin(), ctx->graphs.end(), g) != ctx->graphs.end()) give_back_shorter(g);
+  const auto at = std::find(ctx->graphs.begin(), ctx->graphs.end(), g);
+  if (at != ctx->graphs.end()) {
+    ctx->graphs.erase(at);
+    ctx->shorter_bytes -= g->shorter_bytes;
+  }
   free_graph_arrays(&g->g, st);
   ctx->used -= std::min(ctx->used, g->bytes);
   if (g->g.vlabel) dfree(ctx, g->g.vlabel, g->g.n);
@@ -1598,19 +1605,18 @@ void ctx_release_workspace(rpq_ctx *ctx) {
 }
 const DevGraph &graph_dev(const rpq_graph *g) { return g->g; }
 
-ShorterChunks::ShorterChunks(rpq_ctx *ctx, const rpq_graph *g) : ctx_(ctx), g_(g) {
-  if (ctx == g->ctx) return;  // one call at a time: only its own allocations free them
-  std::lock_guard<std::mutex> lk(g->mu);
-  held_ = !g->giving_back && g->g.chunks_in.shorter.rec;
-  if (held_) g->users++;
+ChunkUse::ChunkUse(rpq_ctx *ctx, const rpq_graph *g) : ctx_(ctx), g_(g) {
+  if (ctx == g->ctx) return;  // one call at a time: only its own allocations change them
+  std::unique_lock<std::mutex> lk(g->mu);
+  g->cv.wait(lk, [&] { return !g->giving_back; });
+  g->users++;
 }
-ShorterChunks::~ShorterChunks() {
-  if (!held_) return;
+ChunkUse::~ChunkUse() {
+  if (ctx_ == g_->ctx) return;
   cudaStreamSynchronize(ctx_->stream);  // an evaluation that failed may have left a launch running
   std::lock_guard<std::mutex> lk(g_->mu);
   if (--g_->users == 0) g_->cv.notify_all();
 }
-bool ShorterChunks::there() const { return ctx_ == g_->ctx ? g_->g.chunks_in.shorter.rec != nullptr : held_; }
 
 const HostQuery &query_host(const rpq_query *q) { return q->hq; }
 
@@ -1852,8 +1858,8 @@ int rpq_lane_stats_multi(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Mu
   p.lane_by_source = ctx->lane_by_source;
   p.time_limit_ns = ctx->time_limit_ns;
   p.q = un;
-  const ShorterChunks shorter(ctx, gr);
-  set_chunks(p, g.chunks_in, total_lanes, shorter.there());
+  const ChunkUse use(ctx, gr);
+  set_chunks(p, g.chunks_in, total_lanes);
   const int grid = bfs_grid(blocks, 1, G, n, label_edges(p));
   p.nblocks = (unsigned)grid;
   p.qg = d_desc;
@@ -2122,8 +2128,8 @@ static int lane_launch(rpq_ctx *ctx, const rpq_graph *gr, const std::vector<Lane
   p.lane_by_source = ctx->lane_by_source;
   p.time_limit_ns = ctx->time_limit_ns;
   p.q = un;
-  const ShorterChunks shorter(ctx, gr);
-  set_chunks(p, g.chunks_in, k, shorter.there(), staged);
+  const ChunkUse use(ctx, gr);
+  set_chunks(p, g.chunks_in, k, staged);
   const int grid = bfs_grid(blocks, nw, G, n, label_edges(p));
   p.nblocks = (unsigned)grid;
   if (kernel == LaneKernel::plain && grid <= ctx_sm_share(ctx) * bpsm[(int)LaneKernel::few]) kernel = LaneKernel::few;

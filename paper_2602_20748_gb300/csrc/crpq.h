@@ -68,23 +68,21 @@ void *ctx_static_scratch(rpq_ctx *ctx);
 void ctx_release_workspace(rpq_ctx *ctx);
 int static_scratch_prepare(void **addr, std::string *msg);
 const DevGraph &graph_dev(const rpq_graph *g);
-// The use of a graph's chunk lists of shorter rows by an evaluation on ctx: the
-// graph's own context gives them back when its budget needs the room, in its
-// stream's order; evaluations on other contexts keep them until they are done.
-class ShorterChunks {
+// An evaluation's use of a graph's chunk lists, which the graph's own context may
+// build again without the shorter rows when its budget needs their room: in its
+// stream's order for its own evaluations (which ask for the lists when they
+// allocate nothing more before a launch), and not while evaluations on other
+// contexts read them.
+class ChunkUse {
  public:
-  ShorterChunks(rpq_ctx *ctx, const rpq_graph *g);
-  ~ShorterChunks();
-  ShorterChunks(const ShorterChunks &) = delete;
-  ShorterChunks &operator=(const ShorterChunks &) = delete;
-  // Whether a launch that is issued next may read them (asked when no more
-  // memory is allocated before it).
-  bool there() const;
+  ChunkUse(rpq_ctx *ctx, const rpq_graph *g);
+  ~ChunkUse();
+  ChunkUse(const ChunkUse &) = delete;
+  ChunkUse &operator=(const ChunkUse &) = delete;
 
  private:
   rpq_ctx *ctx_;
   const rpq_graph *g_;
-  bool held_ = false;  // counted in the graph's users
 };
 const HostQuery &query_host(const rpq_query *q);
 int rpq_rows_for_sources(rpq_ctx *ctx, const rpq_graph *g, const rpq_query *q, std::vector<uint32_t> &srcs,

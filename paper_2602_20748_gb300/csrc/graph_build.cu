@@ -131,12 +131,12 @@ __global__ void label_bounds(const uint32_t *__restrict__ off, uint32_t n, uint3
 
 // Chunk lists of long rows, all labels at once (blockIdx.y = label): a list per
 // label and class, rows of at least LONG_ROW edges (class 0) and rows of
-// HEAVY_ROW .. LONG_ROW - 1 (class 1).  Without out0 and out1,
-// next[2 * label + class] counts the chunks and light[label] the edges in rows
-// below HEAVY_ROW; with them, next is the place of the list's next record
-// (vertex, first edge, end edge), taken a warp at a time.
+// HEAVY_ROW .. LONG_ROW - 1 (class 1).  Without out, next[2 * label + class]
+// counts the chunks and light[label] the edges in rows below HEAVY_ROW; with out,
+// next is the place of the list's next record (vertex, first edge, end edge),
+// taken a warp at a time, and classes from n_cls on are not listed.
 __global__ void row_chunks(const uint32_t *__restrict__ off, uint32_t n, u32 *__restrict__ next, u32 *__restrict__ light,
-                           uint32_t *__restrict__ out0, uint32_t *__restrict__ out1) {
+                           uint32_t *__restrict__ out, int n_cls) {
   const uint32_t *row = off + (u64)blockIdx.y * (n + 1);
   next += 2 * blockIdx.y;
   const u64 step = (u64)gridDim.x * blockDim.x;
@@ -145,7 +145,7 @@ __global__ void row_chunks(const uint32_t *__restrict__ off, uint32_t n, u32 *__
     const u64 v = v0 + lane_id();
     const uint32_t b = v < n ? row[v] : 0u, len = v < n ? row[v + 1] - b : 0u;
     if (len < HEAVY_ROW) few += len;
-    for (int cls = 0; cls < 2; cls++) {
+    for (int cls = 0; cls < n_cls; cls++) {
       const bool mine = cls == 0 ? len >= LONG_ROW : len >= HEAVY_ROW && len < LONG_ROW;
       if (!__any_sync(FULL_MASK, mine)) continue;
       const u32 k = mine ? (len + HCHUNK - 1) / HCHUNK : 0u;
@@ -158,7 +158,6 @@ __global__ void row_chunks(const uint32_t *__restrict__ off, uint32_t n, u32 *__
       u32 base = 0;
       if (lane_id() == 31) base = atomicAdd(&next[cls], at);
       base = __shfl_sync(FULL_MASK, base, 31) + at - k;
-      uint32_t *out = cls == 0 ? out0 : out1;
       if (out)
         for (u32 c = 0; c < k; c++) {
           const u64 r = 3ull * (base + c);
@@ -168,7 +167,7 @@ __global__ void row_chunks(const uint32_t *__restrict__ off, uint32_t n, u32 *__
         }
     }
   }
-  if (out0) return;
+  if (out) return;
   few = warp_sum(few);
   if (lane_id() == 0 && few) atomicAdd(&light[blockIdx.y], few);
 }
@@ -271,41 +270,68 @@ static int bits_for(uint64_t n) {
   return b;
 }
 
+// Allocates c->rec and writes the records of the classes below n_cls of the CSR
+// `off`, whose places c->off holds.
+static cudaError_t list_chunks(const uint32_t *off, uint32_t n, uint32_t L, ChunkLists *c, int n_cls, u32 *next,
+                               cudaStream_t st) {
+  cudaError_t e = cudaMallocAsync(&c->rec, 3 * (u64)std::max(1u, c->off[2 * L]) * 4, st);
+  if (e != cudaSuccess) c->rec = nullptr;
+  if (e == cudaSuccess) e = cudaMemcpyAsync(next, c->off.data(), 8ull * L, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) {
+    row_chunks<<<dim3((unsigned)std::min<u64>(grid_for(n, 256), 608), L), 256, 0, st>>>(off, n, next, nullptr, c->rec,
+                                                                                        n_cls);
+    e = cudaGetLastError();
+  }
+  return e;
+}
+
 // Chunk records of the long rows of every label of the CSR `off`.
-static cudaError_t build_chunks(const uint32_t *off, uint32_t n, uint32_t L, ChunkLists *lists, cudaStream_t st) {
+static cudaError_t build_chunks(const uint32_t *off, uint32_t n, uint32_t L, ChunkLists *c, cudaStream_t st) {
   u32 *next = nullptr;
-  ChunkList *cls[2] = {&lists->longer, &lists->shorter};
-  for (ChunkList *c : cls) c->off.assign(L + 1, 0);
+  c->off.assign(2 * L + 1, 0);
   std::vector<u32> cnt(3 * L, 0);
-  const dim3 grid((unsigned)std::min<u64>(grid_for(n, 256), 608), L);
   cudaError_t e = cudaMallocAsync(&next, 12ull * L, st);
   if (e == cudaSuccess) e = cudaMemsetAsync(next, 0, 12ull * L, st);
   if (e == cudaSuccess) {
-    row_chunks<<<grid, 256, 0, st>>>(off, n, next, next + 2 * L, nullptr, nullptr);
+    row_chunks<<<dim3((unsigned)std::min<u64>(grid_for(n, 256), 608), L), 256, 0, st>>>(off, n, next, next + 2 * L,
+                                                                                        nullptr, 2);
     e = cudaGetLastError();
   }
   if (e == cudaSuccess) e = cudaMemcpyAsync(cnt.data(), next, 12ull * L, cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  lists->light.assign(cnt.begin() + 2 * L, cnt.end());
-  for (int c = 0; c < 2 && e == cudaSuccess; c++) {
-    for (uint32_t l = 0; l < L; l++) {
-      cls[c]->off[l + 1] = cls[c]->off[l] + cnt[2 * l + c];
-      cnt[2 * l + c] = cls[c]->off[l];
-    }
-    e = cudaMallocAsync(&cls[c]->rec, 3 * (u64)std::max(1u, cls[c]->off[L]) * 4, st);
-  }
-  if (e == cudaSuccess) e = cudaMemcpyAsync(next, cnt.data(), 8ull * L, cudaMemcpyHostToDevice, st);
   if (e == cudaSuccess) {
-    row_chunks<<<grid, 256, 0, st>>>(off, n, next, nullptr, cls[0]->rec, cls[1]->rec);
-    e = cudaGetLastError();
+    c->light.assign(cnt.begin() + 2 * L, cnt.end());
+    c->shorter_rows.resize(L);
+    for (uint32_t i = 0; i < 2 * L; i++) c->off[i + 1] = c->off[i] + cnt[i];
+    for (uint32_t l = 0; l < L; l++) c->shorter += c->shorter_rows[l] = cnt[2 * l + 1];  // a chunk each
+    e = list_chunks(off, n, L, c, 2, next, st);
   }
   if (next) cudaFreeAsync(next, st);
   return e;
 }
 
+cudaError_t drop_shorter_chunks(const uint32_t *off, uint32_t n, uint32_t L, ChunkLists *c, cudaStream_t st) {
+  std::vector<uint32_t> longer(2 * L + 1, 0);
+  for (uint32_t l = 0; l < L; l++) longer[2 * l + 1] = longer[2 * l + 2] = longer[2 * l] + c->off[2 * l + 1] - c->off[2 * l];
+  c->off = longer;
+  c->shorter = 0;
+  cudaFreeAsync(c->rec, st);  // first: the new list is no larger than what it leaves
+  c->rec = nullptr;
+  u32 *next = nullptr;
+  cudaError_t e = cudaMallocAsync(&next, 8ull * L, st);
+  if (e == cudaSuccess) e = list_chunks(off, n, L, c, 1, next, st);
+  if (next) cudaFreeAsync(next, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);  // `longer` is read by the copy, and other streams read the list
+  if (e != cudaSuccess) {  // no list: every row is read whole
+    if (c->rec) cudaFreeAsync(c->rec, st);
+    c->rec = nullptr;
+    c->off.assign(2 * L + 1, 0);
+  }
+  return e;
+}
+
 void free_graph_arrays(DevGraph *g, cudaStream_t st) {
-  for (uint32_t **p : {&g->out_off, &g->in_off, &g->out_col, &g->in_col, &g->chunks_in.longer.rec,
-                       &g->chunks_in.shorter.rec, &g->chunks_out.longer.rec, &g->chunks_out.shorter.rec}) {
+  for (uint32_t **p : {&g->out_off, &g->in_off, &g->out_col, &g->in_col, &g->chunks_in.rec, &g->chunks_out.rec}) {
     if (*p) cudaFreeAsync(*p, st);
     *p = nullptr;
   }

@@ -135,14 +135,6 @@ __device__ __forceinline__ const QueryDesc &gdesc(const BfsParams &p, u32 g) {
     return p.q;
 }
 
-// Label l's chunks of long in-rows: their number, and the record (vertex, first
-// edge, end edge) of the k-th, those of the longer rows first.
-__device__ __forceinline__ u32 chunk_count(const BfsParams &p, u32 l) { return p.chunk_n[0][l] + p.chunk_n[1][l]; }
-__device__ __forceinline__ const u32 *chunk_rec(const BfsParams &p, u32 l, u32 k) {
-  const u32 n0 = p.chunk_n[0][l];
-  return k < n0 ? p.chunk_rec[0] + 3ull * (p.chunk_beg[0][l] + k) : p.chunk_rec[1] + 3ull * (p.chunk_beg[1][l] + k - n0);
-}
-
 // Out-degree of v summed over the labels leaving DFA state q; *rows (if
 // given) gets the number of those labels present in the graph.
 __device__ __forceinline__ u32 degsum(const BfsParams &p, const QueryDesc &qd, u32 q, u32 v, u32 *rows = nullptr) {
@@ -767,6 +759,7 @@ __device__ void pull_staged(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 ac
   // out-degree
   __shared__ uint4 s_vertex[BFS_THREADS / 32][32];
   uint4 *vertex = s_vertex[threadIdx.x >> 5];
+  const bool chunked = p.hchunk != nullptr;
   const u64 gword = 8ull * NW * p.G;  // bytes of the G words of one (state, vertex)
   u64 W = 0, mf = 0;
   u32 N = 0, gv = 0, gx = 0, states = 0;
@@ -776,59 +769,61 @@ __device__ void pull_staged(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 ac
   // Long in-rows first (the light rows' shorter items then fill the phase's
   // end): their precomputed chunks, a warp per (target state, transition
   // group, chunk), the sub-warps sharing the list.
-  for (u64 it = grid_warp();; it = next_item(&p.ctl->heavy_cursor[cur], grid_warps(), 1)) {
-    u64 acc_base = 0;
-    const u32 *rec = nullptr;
-    u32 q2 = 0, from = 0;
-    bool found = false;
-    for (u32 q = 0; q < Q && !found; q++)
-      for (u32 j = p.q.in_begin[q]; j < p.q.in_begin[q + 1]; j++) {
-        const u32 l = p.q.in_label[j];
-        if (!(p.q.in_from[j] & active) || l >= p.L) continue;
-        const u64 cnt = chunk_count(p, l);
-        if (it < acc_base + cnt) {
-          found = true;
-          q2 = q;
-          from = p.q.in_from[j] & active;
-          rec = chunk_rec(p, l, (u32)(it - acc_base));
-          break;
-        }
-        acc_base += cnt;
-      }
-    if (!found) break;
-    const u32 w = __ldg(rec), beg = __ldg(rec + 1), len = __ldg(rec + 2) - beg;
-    u64 vis[2], acc[2] = {0, 0};
-    load_vis<2>(p.vis + ((u64)q2 * n + w) * wpv + lane_off, lane_on, vis);
-    if (__all_sync(FULL_MASK, (vis[0] & vis[1]) == ~0ull)) continue;
-    for (u32 fb = from; fb; fb &= fb - 1) {
-      const u64 qb = (u64)(__ffs(fb) - 1) * n;
-      for (u32 e0 = 0; e0 < len; e0 += STAGE) {
-        u32 cnt = 0;
-        __syncwarp();  // the previous list is consumed
-        for (u32 k = e0; k < min(len, e0 + STAGE); k += 32) {
-          u64 row = 0;
-          bool in = k + lane < len;
-          if (in) {
-            row = qb + __ldg(p.in_col + beg + k + lane);
-            if (bits) in = (__ldcg(bits + (row >> 5)) >> (row & 31)) & 1u;
+  if (chunked) {
+    for (u64 it = grid_warp();; it = next_item(&p.ctl->heavy_cursor[cur], grid_warps(), 1)) {
+      u64 acc_base = 0, ci = 0;
+      u32 q2 = 0, from = 0;
+      bool found = false;
+      for (u32 q = 0; q < Q && !found; q++)
+        for (u32 j = p.q.in_begin[q]; j < p.q.in_begin[q + 1]; j++) {
+          const u32 l = p.q.in_label[j];
+          if (!(p.q.in_from[j] & active) || l >= p.L) continue;
+          const u64 cnt = p.hchunk_end[l] - p.hchunk_beg[l];
+          if (it < acc_base + cnt) {
+            found = true;
+            q2 = q;
+            from = p.q.in_from[j] & active;
+            ci = p.hchunk_beg[l] + (it - acc_base);
+            break;
           }
-          const u32 b = __ballot_sync(FULL_MASK, in);
-          if (in) lst[cnt + __popc(b & lanemask_lt())] = row;
-          cnt += __popc(b);
+          acc_base += cnt;
         }
-        __syncwarp();
-        gather_list<6>(F, wpv, lane_off, lst, sg, VPW, lane_on ? cnt : 0, acc);
-        stat_add(stat, ST_ALG_BYTES, cnt * gword);
+      if (!found) break;
+      const u32 *rec = p.hchunk + 3 * ci;
+      const u32 w = __ldg(rec), beg = __ldg(rec + 1), len = __ldg(rec + 2) - beg;
+      u64 vis[2], acc[2] = {0, 0};
+      load_vis<2>(p.vis + ((u64)q2 * n + w) * wpv + lane_off, lane_on, vis);
+      if (__all_sync(FULL_MASK, (vis[0] & vis[1]) == ~0ull)) continue;
+      for (u32 fb = from; fb; fb &= fb - 1) {
+        const u64 qb = (u64)(__ffs(fb) - 1) * n;
+        for (u32 e0 = 0; e0 < len; e0 += STAGE) {
+          u32 cnt = 0;
+          __syncwarp();  // the previous list is consumed
+          for (u32 k = e0; k < min(len, e0 + STAGE); k += 32) {
+            u64 row = 0;
+            bool in = k + lane < len;
+            if (in) {
+              row = qb + __ldg(p.in_col + beg + k + lane);
+              if (bits) in = (__ldcg(bits + (row >> 5)) >> (row & 31)) & 1u;
+            }
+            const u32 b = __ballot_sync(FULL_MASK, in);
+            if (in) lst[cnt + __popc(b & lanemask_lt())] = row;
+            cnt += __popc(b);
+          }
+          __syncwarp();
+          gather_list<6>(F, wpv, lane_off, lst, sg, VPW, lane_on ? cnt : 0, acc);
+          stat_add(stat, ST_ALG_BYTES, cnt * gword);
+        }
       }
+      for (u32 o = SW; o < 32; o <<= 1) {
+        acc[0] |= __shfl_xor_sync(FULL_MASK, acc[0], o);
+        acc[1] |= __shfl_xor_sync(FULL_MASK, acc[1], o);
+      }
+      stat_add(stat, ST_PULL_EDGES, len);
+      stat_add(stat, ST_PULL_VERTICES, 1);
+      stat_add(stat, ST_ALG_BYTES, gword + len * (bits ? 8 : 4));
+      pull_finish<NW, 2>(p, app, FB, nlist, nxt, q2, w, stamp, li, lane_on && sg == 0, my_g, true, vis, acc);
     }
-    for (u32 o = SW; o < 32; o <<= 1) {
-      acc[0] |= __shfl_xor_sync(FULL_MASK, acc[0], o);
-      acc[1] |= __shfl_xor_sync(FULL_MASK, acc[1], o);
-    }
-    stat_add(stat, ST_PULL_EDGES, len);
-    stat_add(stat, ST_PULL_VERTICES, 1);
-    stat_add(stat, ST_ALG_BYTES, gword + len * (bits ? 8 : 4));
-    pull_finish<NW, 2>(p, app, FB, nlist, nxt, q2, w, stamp, li, lane_on && sg == 0, my_g, true, vis, acc);
   }
 
   u32 cv = 32;  // vertices a warp takes at a time (see pull_level)
@@ -848,7 +843,7 @@ __device__ void pull_staged(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 ac
           if (!from || l >= p.L) continue;
           const u32 *off = p.in_off + (u64)l * n1 + v;
           const u32 len = __ldg(off + 1) - __ldg(off);
-          if (len >= p.heavy_row)
+          if (len >= p.heavy_row && chunked)
             shared = true;
           else
             lens += len, tot += len * __popc(from);
@@ -894,7 +889,7 @@ __device__ void pull_staged(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 ac
               if (!from || l >= p.L) continue;
               const u32 *off = p.in_off + (u64)l * n1 + (u32)(c0 + o);
               const u32 beg = __ldg(off), len = __ldg(off + 1) - beg;
-              if (len >= p.heavy_row) continue;
+              if (len >= p.heavy_row && chunked) continue;
               const u32 np = __popc(from);
               if (r < len * np) {
                 col = beg + (np == 1 ? r : r / np);
@@ -1046,6 +1041,7 @@ __device__ void pull_lanes(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
   const u64 wpv = (u64)p.G * NW, gword = 8ull * NW * p.G;
   ulonglong2 *sacc = reinterpret_cast<ulonglong2 *>(scratch) + lane;  // target q2's words at sacc[32 * q2]
   u64 *lst = scratch + LANE_SRC_Q * 2 * 32;                           // [LANE_LIST]
+  const bool chunked = p.hchunk != nullptr;
   u32 *nbits = p.fbits ? p.fbits + (lp ? 0 : p.fbits_words) : nullptr;  // the next frontier's bitmap
   Appender app;
   app.seg = (u64)n * Q * p.G >= grid_warps() * 2 * APPEND_SEG ? p.append_seg : min(p.append_seg, 32u);
@@ -1136,46 +1132,48 @@ __device__ void pull_lanes(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
 
   // Long in-rows first, an item per (label, chunk): the chunk's rows of each
   // active source state are ORed together and masked once.
-  for (u64 it = grid_warp();; it = next_item(&p.ctl->heavy_cursor[cur], grid_warps(), 1)) {
-    u64 acc_base = 0;
-    const u32 *rec = nullptr;
-    u32 l = 0;
-    bool found = false;
-    for (u64 lb = lset; lb && !found; lb &= lb - 1) {
-      l = __ffsll((long long)lb) - 1;
-      const u64 cnt = chunk_count(p, l);
-      found = it < acc_base + cnt;
-      if (found) rec = chunk_rec(p, l, (u32)(it - acc_base));
-      acc_base += cnt;
-    }
-    if (!found) break;
-    const u32 w = __ldg(rec), beg = __ldg(rec + 1), len = __ldg(rec + 2) - beg;
-    for (u32 sm = tab.act[l]; sm; sm &= sm - 1) {
-      const u32 st = __ffs(sm) - 1;
-      u64 g[2] = {0, 0};
-      for (u32 e0 = 0; e0 < len; e0 += LANE_LIST) {
-        u32 cnt = 0;
-        __syncwarp();  // the previous list is consumed
-        for (u32 k = e0; k < min(len, e0 + LANE_LIST); k += 32) {
-          u64 row = 0;
-          bool in = k + lane < len;
-          if (in) {
-            row = (u64)st * n + __ldg(p.in_col + beg + k + lane);
-            if (bits) in = (__ldcg(bits + (row >> 5)) >> (row & 31)) & 1u;
-          }
-          const u32 b = __ballot_sync(FULL_MASK, in);
-          if (in) lst[cnt + __popc(b & lanemask_lt())] = row;
-          cnt += __popc(b);
-        }
-        __syncwarp();
-        gather_list<8>(F, wpv, lane_off, lst, 0, 1, lane_on ? cnt : 0, g);
-        stat_add(stat, ST_ALG_BYTES, cnt * gword);
+  if (chunked) {
+    for (u64 it = grid_warp();; it = next_item(&p.ctl->heavy_cursor[cur], grid_warps(), 1)) {
+      u64 acc_base = 0, ci = 0;
+      u32 l = 0;
+      bool found = false;
+      for (u64 lb = lset; lb && !found; lb &= lb - 1) {
+        l = __ffsll((long long)lb) - 1;
+        const u64 cnt = p.hchunk_end[l] - p.hchunk_beg[l];
+        found = it < acc_base + cnt;
+        if (found) ci = p.hchunk_beg[l] + (it - acc_base);
+        acc_base += cnt;
       }
-      if (__any_sync(FULL_MASK, (g[0] | g[1]) != 0)) apply(l * LANE_SRC_Q + st, make_ulonglong2(g[0], g[1]));
+      if (!found) break;
+      const u32 *rec = p.hchunk + 3 * ci;
+      const u32 w = __ldg(rec), beg = __ldg(rec + 1), len = __ldg(rec + 2) - beg;
+      for (u32 sm = tab.act[l]; sm; sm &= sm - 1) {
+        const u32 st = __ffs(sm) - 1;
+        u64 g[2] = {0, 0};
+        for (u32 e0 = 0; e0 < len; e0 += LANE_LIST) {
+          u32 cnt = 0;
+          __syncwarp();  // the previous list is consumed
+          for (u32 k = e0; k < min(len, e0 + LANE_LIST); k += 32) {
+            u64 row = 0;
+            bool in = k + lane < len;
+            if (in) {
+              row = (u64)st * n + __ldg(p.in_col + beg + k + lane);
+              if (bits) in = (__ldcg(bits + (row >> 5)) >> (row & 31)) & 1u;
+            }
+            const u32 b = __ballot_sync(FULL_MASK, in);
+            if (in) lst[cnt + __popc(b & lanemask_lt())] = row;
+            cnt += __popc(b);
+          }
+          __syncwarp();
+          gather_list<8>(F, wpv, lane_off, lst, 0, 1, lane_on ? cnt : 0, g);
+          stat_add(stat, ST_ALG_BYTES, cnt * gword);
+        }
+        if (__any_sync(FULL_MASK, (g[0] | g[1]) != 0)) apply(l * LANE_SRC_Q + st, make_ulonglong2(g[0], g[1]));
+      }
+      stat_add(stat, ST_PULL_EDGES, len);
+      stat_add(stat, ST_ALG_BYTES, len * 4);
+      if (tmask) flush(w, true);
     }
-    stat_add(stat, ST_PULL_EDGES, len);
-    stat_add(stat, ST_ALG_BYTES, len * 4);
-    if (tmask) flush(w, true);
   }
 
   u32 cv = 32;  // vertices a warp takes at a time (see pull_level)
@@ -1189,7 +1187,7 @@ __device__ void pull_lanes(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
       for (u64 lb = lset; lb; lb &= lb - 1) {
         const u32 *off = p.in_off + (u64)(__ffsll((long long)lb) - 1) * n1 + c0 + lane;
         const u32 len = __ldg(off + 1) - __ldg(off);
-        if (len >= p.heavy_row)
+        if (len >= p.heavy_row && chunked)
           sh = true;
         else
           tot += len;
@@ -1222,7 +1220,7 @@ __device__ void pull_lanes(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
           l = __ffsll((long long)lb) - 1;
           const u32 *off = p.in_off + (u64)l * n1 + c0 + o;
           const u32 beg = __ldg(off), len = __ldg(off + 1) - beg;
-          if (len >= p.heavy_row) continue;
+          if (len >= p.heavy_row && chunked) continue;
           if (r < len) {
             u = __ldg(p.in_col + beg + r);
             sm = tab.act[l];
@@ -1351,6 +1349,7 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
   // at once) on graphs too small to give every warp two such chunks
   u32 cv = 32;
   while (cv > VPW && n < 2 * n_warps * cv) cv >>= 1;
+  const bool chunked = p.hchunk != nullptr;
   const u64 gword = 8ull * NW * p.G;  // bytes of the G words of one (state, vertex)
   u64 edges = 0, words = 0, bytes = 0;
   Appender app;
@@ -1385,7 +1384,7 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
           if (!from || l >= p.L) continue;
           const u32 *off = p.in_off + (u64)l * n1 + v;
           const u32 beg = __ldg(off), len = __ldg(off + 1) - beg;
-          if (len >= p.heavy_row) {
+          if (len >= p.heavy_row && chunked) {
             hmask |= 1u << q2;
             continue;
           }
@@ -1460,7 +1459,7 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
           const u32 l = __ffsll((long long)lset) - 1;
           const u32 *off = p.in_off + (u64)l * n1 + w;
           const u32 beg = __ldg(off), end = __ldg(off + 1);
-          if (beg == end || end - beg >= p.heavy_row) continue;
+          if (beg == end || (end - beg >= p.heavy_row && chunked)) continue;
           u32 S = 0;  // source states of those transitions on label l
           for (u32 q2 = 0; q2 < Q; q2++)
             if ((wmask >> q2) & 1u)
@@ -1522,7 +1521,7 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
           if (!from || l >= p.L) continue;
           const u32 *off = p.in_off + (u64)l * n1 + w;
           const u32 beg = __ldg(off), end = __ldg(off + 1);
-          if (end - beg >= p.heavy_row) continue;
+          if (end - beg >= p.heavy_row && chunked) continue;
           for (u32 i = beg + li; i < end && !hit; i += SW) {
             const u32 u = __ldg(p.in_col + i);
             bytes += 4 + 4 * __popc(from);
@@ -1548,7 +1547,7 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
           if (!from || l >= p.L) continue;
           const u32 *off = p.in_off + (u64)l * n1 + w;
           const u32 beg = __ldg(off), end = __ldg(off + 1);
-          if (end - beg >= p.heavy_row) continue;
+          if (end - beg >= p.heavy_row && chunked) continue;
           // in multi mode each lane gathers through its own group's transitions
           u32 lfrom = from;
           if constexpr (AM == AM_GROUP) lfrom = lane_on ? p.from_tab[((u64)my_g * Q + q2) * p.L + l] & active : 0u;
@@ -1586,9 +1585,9 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
       c0 += n_warps * cv;
   }
 
-  bool chunks_done = false;
+  bool chunks_done = !chunked;
   if constexpr (AM == AM_LANE) {
-    if (p.lane_by_source && Q <= LANE_SRC_Q) {
+    if (chunked && p.lane_by_source && Q <= LANE_SRC_Q) {
       // Long in-rows by source state: an item is a chunk of a label's long
       // in-rows; its frontier words are gathered once per active source
       // state with a transition on that label and masked into every target
@@ -1597,22 +1596,22 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
       for (u32 j = 0; j < p.q.in_begin[Q]; j++)
         if ((p.q.in_from[j] & active) && p.q.in_label[j] < p.L) lact |= 1ull << p.q.in_label[j];
       for (u64 it = warp;; it = next_item(&p.ctl->heavy_cursor[cur], n_warps, 1)) {
-        u64 acc_base = 0;
-        const u32 *rec = nullptr;
+        u64 acc_base = 0, ci = 0;
         u32 ls = 0;
         bool found = false;
         for (u64 lb = lact; lb; lb &= lb - 1) {
           const u32 l = __ffsll((long long)lb) - 1;
-          const u64 cnt = chunk_count(p, l);
+          const u64 cnt = p.hchunk_end[l] - p.hchunk_beg[l];
           if (it < acc_base + cnt) {
             found = true;
             ls = l;
-            rec = chunk_rec(p, l, (u32)(it - acc_base));
+            ci = p.hchunk_beg[l] + (it - acc_base);
             break;
           }
           acc_base += cnt;
         }
         if (!found) break;
+        const u32 *rec = p.hchunk + 3 * ci;
         const u32 w = __ldg(rec), beg = __ldg(rec + 1), end = __ldg(rec + 2);
         // targets with a transition on ls from an active state and lanes not
         // yet visited (the whole warp works on vertex w)
@@ -1686,27 +1685,27 @@ __device__ void pull_level(const BfsParams &p, int lp, u32 cur, u32 nxt, u32 act
   if (!chunks_done) {
     for (u64 it = warp;; it = next_item(&p.ctl->heavy_cursor[cur], n_warps, 1)) {
       // map the item number to (target state, transition group, chunk)
-      u64 acc_base = 0;
-      const u32 *rec = nullptr;
+      u64 acc_base = 0, ci = 0;
       u32 q2s = 0, from = 0, ls = 0, js = 0;
       bool found = false;
       for (u32 q2 = 0; q2 < Q && !found; q2++)
         for (u32 j = p.q.in_begin[q2]; j < p.q.in_begin[q2 + 1]; j++) {
           const u32 l = p.q.in_label[j];
           if (!(p.q.in_from[j] & active) || l >= p.L) continue;
-          const u64 cnt = chunk_count(p, l);
+          const u64 cnt = p.hchunk_end[l] - p.hchunk_beg[l];
           if (it < acc_base + cnt) {
             found = true;
             q2s = q2;
             ls = l;
             js = j;
             from = p.q.in_from[j] & active;
-            rec = chunk_rec(p, l, (u32)(it - acc_base));
+            ci = p.hchunk_beg[l] + (it - acc_base);
             break;
           }
           acc_base += cnt;
         }
       if (!found) break;
+      const u32 *rec = p.hchunk + 3 * ci;
       const u32 w = __ldg(rec), beg = __ldg(rec + 1), end = __ldg(rec + 2);
       const u64 base = ((u64)q2s * n + w) * wpv + lane_off;
       u64 vis[PER];

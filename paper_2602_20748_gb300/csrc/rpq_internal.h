@@ -69,16 +69,19 @@ constexpr uint32_t LONG_ROW = 128;
 constexpr uint32_t FEW_STARTS = 32;  // fewer start vertices than this chunk LONG_ROW rows only
 constexpr uint32_t HCHUNK = 256;
 
-// The chunks of one class of rows, grouped by label: label l's are [off[l],
-// off[l + 1]) (host copy of the L + 1 offsets).
-struct ChunkList {
+// Chunks (vertex, first edge, end edge) of one direction's rows with at least
+// HEAVY_ROW edges, grouped by label and class: label l's chunks of rows of
+// LONG_ROW edges and more are [off[2 l], off[2 l + 1]), those of shorter rows
+// follow up to off[2 l + 2] (host copy of the 2 L + 1 offsets).  One list, so that
+// a launch finds a record with one base and one offset (a list per class made
+// configuration 2 1.2% slower); where the budget needs the room of the shorter
+// rows' chunks it is built again without them.
+struct ChunkLists {
   uint32_t *rec = nullptr;
   std::vector<uint32_t> off;
-};
-struct ChunkLists {
-  ChunkList longer;   // rows of LONG_ROW edges and more
-  ChunkList shorter;  // HEAVY_ROW .. LONG_ROW - 1 edges; given back when the budget needs the room
   std::vector<uint32_t> light;  // per label, the edges in rows below HEAVY_ROW
+  uint32_t shorter = 0;         // chunks of the shorter rows in the list
+  std::vector<uint32_t> shorter_rows;  // per label, the rows of the second class (listed or not)
 };
 
 struct DevGraph {
@@ -90,9 +93,6 @@ struct DevGraph {
   uint32_t *in_off = nullptr;
   uint32_t *in_col = nullptr;
   uint8_t *vlabel = nullptr;
-  // Chunks (vertex, first edge, end edge) of the rows with >= HEAVY_ROW
-  // edges, per direction: of the rows of LONG_ROW edges and more, and of the
-  // shorter ones.
   ChunkLists chunks_in, chunks_out;
   std::vector<uint8_t> vlabel_host;   // vertex labels (host copy), empty if none
   std::vector<uint64_t> label_edges;  // edges per label (host copy)
@@ -179,11 +179,9 @@ struct BfsParams {
   const uint32_t *out_col;
   const uint32_t *in_off;
   const uint32_t *in_col;
-  // chunks of the in_off rows of at least heavy_row edges: per label and
-  // class (longer rows, shorter rows) their records and number
-  const uint32_t *chunk_rec[2];
-  uint32_t chunk_beg[2][RPQ_MAX_LABELS];
-  uint32_t chunk_n[2][RPQ_MAX_LABELS];
+  const uint32_t *hchunk;               // chunks of long in_off rows (nullptr: the list could not be built again)
+  uint32_t hchunk_beg[RPQ_MAX_LABELS];  // per label, the chunks of rows of
+  uint32_t hchunk_end[RPQ_MAX_LABELS];  // at least heavy_row edges
   uint32_t heavy_row;
   bool walk_rows;  // several lane groups: bottom-up levels walk each row (see set_chunks)
   unsigned long long label_edges[RPQ_MAX_LABELS];
@@ -262,9 +260,8 @@ inline uint64_t label_set(const BfsParams &p) {
     if (p.q.in_label[j] < p.L) set |= 1ull << p.q.in_label[j];
   return set;
 }
-// The chunk lists of a launch of `starts` start vertices (shorter: the graph
-// still has its lists of shorter rows), and how launches of several lane groups
-// read the other rows bottom-up.
+// The chunks of a launch of `starts` start vertices, and how launches of several
+// lane groups read the other rows bottom-up.
 //
 // Where rows of 32 to 127 edges are the ordinary ones, more than one vertex in
 // eight over the launch's labels, they stay whole: an item per row costs more
@@ -289,26 +286,23 @@ inline uint64_t label_set(const BfsParams &p) {
 // list rows anyhow (3,000 lanes on 128,000 vertices of degree 50 per label: 54 ms
 // by chunks, 68 without).
 constexpr uint32_t WHOLE_MIN = 1u << 15, WALK_MIN = 1u << 17;
-inline void set_chunks(BfsParams &p, const ChunkLists &c, uint64_t starts, bool shorter, bool lanes_staged = false) {
+inline void set_chunks(BfsParams &p, const ChunkLists &c, uint64_t starts, bool lanes_staged = false) {
   const uint64_t labels = label_set(p);
   uint64_t rows = 0, light = 0, vertices = 0;  // over the labels
   for (uint32_t l = 0; l < p.L; l++)
     if ((labels >> l) & 1u) {
-      rows += c.shorter.off[l + 1] - c.shorter.off[l];
+      rows += c.shorter_rows[l];
       light += c.light[l];
       vertices += p.n;
     }
   const bool whole = rows * 8 > vertices && (p.G == 1 || p.n >= WHOLE_MIN) && !lanes_staged;
-  p.walk_rows = whole || (p.n >= WALK_MIN && light > vertices * (p.G <= 4 ? 8 : 16));
-  shorter = shorter && starts >= FEW_STARTS && !whole;
+  p.walk_rows = whole || !c.rec || (p.n >= WALK_MIN && light > vertices * (p.G <= 4 ? 8 : 16));
+  const bool shorter = c.shorter > 0 && starts >= FEW_STARTS && !whole;
+  p.hchunk = c.rec;
   p.heavy_row = shorter ? HEAVY_ROW : LONG_ROW;
-  p.chunk_rec[0] = c.longer.rec;
-  p.chunk_rec[1] = shorter ? c.shorter.rec : nullptr;
   for (uint32_t l = 0; l < p.L; l++) {
-    p.chunk_beg[0][l] = c.longer.off[l];
-    p.chunk_n[0][l] = c.longer.off[l + 1] - c.longer.off[l];
-    p.chunk_beg[1][l] = shorter ? c.shorter.off[l] : 0;
-    p.chunk_n[1][l] = shorter ? c.shorter.off[l + 1] - c.shorter.off[l] : 0;
+    p.hchunk_beg[l] = c.off[2 * l];
+    p.hchunk_end[l] = c.off[2 * l + (shorter ? 2 : 1)];
   }
 }
 
@@ -476,6 +470,9 @@ cudaError_t launch_chunk_triples(const uint32_t *lanesrc, const unsigned long lo
 int build_graph(DevGraph *g, uint32_t n, uint32_t L, uint64_t m, const uint32_t *d_src, const uint32_t *d_dst,
                 const uint16_t *d_lab, cudaStream_t st, std::string *msg);
 void free_graph_arrays(DevGraph *g, cudaStream_t st);  // all but vlabel
+// Builds the list of the CSR `off` again without the shorter rows (see
+// ChunkLists); the other streams that read the old one are done.
+cudaError_t drop_shorter_chunks(const uint32_t *off, uint32_t n, uint32_t L, ChunkLists *c, cudaStream_t st);
 int graph_key_bits(uint32_t n, uint32_t L);
 
 // Stable LSD radix sort of 64-bit keys over bits [lo_bit, hi_bit); the result

@@ -195,8 +195,8 @@ extern "C" int run_rpq_static(rpq_ctx *ctx, const rpq_graph *g, const rpq_query 
   // chunks of long in-rows belong to the graph: scanned in place, one lane
   // walked a row of up to 10^4 edges alone (64 start vertices on R-MAT 2^18:
   // 3.2 ms a call)
-  const ShorterChunks shorter(ctx, g);
-  set_chunks(p, dg.chunks_in, ns, shorter.there());
+  const ChunkUse use(ctx, g);
+  set_chunks(p, dg.chunks_in, ns);
   const int grid = bfs_grid(blocks, 1, 1, n, label_edges(p));
   p.nblocks = (unsigned)grid;
   STATIC_CK(launch_start(1, p, ns, small, lanesrc, src, st));

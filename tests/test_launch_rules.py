@@ -27,13 +27,14 @@ extern "C" int staged(int nw, unsigned groups, unsigned states, int by_source) {
 // shorter ones too, 4 its rows are walked.
 extern "C" int chunked(unsigned n, unsigned longer, unsigned shorter, unsigned light, unsigned groups,
                        unsigned long long starts, int there, int lanes_staged) {
-  static unsigned rec[2];
+  static unsigned rec;
   rpq::ChunkLists c;
-  c.longer.rec = rec;
-  c.shorter.rec = rec + 1;
-  c.longer.off = {0, longer, 2 * longer};
-  c.shorter.off = {0, shorter, 2 * shorter};
+  c.rec = &rec;
+  c.shorter = there ? 2 * shorter : 0;
+  const unsigned listed = there ? shorter : 0;
+  c.off = {0, longer, longer + listed, 2 * longer + listed, 2 * longer + 2 * listed};
   c.light = {light, 100 * n};
+  c.shorter_rows = {shorter, shorter};
   rpq::BfsParams p{};
   p.n = n;
   p.L = 2;
@@ -41,12 +42,15 @@ extern "C" int chunked(unsigned n, unsigned longer, unsigned shorter, unsigned l
   p.q.n_states = 1;
   p.q.in_begin[1] = 1;
   p.q.in_label[0] = 0;
-  rpq::set_chunks(p, c, starts, there != 0, lanes_staged != 0);
-  const bool shorts = p.heavy_row == rpq::HEAVY_ROW;
-  if (shorts != (p.chunk_rec[1] != nullptr) || p.chunk_n[1][0] != (shorts ? shorter : 0) ||
-      p.chunk_n[0][0] != longer || (!shorts && p.heavy_row != rpq::LONG_ROW))
+  rpq::set_chunks(p, c, starts, lanes_staged != 0);
+  const bool shorts = p.heavy_row == rpq::HEAVY_ROW, walk = p.walk_rows;
+  if (p.hchunk != &rec || p.hchunk_beg[0] != 0 || p.hchunk_end[0] != longer + (shorts ? shorter : 0) ||
+      p.hchunk_beg[1] != longer + listed || (!shorts && p.heavy_row != rpq::LONG_ROW))
     return -1;
-  return (p.chunk_rec[0] ? 1 : 0) | (shorts ? 2 : 0) | (p.walk_rows ? 4 : 0);
+  c.rec = nullptr;
+  rpq::set_chunks(p, c, starts, lanes_staged != 0);
+  if (p.hchunk || !p.walk_rows) return -2;
+  return 1 | (shorts ? 2 : 0) | (walk ? 4 : 0);
 }
 """)
     cuda = os.path.join(os.path.dirname(os.path.realpath(build._nvcc())), "..", "include")
@@ -79,7 +83,7 @@ K, BIG = 1 << 15, 1 << 17
 
 
 @pytest.mark.parametrize("n,longer,shorter,light,groups,starts,there,want", [
-    (K, 3, 0, 0, 2, 100, 1, 3), (K, 3, K // 8, 0, 2, 100, 1, 3), (K, 3, K // 8 + 1, 0, 2, 100, 1, 5),
+    (K, 3, 0, 0, 2, 100, 1, 1), (K, 3, 1, 0, 2, 100, 1, 3), (K, 3, K // 8, 0, 2, 100, 1, 3), (K, 3, K // 8 + 1, 0, 2, 100, 1, 5),
     (K, 0, K - 9, 0, 16, 4096, 1, 5), (K - 8, 3, K // 2, 0, 2, 100, 1, 3), (K - 8, 3, K // 2, 0, 1, 100, 1, 5),
     (K, 3, 50, 0, 1, 31, 1, 1), (K, 3, 50, 0, 1, 32, 1, 3), (K, 3, 50, 0, 2, 100, 0, 1), (K, 3, K, 0, 1, 1, 0, 5),
     (BIG, 3, 50, 8 * BIG, 2, 300, 1, 3), (BIG, 3, 50, 8 * BIG + 1, 2, 300, 1, 7),
