@@ -140,7 +140,9 @@ __global__ void row_chunks(const uint32_t *__restrict__ off, uint32_t n, u32 *__
   const uint32_t *row = off + (u64)blockIdx.y * (n + 1);
   next += 2 * blockIdx.y;
   const u64 step = (u64)gridDim.x * blockDim.x;
+  __shared__ u32 s_few;
   u32 few = 0;
+  if (threadIdx.x == 0) s_few = 0;
   for (u64 v0 = (u64)blockIdx.x * blockDim.x + (threadIdx.x & ~31u); v0 < n; v0 += step) {
     const u64 v = v0 + lane_id();
     const uint32_t b = v < n ? row[v] : 0u, len = v < n ? row[v + 1] - b : 0u;
@@ -168,8 +170,11 @@ __global__ void row_chunks(const uint32_t *__restrict__ off, uint32_t n, u32 *__
     }
   }
   if (out) return;
+  __syncthreads();
   few = warp_sum(few);
-  if (lane_id() == 0 && few) atomicAdd(&light[blockIdx.y], few);
+  if (lane_id() == 0) atomicAdd(&s_few, few);
+  __syncthreads();
+  if (threadIdx.x == 0 && s_few) atomicAdd(&light[blockIdx.y], s_few);
 }
 
 // (label | src | dst) -> (label | dst | src)
