@@ -7,7 +7,7 @@
 // (DFA state, vertex) pairs -- one bit each, Q_i * |V| bits -- and all
 // queries advance together, level by level, in one cooperative kernel over a
 // shared frontier list of (query, state, vertex) entries.  A level is
-// expanded top-down: a warp takes 32 entries, spreads the out-edges of their
+// expanded top-down: a warp takes up to 32 entries, spreads the out-edges of their
 // transition rows evenly over its lanes, and test-and-sets the target bits
 // (a plain read first, the atomic only when the bit is clear); long rows are
 // cut into chunks shared by all warps (spill_chunk).  Results are the
